@@ -119,7 +119,7 @@ enum {
   CKV_KERNEL_COMBINE = 2,       /* normalised scores summed over queries, then pooled */
   CKV_KERNEL_SELECT = 3,        /* pooling + top-k + window append */
   CKV_KERNEL_GATHER = 4,        /* retained K/V rows -> compressed cache */
-  CKV_KERNEL_FUSED = 5          /* all four steps for every unit of a call, one persistent kernel */
+  CKV_KERNEL_FUSED = 5          /* all four steps for every unit of a call (persistent kernels) */
 };
 
 /* Optional launch trace.  When ckv_problem.trace is non-null every kernel
@@ -234,22 +234,32 @@ int compresskv_compress_layer(const ckv_problem* p, const void* q_win, const voi
  * then covers all the layers' units, so the scoring kernel's start-up and
  * tail are paid once.
  * Under CKV_SELECT_PER_GROUP every step of every unit (scoring, normalising
- * and pooling, top-k, window, gather) runs in one persistent kernel
- * (CKV_KERNEL_FUSED): one CTA per SM streams K from the first layer to the
- * last while other warps of the same CTAs merge, select and gather the units
- * whose scores are complete.  It reads K twice per chunk of 16 tiles of 128
- * keys: a first pass sums each query row's exponentials (softmax statistics
- * of the chunk), and once every chunk of the unit is in and the row's
- * denominator merged, a second pass sums the normalised probabilities of
- * each key (Eq. 1-2) in fp32 from K read again (for long calls mostly from
- * DRAM: the step then moves about twice the bytes of K); no exponent table
- * is stored.  The chunk grid is fixed per unit and every chunk's statistics
- * restart, so the scores depend only on the unit itself: compressing a layer
- * alone or among others gives the same bits.  That kernel takes windows W
- * that are multiples of 16, query strides that are multiples of 8 elements,
- * at most 32 query heads per group and SRH lists of at most 192 query rows
- * (|S_g| W: two Q buffers of them beside a ring of two K tiles fill its
- * shared memory); other per-group problems use the separate kernels.
+ * and pooling, top-k, window, gather) runs in one of two persistent kernels
+ * (both traced as CKV_KERNEL_FUSED): one CTA per SM streams K from the first
+ * layer to the last while other warps of the same CTAs select and gather the
+ * units whose scores are complete.
+ * A layer with short prompts takes the resident kernel, which reads K once:
+ * a unit's K tiles are spread over all SMs, their logits stay in tensor
+ * memory while the query rows' sums of exponentials are added up over the
+ * SMs, and the normalised probabilities of each key (Eq. 1-2) are then summed
+ * in fp32 from the same logits.  "Short": the layer's longest prompt has at
+ * most 32768 tokens when its widest group has at most 32 query rows (|S_g| W;
+ * 16384 with the LSE given), 16384 at 64 rows, 8192 at 128, 4096 at 192.
+ * Other layers take the two-pass kernel, which reads K twice per chunk of 16
+ * tiles of 128 keys: a first pass sums each query row's exponentials (softmax
+ * statistics of the chunk), and once every chunk of the unit is in and the
+ * row's denominator merged, a second pass sums the normalised probabilities
+ * from K read again (for long calls mostly from DRAM: the step then moves
+ * about twice the bytes of K).  A call with layers of both kinds launches
+ * both kernels, one after the other.
+ * Neither stores exponentials.  The kernel and the grid of chunks follow
+ * from the layer alone, and neither kernel's scores depend on the order in
+ * which chunks complete: compressing a layer alone or among others gives the
+ * same bits.  The kernels take windows W that are multiples of 16, query
+ * strides that are multiples of 8 elements, at most 32 query heads per group
+ * and SRH lists of at most 192 query rows (two Q buffers of them beside a
+ * ring of two K tiles fill the shared memory); other per-group problems use
+ * the separate kernels.  The resident kernel is a cooperative launch.
  * n_masks: 1 <= n_masks, dividing batch (else CKV_ERR_INVALID_ARG); at most
  *   256 under CKV_SELECT_PER_GROUP and 4 under CKV_SELECT_PER_LAYER (or when
  *   the separate kernels run) (else CKV_ERR_UNSUPPORTED).
@@ -351,8 +361,8 @@ int compresskv_compress_layer_noalloc(const ckv_problem* p, const void* q_win, c
  * CKV_OK (or CKV_ERR_CUDA if the copy fails). */
 int compresskv_read_device_status(const void* workspace, void* stream, int32_t* status);
 
-/* Test hook for the failure path of the persistent per-group kernel
- * (CKV_KERNEL_FUSED): the next call that launches it runs with every bounded
+/* Test hook for the failure path of the persistent per-group kernels
+ * (CKV_KERNEL_FUSED): the next call that launches one runs with every bounded
  * wait limited to wait_ns (instead of 2 s), and its first CTA's claimer
  * first waits for a counter that nothing sets -- before any copy or UMMA is
  * issued -- so the wait runs out: the call stops every CTA, its device status

@@ -96,6 +96,7 @@ int device_facts(DeviceFacts** out) {
     f.smem_optin = optin;
     if (score_set_smem_limit(static_cast<size_t>(optin)) != cudaSuccess) return CKV_ERR_CUDA;
     if (fused_set_smem_limit(static_cast<size_t>(optin)) != cudaSuccess) return CKV_ERR_CUDA;
+    if (resident_set_smem_limit(static_cast<size_t>(optin)) != cudaSuccess) return CKV_ERR_CUDA;
     if (combine_set_smem_limit(static_cast<size_t>(optin), &f.combine_smem_max) != cudaSuccess)
       return CKV_ERR_CUDA;
     if (select_set_smem_limit(static_cast<size_t>(select_max_smem_floats()) * 4) != cudaSuccess)
@@ -328,14 +329,40 @@ FusedLayout fused_layout(const Info& I) {
   return F;
 }
 
-// Max pooling: after both layouts, one raw-score row per SRH head slot (at
+// Layout of the resident call's workspace (it aliases the ones above).
+struct ResidentLayout {
+  size_t raw, pooled, acc, pairs, ctr, total;
+};
+
+ResidentLayout resident_layout(const Info& I) {
+  ResidentLayout F;
+  const size_t rows = static_cast<size_t>((std::min(I.G * I.W, kResidentMaxRows) + 31) & ~31);
+  const size_t units = static_cast<size_t>(I.B) * I.Hkv;
+  const size_t scores = align256(static_cast<size_t>(I.Hkv) * I.p_total * sizeof(float));
+  F.raw = kHeaderBytes;
+  F.pooled = F.raw + scores;
+  F.acc = F.pooled + scores;
+  F.pairs = F.acc + align256(units * kAccWords * rows * 8);
+  F.ctr = F.pairs + align256(static_cast<size_t>(kResidentMaxGrid) * kPairRing * rows * sizeof(float2));
+  F.total = F.ctr + align256(2 * units * sizeof(int));
+  return F;
+}
+
+// The layouts alias one another; selection across groups (with average
+// pooling) does not run the resident kernel.
+size_t base_bytes(const Info& I) {
+  const size_t base = std::max(workspace_layout(I).total, fused_layout(I).total);
+  return I.layer && !I.pool_max ? base : std::max(base, resident_layout(I).total);
+}
+
+// Max pooling: after these layouts, one raw-score row per SRH head slot (at
 // most G) of every group.
 size_t maxpool_slots_offset(const Info& I) {
-  return align256(std::max(workspace_layout(I).total, fused_layout(I).total));
+  return align256(base_bytes(I));
 }
 
 size_t workspace_bytes(const Info& I) {
-  const size_t base = std::max(workspace_layout(I).total, fused_layout(I).total);
+  const size_t base = base_bytes(I);
   if (!I.pool_max) return base;
   return maxpool_slots_offset(I) +
          align256(static_cast<size_t>(I.G) * I.Hkv * I.p_total * sizeof(float));
@@ -891,11 +918,98 @@ int run_gather(const ckv_problem* p, const Info& I, const int32_t* indices,
   return traced(tr, CKV_KERNEL_GATHER, [&] { return launch_gather(P, rows, stream); });
 }
 
-// Per-group selection of a (multi-layer) fused call in one persistent kernel
-// (fused_kernel.cu).  Sets *handled = false, enqueueing nothing, when the
-// problem is outside what that kernel takes (the caller then uses the
-// scoring / combine / selection kernels).  `lse` given: the window queries'
-// log-sum-exp replaces the first pass.
+// Which of the two persistent kernels a layer takes: the resident one
+// (resident_kernel.cu: K read once, the logits kept in tensor memory until
+// the softmax sums are complete) for short prompts, else the two-pass one
+// (fused_kernel.cu).  The lines are by the layer's longest prompt and the query
+// rows of its widest group, and by nothing else of the call, so that a layer
+// gives the same bits alone or among others; a call with layers of both kinds
+// launches both.  (The prompts of one layer go together: taking a 28-layer
+// batch's shorter prompts apart cost two tails, 3195 -> 3285 us.)  Two-pass / resident time in us (1 layer; 32 layers; 8 KV heads):
+//   32 rows      16384: 85/67, 568/319    32768: 98/90, 699/586
+//                65536: 128/135
+//   32, LSE      16384: 66/65, 348/277    24576: 71/75, 381/395
+//   64 rows      16384: 1.2 to 1.8 times faster    32768: 0.91 to 1.2
+//   128 rows      8192: 1.6, 1.22 times            16384: 0.63 (32 layers)
+//   192 rows      4096: 2.5, 1.5 times              8192: 0.78 (32 layers)
+// The resident kernel loses on long prompts because a unit's logits must all
+// be on the chip at once: beyond a few tiles per SM the chunks of different
+// units no longer overlap.
+constexpr int kResidentMinGrid = 32;  // CTAs that hold a unit of every admitted size
+static_assert(kResidentMaxRows <= kMaxQRows, "resident rows");
+
+bool takes_resident(int rows, int len, bool given_lse) {
+  if (rows <= 32) return len <= (given_lse ? 16384 : 32768);
+  if (rows <= 64) return len <= 16384;
+  if (rows <= 128) return len <= 8192;
+  return rows <= kResidentMaxRows && len <= 4096;
+}
+
+// K tiles per chunk of a resident sequence: up to four (what a chunk costs
+// beside its tiles is then small); fewer where a unit has few tiles (they
+// then reach more SMs) or its layer has wide groups (the tensor memory must
+// hold two chunks).  At most 32 chunks a unit (64 of 32 rows, of which the
+// tensor memory holds four): kResidentMinGrid CTAs hold any.
+int resident_chunk_tiles(int rows, int len) {
+  const int tiles = (len + kTileTokens - 1) / kTileTokens;
+  const int most = rows <= 64 ? kResidentChunkTiles : (rows <= 128 ? 2 : 1);
+  return std::min(most, tiles <= 32 ? 1 : (tiles <= 64 ? 2 : 4));
+}
+
+// What the two persistent kernels' parameters have in common.
+template <class Params>
+void fill_common(Params& P, const ckv_problem* p, const Info& I, const SrhLists& S,
+                 const std::vector<int>& co, int32_t* indices, const void* k, const void* v,
+                 void* k_out, void* v_out, const LseInput& lse, bool do_select) {
+  P.lse = lse.lse;
+  P.lse_bs = lse.batch_stride;
+  P.lse_hs = lse.head_stride;
+  P.given_lse = lse.lse ? 1 : 0;
+  P.k = static_cast<const uint4*>(k);
+  P.v = static_cast<const uint4*>(v);
+  P.k_out = static_cast<uint4*>(k_out);
+  P.v_out = static_cast<uint4*>(v_out);
+  P.tok_stride_v16 = p->kv_token_stride / 8;
+  P.head_stride_v16 = p->kv_head_stride / 8;
+  P.indices = indices;
+  {
+    const long long stall = g_stall_next_ns.exchange(0);
+    P.wait_ns = stall > 0 ? static_cast<unsigned long long>(stall) : kWaitTimeoutNs;
+    P.stall = stall > 0 ? 1 : 0;
+  }
+  P.c = static_cast<float>(static_cast<double>(I.scale) * 1.4426950408889634);
+  P.window = I.W;
+  P.pool_width = I.P;
+  P.num_kv_heads = I.Hkv;
+  P.group_size = I.G;
+  P.p_total = static_cast<int>(I.p_total);
+  P.o_total = co[I.B];
+  P.is_bf16 = I.bf16 ? 1 : 0;
+  P.n_units = I.B * I.Hkv;
+  P.batch = I.B;
+  P.do_select = do_select ? 1 : 0;
+  P.chunk_off[0] = 0;
+  for (int s = 0; s <= I.B; ++s) {
+    P.cu_seqlens[s] = I.cu[s];
+    P.cu_prefix[s] = I.cu_prefix[s];
+    P.cu_out[s] = co[s];
+  }
+  P.seqs_per_mask = I.spm;
+  for (int m = 0; m < I.n_masks; ++m) {
+    for (int g = 0; g < I.Hkv; ++g) {
+      const int v_ = m * I.Hkv + g;
+      uint32_t bits = 0u;
+      for (int j = S.off[v_]; j < S.off[v_ + 1]; ++j) bits |= 1u << (S.heads[j] - g * I.G);
+      P.srh_bits[v_] = bits;
+    }
+  }
+}
+
+// Per-group selection of a (multi-layer) fused call in the persistent kernels
+// (fused_kernel.cu, resident_kernel.cu).  Sets *handled = false, enqueueing
+// nothing, when the problem is outside what they take (the caller then uses
+// the scoring / combine / selection kernels).  `lse` given: the window
+// queries' log-sum-exp replaces the first pass.
 int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void* q_win,
               const void* k, const void* v, const std::vector<int>& co, int32_t* indices,
               void* k_out, void* v_out, float* raw_user, float* pooled_user, void* ws,
@@ -911,18 +1025,49 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
       p->q_win_stride <= 0 || p->q_head_stride <= 0 ||
       (I.B > 1 && (p->q_batch_stride % 8 != 0 || p->q_batch_stride <= 0)))
     return CKV_OK;
-  int max_rows = 16;
-  for (int v_ = 0; v_ < I.n_masks * I.Hkv; ++v_) max_rows = std::max(max_rows, S.rows[v_]);
+  DeviceFacts* Fd = nullptr;
+  int rc = device_facts(&Fd);
+  if (rc != CKV_OK) return rc;
+  // the kernel of every layer (mask), and the query rows of each kernel's
+  // widest group
+  const int r_grid = std::min(Fd->sms, kResidentMaxGrid);
+  std::vector<int> seq_rows(I.B, 0);
+  std::vector<uint8_t> in_resident(I.B, 0);
+  int max_rows = 16, r_rows = 16, n_resident = 0;
+  for (int s0 = 0; s0 < I.B; s0 += I.spm) {
+    int rows = 0, longest = 0;
+    for (int g = 0; g < I.Hkv; ++g) rows = std::max(rows, S.rows[I.vgroup(s0, g)]);
+    for (int s_ = s0; s_ < s0 + I.spm; ++s_) longest = std::max(longest, I.len[s_]);
+    const bool res =
+        r_grid >= kResidentMinGrid && takes_resident(rows, longest, lse.lse != nullptr);
+    int& most = res ? r_rows : max_rows;
+    most = std::max(most, rows);
+    if (res) n_resident += I.spm;
+    for (int s_ = s0; s_ < s0 + I.spm; ++s_) {
+      seq_rows[s_] = rows;
+      in_resident[s_] = res ? 1 : 0;
+    }
+  }
+  auto half_bytes = [](int rows) { return ((((rows + 15) & ~15) * 128) + 1023) & ~1023; };
+  // resident: three Q buffers beside four to eight K tiles, else two beside
+  // at least two
+  const int r_half = half_bytes(r_rows);
+  const int acc_rows = (r_rows + 31) & ~31;
+  int r_stages = 0, r_bufs = 0;
+  for (int nq = 3; nq >= 2 && r_stages == 0; --nq)
+    for (int st = 8; st >= (nq == 3 ? 4 : 2) && r_stages == 0; --st)
+      if (resident_smem_bytes(r_half, nq, st, acc_rows) <= static_cast<size_t>(Fd->smem_optin)) {
+        r_stages = st;
+        r_bufs = nq;
+      }
+  if (r_stages == 0) return CKV_ERR_CUDA;  // cannot happen on sm_103: kResidentMaxRows fit
   const int npad_max = (max_rows + 15) & ~15;
-  const int q_half = ((npad_max * 128) + 1023) & ~1023;
+  const int q_half = half_bytes(max_rows);
   const int row_stride = (max_rows + 31) & ~31;
   // TMEM: 512 columns of accumulator buffers, tstride columns each
   const int tstride = npad_max <= 64 ? 64 : (npad_max <= 128 ? 128 : 256);
   const int nwg = 2;  // epilogue warpgroups that take tiles
   const int nbuf = 512 / tstride;
-  DeviceFacts* Fd = nullptr;
-  int rc = device_facts(&Fd);
-  if (rc != CKV_OK) return rc;
   // three Q buffers when they fit beside a ring of at least four K tiles,
   // else two beside at least two; an even number of stages (each UMMA warp
   // has half of them)
@@ -946,70 +1091,62 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
     return CKV_ERR_WORKSPACE;
   char* wb = static_cast<char*>(ws);
 
+  Tracer tr{p->trace, stream};
+  if (n_resident > 0) {
+    const ResidentLayout RL = resident_layout(I);
+    static thread_local ResidentParams P;  // large (about 13 KB): kept off the stack
+    std::memset(&P, 0, sizeof(P));
+    if ((rc = make_k_map(I, p, k, &P.tmap_k)) != CKV_OK) return rc;
+    if ((rc = make_q_map(I, p, q_win, &P.tmap_q)) != CKV_OK) return rc;
+    fill_common(P, p, I, S, co, indices, k, v, k_out, v_out, lse, do_select);
+    P.raw = raw_user ? raw_user : reinterpret_cast<float*>(wb + RL.raw);
+    P.raw_scratch = raw_user ? 0 : 1;
+    P.pooled = pooled_user ? pooled_user : reinterpret_cast<float*>(wb + RL.pooled);
+    P.status = reinterpret_cast<int*>(wb);
+    P.ctr = reinterpret_cast<int*>(wb + kFusedCtrOffset);
+    P.unit_ctr = reinterpret_cast<int*>(wb + RL.ctr);
+    P.acc = reinterpret_cast<unsigned long long*>(wb + RL.acc);
+    P.acc_rows = acc_rows;
+    P.pairs = reinterpret_cast<float2*>(wb + RL.pairs);
+    long long out = 0;  // rows of the sequences this launch selects
+    for (int s_ = 0; s_ < I.B; ++s_) {
+      const int ct = in_resident[s_] ? resident_chunk_tiles(seq_rows[s_], I.len[s_]) : 0;
+      const int tiles = I.n[s_] > 0 ? (I.len[s_] + kTileTokens - 1) / kTileTokens : 0;
+      P.seq_chunk[s_] = static_cast<uint8_t>(ct);
+      P.chunk_off[s_ + 1] = P.chunk_off[s_] + (ct ? I.Hkv * ((tiles + ct - 1) / ct) : 0);
+      if (ct) out += co[s_ + 1] - co[s_];
+    }
+    P.n_chunks = P.chunk_off[I.B];
+    P.q_half_bytes = r_half;
+    P.q_bufs = r_bufs;
+    P.stages = r_stages;
+    const size_t smem = resident_smem_bytes(r_half, r_bufs, r_stages, acc_rows);
+    if (P.n_units > 0 && (P.n_chunks > 0 || (do_select && out > 0)))
+      rc = traced(tr, CKV_KERNEL_FUSED, [&] { return launch_resident(P, r_grid, smem, stream); });
+    if (rc != CKV_OK || n_resident == I.B) return rc;
+  }
+
   static thread_local FusedParams P;  // large (about 15 KB): kept off the stack
   std::memset(&P, 0, sizeof(P));
   if ((rc = make_k_map(I, p, k, &P.tmap_k)) != CKV_OK) return rc;
   if ((rc = make_q_map(I, p, q_win, &P.tmap_q)) != CKV_OK) return rc;
-  P.q = static_cast<const uint16_t*>(q_win);
-  P.q_bs = p->q_batch_stride;
-  P.q_hs = p->q_head_stride;
-  P.q_ws = p->q_win_stride;
-  P.lse = lse.lse;
-  P.lse_bs = lse.batch_stride;
-  P.lse_hs = lse.head_stride;
-  P.given_lse = lse.lse ? 1 : 0;
-  P.k = static_cast<const uint4*>(k);
-  P.v = static_cast<const uint4*>(v);
-  P.k_out = static_cast<uint4*>(k_out);
-  P.v_out = static_cast<uint4*>(v_out);
-  P.tok_stride_v16 = p->kv_token_stride / 8;
-  P.head_stride_v16 = p->kv_head_stride / 8;
-  P.indices = indices;
+  fill_common(P, p, I, S, co, indices, k, v, k_out, v_out, lse, do_select);
   P.raw = raw_user ? raw_user : reinterpret_cast<float*>(wb + FL.raw);
   P.raw_scratch = raw_user ? 0 : 1;
-  {
-    const long long stall = g_stall_next_ns.exchange(0);
-    P.wait_ns = stall > 0 ? static_cast<unsigned long long>(stall) : kWaitTimeoutNs;
-    P.stall = stall > 0 ? 1 : 0;
-  }
   P.pooled = pooled_user ? pooled_user : reinterpret_cast<float*>(wb + FL.pooled);
   P.status = reinterpret_cast<int*>(wb);
   P.ctr = reinterpret_cast<int*>(wb + kFusedCtrOffset);
   P.partials = reinterpret_cast<float2*>(wb + FL.partials);
   P.bias = reinterpret_cast<float*>(wb + FL.bias);
   P.part_stride = FL.part_stride;
-  P.c = static_cast<float>(static_cast<double>(I.scale) * 1.4426950408889634);
-  P.window = I.W;
-  P.pool_width = I.P;
-  P.num_kv_heads = I.Hkv;
-  P.group_size = I.G;
-  P.p_total = static_cast<int>(I.p_total);
-  P.o_total = co[I.B];
-  P.is_bf16 = I.bf16 ? 1 : 0;
-  P.n_units = I.B * I.Hkv;
-  P.batch = I.B;
-  P.do_select = do_select ? 1 : 0;
-  P.chunk_off[0] = 0;
+  long long out = 0;  // rows of the sequences this launch selects
   for (int s_ = 0; s_ < I.B; ++s_) {
-    P.cu_seqlens[s_] = I.cu[s_];
-    P.cu_prefix[s_] = I.cu_prefix[s_];
-    P.cu_out[s_] = co[s_];
-    P.chunk_off[s_ + 1] = P.chunk_off[s_] + I.Hkv * chunks_per_unit(I, s_);
+    const int chunks = in_resident[s_] ? 0 : I.Hkv * chunks_per_unit(I, s_);
+    P.chunk_off[s_ + 1] = P.chunk_off[s_] + chunks;
+    if (!in_resident[s_]) out += co[s_ + 1] - co[s_];
   }
-  P.cu_seqlens[I.B] = I.cu[I.B];
-  P.cu_prefix[I.B] = I.cu_prefix[I.B];
-  P.cu_out[I.B] = co[I.B];
   P.n_chunks = P.chunk_off[I.B];
-  if (P.n_chunks != FL.n_chunks) return CKV_ERR_WORKSPACE;  // cannot happen: same plan
-  P.seqs_per_mask = I.spm;
-  for (int m = 0; m < I.n_masks; ++m) {
-    for (int g = 0; g < I.Hkv; ++g) {
-      const int v_ = m * I.Hkv + g;
-      uint32_t bits = 0u;
-      for (int j = S.off[v_]; j < S.off[v_ + 1]; ++j) bits |= 1u << (S.heads[j] - g * I.G);
-      P.srh_bits[v_] = bits;
-    }
-  }
+  if (P.n_chunks > FL.n_chunks) return CKV_ERR_WORKSPACE;  // cannot happen: same plan
   P.q_half_bytes = q_half;
   P.q_bufs = q_bufs;
   P.row_stride = row_stride;
@@ -1017,9 +1154,8 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   P.tstride = tstride;
   P.nbuf = nbuf;
   P.nwg = nwg;
-  if (P.n_units == 0 || (P.n_chunks == 0 && (!do_select || co[I.B] == 0))) return CKV_OK;
+  if (P.n_units == 0 || (P.n_chunks == 0 && (!do_select || out == 0))) return CKV_OK;
   const size_t smem = fused_smem_bytes(q_half, q_bufs, stages, row_stride, nwg);
-  Tracer tr{p->trace, stream};
   return traced(tr, CKV_KERNEL_FUSED, [&] { return launch_fused(P, Fd->sms, smem, stream); });
 }
 

@@ -202,7 +202,9 @@ struct FusedParams {
   int cu_seqlens[kFusedMaxSeqs + 1];
   int cu_prefix[kFusedMaxSeqs + 1];
   int cu_out[kFusedMaxSeqs + 1];
-  int chunk_off[kFusedMaxSeqs + 1];   // first chunk of sequence s (units of s are consecutive)
+  // first chunk of sequence s (units of s are consecutive); a sequence with
+  // a prefix and no chunks is not one of this launch
+  int chunk_off[kFusedMaxSeqs + 1];
   uint32_t srh_bits[kFusedMaxLists];  // per (mask, group): bit i = query head group*G + i is SRH
 };
 
@@ -211,11 +213,66 @@ size_t fused_smem_bytes(int q_half_bytes, int q_bufs, int stages, int row_stride
 constexpr int kFusedPartsPerChunk = 4;  // first-pass pairs per chunk (epilogue warpgroups)
 cudaError_t fused_set_smem_limit(size_t bytes);
 
+// ---------------------------------------------------------------------------
+// Resident layer call: the same result as the fused call for short prompts,
+// with the logits held in tensor memory between the softmax statistics and
+// the scores (resident_kernel.cu).
+constexpr int kResidentChunkTiles = 4;  // most K tiles in a scoring chunk
+constexpr int kAccWords = 8;            // 64-bit accumulator words per unit and query row
+constexpr int kPairRing = 20;           // chunk sums a CTA keeps (more than it holds in tensor memory)
+constexpr int kResidentMaxGrid = 152;   // CTAs, at most
+constexpr int kResidentMaxRows = 192;   // query rows of a group, at most
+constexpr int kSelRegion = 38 * 1024;   // shared memory of the select warps
+
+struct ResidentParams {
+  CUtensorMap tmap_k;          // 3-D map over K: (d, kv head, token)
+  CUtensorMap tmap_q;          // 4-D map over the window queries: (d, w, head, sequence)
+  const float* lse;            // given-LSE mode: natural-log LSE per (sequence, head, window row)
+  long long lse_bs, lse_hs;    // its strides (elements); window rows contiguous
+  const uint4* k;              // gather sources (K on the device; V may be mapped host memory)
+  const uint4* v;
+  uint4* k_out;
+  uint4* v_out;
+  long long tok_stride_v16, head_stride_v16;  // K/V strides in 16-byte units
+  int32_t* indices;            // [num_kv_heads][o_total]
+  float* raw;                  // raw scores, score layout (caller's buffer or workspace)
+  float* pooled;               // pooled scores, score layout (caller's buffer or workspace)
+  int* status;                 // device status word
+  int* ctr;                    // header words (abort, start)
+  int* unit_ctr;               // per unit: chunks scored; then per unit: ticket of its second round
+  unsigned long long* acc;     // [unit][kAccWords][acc_rows]: the units' sums of exponentials
+  int acc_rows;                // row length of the accumulators (a multiple of 32)
+  float c;                     // scale * log2(e)
+  int window, pool_width, num_kv_heads, group_size, p_total, o_total, is_bf16;
+  int n_units, n_chunks, batch;
+  int do_select;               // 0: scores only (no selection, no gather)
+  int raw_scratch;             // raw scores in the workspace: a unit's row may hold its candidates
+  unsigned long long wait_ns;  // limit of every bounded wait of the call
+  int stall;                   // test hook: CTA 0's scheduler first waits for a counter nothing sets
+  int given_lse;               // 1: no first pass; denominators from `lse`
+  int q_half_bytes;            // bytes of one 64-column half of a Q buffer
+  int q_bufs;                  // Q buffers (2 or 3)
+  int stages;                  // K tiles in the shared-memory ring
+  float2* pairs;               // [CTA][kPairRing][acc_rows]: (M, S) of the CTA's latest chunks
+  int seqs_per_mask;
+  int cu_seqlens[kFusedMaxSeqs + 1];
+  int cu_prefix[kFusedMaxSeqs + 1];
+  int cu_out[kFusedMaxSeqs + 1];
+  int chunk_off[kFusedMaxSeqs + 1];   // first chunk of sequence s (units of s are consecutive)
+  uint8_t seq_chunk[kFusedMaxSeqs];   // K tiles per chunk; 0: not a sequence of this launch
+  uint32_t srh_bits[kFusedMaxLists];  // per (mask, group): bit i = query head group*G + i is SRH
+};
+
+cudaError_t launch_resident(const ResidentParams& p, int grid, size_t smem, cudaStream_t s);
+size_t resident_smem_bytes(int q_half_bytes, int q_bufs, int stages, int acc_rows);
+cudaError_t resident_set_smem_limit(size_t bytes);
+
 // Kernel parameters travel by value; CUDA takes at most 32764 bytes of them.
 static_assert(sizeof(ScoreParams) <= 32764, "scoring kernel parameters");
 static_assert(sizeof(CombineParams) <= 32764, "combine kernel parameters");
 static_assert(sizeof(SelectParams) <= 32764, "selection kernel parameters");
 static_assert(sizeof(FusedParams) <= 32764, "fused kernel parameters");
+static_assert(sizeof(ResidentParams) <= 32764, "resident kernel parameters");
 
 // Max pooling of each SRH head's window scores, summed over the heads: head
 // slot i of list (mask m, group g) holds the raw scores of that list's i-th

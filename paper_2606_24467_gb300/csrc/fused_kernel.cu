@@ -593,6 +593,7 @@ __device__ __noinline__ void select_unit(const Fused& F, int u, uint8_t* creg, i
   const int L = F.len(s);
   const int W = p.window;
   const int n = F.prefix(s);
+  if (n > 0 && F.chunks_per_unit(s) == 0) return;  // not of this launch
   const int out0 = p.cu_out[s];
   const int kept = p.cu_out[s + 1] - out0;
   const long long soff = static_cast<long long>(g) * p.p_total + p.cu_prefix[s];

@@ -1,0 +1,477 @@
+// Selection of one unit (sequence, KV group) by the worker warps of the
+// persistent kernels: pooling, top-k by pooled score, window, K/V gather
+// (CompressKV Sec. 3.3 and 4).  256 threads that share named barrier kBarC.
+#pragma once
+
+#include "ckv_device.cuh"
+#include "select_common.cuh"
+
+namespace ckv {
+namespace {
+
+constexpr int kCThreads = 256;     // worker threads of a CTA
+constexpr int kBarC = 3;           // their named barrier
+constexpr int kSelSamples = 1024;  // samples of a unit's pooled scores for the select threshold
+
+constexpr int kSelGroups = 2048;  // groups of consecutive keys whose largest score is kept
+struct SelShared {
+  uint32_t key[kFusedCandCap];   // (all the keys of a unit of at most kSelWhole: with pos)
+  int pos[kFusedCandCap];        // (while choosing a bound: samples)
+  uint32_t gmax[kSelGroups];     // (of a unit of at most kSelWhole, and
+  float stage_end[64];           // stage_end, while pooling: raw scores of a slice)
+  RadixShared rs;
+  int wcnt[8], wbase[8];
+  int wcnt_ge[8];  // per-warp counts at the best threshold with at least k keys above
+};
+static_assert(sizeof(SelShared) <= kSelRegion, "select scratch");
+static_assert(kSelSamples <= kFusedCandCap, "samples live in the position array");
+constexpr int kPoolSlice = 2048;  // keys pooled at a time
+constexpr int kSelWhole = 2 * kFusedCandCap;  // prefix keys of a unit whose keys all fit
+static_assert(kPoolSlice + 62 <= kFusedCandCap, "a slice and its halo fit the position array");
+static_assert(kPoolSlice + 62 <= kSelGroups + 64, "... and the group maxima's place");
+static_assert(62 < kCThreads, "a slice's halo is one load per thread");
+
+
+// The call's parameters that the selection needs (in shared memory: read
+// through a reference to the kernel's parameters they would come through L1).
+struct SelCall {
+  int* status;
+  int num_kv_heads, pool_width, raw_scratch;
+  const uint4* k;
+  const uint4* v;
+  uint4* k_out;
+  uint4* v_out;
+  long long tok_stride_v16, head_stride_v16;
+};
+
+__device__ __forceinline__ void cbar() { named_bar_sync(kBarC, kCThreads); }
+
+// Zero the radix state (the workers' form of radix_init).
+__device__ __forceinline__ void radix_init_grp(RadixShared& sh, int ct) {
+  for (int i = ct; i < 2 * 256; i += kCThreads) sh.hist[i >> 8][i & 255] = 0u;
+  if (ct < 2) {
+    sh.key_or[ct] = 0u;
+    sh.key_and[ct] = 0xFFFFFFFFu;
+  }
+}
+
+// The workers' form of cta_kth_largest (256 threads, named barrier): the
+// r-th largest of min(keys[j] - sub, clamp), j < count; *rem = how many of
+// the keys equal to it are among the r largest.
+__device__ __noinline__ uint32_t grp_kth_largest(const uint32_t* keys, int count, uint32_t sub,
+                                                 uint32_t clamp, int r, RadixShared& sh, int slot,
+                                                 int& pc, int* rem, int ct, bool global_keys) {
+  const int lane = ct & 31;
+  const int iters = (count + 255) >> 8;
+  auto key_at = [&](int j) -> uint32_t {
+    const uint32_t k = global_keys ? __ldcg(keys + j) : keys[j];
+    return min(k - sub, clamp);
+  };
+  uint32_t ko = 0u, ka = 0xFFFFFFFFu;
+#pragma unroll 2
+  for (int i = 0; i < iters; ++i) {
+    const int j = (i << 8) + ct;
+    if (j < count) {
+      const uint32_t key = key_at(j);
+      ko |= key;
+      ka &= key;
+    }
+  }
+  ko = __reduce_or_sync(0xffffffffu, ko);
+  ka = __reduce_and_sync(0xffffffffu, ka);
+  if (lane == 0) {
+    atomicOr(&sh.key_or[slot], ko);
+    atomicAnd(&sh.key_and[slot], ka);
+  }
+  cbar();
+  const uint32_t diff = sh.key_or[slot] ^ sh.key_and[slot];
+  const uint32_t kand = sh.key_and[slot];
+  int remaining = r;
+  if (diff == 0u) {
+    *rem = remaining;
+    return kand;
+  }
+  int hb = 31 - __clz(diff);
+  uint32_t pmask = hb == 31 ? 0u : ~((2u << hb) - 1u);
+  uint32_t prefix = kand & pmask;
+#pragma unroll 1
+  while (hb >= 0) {
+    const int width = min(8, hb + 1);
+    const int shf = hb + 1 - width;
+    const uint32_t fm = (1u << width) - 1u;
+    uint32_t* hh = sh.hist[pc & 3];
+    constexpr int kB = 4;  // keys per thread loaded before they are counted
+#pragma unroll 1
+    for (int i0 = 0; i0 < iters; i0 += kB) {
+      uint32_t bin[kB];
+      bool m[kB];
+#pragma unroll
+      for (int q = 0; q < kB; ++q) {
+        const int j = ((i0 + q) << 8) + ct;
+        const uint32_t key = j < count ? key_at(j) : 0u;
+        m[q] = j < count && (key & pmask) == prefix;
+        bin[q] = (key >> shf) & fm;
+      }
+#pragma unroll
+      for (int q = 0; q < kB; ++q) {
+        // one add per distinct bin of the warp (no same-address serialisation)
+        const uint32_t act = __ballot_sync(0xffffffffu, m[q]);
+        if (act == 0u) continue;
+        const uint32_t lb = __shfl_sync(0xffffffffu, bin[q], __ffs(act) - 1);
+        if (__all_sync(0xffffffffu, !m[q] || bin[q] == lb)) {
+          if (lane == __ffs(act) - 1) atomicAdd(&hh[lb], static_cast<uint32_t>(__popc(act)));
+        } else if (m[q]) {
+          const uint32_t same = __match_any_sync(act, bin[q]);
+          if (lane == __ffs(same) - 1)
+            atomicAdd(&hh[bin[q]], static_cast<uint32_t>(__popc(same)));
+        }
+      }
+    }
+    sh.hist[(pc + 2) & 3][ct] = 0u;
+    cbar();
+    int bin, above;
+    warp_pick_bin256(hh, remaining, lane, &bin, &above);
+    remaining -= above;
+    prefix |= static_cast<uint32_t>(bin) << shf;
+    pmask |= fm << shf;
+    hb = shf - 1;
+    ++pc;
+  }
+  *rem = remaining;
+  return prefix;
+}
+
+// Ordered emission of the selected entries of a key list in position order:
+// entry j (key keys[j], position pos[j], or j without a list) is selected when
+// its key is above tau, or equal to tau and fewer than need_eq equal keys
+// precede it.  Selected entries go to out[0..k) in list order.  Each warp has
+// a contiguous part of the list: it counts, then (one barrier later) emits.
+__device__ __noinline__ void emit_selected(int count, uint32_t tau, int need_eq, int32_t* out, int k,
+                                           SelShared& sh, int ct, const uint32_t* keys,
+                                           const int* pos) {
+  const int cw = ct >> 5;
+  const int lane = ct & 31;
+  const int seg = (count + 255) >> 8 << 5;  // entries per warp
+  const int j0 = min(count, cw * seg);
+  const int j1 = min(count, j0 + seg);
+  int o = 0, eq_seen = 0;
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    int gt_n = 0, eq_n = 0;
+#pragma unroll 2
+    for (int jb = j0; jb < j1; jb += 32) {
+      const int j = jb + lane;
+      const uint32_t key = j < j1 ? keys[j] : 0u;
+      const uint32_t mgt = __ballot_sync(0xffffffffu, j < j1 && key > tau);
+      const uint32_t meq = __ballot_sync(0xffffffffu, j < j1 && key == tau);
+      if (pass == 0) {
+        gt_n += __popc(mgt);
+        eq_n += __popc(meq);
+      } else if ((mgt | meq) != 0u) {
+        const uint32_t lt = lanemask_lt(lane);
+        const bool take = (meq >> lane & 1u) && eq_seen + __popc(meq & lt) < need_eq;
+        const uint32_t msel = mgt | __ballot_sync(0xffffffffu, take);
+        const int slot = o + __popc(msel & lt);
+        if ((msel >> lane & 1u) && slot < k) out[slot] = pos ? pos[j] : j;
+        o += __popc(msel);
+        eq_seen += __popc(meq);
+      }
+    }
+    if (pass == 0) {
+      if (lane == 0) {
+        sh.wcnt[cw] = gt_n;
+        sh.wbase[cw] = eq_n;
+      }
+      cbar();
+#pragma unroll
+      for (int w = 0; w < 8; ++w) {
+        const int g = sh.wcnt[w], q = sh.wbase[w];
+        if (w < cw) {
+          o += g + max(0, min(need_eq - eq_seen, q));
+          eq_seen += q;
+        }
+      }
+    }
+  }
+}
+
+// Copy the K and V rows of out[0..count) (positions in the sequence) to the
+// compressed cache rows out0 .. out0 + count - 1 of group g: a warp per row
+// (lanes 0-15 its K, 16-31 its V, 16 bytes each), eight rows in flight.  A
+// position outside the sequence (never, for a correct selection) is skipped
+// and recorded.
+__device__ __noinline__ void gather_rows(const SelCall& p, int seq0, int L, int g,
+                                         const int32_t* out, int out0, int count, int ct) {
+  constexpr int kBatch = 8;
+  constexpr int kRow16 = kHeadDim * 2 / 16;
+  const int lane = ct & 31;
+  const int part = lane & 15;
+  const uint4* src = (lane < 16 ? p.k : p.v) + static_cast<long long>(seq0) * p.tok_stride_v16 +
+                     static_cast<long long>(g) * p.head_stride_v16 + part;
+  uint4* dst = (lane < 16 ? p.k_out : p.v_out) +
+               (static_cast<long long>(out0) * p.num_kv_heads + g) * kRow16 + part;
+  const long long stride = p.tok_stride_v16;
+  const int dstride = p.num_kv_heads * kRow16;
+  bool bad = false;
+#pragma unroll 1
+  for (int i0 = ct >> 5; i0 < count; i0 += kBatch * (kCThreads / 32)) {
+    int tok[kBatch];
+    uint4 v[kBatch];
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) {
+      const int i = i0 + k * (kCThreads / 32);
+      tok[k] = i < count ? out[i] : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) {
+      const bool ok = tok[k] >= 0 && tok[k] < L;
+      bad |= !ok;
+      tok[k] = ok ? tok[k] : -1;
+      if (ok && i0 + k * (kCThreads / 32) < count) v[k] = __ldg(src + tok[k] * stride);
+    }
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) {
+      const int i = i0 + k * (kCThreads / 32);
+      if (i < count && tok[k] >= 0) dst[static_cast<long long>(i) * dstride] = v[k];
+    }
+  }
+  if (bad) atomicCAS(p.status, 0, CKV_DEV_ERR_INDEX);
+}
+
+// The keys >= lo of the 32-key rows [r0, r1) of a unit (one warp, eight rows
+// in flight), skipping the rows of groups (2^e rows) whose largest key is
+// below lo.  Counts from o on; with ckey, the keys and their positions go to
+// slots o, o + 1, ... below cap, in position order.
+__device__ __noinline__ int scan_rows(const uint32_t* keys, int n, int r0, int r1, int e,
+                                      const uint32_t* gmax, uint32_t lo, int o, uint32_t* ckey,
+                                      int* cpos, int cap, int lane) {
+  constexpr int kU = 8;
+#pragma unroll 1
+  for (int r = r0; r < r1; r += 32) {
+    uint32_t m = __ballot_sync(0xffffffffu, r + lane < r1 && gmax[(r + lane) >> e] >= lo);
+#pragma unroll 1
+    while (m != 0u) {
+      uint32_t kv[kU];
+      int at[kU];
+#pragma unroll
+      for (int q = 0; q < kU; ++q) {
+        at[q] = m != 0u ? (r + __ffs(m) - 1) * 32 + lane : n;
+        m &= m - 1u;
+        kv[q] = at[q] < n ? __ldcg(keys + at[q]) : 0u;
+      }
+#pragma unroll
+      for (int q = 0; q < kU; ++q) {
+        const bool c = at[q] < n && kv[q] >= lo;
+        const uint32_t mm = __ballot_sync(0xffffffffu, c);
+        const int slot = o + __popc(mm & lanemask_lt(lane));
+        if (ckey && c && slot < cap) {
+          ckey[slot] = kv[q];
+          cpos[slot] = at[q];
+        }
+        o += __popc(mm);
+      }
+    }
+  }
+  return o;
+}
+
+struct SelUnit {
+  int g, seq0, L, W, out0, kept;
+};
+
+// Pools the unit's raw scores (sum from j - h to j + h, zeros outside [0, n),
+// over P), slice by slice through shared memory with the next slice's loads in
+// flight; writes them to `pooled` and, as keys, to `keys` when the unit is
+// small enough for it (n <= kSelWhole), else keeps the largest of every group of
+// 32 << e keys.
+__device__ __noinline__ void pool_unit(const float* raw, float* pooled, int n, int e, int h, float fP,
+                                       SelShared& sh, int ct) {
+  constexpr int kPer = kPoolSlice / kCThreads;  // keys per thread and slice
+  const int lane = ct & 31;
+  const bool keep = n <= kSelWhole;
+  float* const stage = keep ? reinterpret_cast<float*>(sh.gmax) : reinterpret_cast<float*>(sh.pos);
+  float nx[kPer + 1];
+  auto load = [&](int base) {
+#pragma unroll
+    for (int q = 0; q <= kPer; ++q) {
+      const int i = q * kCThreads + ct;
+      const int j = base - h + i;
+      nx[q] = i < kPoolSlice + 2 * h && j >= 0 && j < n ? __ldcg(raw + j) : 0.f;
+    }
+  };
+  load(0);
+#pragma unroll 1
+  for (int base = 0; base < n; base += kPoolSlice) {
+    cbar();  // the slice before is read
+#pragma unroll
+    for (int q = 0; q <= kPer; ++q) {
+      const int i = q * kCThreads + ct;
+      if (i < kPoolSlice + 2 * h) stage[i] = nx[q];
+    }
+    cbar();
+    if (base + kPoolSlice < n) load(base + kPoolSlice);
+    float s[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) s[q] = 0.f;
+    const float* a = stage + ct;
+#pragma unroll 1
+    for (int t = 0; t <= 2 * h; ++t, ++a) {
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) s[q] += a[q * kCThreads];
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int j = base + q * kCThreads + ct;
+      if (j - lane >= n) break;
+      const bool in = j < n;
+      const float v = s[q] / fP;
+      if (in) {
+        pooled[j] = v;
+        if (keep) sh.key[j] = __float_as_uint(v);
+      }
+      if (!keep) {
+        const uint32_t m = __reduce_max_sync(0xffffffffu, in ? __float_as_uint(v) : 0u);
+        if (lane == 0) atomicMax(&sh.gmax[j >> (5 + e)], m);
+      }
+    }
+  }
+}
+
+// Selection of a unit.  Pooling, then the top-k: a unit of at most
+// kSelWhole prefix keys by an exact radix search of its keys in shared
+// memory; a longer one by a lower bound of the k-th largest score -- the k-th
+// largest group maximum (k groups have a key at least that large) or, with
+// fewer groups than k, a rank among samples -- then the candidates in position
+// order and the radix search among them (among all the unit's scores when the
+// bound keeps too few or too many); then the window and the K/V rows.  Pooled
+// scores are >= 0: their bit patterns order like their values.
+__device__ __noinline__ void select_unit(const SelCall& p, const SelUnit U, float* raw,
+                                         float* pooled, int32_t* out, uint8_t* creg, int ct) {
+  SelShared& sh = *reinterpret_cast<SelShared*>(creg);
+  const int cw = ct >> 5;
+  const int lane = ct & 31;
+  const int L = U.L;
+  const int W = U.W;
+  const int n = max(L - W, 0);
+  int e = 0;  // groups of 2^e rows of 32 keys
+  while (((n + 31) >> 5) > (kSelGroups << e)) ++e;
+  const int nr = (n + 31) >> 5;
+  const int ng = (nr + (1 << e) - 1) >> e;
+  for (int i = ct; i < ng; i += kCThreads) sh.gmax[i] = 0u;
+  pool_unit(raw, pooled, n, e, (p.pool_width - 1) >> 1, static_cast<float>(p.pool_width), sh, ct);
+  __threadfence_block();
+  cbar();
+  const int kept = U.kept;
+  if (kept >= L) {  // keep everything
+    for (int i = ct; i < L; i += kCThreads) out[i] = i;
+    __threadfence_block();
+    cbar();
+    gather_rows(p, U.seq0, L, U.g, out, U.out0, L, ct);
+    return;
+  }
+  const int k = kept - W;  // 0 <= k < n
+  for (int w = ct; w < W; w += kCThreads) out[k + w] = n + w;
+  if (k > 0) {
+    const uint32_t* keys = reinterpret_cast<const uint32_t*>(pooled);
+    uint32_t* samp = reinterpret_cast<uint32_t*>(sh.pos);
+    const int seg = (nr + 7) >> 3;  // rows per warp
+    const int r0 = min(nr, cw * seg);
+    const int r1 = min(nr, r0 + seg);
+    int pc = 0, need_eq = 0;
+    uint32_t lo = 0, lo_ge = 0;
+    int total = 0, tot_ge = -1;
+    bool fast = false;
+    const bool whole = n <= kSelWhole;  // every key is in shared memory
+    bool by_group = ng >= k;
+    const int ns = min(kSelSamples, n);
+    const float mu = static_cast<float>(k) * static_cast<float>(ns) / static_cast<float>(n);
+    int rs = min(ns, static_cast<int>(ceilf(mu + 3.f * sqrtf(mu))) + 2);
+#pragma unroll 1
+    for (int attempt = whole ? 2 : (by_group ? -1 : 0); attempt < 2; ++attempt) {
+      if (attempt == 0)
+        for (int i = ct; i < ns; i += kCThreads)
+          samp[i] = __ldcg(keys + static_cast<int>((static_cast<long long>(i) * n) / ns));
+      radix_init_grp(sh.rs, ct);
+      pc = 0;
+      cbar();
+      by_group = attempt < 0;
+      lo = grp_kth_largest(by_group ? sh.gmax : samp, by_group ? ng : ns, 0u, 0xFFFFFFFFu,
+                           by_group ? k : rs, sh.rs, 0, pc, &need_eq, ct, false);
+      const int wc = scan_rows(keys, n, r0, r1, e, sh.gmax, lo, 0, nullptr, nullptr, 0, lane);
+      if (lane == 0) sh.wcnt[cw] = wc;
+      cbar();
+      total = 0;
+      for (int w = 0; w < 8; ++w) total += sh.wcnt[w];
+      if (total >= k && (tot_ge < 0 || total < tot_ge)) {
+        lo_ge = lo;
+        tot_ge = total;
+        if (ct < 8) sh.wcnt_ge[ct] = sh.wcnt[ct];
+      }
+      fast = total >= k && total <= kFusedCandCap;
+      if (fast) break;
+      cbar();  // every thread has read the counts
+      if (by_group) continue;
+      // aim at the middle of [k, capacity] from the density this attempt saw
+      const float per = static_cast<float>(max(total, 1)) / static_cast<float>(rs);
+      int want = static_cast<int>(ceilf(0.5f * static_cast<float>(k + kFusedCandCap) / per));
+      want = total < k ? max(want, rs + 1) : min(want, rs - 1);
+      if (want < 1 || want > ns || want == rs) break;
+      rs = want;
+    }
+    // the candidates' radix starts afresh
+    cbar();
+    radix_init_grp(sh.rs, ct);
+    pc = 0;
+    need_eq = 0;
+    // The candidates (keys >= lo) in position order: in shared memory when at
+    // most kFusedCandCap, else -- when the raw scores are workspace, last read
+    // above -- in the unit's raw-score row, keys in its first half and
+    // positions in its second; else all of the unit's keys.
+    const uint32_t* ckey = keys;
+    const int* cpos = nullptr;
+    int count = n;
+    bool in_shared = true;
+    if (whole) {
+      ckey = sh.key;
+    } else if (!fast && p.raw_scratch && tot_ge >= k && tot_ge <= n / 2) {
+      lo = lo_ge;
+      total = tot_ge;
+      if (ct < 8) sh.wcnt[ct] = sh.wcnt_ge[ct];
+      ckey = reinterpret_cast<uint32_t*>(raw);
+      cpos = reinterpret_cast<int*>(raw + n / 2);
+      count = total;
+      in_shared = false;
+    } else if (fast) {
+      ckey = sh.key;
+      cpos = sh.pos;
+      count = total;
+    } else {
+      in_shared = false;
+    }
+    cbar();
+    if (cpos) {
+      int o = 0;
+      for (int w = 0; w < cw; ++w) o += sh.wcnt[w];
+      scan_rows(keys, n, r0, r1, e, sh.gmax, lo, o, const_cast<uint32_t*>(ckey),
+                const_cast<int*>(cpos), total, lane);
+      __threadfence_block();
+      cbar();
+    } else {
+      lo = 0u;
+    }
+    // offsets above the bound, clamped to 16 bits: at most two radix passes
+    const uint32_t clamp = cpos ? 0xFFFFu : 0xFFFFFFFFu;
+    const uint32_t td =
+        grp_kth_largest(ckey, count, lo, clamp, k, sh.rs, 0, pc, &need_eq, ct, !in_shared);
+    uint32_t tau = lo + td;
+    if (cpos && td == clamp)
+      tau = grp_kth_largest(ckey, count, 0u, 0xFFFFFFFFu, k, sh.rs, 1, pc, &need_eq, ct, !in_shared);
+    emit_selected(count, tau, need_eq, out, k, sh, ct, ckey, cpos);
+  }
+  __threadfence_block();
+  cbar();  // the indices written above are read back by the copy
+  gather_rows(p, U.seq0, L, U.g, out, U.out0, kept, ct);
+}
+
+}  // namespace
+}  // namespace ckv

@@ -1,0 +1,100 @@
+"""The persistent kernel for short prompts (logits kept in tensor memory) and
+the line between it and the two-pass kernel, against the float64 oracle (needs
+a GB300)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2606_24467_gb300 as ckv
+import workloads as wl
+from oracle import compare
+from test_gpu_fused import _block, _check_block, _pack, _run_call
+
+pytestmark = pytest.mark.gpu
+
+BLOCK_KEYS = ("raw", "pooled", "indices", "k_out", "v_out", "cu_out")
+
+
+def _make(name, lens, **over):
+    cfg = wl.get(name).scaled(seq_len=0, batch=len(lens), **over)
+    masks = wl.srh_masks(cfg)
+    budgets = wl.layer_budgets(cfg, lens)
+    return cfg, [wl.make_layer(cfg, l, lengths=lens, masks=masks, budgets=budgets)
+                 for l in range(cfg.n_layers)]
+
+
+@pytest.mark.parametrize("window,heads,lens", [
+    # tile edges; chunks of one, two and four tiles; the longest prompt whose
+    # scores the selection holds in shared memory (6144 keys before the window)
+    (16, (1, 1), [17, 127, 128, 129, 4096, 4097, 6160, 6161, 8193]),
+    # 32 and 64 rows: the line of 64 rows and a prompt that only 32 rows keep
+    (32, (1, 2), [33, 8192, 16384, 16385]),
+    # 64, 128 and 192 rows in one call: the lines of 192 and of 128 rows
+    (64, (1, 3), [65, 4096, 4097, 8192, 8193]),
+])
+def test_sizes_around_tiles_chunks_and_the_kernels_line(cuda_device, window, heads, lens):
+    cfg, layers = _make("c5", lens, n_layers=2, window=window, srh_per_group=heads,
+                        budget_mean=300)
+    big, cu_out, cu = _run_call(layers, cfg, cuda_device)
+    for l, lay in enumerate(layers):
+        _check_block(_block(big, cu_out, cu, l, cfg.batch, window), lay, cfg)
+    alone, cu_out1, cu1 = _run_call(layers[1:], cfg, cuda_device)
+    a = _block(alone, cu_out1, cu1, 0, cfg.batch, window)
+    b = _block(big, cu_out, cu, 1, cfg.batch, window)
+    for key in BLOCK_KEYS:
+        assert np.array_equal(a[key], b[key]), key
+
+
+@pytest.mark.parametrize("shift", [-90.0, 90.0])
+def test_sums_outside_the_fixed_point_bins(cuda_device, shift):
+    """Every other window row's logits moved by about `shift`: its sums of
+    exponentials leave the range of the accumulators' bins (2^-10 down to the
+    grid's end, 2^118 up), so it takes the second round; its neighbours don't.
+
+    Bound: a logit is eight accumulations of at most |q| |k| in fp32, scaled
+    once and rounded once against the exponent's reference, so off by at most
+    10 ulp of |q| |k| / sqrt(d); a score is a ratio of two exponentials of it."""
+    cfg, layers = _make("c2", [700, 5000], n_layers=1, srh_per_group=(1, 2), budget_mean=200)
+    lay = layers[0]
+    u = torch.sign(torch.randn(128, generator=torch.Generator().manual_seed(7)))
+    dt = lay["k"].dtype
+    lay["k"] = (lay["k"].float() + 2.0 * u).to(dt)
+    q = lay["q_win"].float()
+    q[:, :, ::2] += shift * 128 ** 0.5 / 256.0 * u
+    lay["q_win"] = q.to(dt)
+    out, cu_out, cu = _run_call(layers, cfg, cuda_device)
+    blk = _block(out, cu_out, cu, 0, cfg.batch, cfg.window)
+    res = oracle.compress_layer(lay["q_win"].float().numpy(), lay["k"].float().numpy(),
+                                lay["v"].float().numpy(), lay["cu_seqlens"], lay["srh_mask"],
+                                lay["budgets"], cfg.window, cfg.pool_width)
+    norms = lay["q_win"].float().norm(dim=-1).max() * lay["k"].float().norm(dim=-1).max()
+    rtol = 2 * 10 * 2.0 ** -23 * float(norms) / 128 ** 0.5 + 1e-5
+    compare.check_scores("raw", blk["raw"], res.raw, rtol=rtol, atol=1e-8)
+    compare.check_scores("pooled", blk["pooled"], res.pooled, rtol=rtol, atol=1e-8)
+
+
+def test_calls_on_two_streams_at_once(cuda_device):
+    """Two calls in flight on two streams with a workspace each (every one
+    needs all its CTAs resident): the bits of the calls made one by one."""
+    dev = cuda_device
+    runs = []
+    for seed, lens in enumerate(([1500, 3000], [900, 16385])):
+        cfg, layers = _make("c2", lens, n_layers=2 + seed, budget_mean=200)
+        want, _, _ = _run_call(layers, cfg, dev)
+        q, k, v, cu, b, m = _pack(layers, dev)
+        prob = ckv.Problem(q, k, cu, cfg.window, cfg.pool_width)
+        out = ckv.LayerOutputs(prob, b, 128, k.dtype, dev, scores=True)
+        runs.append((len(layers), prob, q, k, v, m, b, out, ckv.workspace(prob, dev), want,
+                     torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    for _ in range(10):
+        for n, prob, q, k, v, m, b, out, ws, _, stream in runs:
+            with torch.cuda.stream(stream):
+                ckv.compress_layers(prob, n, q, k, v, m, b, out.indices, out.k_out, out.v_out, ws,
+                                    raw=out.raw, pooled=out.pooled)
+    torch.cuda.synchronize()
+    for _, _, _, _, _, _, _, out, ws, want, _ in runs:
+        assert ckv.read_device_status(ws) == 0
+        for key in ("raw", "pooled", "indices", "k_out", "v_out"):
+            assert torch.equal(getattr(out, key), getattr(want, key)), key
