@@ -945,15 +945,18 @@ bool takes_resident(int rows, int len, bool given_lse) {
   return rows <= kResidentMaxRows && len <= 4096;
 }
 
-// K tiles per chunk of a resident sequence: up to four (what a chunk costs
-// beside its tiles is then small); fewer where a unit has few tiles (they
-// then reach more SMs) or its layer has wide groups (the tensor memory must
-// hold two chunks).  At most 32 chunks a unit (64 of 32 rows, of which the
-// tensor memory holds four): kResidentMinGrid CTAs hold any.
-int resident_chunk_tiles(int rows, int len) {
-  const int tiles = (len + kTileTokens - 1) / kTileTokens;
+// K tiles per chunk of a resident layer: up to four, as a chunk costs about
+// as much again as its tiles (32 layers of 8 prompts of 300 to 4000 tokens:
+// 1144 us with one tile a chunk, 788 with two, 617 with four); fewer where the
+// layer has few tiles over all its units (they then reach more SMs: a single
+// 777-token layer 27.8 us with one tile a chunk, 28.3 with two, 30.9 with
+// four; a 4096-token one 37.5 with two, 38.9 with four, but 32 of the
+// latter 137 with two, 114 with four) or wide groups (the tensor memory must
+// hold two chunks).  A unit then has at most 64 chunks (128 of 32 rows, of
+// which the tensor memory holds eight): kResidentMinGrid CTAs hold any.
+int resident_chunk_tiles(int rows, long long layer_tiles) {
   const int most = rows <= 64 ? kResidentChunkTiles : (rows <= 128 ? 2 : 1);
-  return std::min(most, tiles <= 32 ? 1 : (tiles <= 64 ? 2 : 4));
+  return std::min(most, layer_tiles <= 64 ? 1 : (layer_tiles <= 256 ? 2 : 4));
 }
 
 // What the two persistent kernels' parameters have in common.
@@ -1031,20 +1034,25 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   // the kernel of every layer (mask), and the query rows of each kernel's
   // widest group
   const int r_grid = std::min(Fd->sms, kResidentMaxGrid);
-  std::vector<int> seq_rows(I.B, 0);
+  std::vector<int> seq_ct(I.B, 0);  // K tiles per chunk
   std::vector<uint8_t> in_resident(I.B, 0);
   int max_rows = 16, r_rows = 16, n_resident = 0;
   for (int s0 = 0; s0 < I.B; s0 += I.spm) {
     int rows = 0, longest = 0;
     for (int g = 0; g < I.Hkv; ++g) rows = std::max(rows, S.rows[I.vgroup(s0, g)]);
-    for (int s_ = s0; s_ < s0 + I.spm; ++s_) longest = std::max(longest, I.len[s_]);
+    long long tiles = 0;
+    for (int s_ = s0; s_ < s0 + I.spm; ++s_) {
+      longest = std::max(longest, I.len[s_]);
+      if (I.n[s_] > 0)
+        tiles += static_cast<long long>(I.Hkv) * ((I.len[s_] + kTileTokens - 1) / kTileTokens);
+    }
     const bool res =
         r_grid >= kResidentMinGrid && takes_resident(rows, longest, lse.lse != nullptr);
     int& most = res ? r_rows : max_rows;
     most = std::max(most, rows);
     if (res) n_resident += I.spm;
     for (int s_ = s0; s_ < s0 + I.spm; ++s_) {
-      seq_rows[s_] = rows;
+      seq_ct[s_] = resident_chunk_tiles(rows, tiles);
       in_resident[s_] = res ? 1 : 0;
     }
   }
@@ -1110,7 +1118,7 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
     P.pairs = reinterpret_cast<float2*>(wb + RL.pairs);
     long long out = 0;  // rows of the sequences this launch selects
     for (int s_ = 0; s_ < I.B; ++s_) {
-      const int ct = in_resident[s_] ? resident_chunk_tiles(seq_rows[s_], I.len[s_]) : 0;
+      const int ct = in_resident[s_] ? seq_ct[s_] : 0;
       const int tiles = I.n[s_] > 0 ? (I.len[s_] + kTileTokens - 1) / kTileTokens : 0;
       P.seq_chunk[s_] = static_cast<uint8_t>(ct);
       P.chunk_off[s_ + 1] = P.chunk_off[s_] + (ct ? I.Hkv * ((tiles + ct - 1) / ct) : 0);

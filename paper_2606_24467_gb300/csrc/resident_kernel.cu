@@ -71,7 +71,7 @@
 // What bounds it: a short call the chain of its steps (one 777-token layer,
 // 28 us against 67 in the two-pass kernel: start 4, scores 7, selection 11,
 // of which the radix search 5), a full one the epilogue's exponentials and
-// tensor-memory loads (32 layers of 8 prompts of 300 to 4000 tokens: 1.1
+// tensor-memory loads (32 layers of 8 prompts of 300 to 4000 tokens: 0.62
 // ms against 3.5), as K is read once.
 // Every wait is bounded (ResidentParams::wait_ns, kWaitTimeoutNs unless a test
 // shortens it) and on expiry records CKV_ERR_DEVICE_TIMEOUT and stops the

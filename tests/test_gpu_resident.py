@@ -25,9 +25,13 @@ def _make(name, lens, **over):
 
 
 @pytest.mark.parametrize("window,heads,lens", [
-    # tile edges; chunks of one, two and four tiles; the longest prompt whose
-    # scores the selection holds in shared memory (6144 keys before the window)
-    (16, (1, 1), [17, 127, 128, 129, 4096, 4097, 6160, 6161, 8193]),
+    # tile edges in chunks of one tile (layers of at most 64 tiles), of two
+    # (at most 256) and of four
+    (16, (1, 1), [17, 127, 128, 129]),
+    (32, (1, 2), [129, 600, 1153]),
+    # the longest prompt whose scores the selection holds in shared memory
+    # (6144 keys before the window)
+    (16, (1, 1), [513, 4096, 4097, 6160, 6161, 8193]),
     # 32 and 64 rows: the line of 64 rows and a prompt that only 32 rows keep
     (32, (1, 2), [33, 8192, 16384, 16385]),
     # 64, 128 and 192 rows in one call: the lines of 192 and of 128 rows
