@@ -13,6 +13,7 @@ constexpr int kCThreads = 256;     // worker threads of a CTA
 constexpr int kBarC = 3;           // their named barrier
 constexpr int kSelSamples = 1024;  // samples of a unit's pooled scores for the select threshold
 
+constexpr int kSelWhole = 2 * kFusedCandCap;  // prefix keys of a unit whose keys all fit
 constexpr int kSelGroups = 2048;  // groups of consecutive keys whose largest score is kept
 struct SelShared {
   uint32_t key[kFusedCandCap];   // (all the keys of a unit of at most kSelWhole: with pos)
@@ -22,11 +23,11 @@ struct SelShared {
   RadixShared rs;
   int wcnt[8], wbase[8];
   int wcnt_ge[8];  // per-warp counts at the best threshold with at least k keys above
+  alignas(16) uint32_t cnt[2][2][8];  // per-warp results of a bisection step
 };
 static_assert(sizeof(SelShared) <= kSelRegion, "select scratch");
 static_assert(kSelSamples <= kFusedCandCap, "samples live in the position array");
 constexpr int kPoolSlice = 2048;  // keys pooled at a time
-constexpr int kSelWhole = 2 * kFusedCandCap;  // prefix keys of a unit whose keys all fit
 static_assert(kPoolSlice + 62 <= kFusedCandCap, "a slice and its halo fit the position array");
 static_assert(kPoolSlice + 62 <= kSelGroups + 64, "... and the group maxima's place");
 static_assert(62 < kCThreads, "a slice's halo is one load per thread");
@@ -56,16 +57,15 @@ __device__ __forceinline__ void radix_init_grp(RadixShared& sh, int ct) {
 }
 
 // The workers' form of cta_kth_largest (256 threads, named barrier): the
-// r-th largest of min(keys[j] - sub, clamp), j < count; *rem = how many of
-// the keys equal to it are among the r largest.
+// r-th largest of min(keys[j] - sub, clamp), j < count, of keys in global
+// memory; *rem = how many of the keys equal to it are among the r largest.
 __device__ __noinline__ uint32_t grp_kth_largest(const uint32_t* keys, int count, uint32_t sub,
                                                  uint32_t clamp, int r, RadixShared& sh, int slot,
-                                                 int& pc, int* rem, int ct, bool global_keys) {
+                                                 int& pc, int* rem, int ct) {
   const int lane = ct & 31;
   const int iters = (count + 255) >> 8;
   auto key_at = [&](int j) -> uint32_t {
-    const uint32_t k = global_keys ? __ldcg(keys + j) : keys[j];
-    return min(k - sub, clamp);
+    return min(__ldcg(keys + j) - sub, clamp);
   };
   uint32_t ko = 0u, ka = 0xFFFFFFFFu;
 #pragma unroll 2
@@ -140,6 +140,81 @@ __device__ __noinline__ uint32_t grp_kth_largest(const uint32_t* keys, int count
   *rem = remaining;
   return prefix;
 }
+
+// Bisection for the r-th largest of keys[0..count) (shared memory, at most
+// kPer * 256), r <= count: each thread holds its keys in registers and a step
+// counts the keys at least the middle of the range (one barrier).  Returns
+// tau and *need_eq such that the keys above tau and the first *need_eq equal
+// to it are the r largest; stops early when a step finds r to r + slack keys
+// at least its middle (the keys above tau are then that many).  Some 20 steps
+// of 0.1 us, where radix passes of 8 bits over shared memory took 1 us each
+// and more with the keys: 14.8 -> 3 us at 4064 keys.
+template <int kPer>
+__device__ __noinline__ uint32_t bisect_kth(const uint32_t* keys, int count, int r, int slack,
+                                            SelShared& sh, int* need_eq, int ct) {
+  const int cw = ct >> 5;
+  const int lane = ct & 31;
+  uint32_t kv[kPer];
+  uint32_t mn = 0xFFFFFFFFu, mx = 0u;
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const int j = i * kCThreads + ct;
+    kv[i] = j < count ? keys[j] : 0u;  // (never counted: the middle is at least 1)
+    if (j < count) mn = min(mn, kv[i]);
+    mx = max(mx, kv[i]);
+  }
+  mn = __reduce_min_sync(0xffffffffu, mn);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0) {
+    sh.cnt[0][0][cw] = mn;
+    sh.cnt[0][1][cw] = mx;
+  }
+  cbar();
+  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    lo = min(lo, sh.cnt[0][0][w]);
+    hi = max(hi, sh.cnt[0][1][w]);
+  }
+  int above = 0;  // keys above hi
+  int step = 1;
+#pragma unroll 1
+  while (lo < hi) {
+    const uint32_t mid = hi - ((hi - lo) >> 1);  // lo < mid <= hi
+    int c = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) c += kv[i] >= mid ? 1 : 0;
+    c = __reduce_add_sync(0xffffffffu, c);
+    uint32_t* const cnt = sh.cnt[step & 1][0];
+    if (lane == 0) cnt[cw] = static_cast<uint32_t>(c);
+    cbar();
+    const uint4 a = *reinterpret_cast<const uint4*>(cnt);
+    const uint4 b = *reinterpret_cast<const uint4*>(cnt + 4);
+    c = static_cast<int>((a.x + a.y) + (a.z + a.w) + (b.x + b.y) + (b.z + b.w));
+    if (c >= r) {
+      lo = mid;
+      if (c <= r + slack) {
+        *need_eq = 0;
+        cbar();  // (the counts are rewritten by the next search)
+        return mid - 1u;
+      }
+    } else {
+      hi = mid - 1u;
+      above = c;
+    }
+    ++step;
+  }
+  *need_eq = r - above;
+  cbar();
+  return lo;
+}
+__device__ __forceinline__ uint32_t shared_kth(const uint32_t* keys, int count, int r, int slack,
+                                               SelShared& sh, int* need_eq, int ct) {
+  if (count <= 4 * kCThreads) return bisect_kth<4>(keys, count, r, slack, sh, need_eq, ct);
+  if (count <= 12 * kCThreads) return bisect_kth<12>(keys, count, r, slack, sh, need_eq, ct);
+  return bisect_kth<24>(keys, count, r, slack, sh, need_eq, ct);
+}
+static_assert(kSelWhole <= 24 * kCThreads && kSelGroups <= 12 * kCThreads, "bisected keys");
 
 // Ordered emission of the selected entries of a key list in position order:
 // entry j (key keys[j], position pos[j], or j without a list) is selected when
@@ -338,12 +413,12 @@ __device__ __noinline__ void pool_unit(const float* raw, float* pooled, int n, i
 }
 
 // Selection of a unit.  Pooling, then the top-k: a unit of at most
-// kSelWhole prefix keys by an exact radix search of its keys in shared
+// kSelWhole prefix keys by bisection over its keys in shared
 // memory; a longer one by a lower bound of the k-th largest score -- the k-th
 // largest group maximum (k groups have a key at least that large) or, with
 // fewer groups than k, a rank among samples -- then the candidates in position
-// order and the radix search among them (among all the unit's scores when the
-// bound keeps too few or too many); then the window and the K/V rows.  Pooled
+// order and the bisection among them (a radix search among those in global
+// memory, or all the unit's scores, when the bound keeps too few or too many); then the window and the K/V rows.  Pooled
 // scores are >= 0: their bit patterns order like their values.
 __device__ __noinline__ void select_unit(const SelCall& p, const SelUnit U, float* raw,
                                          float* pooled, int32_t* out, uint8_t* creg, int ct) {
@@ -391,12 +466,10 @@ __device__ __noinline__ void select_unit(const SelCall& p, const SelUnit U, floa
       if (attempt == 0)
         for (int i = ct; i < ns; i += kCThreads)
           samp[i] = __ldcg(keys + static_cast<int>((static_cast<long long>(i) * n) / ns));
-      radix_init_grp(sh.rs, ct);
-      pc = 0;
       cbar();
       by_group = attempt < 0;
-      lo = grp_kth_largest(by_group ? sh.gmax : samp, by_group ? ng : ns, 0u, 0xFFFFFFFFu,
-                           by_group ? k : rs, sh.rs, 0, pc, &need_eq, ct, false);
+      lo = shared_kth(by_group ? sh.gmax : samp, by_group ? ng : ns, by_group ? k : rs,
+                      by_group ? k >> 4 : 0, sh, &need_eq, ct);
       const int wc = scan_rows(keys, n, r0, r1, e, sh.gmax, lo, 0, nullptr, nullptr, 0, lane);
       if (lane == 0) sh.wcnt[cw] = wc;
       cbar();
@@ -459,13 +532,17 @@ __device__ __noinline__ void select_unit(const SelCall& p, const SelUnit U, floa
     } else {
       lo = 0u;
     }
-    // offsets above the bound, clamped to 16 bits: at most two radix passes
-    const uint32_t clamp = cpos ? 0xFFFFu : 0xFFFFFFFFu;
-    const uint32_t td =
-        grp_kth_largest(ckey, count, lo, clamp, k, sh.rs, 0, pc, &need_eq, ct, !in_shared);
-    uint32_t tau = lo + td;
-    if (cpos && td == clamp)
-      tau = grp_kth_largest(ckey, count, 0u, 0xFFFFFFFFu, k, sh.rs, 1, pc, &need_eq, ct, !in_shared);
+    uint32_t tau;
+    if (in_shared) {
+      tau = shared_kth(ckey, count, k, 0, sh, &need_eq, ct);
+    } else {
+      // offsets above the bound, clamped to 16 bits: at most two radix passes
+      const uint32_t clamp = cpos ? 0xFFFFu : 0xFFFFFFFFu;
+      const uint32_t td = grp_kth_largest(ckey, count, lo, clamp, k, sh.rs, 0, pc, &need_eq, ct);
+      tau = lo + td;
+      if (cpos && td == clamp)
+        tau = grp_kth_largest(ckey, count, 0u, 0xFFFFFFFFu, k, sh.rs, 1, pc, &need_eq, ct);
+    }
     emit_selected(count, tau, need_eq, out, k, sh, ct, ckey, cpos);
   }
   __threadfence_block();
