@@ -77,6 +77,7 @@ class CompressKVError(RuntimeError):
 
 
 _LIB = None
+_FAST = {}
 
 
 def library_path() -> str:
@@ -126,8 +127,20 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
         fn = getattr(lib, name)
         fn.restype = res
         fn.argtypes = args
+        # the wrappers below pass plain addresses: a second prototype of the
+        # same function that takes them as integers
+        fast = lib[name]
+        fast.restype = res
+        fast.argtypes = [vp if a in (pp, i32p) else a for a in args]
+        _FAST[name] = fast
     _LIB = lib
     return lib
+
+
+def _fast(name: str):
+    if _LIB is None:
+        load()
+    return _FAST[name]
 
 
 def status_string(code: int) -> str:
@@ -149,6 +162,29 @@ def _stream(stream) -> c_void_p:
     if stream is None:
         stream = torch.cuda.current_stream()
     return c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+
+
+def _raw_stream(stream) -> int:
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
+
+
+def _addr(t):
+    return None if t is None else t.data_ptr()
+
+
+def _data(a: np.ndarray) -> int:
+    """Address of an array's first element (a.ctypes.data takes 1 us)."""
+    try:
+        return ctypes.addressof(ctypes.c_char.from_buffer(a))
+    except (TypeError, ValueError):  # read-only or empty
+        return a.ctypes.data
+
+
+def _host_i32(arr) -> np.ndarray:
+    """`arr` as contiguous int32 (kept alive by the caller over the C call)."""
+    return np.ascontiguousarray(arr, dtype=np.int32)
 
 
 def _i32(arr) -> tuple:
@@ -202,6 +238,10 @@ class Problem:
     @property
     def ref(self):
         return ctypes.byref(self.struct)
+
+    @property
+    def addr(self) -> int:
+        return ctypes.addressof(self.struct)
 
 
 class Trace:
@@ -263,12 +303,17 @@ def output_layout(problem: Problem, budgets):
     return cu_prefix, cu_out
 
 
-def _mask(srh_mask, problem: "Problem"):
-    """One layer's SRH mask as host bytes; the library reads num_q_heads of them."""
-    m = np.ascontiguousarray(np.asarray(srh_mask).astype(np.uint8).reshape(-1))
-    if m.size != int(problem.struct.num_q_heads):
-        raise CompressKVError(CKV_ERR_INVALID_ARG, "srh_mask must have num_q_heads entries")
-    return m, c_void_p(m.ctypes.data)
+def _mask(srh_mask, problem: "Problem", n_masks: int = 1):
+    """SRH masks as host bytes; the library reads n_masks * num_q_heads of them."""
+    m = np.asarray(srh_mask)
+    if m.dtype != np.uint8:
+        m = m.astype(np.uint8)
+    m = np.ascontiguousarray(m)
+    if n_masks >= 1 and m.size != n_masks * problem.struct.num_q_heads:
+        what = ("srh_mask must have num_q_heads entries" if n_masks == 1
+                else "srh_masks must be [n_masks, num_q_heads]")
+        raise CompressKVError(CKV_ERR_INVALID_ARG, what)
+    return m
 
 
 def _check_lse(problem: "Problem", lse_win, k, rows: int):
@@ -287,36 +332,37 @@ def _check_lse(problem: "Problem", lse_win, k, rows: int):
 
 
 def score(problem: Problem, q_win, k, srh_mask, raw, ws, stream=None):
-    m, mp = _mask(srh_mask, problem)
-    _check(load().compresskv_score(problem.ref, _ptr(q_win), _ptr(k), mp, _ptr(raw), _ptr(ws),
-                                   ws.numel(), _stream(stream)), "compresskv_score")
+    m = _mask(srh_mask, problem)
+    _check(_fast("compresskv_score")(problem.addr, _addr(q_win), _addr(k), _data(m),
+                                     _addr(raw), _addr(ws), ws.numel(), _raw_stream(stream)),
+           "compresskv_score")
 
 
 def select(problem: Problem, raw, budgets, indices, ws, pooled=None, stream=None) -> np.ndarray:
-    b, bp = _i32(budgets)
+    b = _host_i32(budgets)
     cu_out = np.zeros(problem.batch + 1, np.int32)
-    _check(load().compresskv_select(problem.ref, _ptr(raw), bp, _ptr(indices),
-                                    cu_out.ctypes.data_as(POINTER(c_int32)), _ptr(pooled),
-                                    _ptr(ws), ws.numel(), _stream(stream)), "compresskv_select")
+    _check(_fast("compresskv_select")(problem.addr, _addr(raw), _data(b), _addr(indices),
+                                      _data(cu_out), _addr(pooled), _addr(ws), ws.numel(),
+                                      _raw_stream(stream)), "compresskv_select")
     return cu_out
 
 
 def gather(problem: Problem, indices, cu_out, k, v, k_out, v_out, ws=None, stream=None):
-    c, cp = _i32(cu_out)
-    _check(load().compresskv_gather(problem.ref, _ptr(indices), cp, _ptr(k), _ptr(v),
-                                    _ptr(k_out), _ptr(v_out), _ptr(ws), _stream(stream)),
-           "compresskv_gather")
+    c = _host_i32(cu_out)
+    _check(_fast("compresskv_gather")(problem.addr, _addr(indices), _data(c), _addr(k),
+                                      _addr(v), _addr(k_out), _addr(v_out), _addr(ws),
+                                      _raw_stream(stream)), "compresskv_gather")
 
 
 def compress_layer(problem: Problem, q_win, k, v, srh_mask, budgets, indices, k_out, v_out, ws,
                    raw=None, pooled=None, stream=None) -> np.ndarray:
-    m, mp = _mask(srh_mask, problem)
-    b, bp = _i32(budgets)
+    m = _mask(srh_mask, problem)
+    b = _host_i32(budgets)
     cu_out = np.zeros(problem.batch + 1, np.int32)
-    _check(load().compresskv_compress_layer(
-        problem.ref, _ptr(q_win), _ptr(k), _ptr(v), mp, bp, _ptr(indices),
-        cu_out.ctypes.data_as(POINTER(c_int32)), _ptr(k_out), _ptr(v_out), _ptr(raw),
-        _ptr(pooled), _ptr(ws), ws.numel(), _stream(stream)), "compresskv_compress_layer")
+    _check(_fast("compresskv_compress_layer")(
+        problem.addr, _addr(q_win), _addr(k), _addr(v), _data(m), _data(b),
+        _addr(indices), _data(cu_out), _addr(k_out), _addr(v_out), _addr(raw), _addr(pooled),
+        _addr(ws), ws.numel(), _raw_stream(stream)), "compresskv_compress_layer")
     return cu_out
 
 
@@ -327,16 +373,14 @@ def compress_layers(problem: Problem, n_masks: int, q_win, k, v, srh_masks, budg
     ``[n_layers*B, H_q, W, d]``, cu_seqlens repeated per layer with offset
     l*T) and block l selects with ``srh_masks[l]`` (``[n_masks, H_q]``);
     budgets ``[n_layers*B]``; outputs as for compress_layer on that batch."""
-    m = np.ascontiguousarray(np.asarray(srh_masks).astype(np.uint8).reshape(-1))
-    if n_masks >= 1 and m.size != int(n_masks) * int(problem.struct.num_q_heads):
-        raise CompressKVError(CKV_ERR_INVALID_ARG, "srh_masks must be [n_masks, num_q_heads]")
-    b, bp = _i32(budgets)
+    n_masks = int(n_masks)
+    m = _mask(srh_masks, problem, n_masks)
+    b = _host_i32(budgets)
     cu_out = np.zeros(problem.batch + 1, np.int32)
-    _check(load().compresskv_compress_layers(
-        problem.ref, int(n_masks), _ptr(q_win), _ptr(k), _ptr(v), c_void_p(m.ctypes.data), bp,
-        _ptr(indices), cu_out.ctypes.data_as(POINTER(c_int32)), _ptr(k_out), _ptr(v_out),
-        _ptr(raw), _ptr(pooled), _ptr(ws), ws.numel(), _stream(stream)),
-        "compresskv_compress_layers")
+    _check(_fast("compresskv_compress_layers")(
+        problem.addr, n_masks, _addr(q_win), _addr(k), _addr(v), _data(m), _data(b),
+        _addr(indices), _data(cu_out), _addr(k_out), _addr(v_out), _addr(raw), _addr(pooled),
+        _addr(ws), ws.numel(), _raw_stream(stream)), "compresskv_compress_layers")
     return cu_out
 
 
@@ -345,13 +389,13 @@ def compress_layer_noalloc(problem: Problem, q_win, k, v, srh_mask, budgets, ind
                            stream=None) -> np.ndarray:
     """compress_layer without a workspace: the library's static scratch is
     used (for callers that cannot allocate device memory)."""
-    m, mp = _mask(srh_mask, problem)
-    b, bp = _i32(budgets)
+    m = _mask(srh_mask, problem)
+    b = _host_i32(budgets)
     cu_out = np.zeros(problem.batch + 1, np.int32)
-    _check(load().compresskv_compress_layer_noalloc(
-        problem.ref, _ptr(q_win), _ptr(k), _ptr(v), mp, bp, _ptr(indices),
-        cu_out.ctypes.data_as(POINTER(c_int32)), _ptr(k_out), _ptr(v_out), _ptr(raw),
-        _ptr(pooled), _ptr(device_status), _stream(stream)), "compresskv_compress_layer_noalloc")
+    _check(_fast("compresskv_compress_layer_noalloc")(
+        problem.addr, _addr(q_win), _addr(k), _addr(v), _data(m), _data(b),
+        _addr(indices), _data(cu_out), _addr(k_out), _addr(v_out), _addr(raw), _addr(pooled),
+        _addr(device_status), _raw_stream(stream)), "compresskv_compress_layer_noalloc")
     return cu_out
 
 
@@ -373,14 +417,14 @@ def compress_layer_lse(problem: Problem, q_win, k, v, lse_win, srh_mask, budgets
     """compress_layer with the window queries' log-sum-exp given:
     ``lse_win`` is a float32 ``[B, H_q, W]`` tensor (window rows contiguous)."""
     _check_lse(problem, lse_win, k, problem.batch)
-    m, mp = _mask(srh_mask, problem)
-    b, bp = _i32(budgets)
+    m = _mask(srh_mask, problem)
+    b = _host_i32(budgets)
     cu_out = np.zeros(problem.batch + 1, np.int32)
-    _check(load().compresskv_compress_layer_lse(
-        problem.ref, _ptr(q_win), _ptr(k), _ptr(v), _ptr(lse_win), lse_win.stride(0),
-        lse_win.stride(1), mp, bp, _ptr(indices), cu_out.ctypes.data_as(POINTER(c_int32)),
-        _ptr(k_out), _ptr(v_out), _ptr(raw), _ptr(pooled), _ptr(ws), ws.numel(), _stream(stream)),
-        "compresskv_compress_layer_lse")
+    _check(_fast("compresskv_compress_layer_lse")(
+        problem.addr, _addr(q_win), _addr(k), _addr(v), _addr(lse_win), lse_win.stride(0),
+        lse_win.stride(1), _data(m), _data(b), _addr(indices), _data(cu_out),
+        _addr(k_out), _addr(v_out), _addr(raw), _addr(pooled), _addr(ws), ws.numel(),
+        _raw_stream(stream)), "compresskv_compress_layer_lse")
     return cu_out
 
 
@@ -390,16 +434,15 @@ def compress_layers_lse(problem: Problem, n_masks: int, q_win, k, v, lse_win, sr
     """compress_layers with the window queries' log-sum-exp given, packed like
     the batch: ``lse_win`` is float32 ``[n_layers*B, H_q, W]``."""
     _check_lse(problem, lse_win, k, problem.batch)
-    m = np.ascontiguousarray(np.asarray(srh_masks).astype(np.uint8).reshape(-1))
-    if n_masks >= 1 and m.size != int(n_masks) * int(problem.struct.num_q_heads):
-        raise CompressKVError(CKV_ERR_INVALID_ARG, "srh_masks must be [n_masks, num_q_heads]")
-    b, bp = _i32(budgets)
+    n_masks = int(n_masks)
+    m = _mask(srh_masks, problem, n_masks)
+    b = _host_i32(budgets)
     cu_out = np.zeros(problem.batch + 1, np.int32)
-    _check(load().compresskv_compress_layers_lse(
-        problem.ref, int(n_masks), _ptr(q_win), _ptr(k), _ptr(v), _ptr(lse_win),
-        lse_win.stride(0), lse_win.stride(1), c_void_p(m.ctypes.data), bp, _ptr(indices),
-        cu_out.ctypes.data_as(POINTER(c_int32)), _ptr(k_out), _ptr(v_out), _ptr(raw),
-        _ptr(pooled), _ptr(ws), ws.numel(), _stream(stream)), "compresskv_compress_layers_lse")
+    _check(_fast("compresskv_compress_layers_lse")(
+        problem.addr, n_masks, _addr(q_win), _addr(k), _addr(v), _addr(lse_win),
+        lse_win.stride(0), lse_win.stride(1), _data(m), _data(b), _addr(indices),
+        _data(cu_out), _addr(k_out), _addr(v_out), _addr(raw), _addr(pooled), _addr(ws),
+        ws.numel(), _raw_stream(stream)), "compresskv_compress_layers_lse")
     return cu_out
 
 
@@ -425,14 +468,13 @@ def compress_layer_head_budgets(problem: Problem, q_win, k, v, srh_mask, group_b
     """compress_layer with a budget per (sequence, KV group): ``group_budgets``
     is ``[B, H_kv]``; outputs are packed group-major (see head_budget_layout);
     returns cu_out ``[H_kv, B+1]``."""
-    m, mp = _mask(srh_mask, problem)
-    b, bp = _i32(np.asarray(group_budgets).reshape(-1))
+    m = _mask(srh_mask, problem)
+    b = _host_i32(group_budgets)
     cu_out = np.zeros((problem.num_kv_heads, problem.batch + 1), np.int32)
-    _check(load().compresskv_compress_layer_head_budgets(
-        problem.ref, _ptr(q_win), _ptr(k), _ptr(v), mp, bp, _ptr(indices),
-        cu_out.ctypes.data_as(POINTER(c_int32)), _ptr(k_out), _ptr(v_out), _ptr(raw),
-        _ptr(pooled), _ptr(ws), ws.numel(), _stream(stream)),
-        "compresskv_compress_layer_head_budgets")
+    _check(_fast("compresskv_compress_layer_head_budgets")(
+        problem.addr, _addr(q_win), _addr(k), _addr(v), _data(m), _data(b),
+        _addr(indices), _data(cu_out), _addr(k_out), _addr(v_out), _addr(raw), _addr(pooled),
+        _addr(ws), ws.numel(), _raw_stream(stream)), "compresskv_compress_layer_head_budgets")
     return cu_out
 
 

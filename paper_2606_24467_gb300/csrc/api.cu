@@ -925,7 +925,8 @@ int run_gather(const ckv_problem* p, const Info& I, const int32_t* indices,
 // rows of its widest group, and by nothing else of the call, so that a layer
 // gives the same bits alone or among others; a call with layers of both kinds
 // launches both.  (The prompts of one layer go together: taking a 28-layer
-// batch's shorter prompts apart cost two tails, 3195 -> 3285 us.)  Two-pass / resident time in us (1 layer; 32 layers; 8 KV heads):
+// batch's shorter prompts apart cost two tails, 3195 -> 3285 us.)
+// Two-pass / resident time in us (1 layer; 32 layers; 8 KV heads):
 //   32 rows      16384: 85/67, 568/319    32768: 98/90, 699/586
 //                65536: 128/135
 //   32, LSE      16384: 66/65, 348/277    24576: 71/75, 381/395
