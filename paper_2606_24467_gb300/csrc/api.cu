@@ -1078,11 +1078,10 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   const int nwg = 2;  // epilogue warpgroups that take tiles
   const int nbuf = 512 / tstride;
   // three Q buffers when they fit beside a ring of at least four K tiles,
-  // else two beside at least two; an even number of stages (each UMMA warp
-  // has half of them)
+  // else two beside at least two
   int stages = 0, q_bufs = 0;
   for (int nq = 3; nq >= 2 && stages == 0; --nq) {
-    for (int st = 8; st >= (nq == 3 ? 4 : 2); st -= 2) {
+    for (int st = 8; st >= (nq == 3 ? 4 : 2); --st) {
       if (fused_smem_bytes(q_half, nq, st, row_stride, nwg) <=
           static_cast<size_t>(Fd->smem_optin)) {
         stages = st;

@@ -162,7 +162,7 @@ constexpr size_t kFusedCtrBytes = static_cast<size_t>(kFusedCtrHead + 3 * kFused
 // raw-score row); with it the merge / select region leaves room for two Q
 // buffers of 192 query rows (W = 64 with three SRH heads) and two K stages
 constexpr int kFusedCandCap = 3072;
-constexpr int kFusedCRegion = 32 * 1024;  // shared memory of the merge / select warps
+constexpr int kSelRegion = 38 * 1024;  // shared memory of the merge / select warps
 
 struct FusedParams {
   CUtensorMap tmap_k;          // 3-D map over K: (d, kv head, token)
@@ -222,7 +222,6 @@ constexpr int kAccWords = 8;            // 64-bit accumulator words per unit and
 constexpr int kPairRing = 20;           // chunk sums a CTA keeps (more than it holds in tensor memory)
 constexpr int kResidentMaxGrid = 152;   // CTAs, at most
 constexpr int kResidentMaxRows = 192;   // query rows of a group, at most
-constexpr int kSelRegion = 38 * 1024;   // shared memory of the select warps
 
 struct ResidentParams {
   CUtensorMap tmap_k;          // 3-D map over K: (d, kv head, token)

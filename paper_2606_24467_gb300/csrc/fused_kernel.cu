@@ -10,20 +10,19 @@
 // D_q = sum_{j <= p_q} 2^(z_qj c).  The kernel makes two passes over the
 // unit's K, both on tcgen05 tensor cores (logits in TMEM):
 //   pass 1  per query row and epilogue warpgroup the pair (M, S) with
-//           sum 2^(z c) = S 2^M over its tiles of a chunk of kChunkTiles K tiles (the epilogue keeps a reference R
-//           per warp and query, 7 below the largest scaled logit it has seen,
-//           and sums 2^(z c - R) exactly as the scoring kernel of the
-//           separate path does); the workers merge a unit's pairs into
-//           log2 D_q once every chunk of the unit is in;
+//           sum 2^(z c) = S 2^M over its tiles of a chunk of kChunkTiles K
+//           tiles (each epilogue warp sums 2^(z c - R) against a reference R
+//           per query row, its first scaled logit, raised when a sum passes
+//           2^64); the workers merge a unit's pairs into log2 D_q once every
+//           chunk of the unit is in;
 //   pass 2  raw_j = sum_q 2^(z_qj c - log2 D_q) over the unit's prefix keys
 //           j < n = L - W, straight from the logits in fp32; pass 2 of a
 //           chunk is published only once its unit's denominators are merged
 //           (it reads K again: in long calls pass 1 runs too far ahead for
 //           L2 to keep it, so mostly from DRAM);
-// then pooled_j = (sum_{t=-h..h} raw_{j+t}) / P with zeros outside [0, n)
-// (inside a chunk by the epilogue from shared memory, within h of a chunk
-// edge by the select), the k = kept - W largest pooled scores (ties to the
-// lower position) in ascending position, the window, and the K/V rows.
+// then (unit_select.cuh) pooled_j = (sum_{t=-h..h} raw_{j+t}) / P with zeros
+// outside [0, n), the k = kept - W largest pooled scores (ties to the lower
+// position) in ascending position, the window, and the K/V rows.
 // With the window queries' log-sum-exp given (given_lse) pass 1 is skipped
 // and log2 D_q = LSE_q * log2(e).
 //
@@ -33,14 +32,12 @@
 //               up to kDescs ahead, in a descriptor ring;
 //   warp 0      loads each chunk's SRH query rows (one TMA box of W rows per
 //               head and 64-column half) into one of two or three Q buffers
-//               and streams its K tiles, by TMA, into a shared-memory ring
-//               split in two sub-rings, one per UMMA warp (each consumes
-//               its own in order);
-//   warps 1, 2  UMMA issue (M = 128 keys, N = query rows), warp 1 for the
-//               tiles of warpgroup 0 and warp 2 for those of warpgroup 1
-//               (a UMMA of this shape holds the tensor core for a fixed 76
-//               cycles whatever N up to 128, so two issuing threads, each
-//               with its own waits, keep it fed); warp 1 also allocates TMEM;
+//               and streams its K tiles, by TMA, into a shared-memory ring;
+//   warp 1      UMMA issue (M = 128 keys, N = query rows) in tile order, by
+//               the whole warp with one lane issuing, and the TMEM
+//               allocation.  (Two issuers, one per warpgroup, interleaved
+//               their UMMAs, so that both warpgroups' tiles came late and at
+//               the same time, and tensor-memory loads queued behind them.)
 //   warps 4-11  two epilogue warpgroups; tile t of a chunk belongs to
 //               warpgroup t % nwg (nwg = 2), each with its own TMEM buffers;
 //   warps 12-19 workers: they merge a unit's pass-1 pairs into its
@@ -55,6 +52,11 @@
 // is bounded (FusedParams::wait_ns, kWaitTimeoutNs unless a test shortens it)
 // and on expiry records CKV_ERR_DEVICE_TIMEOUT
 // and stops the call.
+// What bounds it: up to 64 query rows DRAM, both passes' reads (32 layers of
+// 32768 tokens, 680 us); 128 and 192 rows the epilogue and, with few K stages
+// beside the Q buffers, the loads' latency (16 layers of 32768 tokens: 433 and
+// 649 us, 567 and 911 with one logit per register and key-per-lane sums and
+// two UMMA issuers).
 // References restart at every chunk and tile t of a chunk always goes to
 // warpgroup t % nwg, so the scores depend only on the chunk grid (fixed per
 // unit), not on which CTA ran a chunk or what else the call holds.
@@ -64,7 +66,8 @@
 #include <cfloat>
 
 #include "ckv_device.cuh"
-#include "select_common.cuh"
+#include "tile_math.cuh"
+#include "unit_select.cuh"
 
 namespace ckv {
 
@@ -74,17 +77,13 @@ constexpr int kFWarps = 20;
 constexpr int kFThreads = 32 * kFWarps;
 constexpr int kProdWarp = 0;
 constexpr int kMmaWarp = 1;
-constexpr int kMmaWarp2 = 2;  // second UMMA issuer (tiles of warpgroup 1)
 constexpr int kClaimWarp = 3;
 constexpr int kEpiWarp0 = 4;  // warps 4..11: two warpgroups (TMEM lane quarter = warp % 4)
 constexpr int kEpiWarps = 8;
 constexpr int kCWarp0 = 12;   // warps 12..19
-constexpr int kCThreads = 256;
 constexpr int kDescs = 2;     // chunk descriptors in flight (claimed ahead; 2 measured faster than 4)
 constexpr int kNwg = 2;       // epilogue warpgroups that take tiles (tile t of a chunk: t % 2)
-constexpr int kSelSamples = 1024;  // samples of a unit's pooled scores for the select threshold
 constexpr int kPub = 6;       // chunks written, not yet published (publish ring)
-constexpr int kBarC = 3;      // named barrier of the worker warps
 constexpr float kShift = 7.0f;
 constexpr float kRaiseSum = 18446744073709551616.0f;  // 2^64: fp32 column sums stay below it before R is raised
 constexpr float kNegInf = -INFINITY;
@@ -106,26 +105,14 @@ struct ChunkDesc {
   int end, pass, s, g, t0, t1, chunk, n_rows;
 };
 
-// Shared memory of the worker warps (a merge or a selection at a time).
-struct SelShared {
-  uint32_t key[kFusedCandCap];
-  int pos[kFusedCandCap];
-  RadixShared rs;
-  int wcnt[8], wbase[8];
-  int wcnt_ge[8];  // per-warp counts at the best threshold with at least k keys above
-  int flag[4];
-  uint32_t lo;
-};
-static_assert(sizeof(SelShared) <= kFusedCRegion, "select scratch");
-static_assert(kSelSamples <= kFusedCandCap, "samples live in the position array");
-static_assert(3 * kMaxQRows * 4 + 16 <= kFusedCRegion, "merge scratch");
+static_assert(3 * kMaxQRows * 4 + 16 <= kSelRegion, "merge scratch");
 
 constexpr int kWposBytes = kMaxQRows * 4;
-constexpr int kChunkBufBytes = 2 * kChunkKeys * 4;  // raw scores of two pass-2 chunks
 constexpr int kBarBytes = 512;
 static_assert((51 + 2 * kPub) * 8 <= kBarBytes, "mbarriers (the publish ring's last) fit their block");
-constexpr int kMiscBytes = 256;  // TMEM address, abort flag, task
-constexpr int kFixedBytes = kWposBytes + kChunkBufBytes + kBarBytes + kMiscBytes +
+constexpr int kMiscBytes = 256;  // TMEM address, abort flag, task, the selection's parameters
+static_assert(64 + sizeof(SelCall) <= kMiscBytes, "misc block");
+constexpr int kFixedBytes = kWposBytes + kBarBytes + kMiscBytes +
                             kDescs * static_cast<int>(sizeof(ChunkDesc));
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
@@ -136,8 +123,6 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 __device__ __forceinline__ int ld_volatile(const int* p) {
   return *reinterpret_cast<const volatile int*>(p);
 }
-
-__device__ __forceinline__ void cbar() { named_bar_sync(kBarC, kCThreads); }
 
 // Index of the i-th set bit of `bits` (i < popc(bits)).
 __device__ __forceinline__ int nth_bit(uint32_t bits, int i) {
@@ -377,392 +362,6 @@ __device__ __noinline__ void merge_unit(const Fused& F, int u, uint8_t* creg, in
   if (ct == 0) atomicExch(F.bias_state(u), 2);
 }
 
-// ---------------------------------------------------------------- select
-// Zero the radix state (the workers' form of radix_init).
-__device__ __forceinline__ void radix_init_grp(RadixShared& sh, int ct) {
-  for (int i = ct; i < 2 * 256; i += kCThreads) sh.hist[i >> 8][i & 255] = 0u;
-  if (ct < 2) {
-    sh.key_or[ct] = 0u;
-    sh.key_and[ct] = 0xFFFFFFFFu;
-  }
-}
-
-// The workers' form of cta_kth_largest (256 threads, named barrier): the
-// r-th largest of min(keys[j] - sub, clamp), j < count; *rem = how many of
-// the keys equal to it are among the r largest.
-__device__ __noinline__ uint32_t grp_kth_largest(const uint32_t* keys, int count, uint32_t sub,
-                                                 uint32_t clamp, int r, RadixShared& sh, int slot,
-                                                 int& pc, int* rem, int ct, bool global_keys) {
-  const int lane = ct & 31;
-  const int iters = (count + 255) >> 8;
-  auto key_at = [&](int j) -> uint32_t {
-    const uint32_t k = global_keys ? __ldcg(keys + j) : keys[j];
-    return min(k - sub, clamp);
-  };
-  uint32_t ko = 0u, ka = 0xFFFFFFFFu;
-#pragma unroll 4
-  for (int i = 0; i < iters; ++i) {
-    const int j = (i << 8) + ct;
-    if (j < count) {
-      const uint32_t key = key_at(j);
-      ko |= key;
-      ka &= key;
-    }
-  }
-  ko = __reduce_or_sync(0xffffffffu, ko);
-  ka = __reduce_and_sync(0xffffffffu, ka);
-  if (lane == 0) {
-    atomicOr(&sh.key_or[slot], ko);
-    atomicAnd(&sh.key_and[slot], ka);
-  }
-  cbar();
-  const uint32_t diff = sh.key_or[slot] ^ sh.key_and[slot];
-  const uint32_t kand = sh.key_and[slot];
-  int remaining = r;
-  if (diff == 0u) {
-    *rem = remaining;
-    return kand;
-  }
-  int hb = 31 - __clz(diff);
-  uint32_t pmask = hb == 31 ? 0u : ~((2u << hb) - 1u);
-  uint32_t prefix = kand & pmask;
-#pragma unroll 1
-  while (hb >= 0) {
-    const int width = min(8, hb + 1);
-    const int shf = hb + 1 - width;
-    const uint32_t fm = (1u << width) - 1u;
-    uint32_t* hh = sh.hist[pc & 3];
-    constexpr int kB = 8;  // keys per thread loaded before they are counted
-#pragma unroll 1
-    for (int i0 = 0; i0 < iters; i0 += kB) {
-      uint32_t kv[kB];
-#pragma unroll
-      for (int q = 0; q < kB; ++q) {
-        const int j = ((i0 + q) << 8) + ct;
-        kv[q] = j < count ? key_at(j) : 0u;
-      }
-#pragma unroll
-      for (int q = 0; q < kB; ++q) {
-        const int j = ((i0 + q) << 8) + ct;
-        const uint32_t key = kv[q];
-        const bool m = j < count && (key & pmask) == prefix;
-        const uint32_t act = __ballot_sync(0xffffffffu, m);
-        if (!act) continue;
-        const uint32_t bin = (key >> shf) & fm;
-        const int leader = __ffs(act) - 1;
-        const uint32_t lb = __shfl_sync(0xffffffffu, bin, leader);
-        if (__all_sync(0xffffffffu, !m || bin == lb)) {
-          if (lane == leader) atomicAdd(&hh[lb], static_cast<uint32_t>(__popc(act)));
-        } else if (m) {
-          // one add per distinct bin of the warp (no same-address serialisation)
-          const uint32_t same = __match_any_sync(act, bin);
-          if (lane == __ffs(same) - 1) atomicAdd(&hh[bin], static_cast<uint32_t>(__popc(same)));
-        }
-      }
-    }
-    sh.hist[(pc + 2) & 3][ct] = 0u;
-    cbar();
-    int bin, above;
-    warp_pick_bin256(hh, remaining, lane, &bin, &above);
-    remaining -= above;
-    prefix |= static_cast<uint32_t>(bin) << shf;
-    pmask |= fm << shf;
-    hb = shf - 1;
-    ++pc;
-  }
-  *rem = remaining;
-  return prefix;
-}
-
-// Ordered emission of the selected entries of a key list in position order:
-// entry j (key key_at(j), position pos_at(j)) is selected when its key is
-// above tau, or equal to tau and fewer than need_eq equal keys precede it.
-// Selected entries go to out[0..k) in list order.
-template <class KeyAt, class PosAt>
-__device__ void emit_selected(int count, uint32_t tau, int need_eq, int32_t* out, int k,
-                              SelShared& sh, int ct, KeyAt key_at, PosAt pos_at) {
-  const int cw = ct >> 5;
-  const int lane = ct & 31;
-  int o = 0, eq_seen = 0;
-  uint32_t next = ct < count ? key_at(ct) : 0u;  // one block of keys loaded ahead
-  for (int j0 = 0; j0 < count; j0 += kCThreads) {
-    const int j = j0 + ct;
-    const bool in = j < count;
-    const uint32_t key = next;
-    if (j + kCThreads < count) next = key_at(j + kCThreads);
-    const bool gt = in && key > tau;
-    const bool eq = in && key == tau;
-    const uint32_t mgt = __ballot_sync(0xffffffffu, gt);
-    const uint32_t meq = __ballot_sync(0xffffffffu, eq);
-    if (lane == 0) {
-      sh.wcnt[cw] = __popc(mgt);
-      sh.wbase[cw] = __popc(meq);
-    }
-    cbar();
-    int gtb = 0, eqb = 0, gtt = 0, eqt = 0;
-    for (int w = 0; w < 8; ++w) {
-      if (w < cw) {
-        gtb += sh.wcnt[w];
-        eqb += sh.wbase[w];
-      }
-      gtt += sh.wcnt[w];
-      eqt += sh.wbase[w];
-    }
-    const int eq_rank = eq_seen + eqb + __popc(meq & lanemask_lt(lane));
-    const bool take_eq = eq && eq_rank < need_eq;
-    const uint32_t msel = mgt | __ballot_sync(0xffffffffu, take_eq);
-    const int eq_taken_before = max(0, min(need_eq - eq_seen, eqb));
-    const int slot = o + gtb + eq_taken_before + __popc(msel & lanemask_lt(lane));
-    if (((msel >> lane) & 1u) && slot < k) out[slot] = pos_at(j);
-    o += gtt + max(0, min(need_eq - eq_seen, eqt));
-    eq_seen += eqt;
-    cbar();
-  }
-}
-
-// Copy the K and V rows of out[0..count) (positions in the sequence) to the
-// compressed cache rows out0 .. out0 + count - 1 of group g.  Eight 16-byte
-// loads in flight per thread: a batch's positions are loaded first, then its
-// rows, and a position outside the sequence (never, for a correct selection)
-// is skipped and recorded after the batch, so no load waits behind another.
-__device__ __noinline__ void gather_rows(const FusedParams& p, int seq0, int L, int g,
-                                         const int32_t* out, int out0, int count, int ct) {
-  constexpr int kChunks = 2 * kHeadDim * 2 / 16;  // 16 K + 16 V chunks per token
-  constexpr int kBatch = 8;
-  const int total = count * kChunks;
-  bool bad = false;
-  for (int base = 0; base < total; base += kBatch * kCThreads) {
-    int tok[kBatch];
-#pragma unroll
-    for (int k = 0; k < kBatch; ++k) {
-      const int e = base + k * kCThreads + ct;
-      tok[k] = e < total ? out[e / kChunks] : 0;
-    }
-    uint4 v[kBatch];
-    long long dst[kBatch];
-    bool is_v[kBatch];
-#pragma unroll
-    for (int k = 0; k < kBatch; ++k) {
-      const int e = base + k * kCThreads + ct;
-      const int i = e / kChunks;
-      const int ch = e - i * kChunks;
-      const bool ok = e < total && tok[k] >= 0 && tok[k] < L;
-      bad |= e < total && !ok;
-      is_v[k] = ch >= kChunks / 2;
-      const int part = ch & (kChunks / 2 - 1);
-      const long long src = static_cast<long long>(seq0 + (ok ? tok[k] : 0)) * p.tok_stride_v16 +
-                            static_cast<long long>(g) * p.head_stride_v16 + part;
-      dst[k] = ok ? (static_cast<long long>(out0 + i) * p.num_kv_heads + g) * (kHeadDim * 2 / 16) +
-                        part
-                  : -1;
-      if (ok) v[k] = __ldg((is_v[k] ? p.v : p.k) + src);
-    }
-#pragma unroll
-    for (int k = 0; k < kBatch; ++k)
-      if (dst[k] >= 0) (is_v[k] ? p.v_out : p.k_out)[dst[k]] = v[k];
-  }
-  if (bad) atomicCAS(p.status, 0, CKV_DEV_ERR_INDEX);
-}
-
-// Pooled score of prefix key j from the raw scores (zeros outside [0, n)),
-// summed in the order the epilogue's chunk pooling uses.
-__device__ __forceinline__ float pool_from_global(const float* raw, int n, int j, int h,
-                                                  float fP) {
-  float acc = 0.f;
-  for (int t = 0; t <= 2 * h; ++t) {
-    const int jj = j - h + t;
-    acc += (jj >= 0 && jj < n) ? __ldcg(raw + jj) : 0.f;
-  }
-  return acc / fP;
-}
-
-// Selection of unit u.  First the pooled scores within h of a chunk edge
-// (the epilogue pooled each chunk's interior), then the top-k by a sampled
-// lower bound: candidates in position order, an exact radix search among
-// them (among all the unit's scores when the bound keeps too few or too
-// many), the window, and the K/V rows.  Pooled scores are >= 0: their bit
-// patterns order like their values.
-__device__ __noinline__ void select_unit(const Fused& F, int u, uint8_t* creg, int ct) {
-  const FusedParams& p = F.p;
-  SelShared& sh = *reinterpret_cast<SelShared*>(creg);
-  const int cw = ct >> 5;
-  const int lane = ct & 31;
-  const int s = u / p.num_kv_heads;
-  const int g = u - s * p.num_kv_heads;
-  const int seq0 = p.cu_seqlens[s];
-  const int L = F.len(s);
-  const int W = p.window;
-  const int n = F.prefix(s);
-  if (n > 0 && F.chunks_per_unit(s) == 0) return;  // not of this launch
-  const int out0 = p.cu_out[s];
-  const int kept = p.cu_out[s + 1] - out0;
-  const long long soff = static_cast<long long>(g) * p.p_total + p.cu_prefix[s];
-  float* pooled = p.pooled + soff;
-  const int h = (p.pool_width - 1) >> 1;
-  const float fP = static_cast<float>(p.pool_width);
-  // chunk-edge pooled scores: [a, a + h) and [b - h, b) of every chunk
-  if (h > 0 && n > 0) {
-    const float* raw = p.raw + soff;
-    const int nct = (n + kChunkKeys - 1) / kChunkKeys;
-    for (int e = ct; e < nct * 2 * h; e += kCThreads) {
-      const int c = e / (2 * h);
-      const int o = e - c * 2 * h;
-      const int a = c * kChunkKeys;
-      const int b = min(a + kChunkKeys, n);
-      const int lo_end = min(a + h, b);
-      const int hi_start = max(b - h, lo_end);
-      const int j = o < h ? a + o : hi_start + (o - h);
-      if (o < h ? j < lo_end : j < b) pooled[j] = pool_from_global(raw, n, j, h, fP);
-    }
-    __threadfence();
-  }
-  cbar();
-  if (!p.do_select) return;
-  int32_t* out = p.indices + static_cast<long long>(g) * p.o_total + out0;
-  if (kept >= L) {  // keep everything
-    for (int i = ct; i < L; i += kCThreads) out[i] = i;
-    __threadfence_block();
-    cbar();
-    gather_rows(p, seq0, L, g, out, out0, L, ct);
-    return;
-  }
-  const int k = kept - W;  // 0 <= k < n
-  for (int w = ct; w < W; w += kCThreads) out[k + w] = n + w;
-  if (k == 0) {
-    __threadfence_block();
-    cbar();
-    gather_rows(p, seq0, L, g, out, out0, W, ct);
-    return;
-  }
-  const uint32_t* keys = reinterpret_cast<const uint32_t*>(pooled);
-  // threshold lo: the rs-th largest of ns samples spread over the unit,
-  // chosen so that the keys >= lo are at least k and at most the shared
-  // candidate capacity; the samples sit in the (not yet used) position array
-  uint32_t* samp = reinterpret_cast<uint32_t*>(sh.pos);
-  const int ns = min(kSelSamples, n);
-  for (int i = ct; i < ns; i += kCThreads)
-    samp[i] = __ldcg(keys + static_cast<int>((static_cast<long long>(i) * n) / ns));
-  radix_init_grp(sh.rs, ct);
-  cbar();
-  int pc = 0, need_eq = 0;
-  const float mu = static_cast<float>(k) * static_cast<float>(ns) / static_cast<float>(n);
-  int rs = min(ns, static_cast<int>(ceilf(mu + 3.f * sqrtf(mu))) + 2);
-  uint32_t lo = 0, lo_ge = 0;
-  int total = 0, tot_ge = -1;
-  constexpr int kU = 8;  // loads in flight per lane
-  const int seg = ((n + 8 * 32 * kU - 1) / (8 * 32 * kU)) * 32 * kU;  // positions per warp
-  const int wlo = min(n, cw * seg);
-  const int whi = min(n, wlo + seg);
-  bool fast = false;
-  for (int attempt = 0; attempt < 2; ++attempt) {
-    // (same sample set every attempt: the radix's OR/AND of slot 0 stay valid)
-    lo = grp_kth_largest(samp, ns, 0u, 0xFFFFFFFFu, rs, sh.rs, 0, pc, &need_eq, ct, false);
-    int wc = 0;
-    for (int b0 = wlo; b0 < whi; b0 += 32 * kU) {
-      uint32_t kv[kU];
-#pragma unroll
-      for (int q = 0; q < kU; ++q) {
-        const int i = b0 + q * 32 + lane;
-        kv[q] = i < whi ? __ldcg(keys + i) : 0u;
-      }
-#pragma unroll
-      for (int q = 0; q < kU; ++q)
-        wc += __popc(__ballot_sync(0xffffffffu, b0 + q * 32 + lane < whi && kv[q] >= lo));
-    }
-    if (lane == 0) sh.wcnt[cw] = wc;
-    cbar();
-    total = 0;
-    for (int w = 0; w < 8; ++w) total += sh.wcnt[w];
-    if (total >= k && (tot_ge < 0 || total < tot_ge)) {
-      lo_ge = lo;
-      tot_ge = total;
-      if (ct < 8) sh.wcnt_ge[ct] = sh.wcnt[ct];
-    }
-    if (total >= k && total <= kFusedCandCap) {
-      fast = true;
-      break;
-    }
-    // aim at the middle of [k, capacity] from the density this attempt saw
-    const float per = static_cast<float>(max(total, 1)) / static_cast<float>(rs);
-    int want = static_cast<int>(ceilf(0.5f * static_cast<float>(k + kFusedCandCap) / per));
-    want = total < k ? max(want, rs + 1) : min(want, rs - 1);
-    if (want < 1 || want > ns || want == rs) break;
-    rs = want;
-    cbar();  // every thread has read the counts
-  }
-  // the candidates' radix starts afresh
-  radix_init_grp(sh.rs, ct);
-  pc = 0;
-  need_eq = 0;
-  cbar();
-  // The candidates (keys >= lo) in position order: in shared memory when at
-  // most kFusedCandCap, else -- when the raw scores are workspace the select
-  // no longer reads (the chunk edges above were its last use) -- in the
-  // unit's raw-score row, keys in its first half and positions in its second.
-  uint32_t* ckey = sh.key;
-  int* cpos = sh.pos;
-  bool cglob = false;
-  if (!fast && p.raw_scratch && tot_ge >= k && tot_ge <= n / 2) {
-    lo = lo_ge;
-    total = tot_ge;
-    ckey = reinterpret_cast<uint32_t*>(p.raw + soff);
-    cpos = reinterpret_cast<int*>(ckey + n / 2);
-    cglob = true;
-    if (ct < 8) sh.wcnt[ct] = sh.wcnt_ge[ct];
-    cbar();
-    fast = true;
-  }
-  uint32_t tau;
-  if (fast) {
-    int o = 0;
-    for (int w = 0; w < cw; ++w) o += sh.wcnt[w];
-    for (int b0 = wlo; b0 < whi; b0 += 32 * kU) {
-      uint32_t kv[kU];
-#pragma unroll
-      for (int q = 0; q < kU; ++q) {
-        const int i = b0 + q * 32 + lane;
-        kv[q] = i < whi ? __ldcg(keys + i) : 0u;
-      }
-#pragma unroll
-      for (int q = 0; q < kU; ++q) {
-        const int i = b0 + q * 32 + lane;
-        const bool c = i < whi && kv[q] >= lo;
-        const uint32_t mm = __ballot_sync(0xffffffffu, c);
-        const int slot = o + __popc(mm & lanemask_lt(lane));
-        if (c && slot < total) {
-          ckey[slot] = kv[q];
-          cpos[slot] = i;
-        } else if (c) {  // more keys above lo than counted: cannot happen; record
-          atomicCAS(p.status, 0, CKV_DEV_ERR_INDEX);
-        }
-        o += __popc(mm);
-      }
-    }
-    if (cglob) __threadfence_block();
-    cbar();
-    constexpr uint32_t kClamp = 0xFFFFu;
-    const uint32_t td = grp_kth_largest(ckey, total, lo, kClamp, k, sh.rs, 0, pc, &need_eq, ct,
-                                        cglob);
-    tau = lo + td;
-    if (td == kClamp)
-      tau = grp_kth_largest(ckey, total, 0u, 0xFFFFFFFFu, k, sh.rs, 1, pc, &need_eq, ct, cglob);
-    if (cglob) {
-      emit_selected(total, tau, need_eq, out, k, sh, ct, [&](int j) { return __ldcg(ckey + j); },
-                    [&](int j) { return __ldcg(cpos + j); });
-    } else {
-      emit_selected(total, tau, need_eq, out, k, sh, ct, [&](int j) { return ckey[j]; },
-                    [&](int j) { return cpos[j]; });
-    }
-  } else {
-    tau = grp_kth_largest(keys, n, 0u, 0xFFFFFFFFu, k, sh.rs, 1, pc, &need_eq, ct, true);
-    emit_selected(n, tau, need_eq, out, k, sh, ct, [&](int j) { return __ldcg(keys + j); },
-                  [&](int j) { return j; });
-  }
-  __threadfence_block();
-  cbar();  // the indices written above are read back by the copy
-  gather_rows(p, seq0, L, g, out, out0, kept, ct);
-}
-
 // The workers' next task (one thread): the next unit to select once all its
 // pass-2 chunks are in, else the next unit to merge once all its pass-1
 // chunks are in; waits (bounded) while neither is ready.
@@ -858,13 +457,13 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
   float* sRef = reinterpret_cast<float*>(sQ + 2 * nqb * qh);  // [nrow][rstride]
   float* sAcc = sRef + nrow * rstride;                        // [nrow][rstride]
   int* sWpos = reinterpret_cast<int*>(sAcc + nrow * rstride);
-  float* sChunk = reinterpret_cast<float*>(sWpos + kMaxQRows);  // [2][kChunkKeys]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sChunk + 2 * kChunkKeys);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sWpos + kMaxQRows);
   uint8_t* misc = reinterpret_cast<uint8_t*>(bars) + kBarBytes;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(misc);
   int* abort_cta = reinterpret_cast<int*>(misc + 4);
   int* s_task = reinterpret_cast<int*>(misc + 16);
   int* s_last = reinterpret_cast<int*>(misc + 32);
+  SelCall& sel = *reinterpret_cast<SelCall*>(misc + 64);
   ChunkDesc* descs = reinterpret_cast<ChunkDesc*>(misc + kMiscBytes);
   uint8_t* creg = reinterpret_cast<uint8_t*>(descs + kDescs);
 
@@ -878,7 +477,6 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
   auto qfull = [&](int i) { return bar0 + 8u * (40 + i); };     // Q buffer staged
   auto qempty = [&](int i) { return bar0 + 8u * (43 + i); };    // Q buffer's MMAs done
   auto wgbar = [&](int w) { return bar0 + 8u * (46 + w); };     // epilogue warpgroup sync
-  const uint32_t epibar = bar0 + 8u * 50;                       // all epilogue warps
   auto pubfull = [&](int i) { return bar0 + 8u * (51 + i); };   // chunk's results written
   auto pubempty = [&](int i) { return bar0 + 8u * (51 + kPub + i); };  // chunk published
 
@@ -899,19 +497,20 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
     }
     for (int i = 0; i < kDescs; ++i) {
       mbar_init(dfull(i), 1);
-      mbar_init(dempty(i), 3 + kEpiWarps);  // TMA producer, both MMA warps, epilogue warps
+      mbar_init(dempty(i), 2 + kEpiWarps);  // TMA producer, UMMA warp, epilogue warps
     }
     for (int i = 0; i < 3; ++i) {
       mbar_init(qfull(i), 1);
-      mbar_init(qempty(i), 2);  // one commit from each MMA warp
+      mbar_init(qempty(i), 1);
     }
     for (int i = 0; i < 4; ++i) mbar_init(wgbar(i), 4);
-    mbar_init(epibar, kEpiWarps);
     for (int i = 0; i < kPub; ++i) {
       mbar_init(pubfull(i), kEpiWarps);
       mbar_init(pubempty(i), 1);
     }
     *abort_cta = 0;
+    sel = SelCall{p.status, Hkv, p.pool_width, p.raw_scratch, p.k, p.v, p.k_out, p.v_out,
+                  p.tok_stride_v16, p.head_stride_v16};
     fence_mbar_init();
   }
   for (int q = threadIdx.x; q < kMaxQRows; q += kFThreads) sWpos[q] = q % W;
@@ -979,13 +578,8 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
       const uint64_t pol2 = l2_policy_evict_first();
       const uint64_t polq = l2_policy_evict_last();
       const int G = p.group_size;
-      // Each UMMA warp has its own sub-ring of the K stages (warp w: stages
-      // w, w + 2, ...), consumed strictly in order: a warp that skipped the
-      // other warp's tiles could otherwise wait on a stage whose previous
-      // fill has not landed and mistake an older phase for its own.
-      const int nsw = nst >> 1;
-      int sw0 = 0, sw1 = 0;       // next slot of each sub-ring
-      uint32_t sp0 = 0, sp1 = 0;  // and its phase
+      int st = 0;  // next K stage and its phase
+      uint32_t ph = 0;
       uint32_t k_used = 0, k_phase = 0;  // per stage: filled, parity of its last fill
       int qb = 0;  // Q buffer of the next chunk and its phase
       uint32_t qph = 0;
@@ -1020,9 +614,6 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
         }
         bool stop = false;
         for (int t = d.t0; t < d.t1; ++t) {
-          const int w = (t - d.t0) & 1;  // the UMMA warp (and warpgroup) of the tile
-          const int st = w + 2 * (w ? sw1 : sw0);
-          const uint32_t ph = w ? sp1 : sp0;
           if (!F.wait_bar(empty(st), ph ^ 1u)) {
             stop = true;
             break;
@@ -1034,14 +625,9 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
           tma_load_3d(dst + kHalfTileBytes, &p.tmap_k, full(st), 64, d.g, row, pol);
           k_used |= 1u << st;
           k_phase = (k_phase & ~(1u << st)) | (ph << st);
-          if (w) {
-            if (++sw1 == nsw) {
-              sw1 = 0;
-              sp1 ^= 1u;
-            }
-          } else if (++sw0 == nsw) {
-            sw0 = 0;
-            sp0 ^= 1u;
+          if (++st == nst) {
+            st = 0;
+            ph ^= 1u;
           }
         }
         if (stop) break;
@@ -1066,75 +652,75 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
         if ((q_issued >> b) & 1u) wait_plain(qempty(b), (q_phase >> b) & 1u, tail_ns);
     }
     __syncwarp();
-  } else if (warp == kMmaWarp || warp == kMmaWarp2) {
+  } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------ UMMA issue
-    const int mw = warp == kMmaWarp ? 0 : 1;  // the warpgroup whose tiles this warp issues
-    if (lane == 0) {
-      const uint64_t dk0 = smem_desc_sw128(smem_u32(sK));
-      const int bpw = p.nbuf / kNwg;  // TMEM buffers per warpgroup (a power of two)
-      const int lbpw = __ffs(bpw) - 1;
-      const int nsw = nst >> 1;
-      int st = 0;  // next slot of this warp's K sub-ring (stages mw, mw + 2, ...) and its phase
-      uint32_t sph = 0;
-      int qb = 0;  // Q buffer of the next chunk and its phase
-      uint32_t qph = 0;
-      int kw = 0;  // tiles issued for warpgroup mw
-      int last_b = -1;
-      uint32_t last_use = 0;
-      for (int c = 0;; ++c) {
-        const int ds = c % kDescs;
-        if (!F.wait_bar(dfull(ds), static_cast<uint32_t>(c / kDescs) & 1u)) break;
-        const ChunkDesc d = descs[ds];
-        mbar_arrive(dempty(ds));
-        if (d.end) break;
-        if (!F.wait_bar(qfull(qb), qph)) break;
+    auto wait_all = [&](uint32_t bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, F.wait_bar(bar, parity));
+    };
+    const uint64_t dk0 = smem_desc_sw128(smem_u32(sK));
+    const int bpw = p.nbuf / kNwg;  // TMEM buffers per warpgroup (a power of two)
+    const int lbpw = __ffs(bpw) - 1;
+    int st = 0;  // next K stage and its phase
+    uint32_t sph = 0;
+    int qb = 0;  // Q buffer of the next chunk and its phase
+    uint32_t qph = 0;
+    int kw0 = 0, kw1 = 0;  // tiles issued per warpgroup
+    int last_st = -1;
+    uint32_t last_ph = 0;
+    for (int c = 0;; ++c) {
+      const int ds = c % kDescs;
+      if (!wait_all(dfull(ds), static_cast<uint32_t>(c / kDescs) & 1u)) break;
+      const int end = descs[ds].end, nt = descs[ds].t1 - descs[ds].t0, rows = descs[ds].n_rows;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(dempty(ds));
+      if (end) break;
+      if (!wait_all(qfull(qb), qph)) break;
+      const int Npad = (rows + 15) & ~15;
+      const uint32_t idesc = umma_idesc_f16(kTileTokens, Npad, p.is_bf16 != 0);
+      const uint64_t dq0 = smem_desc_sw128(smem_u32(sQ + qb * 2 * qh));
+      const uint64_t qhalf = static_cast<uint64_t>(qh >> 4);
+      bool stop = false;
+#pragma unroll 1
+      for (int t = 0; t < nt; ++t) {
+        const int mw = t & 1;  // the warpgroup that takes the tile
+        const int kk = mw ? kw1++ : kw0++;
+        const int b = mw + kNwg * (kk & (bpw - 1));
+        const uint32_t use = static_cast<uint32_t>(kk >> lbpw) & 1u;
+        if (!wait_all(tempty(b), use ^ 1u) || !wait_all(full(st), sph)) {
+          stop = true;
+          break;
+        }
         tc_fence_after();
-        const int Npad = (d.n_rows + 15) & ~15;
-        const uint32_t idesc = umma_idesc_f16(kTileTokens, Npad, p.is_bf16 != 0);
-        const uint64_t dq0 = smem_desc_sw128(smem_u32(sQ + qb * 2 * qh));
-        bool stop = false;
-        for (int t = d.t0; t < d.t1; ++t) {
-          if (((t - d.t0) & 1) != mw) continue;  // the other warp's tile
-          const int kk = kw++;
-          const int b = mw + kNwg * (kk & (bpw - 1));
-          const uint32_t use = static_cast<uint32_t>(kk >> lbpw) & 1u;
-          if (!F.wait_bar(tempty(b), use ^ 1u)) {
-            stop = true;
-            break;
-          }
-          const int stp = mw + 2 * st;  // the stage
-          if (!F.wait_bar(full(stp), sph)) {
-            stop = true;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t dt = tbase + static_cast<uint32_t>(b * p.tstride);
-          const uint64_t dk = dk0 + static_cast<uint64_t>((stp * kTileBytes) >> 4);
+        const uint32_t dt = tbase + static_cast<uint32_t>(b * p.tstride);
+        const uint64_t dk = dk0 + static_cast<uint64_t>((st * kTileBytes) >> 4);
+        if (elect_one()) {
 #pragma unroll
           for (int k8 = 0; k8 < kHeadDim / 16; ++k8) {
-            const uint32_t koff = (k8 >> 2) * kHalfTileBytes + (k8 & 3) * 32;
-            const uint32_t qoff = (k8 >> 2) * qh + (k8 & 3) * 32;
-            umma_f16(dt, dk + (koff >> 4), dq0 + (qoff >> 4), idesc, k8 > 0 ? 1u : 0u);
+            const uint64_t koff = ((k8 >> 2) * kHalfTileBytes + (k8 & 3) * 32) >> 4;
+            const uint64_t qoff = (k8 >> 2) * qhalf + (((k8 & 3) * 32) >> 4);
+            umma_f16(dt, dk + koff, dq0 + qoff, idesc, k8 > 0 ? 1u : 0u);
           }
-          umma_commit(empty(stp));
           umma_commit(tfull(b));
-          last_b = b;
-          last_use = use;
-          if (++st == nsw) {
-            st = 0;
-            sph ^= 1u;
-          }
+          umma_commit(empty(st));
         }
-        if (stop) break;
-        umma_commit(qempty(qb));
-        if (++qb == nqb) {
-          qb = 0;
-          qph ^= 1u;
+        __syncwarp();
+        last_st = st;
+        last_ph = sph;
+        if (++st == nst) {
+          st = 0;
+          sph ^= 1u;
         }
       }
-      if (*reinterpret_cast<volatile int*>(abort_cta) && last_b >= 0)
-        wait_plain(tfull(last_b), last_use, 100000000ull);  // MMAs done before TMEM is freed
+      if (stop) break;
+      if (elect_one()) umma_commit(qempty(qb));
+      __syncwarp();
+      if (++qb == nqb) {
+        qb = 0;
+        qph ^= 1u;
+      }
     }
+    if (lane == 0 && *reinterpret_cast<volatile int*>(abort_cta) && last_st >= 0)
+      wait_plain(empty(last_st), last_ph, 100000000ull);  // MMAs done before TMEM is freed
     __syncwarp();
   } else if (warp >= kEpiWarp0 && warp < kEpiWarp0 + kEpiWarps) {
     // ------------------------------------------------------------ epilogue
@@ -1142,30 +728,20 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
     const int wg = ew >> 2;
     const int qd = warp & 3;  // TMEM lane quarter of this warp
     const int tw = (ew & 3) * 32 + lane;
-    const int te = ew * 32 + lane;  // thread among all epilogue threads
     constexpr int nwg = kNwg;
     const bool takes = wg < nwg;  // this warpgroup takes tiles
     float* ref = sRef + (takes ? ew : 0) * rstride;
     float* acc_s = sAcc + (takes ? ew : 0) * rstride;
     const float c = p.c;
+    const uint64_t c2 = pack2(c, c);
+    const int bcol = block_col(lane);
     const int bpw = p.nbuf / nwg;  // a power of two
     const int lbpw = __ffs(bpw) - 1;
-    const int h = (p.pool_width - 1) >> 1;
-    const float fP = static_cast<float>(p.pool_width);
     const int G = p.group_size;
     int kc = 0;       // tiles this warpgroup has taken
     int nsync = 0;    // warpgroup syncs so far (mbarrier phase)
-    int nsync8 = 0;   // all-epilogue syncs so far
-    int n2 = 0;       // pass-2 chunks so far (raw buffer parity)
     bool stop = false;
     // bounded barriers (a warp that stopped cannot hang the others)
-    auto epi_sync = [&]() -> bool {
-      __syncwarp();
-      if (lane == 0) mbar_arrive(epibar);
-      const bool ok = F.wait_bar(epibar, static_cast<uint32_t>(nsync8) & 1u);
-      ++nsync8;
-      return __all_sync(0xffffffffu, ok);
-    };
     // the chunk's results are written: its claimer publishes it (fence, then
     // the unit's counter) off the epilogue's path
     auto publish = [&](int ci) -> bool {
@@ -1219,62 +795,73 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
             break;
           }
           tc_fence_after();
-          const int tok = tile * kTileTokens + qd * 32 + lane;
+          const int tok0 = tile * kTileTokens + qd * 32;  // the warp's first key
           const uint32_t taddr = tbase + (static_cast<uint32_t>(qd * 32) << 16) +
                                  static_cast<uint32_t>(b * p.tstride);
           const bool edge = (tile + 1) * kTileTokens > n;
-          const int vis = n - tok;
-          const bool key = tok < L;
+#pragma unroll 1
           for (int c0 = 0; c0 < N; c0 += 32) {
             uint32_t r[32];  // the logits
-            tmem_load32_async(taddr + c0, r);
-            tmem_wait_ld(r);
-            const int lim = min(32, N - c0);
-            const bool masked = edge || lim < 32;
-            float* rf = ref + c0;
-            float e[32];  // 2^(z c - R)
-            if (first && !masked) {
-              // the warp's first tile of the chunk: lane 0's scaled logit is
-              // the reference of each query row (any reference within 2^64
-              // of the largest keeps the fp32 sums exact enough)
+            tmem_load_block(taddr + c0, r);
+            const int lim = min(32, N - c0);  // 32 or 16
+            float2* rf = reinterpret_cast<float2*>(ref + c0) + (lane & 3);  // columns 8 j + 2 (lane % 4)
+            uint64_t nr[4];
+            if (first && !edge) {
+              // the warp's first tile of the chunk: its first key's scaled
+              // logit is the reference of each query row (any reference
+              // within 2^64 of the largest keeps the fp32 sums exact enough)
 #pragma unroll
-              for (int j = 0; j < 32; ++j) {
-                const float v = __uint_as_float(r[j]) * c;
-                const float rj = __shfl_sync(0xffffffffu, v, 0);
-                e[j] = ex2_approx(v - rj);
-                if (lane == 0) rf[j] = rj;
+              for (int j = 0; j < 4; ++j) {
+                const float r0 = __shfl_sync(0xffffffffu, __uint_as_float(r[4 * j]) * c, lane & 3);
+                const float r1 =
+                    __shfl_sync(0xffffffffu, __uint_as_float(r[4 * j + 1]) * c, lane & 3);
+                nr[j] = pack2(-r0, -r1);
+                if (lane < 4) rf[4 * j] = make_float2(r0, r1);
               }
               __syncwarp();
-            } else if (masked) {
-#pragma unroll
-              for (int j = 0; j < 32; j += 4) {
-                const int4 wq = *reinterpret_cast<const int4*>(sWpos + c0 + j);
-                const float4 rq = *reinterpret_cast<const float4*>(rf + j);
-                const int wv[4] = {wq.x, wq.y, wq.z, wq.w};
-                const float rv[4] = {rq.x, rq.y, rq.z, rq.w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  const bool okk = (j + k) < lim && (!edge || (key && wv[k] >= -vis));
-                  e[j + k] = okk ? ex2_approx(fmaf(__uint_as_float(r[j + k]), c, -rv[k])) : 0.f;
-                }
-              }
             } else {
 #pragma unroll
-              for (int j = 0; j < 32; j += 4) {
-                const float4 rq = *reinterpret_cast<const float4*>(rf + j);
-                e[j + 0] = ex2_approx(fmaf(__uint_as_float(r[j + 0]), c, -rq.x));
-                e[j + 1] = ex2_approx(fmaf(__uint_as_float(r[j + 1]), c, -rq.y));
-                e[j + 2] = ex2_approx(fmaf(__uint_as_float(r[j + 2]), c, -rq.z));
-                e[j + 3] = ex2_approx(fmaf(__uint_as_float(r[j + 3]), c, -rq.w));
+              for (int j = 0; j < 4; ++j) {
+                const float2 x = rf[4 * j];
+                nr[j] = pack2(-x.x, -x.y);
               }
             }
-            float colsum = warp_transpose_sum32(e, lane);  // column c0 + lane
+            float v[8];  // sums of 2^(z c - R) over the lane's keys
+            if (edge) {
+              const uint32_t ok = block_mask(c0, W, lim, tok0, n, L, lane);
+#pragma unroll
+              for (int i = 0; i < 8; ++i) v[i] = 0.f;
+#pragma unroll
+              for (int e = 0; e < 32; ++e) {
+                const int j = (e >> 2) & 3;
+                float n0, n1;
+                unpack2(nr[j], n0, n1);
+                const float x = ex2_approx(fmaf(__uint_as_float(r[e]), c, (e & 1) ? n1 : n0));
+                v[2 * j + (e & 1)] += (ok >> e) & 1u ? x : 0.f;
+              }
+            } else {
+              uint64_t s2[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+              for (int e = 0; e < 32; e += 2) {
+                const int j = (e >> 2) & 3;
+                const uint64_t z = pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1]));
+                s2[j] = add2(s2[j], exp2_2(fma2(z, c2, nr[j])));
+              }
+              if (lim < 32) s2[2] = s2[3] = 0ull;  // not query rows
+#pragma unroll
+              for (int j = 0; j < 4; ++j) unpack2(s2[j], v[2 * j], v[2 * j + 1]);
+            }
+            float colsum = sum_over_keys(v, lane);
+            int col = bcol;
             // an exponent above 2^64 shows in its column's sum (inf/NaN
             // when above 2^128 or with the references still -inf)
-            if (__any_sync(0xffffffffu, !(colsum <= kRaiseSum)))
-              colsum = p1_raise_group(taddr + c0, rf, acc_s + c0, sWpos + c0, lim, edge, key, vis,
-                                      c, lane);
-            acc_s[c0 + lane] += colsum;
+            if (__any_sync(0xffffffffu, !(colsum <= kRaiseSum))) {
+              const int tok = tok0 + lane;
+              colsum = p1_raise_group(taddr + c0, ref + c0, acc_s + c0, sWpos + c0, lim, edge,
+                                      tok < L, n - tok, c, lane);
+              col = lane;
+            }
+            acc_s[c0 + col] += colsum;
             __syncwarp();
           }
           first = false;
@@ -1319,9 +906,6 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
           for (int q = lane; q < N; q += 32) ref[q] = __ldcg(bias + q);
         }
         __syncwarp();
-        float* cbuf = sChunk + (n2 & 1) * kChunkKeys;
-        ++n2;
-        const int a = d.t0 * kTileTokens;  // first key of the chunk
         for (int tile = d.t0 + wg; takes && tile < d.t1; tile += nwg) {
           const int kk = kc++;
           const int b = wg + nwg * (kk & (bpw - 1));
@@ -1332,64 +916,45 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
             break;
           }
           tc_fence_after();
-          const int tok = tile * kTileTokens + qd * 32 + lane;
           const uint32_t taddr = tbase + (static_cast<uint32_t>(qd * 32) << 16) +
                                  static_cast<uint32_t>(b * p.tstride);
-          const bool edge = (tile + 1) * kTileTokens > n;
-          const int vis = n - tok;
-          const bool key = tok < L;
-          float acc[4] = {0.f, 0.f, 0.f, 0.f};
-          // add 2^(z c - log2 D_q) of 32 columns starting at c0 (lim valid)
-          auto add_group = [&](const uint32_t (&r)[32], int c0, int lim) {
-            if (edge || lim < 32) {
+          // 2^(z c - log2 D_q) summed over the query rows.  (Causality needs
+          // no mask: every query row sees every prefix key, and the scores of
+          // later keys are not kept.)
+          uint64_t rs2[4] = {0ull, 0ull, 0ull, 0ull};  // the lane's four keys
+#pragma unroll 1
+          for (int c0 = 0; c0 < N; c0 += 32) {
+            uint32_t r[32];
+            tmem_load_block(taddr + c0, r);
+            const float2* lq = reinterpret_cast<const float2*>(ref + c0) + (lane & 3);
 #pragma unroll
-              for (int j = 0; j < 32; j += 4) {
-                const int4 wq = *reinterpret_cast<const int4*>(sWpos + c0 + j);
-                const float4 lq = *reinterpret_cast<const float4*>(ref + c0 + j);
-                const int wv[4] = {wq.x, wq.y, wq.z, wq.w};
-                const float lv[4] = {lq.x, lq.y, lq.z, lq.w};
+            for (int j = 0; j < 4; ++j) {
+              if (j == 2 && N - c0 == 16) break;  // the last 16 columns are not query rows
+              const float2 x = lq[4 * j];
+              const uint64_t nl = pack2(-x.x, -x.y);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  const bool okk = (j + k) < lim && (!edge || (key && wv[k] >= -vis));
-                  acc[k] += okk ? ex2_approx(fmaf(__uint_as_float(r[j + k]), c, -lv[k])) : 0.f;
-                }
-              }
-            } else {
-#pragma unroll
-              for (int j = 0; j < 32; j += 4) {
-                const float4 lq = *reinterpret_cast<const float4*>(ref + c0 + j);
-                acc[0] += ex2_approx(fmaf(__uint_as_float(r[j + 0]), c, -lq.x));
-                acc[1] += ex2_approx(fmaf(__uint_as_float(r[j + 1]), c, -lq.y));
-                acc[2] += ex2_approx(fmaf(__uint_as_float(r[j + 2]), c, -lq.z));
-                acc[3] += ex2_approx(fmaf(__uint_as_float(r[j + 3]), c, -lq.w));
+              for (int k = 0; k < 4; ++k) {
+                const int e = 16 * (k >> 1) + 4 * j + 2 * (k & 1);
+                const uint64_t z = pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1]));
+                rs2[k] = add2(rs2[k], exp2_2(fma2(z, c2, nl)));
               }
             }
-          };
-          for (int c0 = 0; c0 < N; c0 += 32) {
-            uint32_t r0[32];
-            tmem_load32_async(taddr + c0, r0);
-            tmem_wait_ld(r0);
-            add_group(r0, c0, min(32, N - c0));
           }
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(tempty(b));
-          if (tok < n) {
-            const float rv = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-            p.raw[soff + tok] = rv;
-            cbuf[tok - a] = rv;
+          float rs[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            float x, y;
+            unpack2(rs2[k], x, y);
+            rs[k] = x + y;
           }
+          const float v = sum_over_cols(rs, lane);
+          const int tok = tile * kTileTokens + qd * 32 + block_key(lane);
+          if (tok < n) p.raw[soff + tok] = v;
         }
         if (stop) break;
-        // pooled scores of the chunk's interior [a + h, b - h) from the raw
-        // scores of both warpgroups; the select pools the h keys at each edge
-        if (!epi_sync()) break;
-        const int bnd = min(d.t1 * kTileTokens, n);
-        for (int j = a + h + te; j < bnd - h; j += 32 * kEpiWarps) {
-          float accp = 0.f;
-          for (int t = 0; t <= 2 * h; ++t) accp += cbuf[j - h + t - a];
-          p.pooled[soff + j] = accp / fP;
-        }
         if (!publish(ci)) break;
       }
     }
@@ -1405,8 +970,20 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
       if (type == kTaskEnd) break;
       if (type == kTaskMerge) {
         merge_unit(F, idx, creg, ct);
-      } else {
-        select_unit(F, idx, creg, ct);
+      } else if (p.do_select) {
+        const int s = idx / Hkv;
+        const int g = idx - s * Hkv;
+        if (F.prefix(s) > 0 && F.chunks_per_unit(s) == 0) continue;  // not of this launch
+        SelUnit U;
+        U.g = g;
+        U.seq0 = p.cu_seqlens[s];
+        U.L = F.len(s);
+        U.W = W;
+        U.out0 = p.cu_out[s];
+        U.kept = p.cu_out[s + 1] - U.out0;
+        const long long soff = static_cast<long long>(g) * p.p_total + p.cu_prefix[s];
+        select_unit(sel, U, p.raw + soff, p.pooled + soff,
+                    p.indices + static_cast<long long>(g) * p.o_total + U.out0, creg, ct);
       }
     }
   }
@@ -1436,7 +1013,7 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
 size_t fused_smem_bytes(int q_half_bytes, int q_bufs, int stages, int row_stride, int nwg) {
   return 1024 + static_cast<size_t>(stages) * kTileBytes +
          2 * static_cast<size_t>(q_bufs) * q_half_bytes +
-         2 * static_cast<size_t>(4 * nwg) * row_stride * 4 + kFixedBytes + kFusedCRegion;
+         2 * static_cast<size_t>(4 * nwg) * row_stride * 4 + kFixedBytes + kSelRegion;
 }
 
 cudaError_t fused_set_smem_limit(size_t bytes) {

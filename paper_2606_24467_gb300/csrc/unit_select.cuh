@@ -27,10 +27,11 @@ struct SelShared {
 };
 static_assert(sizeof(SelShared) <= kSelRegion, "select scratch");
 static_assert(kSelSamples <= kFusedCandCap, "samples live in the position array");
-constexpr int kPoolSlice = 2048;  // keys pooled at a time
-static_assert(kPoolSlice + 62 <= kFusedCandCap, "a slice and its halo fit the position array");
-static_assert(kPoolSlice + 62 <= kSelGroups + 64, "... and the group maxima's place");
-static_assert(62 < kCThreads, "a slice's halo is one load per thread");
+constexpr int kPoolStrip = 192;  // keys a warp pools at a time
+constexpr int kPoolBuf = 256;    // ... with up to 62 neighbours, padded
+static_assert(kPoolStrip + 62 <= kPoolBuf && kPoolStrip % 32 == 0, "a strip and its halo");
+static_assert(8 * kPoolBuf <= kFusedCandCap && 8 * kPoolBuf <= kSelGroups + 64,
+              "the warps' strips fit the position array and the group maxima's place");
 
 
 // The call's parameters that the selection needs (in shared memory: read
@@ -45,6 +46,12 @@ struct SelCall {
   long long tok_stride_v16, head_stride_v16;
 };
 
+// `p` points to shared memory: plain shared-memory instructions instead of
+// generic ones, in functions that are not inlined.
+template <class T>
+__device__ __forceinline__ void assume_shared(const T* p) {
+  __builtin_assume(__isShared(p));
+}
 __device__ __forceinline__ void cbar() { named_bar_sync(kBarC, kCThreads); }
 
 // Zero the radix state (the workers' form of radix_init).
@@ -62,6 +69,7 @@ __device__ __forceinline__ void radix_init_grp(RadixShared& sh, int ct) {
 __device__ __noinline__ uint32_t grp_kth_largest(const uint32_t* keys, int count, uint32_t sub,
                                                  uint32_t clamp, int r, RadixShared& sh, int slot,
                                                  int& pc, int* rem, int ct) {
+  assume_shared(&sh);
   const int lane = ct & 31;
   const int iters = (count + 255) >> 8;
   auto key_at = [&](int j) -> uint32_t {
@@ -154,6 +162,8 @@ __device__ __noinline__ uint32_t bisect_kth(const uint32_t* keys, int count, int
                                             SelShared& sh, int* need_eq, int ct) {
   const int cw = ct >> 5;
   const int lane = ct & 31;
+  assume_shared(&sh);
+  assume_shared(keys);
   uint32_t kv[kPer];
   uint32_t mn = 0xFFFFFFFFu, mx = 0u;
 #pragma unroll
@@ -224,6 +234,7 @@ static_assert(kSelWhole <= 24 * kCThreads && kSelGroups <= 12 * kCThreads, "bise
 __device__ __noinline__ void emit_selected(int count, uint32_t tau, int need_eq, int32_t* out, int k,
                                            SelShared& sh, int ct, const uint32_t* keys,
                                            const int* pos) {
+  assume_shared(&sh);
   const int cw = ct >> 5;
   const int lane = ct & 31;
   const int seg = (count + 255) >> 8 << 5;  // entries per warp
@@ -277,6 +288,7 @@ __device__ __noinline__ void emit_selected(int count, uint32_t tau, int need_eq,
 // and recorded.
 __device__ __noinline__ void gather_rows(const SelCall& p, int seq0, int L, int g,
                                          const int32_t* out, int out0, int count, int ct) {
+  assume_shared(&p);
   constexpr int kBatch = 8;
   constexpr int kRow16 = kHeadDim * 2 / 16;
   const int lane = ct & 31;
@@ -320,6 +332,7 @@ __device__ __noinline__ void gather_rows(const SelCall& p, int seq0, int L, int 
 __device__ __noinline__ int scan_rows(const uint32_t* keys, int n, int r0, int r1, int e,
                                       const uint32_t* gmax, uint32_t lo, int o, uint32_t* ckey,
                                       int* cpos, int cap, int lane) {
+  assume_shared(gmax);
   constexpr int kU = 8;
 #pragma unroll 1
   for (int r = r0; r < r1; r += 32) {
@@ -355,60 +368,83 @@ struct SelUnit {
 };
 
 // Pools the unit's raw scores (sum from j - h to j + h, zeros outside [0, n),
-// over P), slice by slice through shared memory with the next slice's loads in
-// flight; writes them to `pooled` and, as keys, to `keys` when the unit is
+// over P); writes them to `pooled` and, as keys, to `keys` when the unit is
 // small enough for it (n <= kSelWhole), else keeps the largest of every group of
-// 32 << e keys.
+// 32 << e keys.  A warp takes every eighth strip of kPoolStrip keys, through
+// its own part of shared memory and with the loads of its next two strips in
+// flight.  Bound by instruction latency (two warps per scheduler): 22-27 us
+// for 32736 keys with the seven taps of the usual width unrolled, 33-42 us
+// with a loop over them.
 __device__ __noinline__ void pool_unit(const float* raw, float* pooled, int n, int e, int h, float fP,
                                        SelShared& sh, int ct) {
-  constexpr int kPer = kPoolSlice / kCThreads;  // keys per thread and slice
+  constexpr int kPer = kPoolStrip / 32;          // keys per lane
+  constexpr int kLoads = kPoolBuf / 32;  // with the halo
+  assume_shared(&sh);
   const int lane = ct & 31;
   const bool keep = n <= kSelWhole;
-  float* const stage = keep ? reinterpret_cast<float*>(sh.gmax) : reinterpret_cast<float*>(sh.pos);
-  float nx[kPer + 1];
-  auto load = [&](int base) {
+  float* const stage =
+      (keep ? reinterpret_cast<float*>(sh.gmax) : reinterpret_cast<float*>(sh.pos)) +
+      (ct >> 5) * kPoolBuf;
+  float na[kLoads], nb[kLoads];
+  auto load = [&](float (&nx)[kLoads], int base) {
 #pragma unroll
-    for (int q = 0; q <= kPer; ++q) {
-      const int i = q * kCThreads + ct;
+    for (int q = 0; q < kLoads; ++q) {
+      const int i = q * 32 + lane;
       const int j = base - h + i;
-      nx[q] = i < kPoolSlice + 2 * h && j >= 0 && j < n ? __ldcg(raw + j) : 0.f;
+      nx[q] = i < kPoolStrip + 2 * h && j >= 0 && j < n ? __ldcg(raw + j) : 0.f;
     }
   };
-  load(0);
-#pragma unroll 1
-  for (int base = 0; base < n; base += kPoolSlice) {
-    cbar();  // the slice before is read
+  auto step = [&](float (&nx)[kLoads], int base) {
+    __syncwarp();  // the strip before is read
 #pragma unroll
-    for (int q = 0; q <= kPer; ++q) {
-      const int i = q * kCThreads + ct;
-      if (i < kPoolSlice + 2 * h) stage[i] = nx[q];
-    }
-    cbar();
-    if (base + kPoolSlice < n) load(base + kPoolSlice);
+    for (int q = 0; q < kLoads; ++q) stage[q * 32 + lane] = nx[q];
+    __syncwarp();
+    load(nx, base + 16 * kPoolStrip);
     float s[kPer];
 #pragma unroll
     for (int q = 0; q < kPer; ++q) s[q] = 0.f;
-    const float* a = stage + ct;
+    const float* a = stage + lane;
+    if (h == 3) {  // the usual width, without a load's latency per tap
+#pragma unroll
+      for (int t = 0; t < 7; ++t)
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) s[q] += a[q * 32 + t];
+    } else {
+#pragma unroll 4
+      for (int t = 0; t <= 2 * h; ++t)
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) s[q] += a[q * 32 + t];
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) s[q] = s[q] / fP;
+    if (keep) {
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        const int j = base + q * 32 + lane;
+        if (j < n) pooled[j] = s[q];
+        if (j < n) sh.key[j] = __float_as_uint(s[q]);
+      }
+    } else {
+      uint32_t top = 0u;  // lane q: the largest of row q
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        const int j = base + q * 32 + lane;
+        const bool in = j < n;
+        if (in) pooled[j] = s[q];
+        const uint32_t m = __reduce_max_sync(0xffffffffu, in ? __float_as_uint(s[q]) : 0u);
+        top = lane == q ? m : top;
+      }
+      if (lane < kPer && base + 32 * lane < n)
+        atomicMax(&sh.gmax[(base + 32 * lane) >> (5 + e)], top);
+    }
+  };
+  const int base0 = (ct >> 5) * kPoolStrip;
+  load(na, base0);
+  load(nb, base0 + 8 * kPoolStrip);
 #pragma unroll 1
-    for (int t = 0; t <= 2 * h; ++t, ++a) {
-#pragma unroll
-      for (int q = 0; q < kPer; ++q) s[q] += a[q * kCThreads];
-    }
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      const int j = base + q * kCThreads + ct;
-      if (j - lane >= n) break;
-      const bool in = j < n;
-      const float v = s[q] / fP;
-      if (in) {
-        pooled[j] = v;
-        if (keep) sh.key[j] = __float_as_uint(v);
-      }
-      if (!keep) {
-        const uint32_t m = __reduce_max_sync(0xffffffffu, in ? __float_as_uint(v) : 0u);
-        if (lane == 0) atomicMax(&sh.gmax[j >> (5 + e)], m);
-      }
-    }
+  for (int base = base0; base < n; base += 16 * kPoolStrip) {
+    step(na, base);
+    if (base + 8 * kPoolStrip < n) step(nb, base + 8 * kPoolStrip);
   }
 }
 
@@ -422,6 +458,8 @@ __device__ __noinline__ void pool_unit(const float* raw, float* pooled, int n, i
 // scores are >= 0: their bit patterns order like their values.
 __device__ __noinline__ void select_unit(const SelCall& p, const SelUnit U, float* raw,
                                          float* pooled, int32_t* out, uint8_t* creg, int ct) {
+  assume_shared(creg);
+  assume_shared(&p);
   SelShared& sh = *reinterpret_cast<SelShared*>(creg);
   const int cw = ct >> 5;
   const int lane = ct & 31;
@@ -433,6 +471,7 @@ __device__ __noinline__ void select_unit(const SelCall& p, const SelUnit U, floa
   const int nr = (n + 31) >> 5;
   const int ng = (nr + (1 << e) - 1) >> e;
   for (int i = ct; i < ng; i += kCThreads) sh.gmax[i] = 0u;
+  cbar();
   pool_unit(raw, pooled, n, e, (p.pool_width - 1) >> 1, static_cast<float>(p.pool_width), sh, ct);
   __threadfence_block();
   cbar();
