@@ -246,6 +246,7 @@ __device__ __forceinline__ void arrive(uint64_t* bar) { mbar_arrive(smem_u32(bar
 // One more turn of a wait that began at t0: false when the call stopped or
 // the wait ran out (the status word and the abort word are then set).
 __device__ __noinline__ bool still_waiting(ResidentShared& sh, uint64_t t0) {
+  assume_shared(&sh);
   volatile int* mine = &sh.abort_cta;
   if (*mine) return false;
   if (aborted(sh)) {
@@ -277,6 +278,7 @@ __device__ __forceinline__ bool mbar_suspended_wait(uint32_t bar, uint32_t parit
 // Bounded wait (another CTA's progress) until *ptr >= target; false when the
 // call was aborted or the wait ran out.
 __device__ __noinline__ bool wait_counter(ResidentShared& sh, const int* ptr, int target) {
+  assume_shared(&sh);
   if (ld_acquire(ptr) >= target) return true;
   const uint64_t t0 = globaltimer_ns();
   for (;;) {
@@ -287,6 +289,7 @@ __device__ __noinline__ bool wait_counter(ResidentShared& sh, const int* ptr, in
 }
 // Bounded wait on one of this CTA's mbarriers; a timeout stops the call.
 __device__ __noinline__ bool wait_more(ResidentShared& sh, uint32_t a, uint32_t parity) {
+  assume_shared(&sh);
   const uint64_t t0 = globaltimer_ns();
   for (;;) {
     if (mbar_suspended_wait(a, parity)) return true;
@@ -306,11 +309,15 @@ __device__ __forceinline__ bool wait_all(ResidentShared& sh, const uint64_t* bar
 
 // Row i of pairs, and the denominators of warpgroup wg's k-th unit.
 __device__ __forceinline__ float2* pair_row(ResidentShared& sh, int i) {
-  return sh.call.rows + i * sh.call.acc_rows;
+  float2* const r = sh.call.rows + i * sh.call.acc_rows;
+  assume_shared(r);
+  return r;
 }
 // (acc_rows values of -R, then acc_rows of w)
 __device__ __forceinline__ float* den_row(ResidentShared& sh, int wg, int k) {
-  return reinterpret_cast<float*>(pair_row(sh, (wg ? kDenRow : 0) + k));
+  float* const r = reinterpret_cast<float*>(pair_row(sh, (wg ? kDenRow : 0) + k));
+  assume_shared(r);
+  return r;
 }
 
 // Position in a ring of n slots and the parity of its use.
@@ -407,6 +414,7 @@ struct Group {
 // the logits still in tensor memory; (0, 0) when no key is attended.
 __device__ __noinline__ void p1_slow(ResidentShared& sh, const ChunkDesc& d, int quarter,
                                      int lane, uint32_t bad, float2* out) {
+  assume_shared(&sh);
   const int window = sh.call.window;
   const float c = sh.call.c;
   const int nt = d.nt, n = d.n, L = d.L;
@@ -471,6 +479,7 @@ __device__ __noinline__ void p1_slow(ResidentShared& sh, const ChunkDesc& d, int
 // it.
 __device__ __noinline__ bool slow_denominators(ResidentShared& sh, const ChunkDesc& d, float* out,
                                                int lane) {
+  assume_shared(&sh);
   const int grid = static_cast<int>(gridDim.x);
   const int nown = (d.x_last - d.x) / grid + 1;
   const int first = d.x / grid;  // this chunk's number among the CTA's
@@ -550,6 +559,7 @@ __device__ __noinline__ bool slow_denominators(ResidentShared& sh, const ChunkDe
 // (-R_q, w_q) of a unit's query rows from the given LSE (one warp).
 __device__ __noinline__ void lse_denominators(ResidentShared& sh, const ChunkDesc& d, float* out,
                                               int lane) {
+  assume_shared(&sh);
   const CallInfo& p = sh.call;
   const float* lse = p.lse + static_cast<long long>(d.s) * p.lse_bs +
                      static_cast<long long>(d.g) * p.group_size * p.lse_hs;
@@ -782,6 +792,7 @@ __device__ __forceinline__ void wait_plain(const uint64_t* bar, uint32_t parity,
 // Q buffers, tcgen05.commit arrivals that nobody else waits for at the end.
 __device__ __noinline__ void drain_loads(ResidentShared& sh, uint32_t k_used, uint32_t k_phase,
                                          uint32_t q_used, uint32_t q_phase) {
+  assume_shared(&sh);
   const bool ab = ld_volatile(&sh.abort_cta) != 0;
 #pragma unroll 1
   for (int pass = ab ? 0 : 1; pass < 2; ++pass) {
@@ -799,6 +810,7 @@ __device__ __noinline__ void drain_loads(ResidentShared& sh, uint32_t k_used, ui
 }
 
 __device__ __noinline__ void producer_role(ResidentShared& sh, int lane) {
+  assume_shared(&sh);
   const CallInfo& p = sh.call;
   const int nst = p.stages, nqb = p.q_bufs, qh = p.q_half_bytes;
   uint8_t* const sK = p.sK;
@@ -865,6 +877,7 @@ __device__ __noinline__ void producer_role(ResidentShared& sh, int lane) {
 // issuing warp would not help: tensor-memory loads queue behind the UMMAs
 // issued, and took 600 to 1000 clocks instead of 190 with two issuers.
 __device__ __noinline__ void mma_role(ResidentShared& sh, int lane) {
+  assume_shared(&sh);
   const CallInfo& p = sh.call;
   const int nqb = p.q_bufs, qh = p.q_half_bytes, nst = p.stages;
   const bool bf16 = p.is_bf16 != 0;
@@ -962,6 +975,7 @@ __device__ __noinline__ float2 sum_pairs(const float2* src, int rows) {
 }
 
 __device__ __noinline__ void sum_role(ResidentShared& sh, int lane) {
+  assume_shared(&sh);
   const CallInfo& p = sh.call;
   const int rows = p.acc_rows;
   int k1 = 0;  // pass-1 chunks so far
@@ -1007,6 +1021,7 @@ __device__ __noinline__ void sum_role(ResidentShared& sh, int lane) {
 
 // Warpgroup 0 without a given LSE.
 __device__ __noinline__ void pass1_role(ResidentShared& sh, int warp, int lane) {
+  assume_shared(&sh);
   const uint32_t tbase = sh.call.tbase;
   const float c = sh.call.c;
   Group g{sh, 0, warp & 3, lane};
@@ -1040,6 +1055,7 @@ __device__ __noinline__ void pass1_role(ResidentShared& sh, int warp, int lane) 
 // Warpgroup 1 (warpgroup 0 too when the LSE is given: every other chunk).
 template <int w>
 __device__ __noinline__ void pass2_role(ResidentShared& sh, int warp, int lane) {
+  assume_shared(&sh);
   const uint32_t tbase = sh.call.tbase;
   const float c = sh.call.c;
   Group g{sh, w, warp & 3, lane};
@@ -1092,6 +1108,7 @@ __device__ __noinline__ void pass2_role(ResidentShared& sh, int warp, int lane) 
 // warpgroup's arrivals (CTA-scope release/acquire) one GPU-scope fence covers
 // the chunks that are ready, then each adds to its unit's count.
 __device__ __noinline__ void announce_role(ResidentShared& sh, int* p2done, int lane) {
+  assume_shared(&sh);
   if (lane == 0 && wait_bar(sh, &sh.startbar, 0)) {  // every CTA has zeroed its counts
     int next = 0, issued = 0;  // first chunk not yet announced, pass-2 chunks listed
     for (int ci = 0;;) {
@@ -1120,6 +1137,7 @@ __device__ __noinline__ void announce_role(ResidentShared& sh, int* p2done, int 
 
 // Two warps, each every other unit of a warpgroup (its buffer of two).
 __device__ __noinline__ void denominator_role(ResidentShared& sh, int mine, int lane) {
+  assume_shared(&sh);
   const bool given_lse = sh.call.given_lse != 0;
   int unit[2] = {-1, -1}, k[2] = {0, 0};  // per warpgroup: last unit, units so far
   bool ok = given_lse || wait_bar(sh, &sh.startbar, 0);  // no stale sums from here on

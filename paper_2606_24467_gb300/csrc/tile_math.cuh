@@ -8,6 +8,13 @@
 namespace ckv {
 namespace {
 
+// `p` points to shared memory: plain shared-memory instructions instead of
+// generic ones, in functions that are not inlined.
+template <class T>
+__device__ __forceinline__ void assume_shared(const T* p) {
+  __builtin_assume(__isShared(p));
+}
+
 // Two fp32 numbers in a register pair, and packed arithmetic on them.
 __device__ __forceinline__ uint64_t pack2(float a, float b) {
   uint64_t r;

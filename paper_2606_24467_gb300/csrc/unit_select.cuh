@@ -5,6 +5,7 @@
 
 #include "ckv_device.cuh"
 #include "select_common.cuh"
+#include "tile_math.cuh"
 
 namespace ckv {
 namespace {
@@ -46,12 +47,6 @@ struct SelCall {
   long long tok_stride_v16, head_stride_v16;
 };
 
-// `p` points to shared memory: plain shared-memory instructions instead of
-// generic ones, in functions that are not inlined.
-template <class T>
-__device__ __forceinline__ void assume_shared(const T* p) {
-  __builtin_assume(__isShared(p));
-}
 __device__ __forceinline__ void cbar() { named_bar_sync(kBarC, kCThreads); }
 
 // Zero the radix state (the workers' form of radix_init).
