@@ -243,8 +243,8 @@ int compresskv_compress_layer(const ckv_problem* p, const void* q_win, const voi
  * memory while the query rows' sums of exponentials are added up over the
  * SMs, and the normalised probabilities of each key (Eq. 1-2) are then summed
  * in fp32 from the same logits.  "Short": the layer's longest prompt has at
- * most 32768 tokens when its widest group has at most 32 query rows (|S_g| W;
- * 16384 with the LSE given), 16384 at 64 rows, 8192 at 128, 4096 at 192.
+ * most 49152 tokens when its widest group has at most 64 query rows (|S_g| W),
+ * 8192 at 128 rows, 4096 at 192 (24576, 12288 and 6144 with the LSE given).
  * Other layers take the two-pass kernel, which reads K twice per chunk of 16
  * tiles of 128 keys: a first pass sums each query row's exponentials (softmax
  * statistics of the chunk), and once every chunk of the unit is in and the

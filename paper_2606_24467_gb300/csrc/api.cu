@@ -927,23 +927,24 @@ int run_gather(const ckv_problem* p, const Info& I, const int32_t* indices,
 // launches both.  (The prompts of one layer go together: taking a 28-layer
 // batch's shorter prompts apart cost two tails, 3195 -> 3285 us.)
 // Two-pass / resident time in us (1 layer; 32 layers; 8 KV heads):
-//   32 rows      16384: 85/67, 568/319    32768: 98/90, 699/586
-//                65536: 128/135
-//   32, LSE      16384: 66/65, 348/277    24576: 71/75, 381/395
-//   64 rows      16384: 1.2 to 1.8 times faster    32768: 0.91 to 1.2
-//   128 rows      8192: 1.6, 1.22 times            16384: 0.63 (32 layers)
-//   192 rows      4096: 2.5, 1.5 times              8192: 0.78 (32 layers)
+//   32 rows      32768: 89/68, 723/496      49152: 108/84, 1009/725
+//   64 rows      32768: 91/76, 683/661      49152: 111/95, 971/977
+//   128 rows      8192: 79/49, 486/368      12288: 81/59, 496/551
+//   192 rows      4096: 85/41, 480/411       6144: 88/51, 489/604
+// with the LSE given, when the two-pass kernel reads K once as well:
+//   64 rows      24576: 63/57, 339/338      32768: 71/67, 396/437
+//   128 rows     12288: 55/46, 276/243      16384: 56/49, 285/318
+//   192 rows      6144: 51/36, 265/208       8192: 58/44, 267/271
 // The resident kernel loses on long prompts because a unit's logits must all
 // be on the chip at once: beyond a few tiles per SM the chunks of different
 // units no longer overlap.
-constexpr int kResidentMinGrid = 32;  // CTAs that hold a unit of every admitted size
+constexpr int kResidentMinGrid = 96;  // CTAs that hold a unit of every admitted size
 static_assert(kResidentMaxRows <= kMaxQRows, "resident rows");
 
 bool takes_resident(int rows, int len, bool given_lse) {
-  if (rows <= 32) return len <= (given_lse ? 16384 : 32768);
-  if (rows <= 64) return len <= 16384;
-  if (rows <= 128) return len <= 8192;
-  return rows <= kResidentMaxRows && len <= 4096;
+  if (rows <= 64) return len <= (given_lse ? 24576 : 49152);
+  if (rows <= 128) return len <= (given_lse ? 12288 : 8192);
+  return rows <= kResidentMaxRows && len <= (given_lse ? 6144 : 4096);
 }
 
 // K tiles per chunk of a resident layer: up to four, as a chunk costs about
@@ -953,8 +954,8 @@ bool takes_resident(int rows, int len, bool given_lse) {
 // 777-token layer 27.8 us with one tile a chunk, 28.3 with two, 30.9 with
 // four; a 4096-token one 37.5 with two, 38.9 with four, but 32 of the
 // latter 137 with two, 114 with four) or wide groups (the tensor memory must
-// hold two chunks).  A unit then has at most 64 chunks (128 of 32 rows, of
-// which the tensor memory holds eight): kResidentMinGrid CTAs hold any.
+// hold two chunks).  A unit then has at most 128 chunks of two tiles or 96 of
+// four (the tensor memory holds 2 to 8): kResidentMinGrid CTAs hold any.
 int resident_chunk_tiles(int rows, long long layer_tiles) {
   const int most = rows <= 64 ? kResidentChunkTiles : (rows <= 128 ? 2 : 1);
   return std::min(most, layer_tiles <= 64 ? 1 : (layer_tiles <= 256 ? 2 : 4));

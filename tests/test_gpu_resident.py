@@ -32,8 +32,9 @@ def _make(name, lens, **over):
     # the longest prompt whose scores the selection holds in shared memory
     # (6144 keys before the window)
     (16, (1, 1), [513, 4096, 4097, 6160, 6161, 8193]),
-    # 32 and 64 rows: the line of 64 rows and a prompt that only 32 rows keep
-    (32, (1, 2), [33, 8192, 16384, 16385]),
+    # 32 and 64 rows: the line of both, from either side
+    (32, (1, 2), [33, 16384, 49152]),
+    (32, (1, 2), [33, 49153]),
     # 64, 128 and 192 rows in one call: the lines of 192 and of 128 rows
     (64, (1, 3), [65, 4096, 4097, 8192, 8193]),
 ])
@@ -83,7 +84,7 @@ def test_calls_on_two_streams_at_once(cuda_device):
     needs all its CTAs resident): the bits of the calls made one by one."""
     dev = cuda_device
     runs = []
-    for seed, lens in enumerate(([1500, 3000], [900, 16385])):
+    for seed, lens in enumerate(([1500, 3000], [900, 49153])):
         cfg, layers = _make("c2", lens, n_layers=2 + seed, budget_mean=200)
         want, _, _ = _run_call(layers, cfg, dev)
         q, k, v, cu, b, m = _pack(layers, dev)
