@@ -302,7 +302,7 @@ WorkspaceLayout workspace_layout(const Info& I) {
 // layout above, which the other entry points use).  A function of the problem
 // alone: rows are bounded with every head of a group counted as SRH.
 struct FusedLayout {
-  size_t raw, pooled, partials, bias, total;
+  size_t raw, pooled, rowmax, partials, bias, total;
   long long n_chunks;
   int part_stride;
 };
@@ -311,6 +311,12 @@ int chunks_per_unit(const Info& I, int s) {
   if (I.n[s] <= 0) return 0;
   const int tiles = (I.len[s] + kTileTokens - 1) / kTileTokens;
   return (tiles + kChunkTiles - 1) / kChunkTiles;
+}
+
+size_t row_max_bytes(const Info& I) {
+  const long long scores = static_cast<long long>(I.Hkv) * I.p_total;
+  return align256(static_cast<size_t>(row_max_offset(scores, I.Hkv, 0, I.B) + 1) *
+                  sizeof(uint32_t));
 }
 
 FusedLayout fused_layout(const Info& I) {
@@ -322,7 +328,8 @@ FusedLayout fused_layout(const Info& I) {
   const size_t scores = align256(static_cast<size_t>(I.Hkv) * I.p_total * sizeof(float));
   F.raw = kHeaderBytes;
   F.pooled = F.raw + scores;
-  F.partials = F.pooled + scores;
+  F.rowmax = F.pooled + scores;
+  F.partials = F.rowmax + row_max_bytes(I);
   F.bias = F.partials + align256(static_cast<size_t>(F.n_chunks) * kFusedPartsPerChunk *
                                  F.part_stride * sizeof(float2));
   F.total = F.bias + align256(static_cast<size_t>(units) * F.part_stride * sizeof(float));
@@ -331,7 +338,7 @@ FusedLayout fused_layout(const Info& I) {
 
 // Layout of the resident call's workspace (it aliases the ones above).
 struct ResidentLayout {
-  size_t raw, pooled, acc, pairs, ctr, total;
+  size_t raw, pooled, rowmax, acc, pairs, ctr, total;
 };
 
 ResidentLayout resident_layout(const Info& I) {
@@ -341,10 +348,11 @@ ResidentLayout resident_layout(const Info& I) {
   const size_t scores = align256(static_cast<size_t>(I.Hkv) * I.p_total * sizeof(float));
   F.raw = kHeaderBytes;
   F.pooled = F.raw + scores;
-  F.acc = F.pooled + scores;
+  F.rowmax = F.pooled + scores;
+  F.acc = F.rowmax + row_max_bytes(I);
   F.pairs = F.acc + align256(units * kAccWords * rows * 8);
   F.ctr = F.pairs + align256(static_cast<size_t>(kResidentMaxGrid) * kPairRing * rows * sizeof(float2));
-  F.total = F.ctr + align256(2 * units * sizeof(int));
+  F.total = F.ctr + align256((3 * units + 1) * sizeof(int));
   return F;
 }
 
@@ -961,11 +969,15 @@ int resident_chunk_tiles(int rows, long long layer_tiles) {
   return std::min(most, layer_tiles <= 64 ? 1 : (layer_tiles <= 256 ? 2 : 4));
 }
 
-// What the two persistent kernels' parameters have in common.
+// What the two persistent kernels' parameters have in common; calls of up to
+// piece_units units pool long units in pieces (unit_select.cuh).  16 layers
+// (128 units), by the selection / in pieces: resident kernel 16384 tokens
+// 187/195 us, 32768 339/357; two-pass 65536 tokens 693/670, 32768 with the
+// LSE given 234/223.
 template <class Params>
 void fill_common(Params& P, const ckv_problem* p, const Info& I, const SrhLists& S,
                  const std::vector<int>& co, int32_t* indices, const void* k, const void* v,
-                 void* k_out, void* v_out, const LseInput& lse, bool do_select) {
+                 void* k_out, void* v_out, const LseInput& lse, bool do_select, int piece_units) {
   P.lse = lse.lse;
   P.lse_bs = lse.batch_stride;
   P.lse_hs = lse.head_stride;
@@ -993,6 +1005,11 @@ void fill_common(Params& P, const ckv_problem* p, const Info& I, const SrhLists&
   P.n_units = I.B * I.Hkv;
   P.batch = I.B;
   P.do_select = do_select ? 1 : 0;
+  // (one layer, pooled by the selection / in pieces: 8192 tokens 49/52 us,
+  // 16384 67/65, 32768 90/82, 131072 226/162)
+  int longest = 0;
+  for (int s = 0; s < I.B; ++s) longest = std::max(longest, I.n[s]);
+  P.in_pieces = do_select && longest > 12288 && P.n_units <= piece_units ? 1 : 0;
   P.chunk_off[0] = 0;
   for (int s = 0; s <= I.B; ++s) {
     P.cu_seqlens[s] = I.cu[s];
@@ -1107,10 +1124,12 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
     std::memset(&P, 0, sizeof(P));
     if ((rc = make_k_map(I, p, k, &P.tmap_k)) != CKV_OK) return rc;
     if ((rc = make_q_map(I, p, q_win, &P.tmap_q)) != CKV_OK) return rc;
-    fill_common(P, p, I, S, co, indices, k, v, k_out, v_out, lse, do_select);
+    fill_common(P, p, I, S, co, indices, k, v, k_out, v_out, lse, do_select,
+                Fd->sms / 4);
     P.raw = raw_user ? raw_user : reinterpret_cast<float*>(wb + RL.raw);
     P.raw_scratch = raw_user ? 0 : 1;
     P.pooled = pooled_user ? pooled_user : reinterpret_cast<float*>(wb + RL.pooled);
+    P.rowmax = reinterpret_cast<uint32_t*>(wb + RL.rowmax);
     P.status = reinterpret_cast<int*>(wb);
     P.ctr = reinterpret_cast<int*>(wb + kFusedCtrOffset);
     P.unit_ctr = reinterpret_cast<int*>(wb + RL.ctr);
@@ -1139,10 +1158,12 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   std::memset(&P, 0, sizeof(P));
   if ((rc = make_k_map(I, p, k, &P.tmap_k)) != CKV_OK) return rc;
   if ((rc = make_q_map(I, p, q_win, &P.tmap_q)) != CKV_OK) return rc;
-  fill_common(P, p, I, S, co, indices, k, v, k_out, v_out, lse, do_select);
+  fill_common(P, p, I, S, co, indices, k, v, k_out, v_out, lse, do_select,
+              Fd->sms - 1);
   P.raw = raw_user ? raw_user : reinterpret_cast<float*>(wb + FL.raw);
   P.raw_scratch = raw_user ? 0 : 1;
   P.pooled = pooled_user ? pooled_user : reinterpret_cast<float*>(wb + FL.pooled);
+  P.rowmax = reinterpret_cast<uint32_t*>(wb + FL.rowmax);
   P.status = reinterpret_cast<int*>(wb);
   P.ctr = reinterpret_cast<int*>(wb + kFusedCtrOffset);
   P.partials = reinterpret_cast<float2*>(wb + FL.partials);

@@ -162,6 +162,12 @@ constexpr size_t kFusedCtrBytes = static_cast<size_t>(kFusedCtrHead + 3 * kFused
 // raw-score row); with it the merge / select region leaves room for two Q
 // buffers of 192 query rows (W = 64 with three SRH heads) and two K stages
 constexpr int kFusedCandCap = 3072;
+// Where the row maxima of unit (s, g) start: its score offset in rows of 32,
+// and one more row per unit before it in score order (a unit's last row may be
+// partial).
+__host__ __device__ inline long long row_max_offset(long long soff, int g, int s, int batch) {
+  return (soff >> 5) + static_cast<long long>(g) * batch + s;
+}
 constexpr int kSelRegion = 38 * 1024;  // shared memory of the merge / select warps
 
 struct FusedParams {
@@ -206,6 +212,8 @@ struct FusedParams {
   // a prefix and no chunks is not one of this launch
   int chunk_off[kFusedMaxSeqs + 1];
   uint32_t srh_bits[kFusedMaxLists];  // per (mask, group): bit i = query head group*G + i is SRH
+  uint32_t* rowmax;            // largest pooled score of every 32 keys (row_max_offset)
+  int in_pieces;               // long units are pooled in pieces (few units in the call)
 };
 
 cudaError_t launch_fused(const FusedParams& p, int grid, size_t smem, cudaStream_t s);
@@ -238,7 +246,8 @@ struct ResidentParams {
   float* pooled;               // pooled scores, score layout (caller's buffer or workspace)
   int* status;                 // device status word
   int* ctr;                    // header words (abort, start)
-  int* unit_ctr;               // per unit: chunks scored; then per unit: ticket of its second round
+  int* unit_ctr;               // per unit: chunks scored; ticket of its second round; pieces pooled;
+                               // then the workers' next ticket
   unsigned long long* acc;     // [unit][kAccWords][acc_rows]: the units' sums of exponentials
   int acc_rows;                // row length of the accumulators (a multiple of 32)
   float c;                     // scale * log2(e)
@@ -260,6 +269,8 @@ struct ResidentParams {
   int chunk_off[kFusedMaxSeqs + 1];   // first chunk of sequence s (units of s are consecutive)
   uint8_t seq_chunk[kFusedMaxSeqs];   // K tiles per chunk; 0: not a sequence of this launch
   uint32_t srh_bits[kFusedMaxLists];  // per (mask, group): bit i = query head group*G + i is SRH
+  uint32_t* rowmax;            // largest pooled score of every 32 keys (row_max_offset)
+  int in_pieces;               // long units are pooled in pieces (few units in the call)
 };
 
 cudaError_t launch_resident(const ResidentParams& p, int grid, size_t smem, cudaStream_t s);

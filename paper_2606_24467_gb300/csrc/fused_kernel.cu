@@ -95,11 +95,13 @@ constexpr int kCtrMerge = 2;  // next unit whose denominators to merge
 constexpr int kCtrSel = 3;    // next unit to select
 constexpr int kCtrExit = 4;   // CTAs finished
 constexpr int kCtrAbort = 5;  // set when any wait ran out
+constexpr int kCtrTicket = 7; // the workers' next ticket (pooling in pieces)
 constexpr int kCtrNever = 6;  // never set: the test hook's stall waits for it
 
 constexpr int kTaskEnd = 0;
 constexpr int kTaskMerge = 1;
 constexpr int kTaskSelect = 2;
+constexpr int kTaskPool = 3;
 
 struct ChunkDesc {
   int end, pass, s, g, t0, t1, chunk, n_rows;
@@ -154,6 +156,7 @@ struct Fused {
   __device__ int rows(int s, int g) const { return __popc(p.srh_bits[list(s, g)]) * p.window; }
   __device__ int* ticket(int u) const { return p.ctr + kFusedCtrHead + u; }
   __device__ int* p2done(int u) const { return p.ctr + kFusedCtrHead + p.n_units + u; }
+  // 2 once the unit's denominators are merged, and 4 more per piece pooled
   __device__ int* bias_state(int u) const { return p.ctr + kFusedCtrHead + 2 * p.n_units + u; }
   __device__ bool aborted() const { return ld_volatile(p.ctr + kCtrAbort) != 0; }
   __device__ void raise_abort() const {
@@ -406,6 +409,52 @@ __device__ void claim_task(const Fused& F, int* task) {
   task[1] = 0;
 }
 
+// The same when units are pooled in pieces: the ticket's task (a piece once
+// all the unit's pass-2 chunks are in, a selection once its pieces are
+// pooled), or meanwhile the next unit to merge.
+__device__ void claim_ticket(const Fused& F, TaskPos& T, int* task) {
+  const FusedParams& p = F.p;
+  if (T.t < 0)
+    take_ticket(T, p.ctr + kCtrTicket, p.batch, p.num_kv_heads, [&](int s) {
+      return F.chunks_per_unit(s) > 0 ? pool_pieces(F.prefix(s)) : 0;
+    });
+  const uint64_t t0 = globaltimer_ns();
+  // (every unit's selection is ahead of the first ticket without a task, and
+  // with it every merge)
+  while (T.unit >= 0) {
+    if (F.aborted() || *reinterpret_cast<volatile int*>(F.abort_cta)) break;
+    const bool ready = T.piece < 0 && T.pieces > 0
+                           ? (ld_acquire(F.bias_state(T.unit)) >> 2) >= T.pieces
+                           : ld_acquire(F.p2done(T.unit)) >= kEpiWarps * F.chunks_per_unit(T.s);
+    if (ready) {
+      task[0] = T.piece < 0 ? kTaskSelect : kTaskPool;
+      task[1] = T.unit;
+      task[2] = T.piece;
+      T.t = -1;
+      return;
+    }
+    if (!p.given_lse) {
+      const int m = ld_volatile(p.ctr + kCtrMerge);
+      if (m < p.n_units &&
+          ld_acquire(F.ticket(m)) >= p.nwg * F.chunks_per_unit(m / p.num_kv_heads)) {
+        if (atomicCAS(p.ctr + kCtrMerge, m, m + 1) == m) {
+          task[0] = kTaskMerge;
+          task[1] = m;
+          return;
+        }
+        continue;
+      }
+    }
+    if (globaltimer_ns() - t0 > p.wait_ns) {
+      F.raise_abort();
+      break;
+    }
+    __nanosleep(128);
+  }
+  task[0] = kTaskEnd;
+  task[1] = 0;
+}
+
 // Pass 1, rare: an exponent of this 32-column group passed 2^64 (or the
 // references are still -inf): raise every query's R to kShift below its
 // largest scaled logit among the warp's 32 keys, shrink the sums kept against
@@ -443,6 +492,7 @@ __device__ __forceinline__ void wait_plain(uint32_t bar, uint32_t parity, uint64
   mbar_wait_bounded(bar, parity, &never, nullptr, timeout_ns);
 }
 
+template <bool kPieces>
 __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_constant__ FusedParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -961,11 +1011,19 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
   } else if (warp >= kCWarp0 && warp < kCWarp0 + kCThreads / 32) {
     // ------------------------------------------------------------ merge / select
     const int ct = threadIdx.x - kCWarp0 * 32;
+    TaskPos T{-1, 0, 0, -1, -1, 0};
     for (;;) {
-      if (ct == 0) claim_task(F, s_task);
+      if (ct == 0) {
+        if constexpr (kPieces) {
+          claim_ticket(F, T, s_task);
+        } else {
+          claim_task(F, s_task);
+        }
+      }
       cbar();
       const int type = s_task[0];
       const int idx = s_task[1];
+      const int piece = s_task[2];
       cbar();
       if (type == kTaskEnd) break;
       if (type == kTaskMerge) {
@@ -982,7 +1040,18 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
         U.out0 = p.cu_out[s];
         U.kept = p.cu_out[s + 1] - U.out0;
         const long long soff = static_cast<long long>(g) * p.p_total + p.cu_prefix[s];
-        select_unit(sel, U, p.raw + soff, p.pooled + soff,
+        if constexpr (kPieces) {
+          SelShared& ss = *reinterpret_cast<SelShared*>(creg);
+          uint32_t* const rowmax = p.rowmax + row_max_offset(soff, g, s, p.batch);
+          if (type == kTaskPool) {
+            pool_piece(p.raw + soff, p.pooled + soff, rowmax, U.L - U.W, piece, sel, ss,
+                       F.bias_state(idx), 4, ct);
+            continue;
+          }
+          if (ct == 0) ss.rowmax = rowmax;
+          cbar();
+        }
+        select_unit<kPieces>(sel, U, p.raw + soff, p.pooled + soff,
                     p.indices + static_cast<long long>(g) * p.o_total + U.out0, creg, ct);
       }
     }
@@ -1017,7 +1086,10 @@ size_t fused_smem_bytes(int q_half_bytes, int q_bufs, int stages, int row_stride
 }
 
 cudaError_t fused_set_smem_limit(size_t bytes) {
-  return cudaFuncSetAttribute(fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const cudaError_t e = cudaFuncSetAttribute(
+      fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(bytes));
 }
 
@@ -1029,7 +1101,7 @@ cudaError_t launch_fused(const FusedParams& p, int grid, size_t smem, cudaStream
   cfg.stream = stream;
   cfg.attrs = nullptr;
   cfg.numAttrs = 0;
-  return cudaLaunchKernelEx(&cfg, fused_kernel, p);
+  return cudaLaunchKernelEx(&cfg, p.in_pieces ? fused_kernel<true> : fused_kernel<false>, p);
 }
 
 }  // namespace ckv

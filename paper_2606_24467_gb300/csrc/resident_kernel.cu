@@ -191,7 +191,7 @@ struct ResidentShared {
   uint64_t dnfull[2][2], dnempty[2][2];                // denominators of a unit, per warpgroup
   uint64_t startbar;
   uint32_t tmem;
-  int abort_cta, task;
+  int abort_cta, task, piece;
   int sum_pos;                                         // chunks below have left their pairs
   int p2_unit[kPub];
   ChunkDesc descs[kDescs];
@@ -1170,6 +1170,7 @@ __device__ __noinline__ void denominator_role(ResidentShared& sh, int mine, int 
   __syncwarp();
 }
 
+template <bool kPieces>
 __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_constant__ ResidentParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -1395,8 +1396,8 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
         const long long na = static_cast<long long>(p.n_units) * kAccWords * p.acc_rows / 2;
         for (long long i = who; i < na; i += all) a[i] = make_uint4(0u, 0u, 0u, 0u);
       }
-      for (long long i = who; i < 2 * static_cast<long long>(p.n_units); i += all)
-        p.unit_ctr[i] = 0;
+      const long long nc = (kPieces ? 3 : 2) * static_cast<long long>(p.n_units) + (kPieces ? 1 : 0);
+      for (long long i = who; i < nc; i += all) p.unit_ctr[i] = 0;
       cbar();
       if (ct == 0) {
         __threadfence();
@@ -1413,7 +1414,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
       }
     }
 #pragma unroll 1
-    for (int u = blockIdx.x; p.do_select && u < p.n_units; u += grid) {
+    for (int u = blockIdx.x; !kPieces && p.do_select && u < p.n_units; u += grid) {
       const int s = u / p.num_kv_heads;
       const int g = u - s * p.num_kv_heads;
       if (p.seq_chunk[s] == 0) continue;  // taken by the two-pass kernel
@@ -1431,8 +1432,54 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
       U.out0 = p.cu_out[s];
       U.kept = p.cu_out[s + 1] - U.out0;
       const long long soff = static_cast<long long>(g) * p.p_total + p.cu_prefix[s];
-      select_unit(sh.call.sel, U, p.raw + soff, p.pooled + soff,
+      select_unit<false>(sh.call.sel, U, p.raw + soff, p.pooled + soff,
                   p.indices + static_cast<long long>(g) * p.o_total + U.out0, creg, ct);
+    }
+    TaskPos T{-1, 0, 0, -1, -1, 0};
+#pragma unroll 1
+    while (kPieces) {
+      if (ct == 0) {
+        take_ticket(T, p.unit_ctr + 3 * p.n_units, p.batch, p.num_kv_heads, [&](int s) {
+          return p.seq_chunk[s] == 0
+                     ? 0
+                     : pool_pieces(p.cu_seqlens[s + 1] - p.cu_seqlens[s] - p.window);
+        });
+        bool ok = T.unit >= 0;
+        if (ok)
+          ok = T.piece < 0 && T.pieces > 0
+                   ? wait_counter(sh, p.unit_ctr + 2 * p.n_units + T.unit, T.pieces)
+                   : wait_counter(sh, p.unit_ctr + T.unit,
+                                  (p.chunk_off[T.s + 1] - p.chunk_off[T.s]) / p.num_kv_heads);
+        sh.task = ok ? T.unit : -1;
+        sh.piece = T.piece;
+      }
+      cbar();
+      const int u = sh.task;
+      const int piece = sh.piece;
+      cbar();
+      if (u < 0) break;
+      const int s = u / p.num_kv_heads;
+      const int g = u - s * p.num_kv_heads;
+      if (p.seq_chunk[s] == 0) continue;  // taken by the two-pass kernel
+      SelUnit U;
+      U.g = g;
+      U.seq0 = p.cu_seqlens[s];
+      U.L = p.cu_seqlens[s + 1] - U.seq0;
+      U.W = p.window;
+      U.out0 = p.cu_out[s];
+      U.kept = p.cu_out[s + 1] - U.out0;
+      const long long soff = static_cast<long long>(g) * p.p_total + p.cu_prefix[s];
+      SelShared& ss = *reinterpret_cast<SelShared*>(creg);
+      uint32_t* const rowmax = p.rowmax + row_max_offset(soff, g, s, p.batch);
+      if (piece >= 0) {
+        pool_piece(p.raw + soff, p.pooled + soff, rowmax, U.L - U.W, piece, sh.call.sel, ss,
+                   p.unit_ctr + 2 * p.n_units + u, 1, ct);
+        continue;
+      }
+      if (ct == 0) ss.rowmax = rowmax;
+      cbar();
+      select_unit<true>(sh.call.sel, U, p.raw + soff, p.pooled + soff,
+                        p.indices + static_cast<long long>(g) * p.o_total + U.out0, creg, ct);
     }
   }
 
@@ -1455,7 +1502,10 @@ size_t resident_smem_bytes(int q_half_bytes, int q_bufs, int stages, int acc_row
 }
 
 cudaError_t resident_set_smem_limit(size_t bytes) {
-  return cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const cudaError_t e = cudaFuncSetAttribute(
+      resident_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(resident_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(bytes));
 }
 
@@ -1471,7 +1521,7 @@ cudaError_t launch_resident(const ResidentParams& p, int grid, size_t smem, cuda
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, resident_kernel, p);
+  return cudaLaunchKernelEx(&cfg, p.in_pieces ? resident_kernel<true> : resident_kernel<false>, p);
 }
 
 }  // namespace ckv

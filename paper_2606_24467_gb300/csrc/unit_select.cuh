@@ -25,6 +25,7 @@ struct SelShared {
   int wcnt[8], wbase[8];
   int wcnt_ge[8];  // per-warp counts at the best threshold with at least k keys above
   alignas(16) uint32_t cnt[2][2][8];  // per-warp results of a bisection step
+  uint32_t* rowmax;                   // (pooling in pieces) the unit's row maxima
 };
 static_assert(sizeof(SelShared) <= kSelRegion, "select scratch");
 static_assert(kSelSamples <= kFusedCandCap, "samples live in the position array");
@@ -370,13 +371,17 @@ struct SelUnit {
 // flight.  Bound by instruction latency (two warps per scheduler): 22-27 us
 // for 32736 keys with the seven taps of the usual width unrolled, 33-42 us
 // with a loop over them.
-__device__ __noinline__ void pool_unit(const float* raw, float* pooled, int n, int e, int h, float fP,
-                                       SelShared& sh, int ct) {
+// kRows: only the keys [j0, j1) of such a unit, the largest of every row of 32
+// to rowmax.
+template <bool kRows>
+__device__ __forceinline__ void pool_strips(const float* raw, float* pooled, uint32_t* rowmax,
+                                            int n, int j0, int j1, int e, int h, float fP,
+                                            SelShared& sh, int ct) {
   constexpr int kPer = kPoolStrip / 32;          // keys per lane
   constexpr int kLoads = kPoolBuf / 32;  // with the halo
   assume_shared(&sh);
   const int lane = ct & 31;
-  const bool keep = n <= kSelWhole;
+  const bool keep = !kRows && n <= kSelWhole;
   float* const stage =
       (keep ? reinterpret_cast<float*>(sh.gmax) : reinterpret_cast<float*>(sh.pos)) +
       (ct >> 5) * kPoolBuf;
@@ -429,21 +434,86 @@ __device__ __noinline__ void pool_unit(const float* raw, float* pooled, int n, i
         const uint32_t m = __reduce_max_sync(0xffffffffu, in ? __float_as_uint(s[q]) : 0u);
         top = lane == q ? m : top;
       }
-      if (lane < kPer && base + 32 * lane < n)
-        atomicMax(&sh.gmax[(base + 32 * lane) >> (5 + e)], top);
+      if (lane < kPer && base + 32 * lane < n) {
+        if constexpr (kRows) {
+          rowmax[(base >> 5) + lane] = top;
+        } else {
+          atomicMax(&sh.gmax[(base + 32 * lane) >> (5 + e)], top);
+        }
+      }
     }
   };
-  const int base0 = (ct >> 5) * kPoolStrip;
+  const int base0 = j0 + (ct >> 5) * kPoolStrip;
   load(na, base0);
   load(nb, base0 + 8 * kPoolStrip);
 #pragma unroll 1
-  for (int base = base0; base < n; base += 16 * kPoolStrip) {
+  for (int base = base0; base < j1; base += 16 * kPoolStrip) {
     step(na, base);
-    if (base + 8 * kPoolStrip < n) step(nb, base + 8 * kPoolStrip);
+    if (base + 8 * kPoolStrip < j1) step(nb, base + 8 * kPoolStrip);
+  }
+}
+__device__ __noinline__ void pool_unit(const float* raw, float* pooled, int n, int e, int h, float fP,
+                                       SelShared& sh, int ct) {
+  pool_strips<false>(raw, pooled, nullptr, n, 0, n, e, h, fP, sh, ct);
+}
+
+// Pooling in pieces: when a call has fewer units than CTAs, the units whose
+// keys do not fit shared memory are pooled by all of them, a piece at a time,
+// before one CTA selects (one 131072-token layer: 226 -> 163 us, 32768: 90 ->
+// 82).  With more units it gains nothing, and its code in the kernels costs
+// 5-10% (32 layers of short prompts: 481 -> 536 us), so that they are
+// instantiated with and without it.
+constexpr int kPoolPiece = 32 * kPoolStrip;  // keys of a pooling task
+__device__ __forceinline__ int pool_pieces(int n) {
+  return n <= kSelWhole ? 0 : (n + kPoolPiece - 1) / kPoolPiece;
+}
+// One piece by the 256 threads, which then adds to *count.
+__device__ __noinline__ void pool_piece(const float* raw, float* pooled, uint32_t* rowmax, int n,
+                                        int piece, const SelCall& p, SelShared& sh, int* count,
+                                        int add, int ct) {
+  assume_shared(&p);
+  const int j0 = piece * kPoolPiece;
+  pool_strips<true>(raw, pooled, rowmax, n, j0, min(n, j0 + kPoolPiece), 0, (p.pool_width - 1) >> 1,
+                    static_cast<float>(p.pool_width), sh, ct);
+  __threadfence_block();
+  cbar();
+  if (ct == 0) {
+    fence_acq_rel_gpu();  // (cumulative: the barrier's other writes too)
+    atomicAdd(count, add);
   }
 }
 
-// Selection of a unit.  Pooling, then the top-k: a unit of at most
+// The workers' tasks then, in one order that every CTA takes tickets of: of
+// every unit its pieces, then its selection.  A ticket is taken before its
+// task is ready: claims by compare-and-swap once a task is ready took 1 us
+// apiece (152 CTAs at one counter).
+struct TaskPos {
+  int t;                    // the ticket; -1: none taken
+  int s, off;               // a sequence at or before its own, the tickets before that
+  int unit, piece, pieces;  // its task (unit -1: past the last); piece -1: the selection
+};
+template <class Pieces>
+__device__ __forceinline__ void take_ticket(TaskPos& T, int* counter, int batch, int Hkv,
+                                            Pieces pieces) {
+  T.t = atomicAdd(counter, 1);
+  T.unit = -1;
+  for (; T.s < batch; ++T.s) {
+    T.pieces = pieces(T.s);
+    const int per = T.pieces + 1;
+    const int r = T.t - T.off;
+    if (r < Hkv * per) {
+      const int g = r / per;
+      T.unit = T.s * Hkv + g;
+      T.piece = r - g * per;
+      if (T.piece == T.pieces) T.piece = -1;
+      return;
+    }
+    T.off += Hkv * per;
+  }
+}
+
+// Selection of a unit.  Pooling (of a unit that was not pooled in pieces),
+// then the top-k: a unit of at most
 // kSelWhole prefix keys by bisection over its keys in shared
 // memory; a longer one by a lower bound of the k-th largest score -- the k-th
 // largest group maximum (k groups have a key at least that large) or, with
@@ -451,6 +521,7 @@ __device__ __noinline__ void pool_unit(const float* raw, float* pooled, int n, i
 // order and the bisection among them (a radix search among those in global
 // memory, or all the unit's scores, when the bound keeps too few or too many); then the window and the K/V rows.  Pooled
 // scores are >= 0: their bit patterns order like their values.
+template <bool kPieces>
 __device__ __noinline__ void select_unit(const SelCall& p, const SelUnit U, float* raw,
                                          float* pooled, int32_t* out, uint8_t* creg, int ct) {
   assume_shared(creg);
@@ -465,9 +536,19 @@ __device__ __noinline__ void select_unit(const SelCall& p, const SelUnit U, floa
   while (((n + 31) >> 5) > (kSelGroups << e)) ++e;
   const int nr = (n + 31) >> 5;
   const int ng = (nr + (1 << e) - 1) >> e;
-  for (int i = ct; i < ng; i += kCThreads) sh.gmax[i] = 0u;
-  cbar();
-  pool_unit(raw, pooled, n, e, (p.pool_width - 1) >> 1, static_cast<float>(p.pool_width), sh, ct);
+  if (kPieces && n > kSelWhole) {
+    const uint32_t* const rowmax = sh.rowmax;
+#pragma unroll 4
+    for (int i = ct; i < ng; i += kCThreads) {
+      uint32_t m = 0u;
+      for (int r = i << e; r < min(nr, (i + 1) << e); ++r) m = max(m, __ldcg(rowmax + r));
+      sh.gmax[i] = m;
+    }
+  } else {
+    for (int i = ct; i < ng; i += kCThreads) sh.gmax[i] = 0u;
+    cbar();
+    pool_unit(raw, pooled, n, e, (p.pool_width - 1) >> 1, static_cast<float>(p.pool_width), sh, ct);
+  }
   __threadfence_block();
   cbar();
   const int kept = U.kept;

@@ -35,6 +35,9 @@ def _make(name, lens, **over):
     # 32 and 64 rows: the line of both, from either side
     (32, (1, 2), [33, 16384, 49152]),
     (32, (1, 2), [33, 49153]),
+    # pooling in pieces of 6144 keys (few units, a prompt above 12288), the last
+    # of one key and of one row
+    (16, (1, 1), [2 * 6144 + 17, 2 * 6144 + 48, 6160]),
     # 64, 128 and 192 rows in one call: the lines of 192 and of 128 rows
     (64, (1, 3), [65, 4096, 4097, 8192, 8193]),
 ])
