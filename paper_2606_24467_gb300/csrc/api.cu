@@ -926,21 +926,21 @@ int run_gather(const ckv_problem* p, const Info& I, const int32_t* indices,
   return traced(tr, CKV_KERNEL_GATHER, [&] { return launch_gather(P, rows, stream); });
 }
 
-// Which of the two persistent kernels a layer takes: the resident one
-// (resident_kernel.cu: K read once, the logits kept in tensor memory until
-// the softmax sums are complete) for short prompts, else the two-pass one
-// (fused_kernel.cu).  The lines are by the layer's longest prompt and the query
-// rows of its widest group, and by nothing else of the call, so that a layer
-// gives the same bits alone or among others; a call with layers of both kinds
-// launches both.  (The prompts of one layer go together: taking a 28-layer
-// batch's shorter prompts apart cost two tails, 3195 -> 3285 us.)
+// Whether a layer is one for the resident kernel (resident_kernel.cu: K read
+// once, the logits kept in tensor memory until the softmax sums are complete):
+// short prompts, by its longest prompt and the query rows of its widest group.
+// A call takes it when all its layers are, else the two-pass kernel
+// (fused_kernel.cu).  (Both kernels for a call with layers of both kinds cost
+// a second tail: 32 layers of 15826 tokens with one such layer 568 -> 665 us.)
 // Two-pass / resident time in us (1 layer; 32 layers; 8 KV heads):
 //   32 rows      32768: 89/68, 723/496      49152: 108/84, 1009/725
 //   64 rows      32768: 91/76, 683/661      49152: 111/95, 971/977
+//   96 rows      12288: 78/54, 501/478      16384: 79/59, 515/654
 //   128 rows      8192: 79/49, 486/368      12288: 81/59, 496/551
 //   192 rows      4096: 85/41, 480/411       6144: 88/51, 489/604
 // with the LSE given, when the two-pass kernel reads K once as well:
 //   64 rows      24576: 63/57, 339/338      32768: 71/67, 396/437
+//   96 rows      12288: 54/46, 297/238      16384: 52/49, 293/312
 //   128 rows     12288: 55/46, 276/243      16384: 56/49, 285/318
 //   192 rows      6144: 51/36, 265/208       8192: 58/44, 267/271
 // The resident kernel loses on long prompts because a unit's logits must all
@@ -951,6 +951,7 @@ static_assert(kResidentMaxRows <= kMaxQRows, "resident rows");
 
 bool takes_resident(int rows, int len, bool given_lse) {
   if (rows <= 64) return len <= (given_lse ? 24576 : 49152);
+  if (rows <= 96) return len <= 12288;
   if (rows <= 128) return len <= (given_lse ? 12288 : 8192);
   return rows <= kResidentMaxRows && len <= (given_lse ? 6144 : 4096);
 }
@@ -1050,13 +1051,12 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   DeviceFacts* Fd = nullptr;
   int rc = device_facts(&Fd);
   if (rc != CKV_OK) return rc;
-  // the kernel of every layer (mask), and the query rows of each kernel's
-  // widest group
+  // the call's kernel, and the query rows of its widest group
   const int r_grid = std::min(Fd->sms, kResidentMaxGrid);
   std::vector<int> seq_ct(I.B, 0);  // K tiles per chunk
-  std::vector<uint8_t> in_resident(I.B, 0);
-  int max_rows = 16, r_rows = 16, n_resident = 0;
-  for (int s0 = 0; s0 < I.B; s0 += I.spm) {
+  bool resident = r_grid >= kResidentMinGrid;
+  int max_rows = 16;
+  for (int s0 = 0; s0 < I.B; s0 += I.spm) {  // layer by layer
     int rows = 0, longest = 0;
     for (int g = 0; g < I.Hkv; ++g) rows = std::max(rows, S.rows[I.vgroup(s0, g)]);
     long long tiles = 0;
@@ -1065,29 +1065,11 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
       if (I.n[s_] > 0)
         tiles += static_cast<long long>(I.Hkv) * ((I.len[s_] + kTileTokens - 1) / kTileTokens);
     }
-    const bool res =
-        r_grid >= kResidentMinGrid && takes_resident(rows, longest, lse.lse != nullptr);
-    int& most = res ? r_rows : max_rows;
-    most = std::max(most, rows);
-    if (res) n_resident += I.spm;
-    for (int s_ = s0; s_ < s0 + I.spm; ++s_) {
-      seq_ct[s_] = resident_chunk_tiles(rows, tiles);
-      in_resident[s_] = res ? 1 : 0;
-    }
+    resident = resident && takes_resident(rows, longest, lse.lse != nullptr);
+    max_rows = std::max(max_rows, rows);
+    for (int s_ = s0; s_ < s0 + I.spm; ++s_) seq_ct[s_] = resident_chunk_tiles(rows, tiles);
   }
   auto half_bytes = [](int rows) { return ((((rows + 15) & ~15) * 128) + 1023) & ~1023; };
-  // resident: three Q buffers beside four to eight K tiles, else two beside
-  // at least two
-  const int r_half = half_bytes(r_rows);
-  const int acc_rows = (r_rows + 31) & ~31;
-  int r_stages = 0, r_bufs = 0;
-  for (int nq = 3; nq >= 2 && r_stages == 0; --nq)
-    for (int st = 8; st >= (nq == 3 ? 4 : 2) && r_stages == 0; --st)
-      if (resident_smem_bytes(r_half, nq, st, acc_rows) <= static_cast<size_t>(Fd->smem_optin)) {
-        r_stages = st;
-        r_bufs = nq;
-      }
-  if (r_stages == 0) return CKV_ERR_CUDA;  // cannot happen on sm_103: kResidentMaxRows fit
   const int npad_max = (max_rows + 15) & ~15;
   const int q_half = half_bytes(max_rows);
   const int row_stride = (max_rows + 31) & ~31;
@@ -1097,11 +1079,14 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   const int nbuf = 512 / tstride;
   // three Q buffers when they fit beside a ring of at least four K tiles,
   // else two beside at least two
+  auto smem_bytes = [&](int nq, int st) {
+    return resident ? resident_smem_bytes(q_half, nq, st, row_stride)
+                    : fused_smem_bytes(q_half, nq, st, row_stride, nwg);
+  };
   int stages = 0, q_bufs = 0;
   for (int nq = 3; nq >= 2 && stages == 0; --nq) {
     for (int st = 8; st >= (nq == 3 ? 4 : 2); --st) {
-      if (fused_smem_bytes(q_half, nq, st, row_stride, nwg) <=
-          static_cast<size_t>(Fd->smem_optin)) {
+      if (smem_bytes(nq, st) <= static_cast<size_t>(Fd->smem_optin)) {
         stages = st;
         q_bufs = nq;
         break;
@@ -1118,7 +1103,7 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   char* wb = static_cast<char*>(ws);
 
   Tracer tr{p->trace, stream};
-  if (n_resident > 0) {
+  if (resident) {
     const ResidentLayout RL = resident_layout(I);
     static thread_local ResidentParams P;  // large (about 13 KB): kept off the stack
     std::memset(&P, 0, sizeof(P));
@@ -1134,24 +1119,21 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
     P.ctr = reinterpret_cast<int*>(wb + kFusedCtrOffset);
     P.unit_ctr = reinterpret_cast<int*>(wb + RL.ctr);
     P.acc = reinterpret_cast<unsigned long long*>(wb + RL.acc);
-    P.acc_rows = acc_rows;
+    P.acc_rows = row_stride;
     P.pairs = reinterpret_cast<float2*>(wb + RL.pairs);
-    long long out = 0;  // rows of the sequences this launch selects
     for (int s_ = 0; s_ < I.B; ++s_) {
-      const int ct = in_resident[s_] ? seq_ct[s_] : 0;
       const int tiles = I.n[s_] > 0 ? (I.len[s_] + kTileTokens - 1) / kTileTokens : 0;
-      P.seq_chunk[s_] = static_cast<uint8_t>(ct);
-      P.chunk_off[s_ + 1] = P.chunk_off[s_] + (ct ? I.Hkv * ((tiles + ct - 1) / ct) : 0);
-      if (ct) out += co[s_ + 1] - co[s_];
+      P.seq_chunk[s_] = static_cast<uint8_t>(seq_ct[s_]);
+      P.chunk_off[s_ + 1] =
+          P.chunk_off[s_] + I.Hkv * ((tiles + seq_ct[s_] - 1) / seq_ct[s_]);
     }
     P.n_chunks = P.chunk_off[I.B];
-    P.q_half_bytes = r_half;
-    P.q_bufs = r_bufs;
-    P.stages = r_stages;
-    const size_t smem = resident_smem_bytes(r_half, r_bufs, r_stages, acc_rows);
-    if (P.n_units > 0 && (P.n_chunks > 0 || (do_select && out > 0)))
-      rc = traced(tr, CKV_KERNEL_FUSED, [&] { return launch_resident(P, r_grid, smem, stream); });
-    if (rc != CKV_OK || n_resident == I.B) return rc;
+    P.q_half_bytes = q_half;
+    P.q_bufs = q_bufs;
+    P.stages = stages;
+    if (P.n_units == 0 || (P.n_chunks == 0 && (!do_select || co[I.B] == 0))) return CKV_OK;
+    return traced(tr, CKV_KERNEL_FUSED,
+                  [&] { return launch_resident(P, r_grid, smem_bytes(q_bufs, stages), stream); });
   }
 
   static thread_local FusedParams P;  // large (about 15 KB): kept off the stack
@@ -1169,14 +1151,10 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   P.partials = reinterpret_cast<float2*>(wb + FL.partials);
   P.bias = reinterpret_cast<float*>(wb + FL.bias);
   P.part_stride = FL.part_stride;
-  long long out = 0;  // rows of the sequences this launch selects
-  for (int s_ = 0; s_ < I.B; ++s_) {
-    const int chunks = in_resident[s_] ? 0 : I.Hkv * chunks_per_unit(I, s_);
-    P.chunk_off[s_ + 1] = P.chunk_off[s_] + chunks;
-    if (!in_resident[s_]) out += co[s_ + 1] - co[s_];
-  }
+  for (int s_ = 0; s_ < I.B; ++s_)
+    P.chunk_off[s_ + 1] = P.chunk_off[s_] + I.Hkv * chunks_per_unit(I, s_);
   P.n_chunks = P.chunk_off[I.B];
-  if (P.n_chunks > FL.n_chunks) return CKV_ERR_WORKSPACE;  // cannot happen: same plan
+  if (P.n_chunks != FL.n_chunks) return CKV_ERR_WORKSPACE;  // cannot happen: same plan
   P.q_half_bytes = q_half;
   P.q_bufs = q_bufs;
   P.row_stride = row_stride;
@@ -1184,9 +1162,9 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   P.tstride = tstride;
   P.nbuf = nbuf;
   P.nwg = nwg;
-  if (P.n_units == 0 || (P.n_chunks == 0 && (!do_select || out == 0))) return CKV_OK;
-  const size_t smem = fused_smem_bytes(q_half, q_bufs, stages, row_stride, nwg);
-  return traced(tr, CKV_KERNEL_FUSED, [&] { return launch_fused(P, Fd->sms, smem, stream); });
+  if (P.n_units == 0 || (P.n_chunks == 0 && (!do_select || co[I.B] == 0))) return CKV_OK;
+  return traced(tr, CKV_KERNEL_FUSED,
+                [&] { return launch_fused(P, Fd->sms, smem_bytes(q_bufs, stages), stream); });
 }
 
 }  // namespace

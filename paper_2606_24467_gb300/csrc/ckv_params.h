@@ -173,8 +173,6 @@ constexpr int kSelRegion = 38 * 1024;  // shared memory of the merge / select wa
 struct FusedParams {
   CUtensorMap tmap_k;          // 3-D map over K: (d, kv head, token)
   CUtensorMap tmap_q;          // 4-D map over the window queries: (d, w, head, sequence)
-  const uint16_t* q;           // window queries (f16/bf16 bits)
-  long long q_bs, q_hs, q_ws;  // window-query strides, elements
   const float* lse;            // given-LSE mode: natural-log LSE per (sequence, head, window row)
   long long lse_bs, lse_hs;    // its strides (elements); window rows contiguous
   const uint4* k;              // gather sources (K on the device; V may be mapped host memory)
@@ -208,9 +206,7 @@ struct FusedParams {
   int cu_seqlens[kFusedMaxSeqs + 1];
   int cu_prefix[kFusedMaxSeqs + 1];
   int cu_out[kFusedMaxSeqs + 1];
-  // first chunk of sequence s (units of s are consecutive); a sequence with
-  // a prefix and no chunks is not one of this launch
-  int chunk_off[kFusedMaxSeqs + 1];
+  int chunk_off[kFusedMaxSeqs + 1];   // first chunk of sequence s (units of s are consecutive)
   uint32_t srh_bits[kFusedMaxLists];  // per (mask, group): bit i = query head group*G + i is SRH
   uint32_t* rowmax;            // largest pooled score of every 32 keys (row_max_offset)
   int in_pieces;               // long units are pooled in pieces (few units in the call)
@@ -267,7 +263,7 @@ struct ResidentParams {
   int cu_prefix[kFusedMaxSeqs + 1];
   int cu_out[kFusedMaxSeqs + 1];
   int chunk_off[kFusedMaxSeqs + 1];   // first chunk of sequence s (units of s are consecutive)
-  uint8_t seq_chunk[kFusedMaxSeqs];   // K tiles per chunk; 0: not a sequence of this launch
+  uint8_t seq_chunk[kFusedMaxSeqs];   // K tiles per chunk
   uint32_t srh_bits[kFusedMaxLists];  // per (mask, group): bit i = query head group*G + i is SRH
   uint32_t* rowmax;            // largest pooled score of every 32 keys (row_max_offset)
   int in_pieces;               // long units are pooled in pieces (few units in the call)

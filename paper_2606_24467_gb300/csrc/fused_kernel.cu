@@ -416,7 +416,7 @@ __device__ void claim_ticket(const Fused& F, TaskPos& T, int* task) {
   const FusedParams& p = F.p;
   if (T.t < 0)
     take_ticket(T, p.ctr + kCtrTicket, p.batch, p.num_kv_heads, [&](int s) {
-      return F.chunks_per_unit(s) > 0 ? pool_pieces(F.prefix(s)) : 0;
+      return pool_pieces(F.prefix(s));
     });
   const uint64_t t0 = globaltimer_ns();
   // (every unit's selection is ahead of the first ticket without a task, and
@@ -1031,7 +1031,6 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
       } else if (p.do_select) {
         const int s = idx / Hkv;
         const int g = idx - s * Hkv;
-        if (F.prefix(s) > 0 && F.chunks_per_unit(s) == 0) continue;  // not of this launch
         SelUnit U;
         U.g = g;
         U.seq0 = p.cu_seqlens[s];

@@ -1417,7 +1417,6 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
     for (int u = blockIdx.x; !kPieces && p.do_select && u < p.n_units; u += grid) {
       const int s = u / p.num_kv_heads;
       const int g = u - s * p.num_kv_heads;
-      if (p.seq_chunk[s] == 0) continue;  // taken by the two-pass kernel
       const int nch = (p.chunk_off[s + 1] - p.chunk_off[s]) / p.num_kv_heads;
       if (ct == 0) sh.task = wait_counter(sh, p2done(u), nch) ? 1 : 0;
       cbar();
@@ -1440,9 +1439,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
     while (kPieces) {
       if (ct == 0) {
         take_ticket(T, p.unit_ctr + 3 * p.n_units, p.batch, p.num_kv_heads, [&](int s) {
-          return p.seq_chunk[s] == 0
-                     ? 0
-                     : pool_pieces(p.cu_seqlens[s + 1] - p.cu_seqlens[s] - p.window);
+          return pool_pieces(p.cu_seqlens[s + 1] - p.cu_seqlens[s] - p.window);
         });
         bool ok = T.unit >= 0;
         if (ok)
@@ -1460,7 +1457,6 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
       if (u < 0) break;
       const int s = u / p.num_kv_heads;
       const int g = u - s * p.num_kv_heads;
-      if (p.seq_chunk[s] == 0) continue;  // taken by the two-pass kernel
       SelUnit U;
       U.g = g;
       U.seq0 = p.cu_seqlens[s];

@@ -38,8 +38,12 @@ def _make(name, lens, **over):
     # pooling in pieces of 6144 keys (few units, a prompt above 12288), the last
     # of one key and of one row
     (16, (1, 1), [2 * 6144 + 17, 2 * 6144 + 48, 6160]),
-    # 64, 128 and 192 rows in one call: the lines of 192 and of 128 rows
-    (64, (1, 3), [65, 4096, 4097, 8192, 8193]),
+    # 64, 128 and 192 rows in one call, 64 and 128, 32 to 96: their lines
+    (64, (1, 3), [65, 4096]),
+    (64, (1, 3), [65, 4097]),
+    (64, (1, 2), [65, 8192]),
+    (64, (1, 2), [65, 8193]),
+    (32, (1, 3), [65, 12288]),
 ])
 def test_sizes_around_tiles_chunks_and_the_kernels_line(cuda_device, window, heads, lens):
     cfg, layers = _make("c5", lens, n_layers=2, window=window, srh_per_group=heads,
