@@ -38,10 +38,11 @@ import workloads as wl  # noqa: E402
 METRIC = ("prompt tokens compressed/sec per GB300 and achieved HBM GB/s vs peak at "
           "L=32K–128K")
 UNIT = "tokens/s"
-PROFILE_TRAFFIC = os.path.join(ROOT, "profiles", "fused_llama8b_L32k.md")
-# the timed kernel's own source: a committed traffic figure is shown only
-# while it matches
-KERNEL_SOURCES = ["paper_2606_24467_gb300/csrc/fused_kernel.cu"]
+PROFILE_TRAFFIC = os.path.join(ROOT, "profiles", "resident_llama8b_L32k.md")
+# the timed kernel's own sources: a committed traffic figure is shown only
+# while they match
+KERNEL_SOURCES = ["paper_2606_24467_gb300/csrc/" + f
+                  for f in ("resident_kernel.cu", "unit_select.cuh", "tile_math.cuh")]
 
 
 def parse_args():

@@ -148,7 +148,6 @@ struct GatherParams {
 // re-read from L2), pools, selects and gathers, with work claimed from
 // counters in the workspace.
 constexpr int kChunkTiles = 16;         // K tiles per scoring chunk (references restart per chunk)
-constexpr int kChunkKeys = kChunkTiles * kTileTokens;
 constexpr int kFusedMaxSeqs = kMaxBatch;
 constexpr int kFusedMaxLists = 1024;    // (mask, group) SRH lists of one call
 constexpr int kFusedMaxUnits = kMaxBatch * kMaxKvHeads;

@@ -69,10 +69,12 @@
 // query rows (pass 2) 3 shuffles a tile, where one lane per key takes 31
 // shuffles per block for the first.
 // What bounds it: a short call the chain of its steps (one 777-token layer,
-// 28 us against 67 in the two-pass kernel: start 4, scores 7, selection 11,
-// of which the radix search 5), a full one the epilogue's exponentials and
-// tensor-memory loads (32 layers of 8 prompts of 300 to 4000 tokens: 0.62
-// ms against 3.5), as K is read once.
+// 24 us against 67 in the two-pass kernel before it: start 4, scores 9,
+// selection 8), a full one the time that tensor memory is held: a chunk's
+// logits wait for the sums of the unit's slowest chunk, and the memory holds
+// few chunks (32 layers of 32768 tokens: 619 us, 3.5 TB/s of the K that is
+// read once; 32 layers of 8 prompts of 300 to 4000 tokens: 0.48 ms against
+// 3.5).
 // Every wait is bounded (ResidentParams::wait_ns, kWaitTimeoutNs unless a test
 // shortens it) and on expiry records CKV_ERR_DEVICE_TIMEOUT and stops the
 // call.  A wait depends only on chunks of the same or earlier units, which
