@@ -338,8 +338,11 @@ int compresskv_compress_layer_head_budgets(const ckv_problem* p, const void* q_w
  * inputs and outputs exactly as for compresskv_compress_layer, but no
  * workspace: the scratch is a static device array of CKV_STATIC_SCRATCH_BYTES
  * inside the library, and this call allocates nothing.
- * - A problem whose compresskv_workspace_size exceeds CKV_STATIC_SCRATCH_BYTES
- *   is rejected with CKV_ERR_STATIC_SCRATCH before anything is enqueued.
+ * - A problem whose compresskv_workspace_size, less what only the resident
+ *   kernel takes (some MB with hundreds of units), exceeds
+ *   CKV_STATIC_SCRATCH_BYTES is rejected with CKV_ERR_STATIC_SCRATCH before
+ *   anything is enqueued; one that fits only without that area takes the
+ *   two-pass kernel.
  * - The first call on a device looks up the array's device address (with that
  *   device current); make that first call before any stream capture.  The
  *   address is looked up again when the device's context has changed (after

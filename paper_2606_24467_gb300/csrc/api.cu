@@ -128,6 +128,9 @@ struct Info {
   long long T = 0, p_total = 0;
   // SRH masks: sequence s uses mask s / spm (n_masks masks, spm = B / n_masks)
   int n_masks = 1, spm = 1;
+  // the workspace holds neither the resident kernel's area nor the row maxima
+  // (a static scratch too small for them)
+  bool lean = false;
   int vgroup(int s, int g) const { return srh_group(s, g, spm, Hkv); }
 };
 
@@ -328,11 +331,11 @@ FusedLayout fused_layout(const Info& I) {
   const size_t scores = align256(static_cast<size_t>(I.Hkv) * I.p_total * sizeof(float));
   F.raw = kHeaderBytes;
   F.pooled = F.raw + scores;
-  F.rowmax = F.pooled + scores;
-  F.partials = F.rowmax + row_max_bytes(I);
+  F.partials = F.pooled + scores;
   F.bias = F.partials + align256(static_cast<size_t>(F.n_chunks) * kFusedPartsPerChunk *
                                  F.part_stride * sizeof(float2));
-  F.total = F.bias + align256(static_cast<size_t>(units) * F.part_stride * sizeof(float));
+  F.rowmax = F.bias + align256(static_cast<size_t>(units) * F.part_stride * sizeof(float));
+  F.total = F.rowmax + (I.lean ? 0 : row_max_bytes(I));
   return F;
 }
 
@@ -357,10 +360,14 @@ ResidentLayout resident_layout(const Info& I) {
 }
 
 // The layouts alias one another; selection across groups (with average
-// pooling) does not run the resident kernel.
+// pooling) does not run the persistent kernels, but for the two-pass kernel's
+// former share, which stays reserved.
 size_t base_bytes(const Info& I) {
-  const size_t base = std::max(workspace_layout(I).total, fused_layout(I).total);
-  return I.layer && !I.pool_max ? base : std::max(base, resident_layout(I).total);
+  Info lean = I;
+  lean.lean = true;
+  const size_t base = std::max(workspace_layout(I).total, fused_layout(lean).total);
+  if (I.lean || (I.layer && !I.pool_max)) return base;
+  return std::max({base, fused_layout(I).total, resident_layout(I).total});
 }
 
 // Max pooling: after these layouts, one raw-score row per SRH head slot (at
@@ -1010,7 +1017,7 @@ void fill_common(Params& P, const ckv_problem* p, const Info& I, const SrhLists&
   // 16384 67/65, 32768 90/82, 131072 226/162)
   int longest = 0;
   for (int s = 0; s < I.B; ++s) longest = std::max(longest, I.n[s]);
-  P.in_pieces = do_select && longest > 12288 && P.n_units <= piece_units ? 1 : 0;
+  P.in_pieces = do_select && longest > 12288 && P.n_units <= piece_units && !I.lean ? 1 : 0;
   P.chunk_off[0] = 0;
   for (int s = 0; s <= I.B; ++s) {
     P.cu_seqlens[s] = I.cu[s];
@@ -1054,7 +1061,7 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   // the call's kernel, and the query rows of its widest group
   const int r_grid = std::min(Fd->sms, kResidentMaxGrid);
   std::vector<int> seq_ct(I.B, 0);  // K tiles per chunk
-  bool resident = r_grid >= kResidentMinGrid;
+  bool resident = r_grid >= kResidentMinGrid && !I.lean;
   int max_rows = 16;
   for (int s0 = 0; s0 < I.B; s0 += I.spm) {  // layer by layer
     int rows = 0, longest = 0;
@@ -1362,15 +1369,13 @@ int compresskv_compress_layer(const ckv_problem* p, const void* q_win, const voi
                                     stream);
 }
 
-int compresskv_compress_layers(const ckv_problem* p, int n_masks, const void* q_win,
-                               const void* k, const void* v, const uint8_t* srh_masks,
-                               const int32_t* budgets, int32_t* indices, int32_t* cu_out,
-                               void* k_out, void* v_out, float* raw_scores, float* pooled_scores,
-                               void* workspace, size_t workspace_bytes, void* stream) {
-  NvtxRange nvtx_range(__func__);
-  Info I;
-  int rc = validate(p, I);
-  if (rc != CKV_OK) return rc;
+// compresskv_compress_layers on a validated problem.
+static int compress_layers(Info& I, const ckv_problem* p, int n_masks, const void* q_win,
+                           const void* k, const void* v, const uint8_t* srh_masks,
+                           const int32_t* budgets, int32_t* indices, int32_t* cu_out, void* k_out,
+                           void* v_out, float* raw_scores, float* pooled_scores, void* workspace,
+                           size_t workspace_bytes, void* stream) {
+  int rc = CKV_OK;
   if (n_masks < 1 || I.B % n_masks != 0) return CKV_ERR_INVALID_ARG;
   if (n_masks > kMaxFusedMasks) return CKV_ERR_UNSUPPORTED;
   I.n_masks = n_masks;
@@ -1412,6 +1417,19 @@ int compresskv_compress_layers(const ckv_problem* p, int n_masks, const void* q_
     return run_select(p, I, raw_scores ? raw_scores : ws.raw, nullptr, co, indices,
                       pooled_scores, ws, st, k, v, k_out, v_out);
   return run_select(p, I, nullptr, pooled, co, indices, nullptr, ws, st, k, v, k_out, v_out);
+}
+
+int compresskv_compress_layers(const ckv_problem* p, int n_masks, const void* q_win,
+                               const void* k, const void* v, const uint8_t* srh_masks,
+                               const int32_t* budgets, int32_t* indices, int32_t* cu_out,
+                               void* k_out, void* v_out, float* raw_scores, float* pooled_scores,
+                               void* workspace, size_t workspace_bytes, void* stream) {
+  NvtxRange nvtx_range(__func__);
+  Info I;
+  int rc = validate(p, I);
+  if (rc != CKV_OK) return rc;
+  return compress_layers(I, p, n_masks, q_win, k, v, srh_masks, budgets, indices, cu_out, k_out,
+                         v_out, raw_scores, pooled_scores, workspace, workspace_bytes, stream);
 }
 
 int compresskv_compress_layer_lse(const ckv_problem* p, const void* q_win, const void* k,
@@ -1638,6 +1656,8 @@ extern "C" int compresskv_compress_layer_noalloc(
   Info I;
   int rc = validate(p, I);
   if (rc != CKV_OK) return rc;
+  // (many tiny units need more for the resident kernel than without it)
+  I.lean = workspace_bytes(I) > static_cast<size_t>(CKV_STATIC_SCRATCH_BYTES);
   if (workspace_bytes(I) > static_cast<size_t>(CKV_STATIC_SCRATCH_BYTES))
     return CKV_ERR_STATIC_SCRATCH;
   void* scratch = nullptr;
@@ -1646,9 +1666,9 @@ extern "C" int compresskv_compress_layer_noalloc(
   // The array keeps the previous call's contents; the status word and the
   // counters must start at zero.
   if (cudaMemsetAsync(scratch, 0, kHeaderBytes, st) != cudaSuccess) return CKV_ERR_CUDA;
-  rc = compresskv_compress_layer(p, q_win, k, v, srh_mask, budgets, indices, cu_out, k_out, v_out,
-                                 raw_scores, pooled_scores, scratch,
-                                 static_cast<size_t>(CKV_STATIC_SCRATCH_BYTES), stream);
+  rc = compress_layers(I, p, 1, q_win, k, v, srh_mask, budgets, indices, cu_out, k_out, v_out,
+                       raw_scores, pooled_scores, scratch,
+                       static_cast<size_t>(CKV_STATIC_SCRATCH_BYTES), stream);
   if (rc != CKV_OK) return rc;
   if (device_status &&
       cudaMemcpyAsync(device_status, scratch, sizeof(int32_t), cudaMemcpyDeviceToDevice, st) !=

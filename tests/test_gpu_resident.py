@@ -110,3 +110,24 @@ def test_calls_on_two_streams_at_once(cuda_device):
         assert ckv.read_device_status(ws) == 0
         for key in ("raw", "pooled", "indices", "k_out", "v_out"):
             assert torch.equal(getattr(out, key), getattr(want, key)), key
+
+
+def test_static_scratch_without_the_resident_area(cuda_device):
+    """Many tiny units: the workspace is larger than the static scratch, which
+    holds the two-pass kernel's share of it, so the call without a workspace
+    takes that kernel; both calls agree (fp32 sums in two orders)."""
+    dev = cuda_device
+    cfg, layers = _make("c2", [20] * 512, n_layers=1, num_q_heads=32, num_kv_heads=32, window=16,
+                        srh_per_group=(1, 1), budget_mean=18)
+    want, _, _ = _run_call(layers, cfg, dev)
+    q, k, v, cu, b, m = _pack(layers, dev)
+    prob = ckv.Problem(q, k, cu, cfg.window, cfg.pool_width)
+    assert ckv.workspace_size(prob) > ckv.compresskv.STATIC_SCRATCH_BYTES
+    out = ckv.LayerOutputs(prob, b, 128, k.dtype, dev, scores=True)
+    status = torch.full((1,), -1, dtype=torch.int32, device=dev)
+    ckv.compress_layer_noalloc(prob, q, k, v, m[0], b, out.indices, out.k_out, out.v_out,
+                               raw=out.raw, pooled=out.pooled, device_status=status)
+    torch.cuda.synchronize()
+    assert int(status) == 0
+    torch.testing.assert_close(out.raw, want.raw, rtol=1e-5, atol=1e-9)
+    assert torch.equal(out.indices, want.indices) and torch.equal(out.k_out, want.k_out)
