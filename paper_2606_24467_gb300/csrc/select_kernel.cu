@@ -397,10 +397,9 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_kernel(const __grid_con
 //      keys above it is halfway between k and kScCandCap.
 //      When between k and kScCandCap keys reach lo (the usual case), every
 //      CTA reads all lists (position order across the cluster), finds the
-//      k-th largest key tau and how many keys equal to it are kept (radix
-//      passes over min(key - lo, 2^16 - 1), which resolve tau whenever it is
-//      below lo + 2^16 - 1, else over the keys themselves), and writes its
-//      own selected positions at offsets counted in that list.
+//      k-th largest key tau and how many keys equal to it are kept (by
+//      bisection over keys in registers), and writes its own selected
+//      positions at offsets counted in that list.
 //      Otherwise every CTA runs the same search over all of the unit's
 //      scores (read from global memory) and counts from there.
 //   4. The last CTA appends the window; every CTA copies its own K/V rows.
@@ -424,9 +423,14 @@ struct ScShared {
   RadixShared rs;
   int wcnt[kScWarps];
   int wbase[kScWarps];
+  alignas(16) uint32_t cnt[2][2][8];  // per-warp results of a bisection step
   int red[2][2];              // one pair of sums per use
   int red0;
   uint32_t lo;
+};
+
+struct CtaBarrier {
+  __device__ __forceinline__ void operator()() const { __syncthreads(); }
 };
 
 // Zero state the searches below expect (before the kernel's first barrier).
@@ -652,12 +656,10 @@ __global__ void __launch_bounds__(kScThreads)
     }
     __syncthreads();
     cluster_arrive_release();  // done reading the other CTAs' shared memory
-    // offsets above lo, clamped to 16 bits: at most two passes
-    constexpr uint32_t kClamp = 0xFFFFu;
-    const uint32_t td = cta_kth_largest(sh.all, total, lo, kClamp, k, sh.rs, 0, pc, &need_eq);
-    tau = lo + td;
-    if (td == kClamp)  // tau at or above the clamp: the keys themselves
-      tau = cta_kth_largest(sh.all, total, 0u, 0xFFFFFFFFu, k, sh.rs, 1, pc, &need_eq);
+    tau = total <= 4 * kScThreads
+              ? bisect_largest<4>(sh.all, total, k, 0, sh.cnt, &need_eq, tid, CtaBarrier{})
+              : bisect_largest<kScCandCap / kScThreads>(sh.all, total, k, 0, sh.cnt, &need_eq, tid,
+                                                        CtaBarrier{});
     int a = 0, b = 0;
 #pragma unroll 4
     for (int j = tid; j < before; j += kScThreads) {
