@@ -858,10 +858,12 @@ int run_select(const ckv_problem* p, const Info& I, const float* raw, const floa
     P.cu_out[s] = cu_out[s];
     if (s < I.B) max_n = std::max(max_n, I.n[s]);
   }
-  if (pooled_in && !I.layer && max_n <= 32 * 1024) {
-    // fused layer call, per-group selection: sampled select, one cluster of
+  if (!I.layer && max_n <= 32 * 1024 && (pooled_in || max_n > 8192)) {
+    // per-group selection: sampled select, one cluster of
     // C CTAs per unit (longer prefixes list too many keys above the sampled
-    // bound).  C gives about kScTargetCtas CTAs per launch -- few, busy CTAs
+    // bound).  From raw scores for long units only (score, select and gather
+    // of four units of 16001 tokens 33.9 -> 31.4 us, of 18984 68 -> 64 with
+    // the host's part; 32 units of up to 892 33.9 -> 35.7).  C gives about kScTargetCtas CTAs per launch -- few, busy CTAs
     // leave the SMs to the other calls' kernels (measured on the 32-layer
     // bench: 8 units per launch best with C = 8 of 4/8/16, 32 units with
     // C = 2-4 of 2-16) -- but at least slices of kScMaxSlice positions and
@@ -875,7 +877,7 @@ int run_select(const ckv_problem* p, const Info& I, const float* raw, const floa
       P.cluster = C;
       P.slice = S;
       Tracer tr{p->trace, stream};
-      const size_t smem = select_sampled_smem_bytes(S);
+      const size_t smem = select_sampled_smem_bytes(S, pooled_in ? 0 : S + I.P - 1);
       return traced(tr, CKV_KERNEL_SELECT,
                     [&] { return launch_select_sampled(P, I.B * I.Hkv, smem, stream); });
     }

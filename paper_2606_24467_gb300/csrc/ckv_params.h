@@ -303,7 +303,7 @@ constexpr int kScMaxSlice = 16384;
 constexpr int kScTargetSlice = 2048;  // slice of the cluster-size occupancy query
 constexpr int kScTargetCtas = 80;     // CTAs per sampled-select launch to aim for
 cudaError_t launch_select_sampled(const SelectParams& p, int n_units, size_t smem, cudaStream_t s);
-size_t select_sampled_smem_bytes(int slice);
+size_t select_sampled_smem_bytes(int slice, int raw_floats);
 int select_sampled_max_cluster(int slice);  // 16 when the device takes such clusters, else 8
 cudaError_t launch_gather(const GatherParams& p, long long rows, cudaStream_t s);
 cudaError_t launch_maxpool(const MaxPoolParams& p, int max_n, cudaStream_t s);

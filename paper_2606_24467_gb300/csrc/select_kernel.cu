@@ -385,7 +385,8 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_kernel(const __grid_con
 // the K/V rows copied -- with three cluster barriers (five on a retry)
 // instead of one per radix pass.  One cluster of C <= 16 CTAs per unit; CTA r owns the contiguous
 // slice [r*S, (r+1)*S) of the unit's prefix positions.
-//   1. The slice's pooled scores go to shared memory; each CTA sends 256 / C
+//   1. The slice's pooled scores go to shared memory (pooled there when the
+//      raw scores are given); each CTA sends 256 / C
 //      evenly spaced scores of its slice to every CTA of the cluster.
 //   2. Every CTA takes the same lower bound lo for the k-th largest score:
 //      the r-th largest sample (found by counting, for every sample, the
@@ -492,7 +493,11 @@ __global__ void __launch_bounds__(kScThreads)
   const int out0 = p.head_budgets ? p.unit_out[u].x : p.cu_out[s];
   const int kept = p.head_budgets ? p.unit_out[u].y : p.cu_out[s + 1] - out0;
   int32_t* out = p.indices + (p.head_budgets ? 0 : static_cast<long long>(g) * p.o_total) + out0;
-  const float* pooled = p.pooled_in + static_cast<long long>(g) * p.p_total + p.cu_prefix[s];
+  const long long soff = static_cast<long long>(g) * p.p_total + p.cu_prefix[s];
+  // pooled scores: given, or from the raw ones (then written out as well, for
+  // the caller and for the full search)
+  float* const pooled_w = p.pooled_in ? nullptr : (p.pooled_out ? p.pooled_out : p.pooled_ws) + soff;
+  const float* pooled = p.pooled_in ? p.pooled_in + soff : pooled_w;
   const uint32_t* gkeys = reinterpret_cast<const uint32_t*>(pooled);
   const int S = p.slice;
   const int lo_c = min(n, cr * S);
@@ -500,8 +505,37 @@ __global__ void __launch_bounds__(kScThreads)
 
   pdl_launch_dependents();
   cluster_arrive_relaxed();  // this CTA has started (remote shared memory may be written)
-  pdl_wait();                // pooled scores come from the previous kernel
+  pdl_wait();                // scores come from the previous kernel
 
+  if (pooled_w) {  // pool the slice (select_kernel's sums, in its order)
+    const int r = (p.pool_width - 1) >> 1;
+    const float fP = static_cast<float>(p.pool_width);
+    const float* raw = p.raw + soff;
+    float* const raw_s = s_keys + S;
+    const int span = len > 0 ? len + 2 * r : 0;
+    for (int base = 0; base < span; base += 8 * kScThreads) {
+      float v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int li = base + i * kScThreads + tid;
+        const int j = lo_c - r + li;
+        v[i] = li < span && j >= 0 && j < n ? raw[j] : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int li = base + i * kScThreads + tid;
+        if (li < span) raw_s[li] = v[i];
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i < len; i += kScThreads) {
+      float a = 0.f;
+      for (int t = 0; t <= 2 * r; ++t) a += raw_s[i + t];
+      const float pv = a / fP;
+      s_keys[i] = pv;
+      pooled_w[lo_c + i] = pv;
+    }
+  }
   if (kept >= L) {  // keep everything (uniform over the cluster)
     const int per = (L + C - 1) / C;
     const int a0 = min(L, cr * per);
@@ -530,8 +564,10 @@ __global__ void __launch_bounds__(kScThreads)
   const int per_cta = kScSampleTotal / C;
   sc_init_shared(sh, C * per_cta);
   int pc = 0;  // radix passes run so far (histogram rotation)
-  for (int i = tid; i < len; i += kScThreads) cp_async4(smem_u32(s_keys + i), pooled + lo_c + i);
-  cp_async_wait_all();
+  if (!pooled_w) {
+    for (int i = tid; i < len; i += kScThreads) cp_async4(smem_u32(s_keys + i), pooled + lo_c + i);
+    cp_async_wait_all();
+  }
   __syncthreads();
   auto key_at = [&](int i) { return __float_as_uint(s_keys[i]); };
   const int ns_c = min(per_cta, len);
@@ -672,7 +708,7 @@ __global__ void __launch_bounds__(kScThreads)
     tau = cta_kth_largest(gkeys, n, 0u, 0xFFFFFFFFu, k, sh.rs, 1, pc, &need_eq);
     int a = 0, b = 0;
     for (int j = tid; j < lo_c; j += kScThreads) {
-      const uint32_t key = __ldg(gkeys + j);
+      const uint32_t key = __ldcg(gkeys + j);  // (another CTA may have pooled it)
       a += key > tau ? 1 : 0;
       b += key == tau ? 1 : 0;
     }
@@ -743,8 +779,9 @@ __global__ void __launch_bounds__(kScThreads)
 
 }  // namespace
 
-size_t select_sampled_smem_bytes(int slice) {
-  return ((sizeof(ScShared) + 15) & ~size_t(15)) + static_cast<size_t>(slice) * sizeof(float);
+size_t select_sampled_smem_bytes(int slice, int raw_floats) {
+  return ((sizeof(ScShared) + 15) & ~size_t(15)) +
+         (static_cast<size_t>(slice) + raw_floats) * sizeof(float);
 }
 
 int select_sampled_max_cluster(int slice) {
@@ -753,7 +790,7 @@ int select_sampled_max_cluster(int slice) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kScMaxC);
   cfg.blockDim = dim3(kScThreads);
-  cfg.dynamicSmemBytes = select_sampled_smem_bytes(slice);
+  cfg.dynamicSmemBytes = select_sampled_smem_bytes(slice, 0);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = kScMaxC;
@@ -793,7 +830,8 @@ int select_max_smem_floats() { return (227 * 1024 - kSelStaticSmem - 1024) / 4; 
 cudaError_t select_set_smem_limit(size_t bytes) {
   cudaError_t e = cudaFuncSetAttribute(select_sampled_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(select_sampled_smem_bytes(kScMaxSlice)));
+                                       static_cast<int>(select_sampled_smem_bytes(
+                                           kScMaxSlice, kScMaxSlice + 62)));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(select_sampled_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
