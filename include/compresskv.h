@@ -255,11 +255,12 @@ int compresskv_compress_layer(const ckv_problem* p, const void* q_win, const voi
  * Neither stores exponentials.  The grid of chunks follows from the layer
  * alone, and neither kernel's scores depend on the order in which chunks
  * complete: compressing a layer alone or among others that take the same
- * kernel gives the same bits.  The kernels take windows W that are multiples of 16, query
- * strides that are multiples of 8 elements, at most 32 query heads per group
- * and SRH lists of at most 192 query rows (two Q buffers of them beside a
- * ring of two K tiles fill the shared memory); other per-group problems use
- * the separate kernels.  The resident kernel is a cooperative launch.
+ * kernel gives the same bits.  The kernels take windows W that are multiples
+ * of 16, query strides that are multiples of 8 elements, at most 32 query
+ * heads per group and SRH lists of at most 192 query rows (two Q buffers of
+ * them beside a ring of two K tiles fill the shared memory); other per-group
+ * problems use the separate kernels.  The resident kernel is a cooperative
+ * launch.
  * n_masks: 1 <= n_masks, dividing batch (else CKV_ERR_INVALID_ARG); at most
  *   256 under CKV_SELECT_PER_GROUP and 4 under CKV_SELECT_PER_LAYER (or when
  *   the separate kernels run) (else CKV_ERR_UNSUPPORTED).

@@ -41,8 +41,10 @@ std::atomic<long long> g_stall_next_ns{0};
 // last-CTA-per-unit merge resets the tickets it uses).
 constexpr size_t kTicketOffset = 256;
 constexpr size_t kStatusBytes = kTicketOffset + static_cast<size_t>(kMaxItems) * sizeof(int);
-// ... followed by the fused call's counters; the whole header is zeroed by
-// compresskv_workspace_init and left zero by every call that completes.
+// ... followed by the persistent kernels' words; the whole header is zeroed by
+// compresskv_workspace_init and left zero by every call that completes, but
+// for the resident kernel's start counter and the number of its last call that
+// stopped.
 constexpr size_t kFusedCtrOffset = kStatusBytes;
 constexpr size_t kHeaderBytes = ((kFusedCtrOffset + kFusedCtrBytes) + 255) & ~static_cast<size_t>(255);
 
