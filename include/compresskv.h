@@ -260,7 +260,8 @@ int compresskv_compress_layer(const ckv_problem* p, const void* q_win, const voi
  * heads per group and SRH lists of at most 192 query rows (two Q buffers of
  * them beside a ring of two K tiles fill the shared memory); other per-group
  * problems use the separate kernels.  The resident kernel is a cooperative
- * launch.
+ * launch: it starts when every SM has room for one of its CTAs, and where the
+ * stream's context has fewer SMs than the device the two-pass kernel runs.
  * n_masks: 1 <= n_masks, dividing batch (else CKV_ERR_INVALID_ARG); at most
  *   256 under CKV_SELECT_PER_GROUP and 4 under CKV_SELECT_PER_LAYER (or when
  *   the separate kernels run) (else CKV_ERR_UNSUPPORTED).

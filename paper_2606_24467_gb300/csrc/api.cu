@@ -1048,7 +1048,7 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
               const void* k, const void* v, const std::vector<int>& co, int32_t* indices,
               void* k_out, void* v_out, float* raw_user, float* pooled_user, void* ws,
               size_t ws_bytes, cudaStream_t stream, bool* handled, bool do_select = true,
-              const LseInput& lse = LseInput{}) {
+              const LseInput& lse = LseInput{}, bool allow_resident = true) {
   *handled = false;
   if (I.layer || I.G > 32 || I.n_masks * I.Hkv > kFusedMaxLists || I.B > kFusedMaxSeqs)
     return CKV_OK;
@@ -1065,7 +1065,7 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   // the call's kernel, and the query rows of its widest group
   const int r_grid = std::min(Fd->sms, kResidentMaxGrid);
   std::vector<int> seq_ct(I.B, 0);  // K tiles per chunk
-  bool resident = r_grid >= kResidentMinGrid && !I.lean;
+  bool resident = allow_resident && r_grid >= kResidentMinGrid && !I.lean;
   int max_rows = 16;
   for (int s0 = 0; s0 < I.B; s0 += I.spm) {  // layer by layer
     int rows = 0, longest = 0;
@@ -1143,8 +1143,16 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
     P.q_bufs = q_bufs;
     P.stages = stages;
     if (P.n_units == 0 || (P.n_chunks == 0 && (!do_select || co[I.B] == 0))) return CKV_OK;
-    return traced(tr, CKV_KERNEL_FUSED,
-                  [&] { return launch_resident(P, r_grid, smem_bytes(q_bufs, stages), stream); });
+    cudaError_t e = cudaSuccess;
+    rc = traced(tr, CKV_KERNEL_FUSED, [&] {
+      return e = launch_resident(P, r_grid, smem_bytes(q_bufs, stages), stream);
+    });
+    if (e != cudaErrorCooperativeLaunchTooLarge) return rc;
+    // the stream's context has fewer SMs than the device: the two-pass kernel
+    // runs with any number of CTAs at once
+    (void)cudaGetLastError();
+    return run_fused(p, I, S, q_win, k, v, co, indices, k_out, v_out, raw_user, pooled_user, ws,
+                     ws_bytes, stream, handled, do_select, lse, false);
   }
 
   static thread_local FusedParams P;  // large (about 15 KB): kept off the stack
