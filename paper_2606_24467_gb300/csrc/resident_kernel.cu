@@ -30,16 +30,18 @@
 //
 // The sum over the SMs (kAccWords 64-bit words per unit and query row): a
 // chunk's S_q, an fp32 number, is rounded to an integer multiple of a power
-// of two that its exponent selects (one of kAccBins bins; at least 20
-// significant bits, 44 in the middle of the range) and added to the bin's
-// word, whose low bits count the contributions.  Integer addition has no
+// of two that its exponent selects (one of kAccBins bins, spaced so that no
+// bit of a sum of 2^-10 or more is lost) and added to the bin's word, whose low
+// bits count the contributions.  Integer addition has no
 // order, so D_q is the same whatever the order of arrival; a reader that
 // finds as many contributions as the unit has chunks has the complete sum, so
 // one reduction and one read carry it between SMs, with no fence, ticket or
 // merge in between (measured on 152 SMs: 2.1 us for 64 rows with a ticket and
 // fence, 6 us when every SM reads every other's partial sums).  Rows whose
-// sums leave the bins' range (logits beyond about +-40) are added up again
-// against the unit's largest chunk exponent (slow_denominators).
+// sums leave the bins' range are added up again against the unit's largest
+// chunk exponent (slow_denominators): a chunk's sum of 2^142 and more in a
+// unit of one chunk, of 2^86 in one of 128, or a D below 2^-48 and 2^-27 in
+// these (every logit above about +60 or below about -25).
 //
 // One CTA per SM runs for the whole call (a cooperative launch: the chunks of
 // a unit wait for one another, so all CTAs have to be resident).  Warps:
@@ -338,13 +340,14 @@ struct Ring {
 // The bins of a unit of nch chunks: cb bits count contributions; a
 // contribution has at most vb bits, so nch of them do not overflow into one
 // another (nch 2^vb <= 2^(64 - cb)); bin 0 holds sums below 2^kAccE0, bin
-// k >= 1 those in [2^(kAccE0 + (k - 1) width), 2^(kAccE0 + k width)).
+// k >= 1 those in [2^(kAccE0 + (k - 1) width), 2^(kAccE0 + k width)), which
+// have at least vb - width = 24 bits there: an fp32 sum is added exactly.
 struct Bins {
   int cb, vb, width;
   __device__ explicit Bins(int nch) {
     cb = 32 - __clz(nch);
     vb = 64 - 2 * cb;
-    width = vb - 20;
+    width = vb - 24;
   }
   __device__ int grid(int k) const { return kAccE0 + k * width - vb; }
 };

@@ -61,8 +61,8 @@ def test_sizes_around_tiles_chunks_and_the_kernels_line(cuda_device, window, hea
 @pytest.mark.parametrize("shift", [-90.0, 90.0])
 def test_sums_outside_the_fixed_point_bins(cuda_device, shift):
     """Every other window row's logits moved by about `shift`: its sums of
-    exponentials leave the range of the accumulators' bins (2^-10 down to the
-    grid's end, 2^118 up), so it takes the second round; its neighbours don't.
+    exponentials leave the range of the accumulators' bins, so it takes the
+    second round; its neighbours don't.
 
     Bound: a logit is eight accumulations of at most |q| |k| in fp32, scaled
     once and rounded once against the exponent's reference, so off by at most
@@ -84,6 +84,43 @@ def test_sums_outside_the_fixed_point_bins(cuda_device, shift):
     rtol = 2 * 10 * 2.0 ** -23 * float(norms) / 128 ** 0.5 + 1e-5
     compare.check_scores("raw", blk["raw"], res.raw, rtol=rtol, atol=1e-8)
     compare.check_scores("pooled", blk["pooled"], res.pooled, rtol=rtol, atol=1e-8)
+
+
+def test_chunk_sums_lose_no_bits(cuda_device):
+    """Units whose keys are all alike: every chunk's sum of exponentials is a
+    power of two times one exponential, just above a power of two at which the
+    accumulators' bins could begin (2^24 for a unit of 20 chunks), so each
+    score is 2^(z c) over an exactly known count of the same, however large.
+
+    Bound: what remains is the rounding of D and of its reciprocal, of the
+    product with it and of the sums over 16 rows, some six of at most 2^-24
+    each and independent over the units: an rms below sqrt(6) 2^-24 =
+    1.5e-7.  Sums kept to 20 bits are off by up to 8 / S, 2.3e-7 rms."""
+    dev = cuda_device
+    n_layers, n_kv, window, L, d = 64, 2, 16, 2560, 128
+    scale = float(np.float32(0.125 / np.log2(np.e)))
+    assert np.float32(scale * np.log2(np.e)) == 0.125  # z c exact
+    k = torch.ones((n_layers * L, n_kv, d), dtype=torch.bfloat16, device=dev)
+    q = torch.full((n_layers, n_kv, window, d), 1.0, dtype=torch.bfloat16, device=dev)
+    frac = torch.arange(n_layers * n_kv, device=dev).view(n_layers, n_kv, 1) / 64.0
+    q[..., 0] = 136.0 - 127.0 + 0.0  # z = 136 and a fraction, z c = 17 and up
+    q[..., 1] = 1.0 + (frac % 1.0).to(torch.bfloat16)
+    q[..., 2] = 1.0 + torch.floor(frac).to(torch.bfloat16) / 128.0
+    z = q[:, :, 0].double().sum(-1)
+    assert float(z.min()) >= 17 * 8 and float(z.max()) < 17.3 * 8
+    cu = np.arange(n_layers + 1, dtype=np.int32) * L
+    budgets = np.full(n_layers, window + 1, np.int32)
+    prob = ckv.Problem(q, k, cu, window, 7, scale=scale)
+    out = ckv.LayerOutputs(prob, budgets, d, k.dtype, dev, scores=True)
+    ws = ckv.workspace(prob, dev)
+    ckv.compress_layers(prob, n_layers, q, k, k, np.ones((n_layers, n_kv), np.uint8), budgets,
+                        out.indices, out.k_out, out.v_out, ws, raw=out.raw, pooled=out.pooled)
+    torch.cuda.synchronize()
+    assert ckv.read_device_status(ws) == 0
+    n = L - window
+    want = sum(1.0 / (n + w + 1) for w in range(window))
+    err = out.raw.double().view(n_kv, n_layers, n) / want - 1.0
+    assert float(err.pow(2).mean().sqrt()) < 1.5e-7
 
 
 def test_calls_on_two_streams_at_once(cuda_device):
