@@ -226,6 +226,11 @@ __device__ __forceinline__ unsigned long long ld_relaxed64(const unsigned long l
 __device__ __forceinline__ void red_add64(unsigned long long* p, unsigned long long v) {
   asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
+// Between threads of one CTA: what this thread has waited for happens before
+// what the observer of its next relaxed write does after such a fence.
+__device__ __forceinline__ void fence_acq_rel_cta() {
+  asm volatile("fence.acq_rel.cta;" ::: "memory");
+}
 __device__ __forceinline__ int ld_volatile(const int* p) {
   return *reinterpret_cast<const volatile int*>(p);
 }
@@ -622,6 +627,7 @@ __device__ __forceinline__ bool denominators(ResidentShared& sh, const ChunkDesc
     slow |= v[kAccOut] != 0ull || !(D >= dmin && D < 1.0e38f);
     split_denominator(D, out + q, out + rows + q);
   }
+  fence_acq_rel_cta();  // (see sum_role)
   if (!__all_sync(0xffffffffu, ok)) return false;
   if (__any_sync(0xffffffffu, slow)) return slow_denominators(sh, d, out, lane);
   return true;
@@ -1001,6 +1007,10 @@ __device__ __noinline__ void sum_role(ResidentShared& sh, int lane) {
       const float2* src = pair_row(sh, b * 4);
       ok = wait_all(sh, &sh.p1full[b], static_cast<uint32_t>(k1 >> 1) & 1u);
       if (!ok) break;
+      // pass 1's reads of the chunk's tiles, and the UMMAs it has waited for,
+      // come before pass 2's reads (which begin once a warp of this CTA has
+      // seen the sums below) and the tiles' release
+      fence_acq_rel_cta();
 #pragma unroll 1
       for (int q = lane; q < n_rows; q += 32) {
         const float2 v0 = src[q], v1 = src[rows + q], v2 = src[2 * rows + q], v3 = src[3 * rows + q];
