@@ -981,6 +981,17 @@ int resident_chunk_tiles(int rows, long long layer_tiles) {
   return std::min(most, layer_tiles <= 64 ? 1 : (layer_tiles <= 256 ? 2 : 4));
 }
 
+// The tensor cores' fp32 sums are truncated: a logit's magnitude comes out low
+// by about this share of it (128 products in eight steps; mean over keys along
+// the query, logits 3 to 9: 1.1e-7 to 1.3e-7 in bf16, 1.7e-7 to 2.3e-7 in f16).
+// The scale makes up for it where the denominators have no error of that size
+// of their own: the scores' relative 2-norm error against 64 bits over the
+// declared cases 3.0e-7 to 1.1e-6 -> 1.3e-7 to 6.0e-7 (resident kernel), 8e-7
+// -> 3e-7 (LSE given).  The two-pass kernel's merged denominators are low by
+// 4e-7 (approximate logarithms), which outweighs it: 3.1e-7 without, 3.9e-7
+// with it.
+constexpr double kUmmaTruncation = 1.2e-7;
+
 // What the two persistent kernels' parameters have in common; calls of up to
 // piece_units units pool long units in pieces (unit_select.cuh).  16 layers
 // (128 units), by the selection / in pieces: resident kernel 16384 tokens
@@ -989,7 +1000,8 @@ int resident_chunk_tiles(int rows, long long layer_tiles) {
 template <class Params>
 void fill_common(Params& P, const ckv_problem* p, const Info& I, const SrhLists& S,
                  const std::vector<int>& co, int32_t* indices, const void* k, const void* v,
-                 void* k_out, void* v_out, const LseInput& lse, bool do_select, int piece_units) {
+                 void* k_out, void* v_out, const LseInput& lse, bool do_select, int piece_units,
+                 bool exact_denominators) {
   P.lse = lse.lse;
   P.lse_bs = lse.batch_stride;
   P.lse_hs = lse.head_stride;
@@ -1006,7 +1018,8 @@ void fill_common(Params& P, const ckv_problem* p, const Info& I, const SrhLists&
     P.wait_ns = stall > 0 ? static_cast<unsigned long long>(stall) : kWaitTimeoutNs;
     P.stall = stall > 0 ? 1 : 0;
   }
-  P.c = static_cast<float>(static_cast<double>(I.scale) * 1.4426950408889634);
+  P.c = static_cast<float>(static_cast<double>(I.scale) * 1.4426950408889634 *
+                           (exact_denominators ? 1.0 + kUmmaTruncation : 1.0));
   P.window = I.W;
   P.pool_width = I.P;
   P.num_kv_heads = I.Hkv;
@@ -1121,7 +1134,7 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
     if ((rc = make_k_map(I, p, k, &P.tmap_k)) != CKV_OK) return rc;
     if ((rc = make_q_map(I, p, q_win, &P.tmap_q)) != CKV_OK) return rc;
     fill_common(P, p, I, S, co, indices, k, v, k_out, v_out, lse, do_select,
-                Fd->sms / 4);
+                Fd->sms / 4, true);
     P.raw = raw_user ? raw_user : reinterpret_cast<float*>(wb + RL.raw);
     P.raw_scratch = raw_user ? 0 : 1;
     P.pooled = pooled_user ? pooled_user : reinterpret_cast<float*>(wb + RL.pooled);
@@ -1160,7 +1173,7 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   if ((rc = make_k_map(I, p, k, &P.tmap_k)) != CKV_OK) return rc;
   if ((rc = make_q_map(I, p, q_win, &P.tmap_q)) != CKV_OK) return rc;
   fill_common(P, p, I, S, co, indices, k, v, k_out, v_out, lse, do_select,
-              Fd->sms - 1);
+              Fd->sms - 1, lse.lse != nullptr);
   P.raw = raw_user ? raw_user : reinterpret_cast<float*>(wb + FL.raw);
   P.raw_scratch = raw_user ? 0 : 1;
   P.pooled = pooled_user ? pooled_user : reinterpret_cast<float*>(wb + FL.pooled);

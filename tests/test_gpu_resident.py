@@ -123,6 +123,40 @@ def test_chunk_sums_lose_no_bits(cuda_device):
     assert float(err.pow(2).mean().sqrt()) < 1.5e-7
 
 
+@pytest.mark.parametrize("dtype,n,bias", [(torch.bfloat16, 8000, 0.8e-7),
+                                          (torch.bfloat16, 26000, 0.8e-7),
+                                          (torch.float16, 8000, 1.6e-7),
+                                          (torch.float16, 26000, 1.6e-7)])
+def test_truncated_logits_are_made_up_for(cuda_device, dtype, n, bias):
+    """Given-LSE scores with LSE = 0 and W equal query rows are W e^z: the mean
+    of (log(score / W) - z) / z over keys along the query, |z| from 3 to 9, in
+    the resident (n <= 24576) and in the two-pass kernel.  The tensor cores'
+    truncated sums alone give -1.2e-7 (bf16) and -2.0e-7 (f16); bound: half a
+    unit of the fp32 scale's last place (0.6e-7) beside what the types differ
+    from the mean correction."""
+    dev, d, window, heads = cuda_device, 128, 16, 8
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(3)
+    q1 = 1.5 * torch.randn((1, heads, 1, d), generator=gen, device=dev)
+    q = q1.expand(1, heads, window, d).contiguous().to(dtype)
+    norm = q1[0, :, 0].norm(dim=-1, keepdim=True)
+    along = torch.linspace(-9, 9, n + window, device=dev)[:, None, None] * (d ** 0.5 / norm)
+    k = 0.5 * torch.randn((n + window, heads, d), generator=gen, device=dev)
+    k = (k + along * (q1[0, :, 0] / norm)).to(dtype)
+    budgets = np.array([window + 64], np.int32)
+    prob = ckv.Problem(q, k, np.array([0, n + window], np.int32), window, 7)
+    out = ckv.LayerOutputs(prob, budgets, d, dtype, dev, scores=True)
+    ws = ckv.workspace(prob, dev)
+    ckv.compress_layer_lse(prob, q, k, k, torch.zeros((1, heads, window), device=dev),
+                           np.ones(heads, np.uint8), budgets, out.indices, out.k_out, out.v_out,
+                           ws, raw=out.raw, pooled=out.pooled)
+    torch.cuda.synchronize()
+    assert ckv.read_device_status(ws) == 0
+    z = torch.einsum("nhd,hd->hn", k[:n].double(), q[0, :, 0].double()) / d ** 0.5
+    err = (torch.log(out.raw.double() / window) - z) / z
+    assert abs(float(err[(z.abs() > 3) & (z.abs() < 9)].mean())) < bias
+
+
 def test_calls_on_two_streams_at_once(cuda_device):
     """Two calls in flight on two streams with a workspace each (every one
     needs all its CTAs resident): the bits of the calls made one by one."""
