@@ -992,15 +992,21 @@ int resident_chunk_tiles(int rows, long long layer_tiles) {
 // with it.
 constexpr double kUmmaTruncation = 1.2e-7;
 
-// What the two persistent kernels' parameters have in common; calls of up to
-// piece_units units pool long units in pieces (unit_select.cuh).  16 layers
-// (128 units), by the selection / in pieces: resident kernel 16384 tokens
-// 187/195 us, 32768 339/357; two-pass 65536 tokens 693/670, 32768 with the
-// LSE given 234/223.
+// What the two persistent kernels' parameters have in common.  in_pieces:
+// whether the kernel pools long units in pieces (unit_select.cuh), for calls
+// with few units for the SMs and, where the workers and not the epilogue bound
+// the two-pass kernel (up to 64 query rows), for any.  By the selection / in
+// pieces in us:
+//   resident kernel, 128 units   16384 tokens 187/195      32768: 339/357
+//   two-pass, 128 units          65536 tokens 693/670
+//   256 units of 64 rows         131072 tokens 2533/2454   LSE given 1459/1387
+//   the same, pooling width 63   2892/2488                 1818/1517
+//   896 units of 64 rows         8192 to 65536: 3026/2997
+//   2560 units of 64 to 192 rows 32768: 8736/8956
 template <class Params>
 void fill_common(Params& P, const ckv_problem* p, const Info& I, const SrhLists& S,
                  const std::vector<int>& co, int32_t* indices, const void* k, const void* v,
-                 void* k_out, void* v_out, const LseInput& lse, bool do_select, int piece_units,
+                 void* k_out, void* v_out, const LseInput& lse, bool do_select, bool in_pieces,
                  bool exact_denominators) {
   P.lse = lse.lse;
   P.lse_bs = lse.batch_stride;
@@ -1034,7 +1040,7 @@ void fill_common(Params& P, const ckv_problem* p, const Info& I, const SrhLists&
   // 16384 67/65, 32768 90/82, 131072 226/162)
   int longest = 0;
   for (int s = 0; s < I.B; ++s) longest = std::max(longest, I.n[s]);
-  P.in_pieces = do_select && longest > 12288 && P.n_units <= piece_units && !I.lean ? 1 : 0;
+  P.in_pieces = do_select && longest > 12288 && in_pieces && !I.lean ? 1 : 0;
   P.chunk_off[0] = 0;
   for (int s = 0; s <= I.B; ++s) {
     P.cu_seqlens[s] = I.cu[s];
@@ -1134,7 +1140,7 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
     if ((rc = make_k_map(I, p, k, &P.tmap_k)) != CKV_OK) return rc;
     if ((rc = make_q_map(I, p, q_win, &P.tmap_q)) != CKV_OK) return rc;
     fill_common(P, p, I, S, co, indices, k, v, k_out, v_out, lse, do_select,
-                Fd->sms / 4, true);
+                I.B * I.Hkv <= Fd->sms / 4, true);
     P.raw = raw_user ? raw_user : reinterpret_cast<float*>(wb + RL.raw);
     P.raw_scratch = raw_user ? 0 : 1;
     P.pooled = pooled_user ? pooled_user : reinterpret_cast<float*>(wb + RL.pooled);
@@ -1173,7 +1179,7 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   if ((rc = make_k_map(I, p, k, &P.tmap_k)) != CKV_OK) return rc;
   if ((rc = make_q_map(I, p, q_win, &P.tmap_q)) != CKV_OK) return rc;
   fill_common(P, p, I, S, co, indices, k, v, k_out, v_out, lse, do_select,
-              Fd->sms - 1, lse.lse != nullptr);
+              max_rows <= 64 || I.B * I.Hkv < Fd->sms, lse.lse != nullptr);
   P.raw = raw_user ? raw_user : reinterpret_cast<float*>(wb + FL.raw);
   P.raw_scratch = raw_user ? 0 : 1;
   P.pooled = pooled_user ? pooled_user : reinterpret_cast<float*>(wb + FL.pooled);

@@ -45,9 +45,10 @@
 //               gather a unit once all its pass-2 chunks are in (one CTA per
 //               unit).
 // A pass-2 chunk is published once its claimer has seen (acquire) its unit's
-// denominators merged; workers claim a merge or a selection only
-// when it is ready.  Every wait therefore depends only on
-// work claimed earlier by a running CTA that never waits on later work, so a
+// denominators merged; workers claim a merge only when it is ready, take
+// tickets of the selections in order and merge while their own is not ready.
+// Every wait therefore depends only on work claimed earlier by a running CTA
+// that never waits on later work, so a
 // call completes whatever the number of CTAs resident at once; every wait
 // is bounded (FusedParams::wait_ns, kWaitTimeoutNs unless a test shortens it)
 // and on expiry records CKV_ERR_DEVICE_TIMEOUT
@@ -92,10 +93,9 @@ constexpr float kNegInf = -INFINITY;
 constexpr int kCtrPass1 = 0;  // next pass-1 chunk
 constexpr int kCtrPass2 = 1;  // next pass-2 chunk
 constexpr int kCtrMerge = 2;  // next unit whose denominators to merge
-constexpr int kCtrSel = 3;    // next unit to select
 constexpr int kCtrExit = 4;   // CTAs finished
 constexpr int kCtrAbort = 5;  // set when any wait ran out
-constexpr int kCtrTicket = 7; // the workers' next ticket (pooling in pieces)
+constexpr int kCtrTicket = 7; // the workers' next ticket
 constexpr int kCtrNever = 6;  // never set: the test hook's stall waits for it
 
 constexpr int kTaskEnd = 0;
@@ -365,68 +365,34 @@ __device__ __noinline__ void merge_unit(const Fused& F, int u, uint8_t* creg, in
   if (ct == 0) atomicExch(F.bias_state(u), 2);
 }
 
-// The workers' next task (one thread): the next unit to select once all its
-// pass-2 chunks are in, else the next unit to merge once all its pass-1
-// chunks are in; waits (bounded) while neither is ready.
-__device__ void claim_task(const Fused& F, int* task) {
-  const FusedParams& p = F.p;
-  uint64_t t0 = 0;
-  for (;;) {
-    if (F.aborted() || *reinterpret_cast<volatile int*>(F.abort_cta)) break;
-    const int u = ld_volatile(p.ctr + kCtrSel);
-    if (u >= p.n_units) break;  // every unit selected (and therefore merged)
-    const int s = u / p.num_kv_heads;
-    if (ld_acquire(F.p2done(u)) >= kEpiWarps * F.chunks_per_unit(s)) {  // kEpiWarps per pass-2 chunk
-      if (atomicCAS(p.ctr + kCtrSel, u, u + 1) == u) {
-        task[0] = kTaskSelect;
-        task[1] = u;
-        return;
-      }
-      continue;
-    }
-    if (!p.given_lse) {
-      const int m = ld_volatile(p.ctr + kCtrMerge);
-      if (m < p.n_units &&
-          ld_acquire(F.ticket(m)) >= p.nwg * F.chunks_per_unit(m / p.num_kv_heads)) {
-        if (atomicCAS(p.ctr + kCtrMerge, m, m + 1) == m) {
-          task[0] = kTaskMerge;
-          task[1] = m;
-          return;
-        }
-        continue;
-      }
-    }
-    const uint64_t now = globaltimer_ns();
-    if (t0 == 0) {
-      t0 = now;
-    } else if (now - t0 > p.wait_ns) {
-      F.raise_abort();
-      break;
-    }
-    __nanosleep(128);
-  }
-  task[0] = kTaskEnd;
-  task[1] = 0;
-}
-
-// The same when units are pooled in pieces: the ticket's task (a piece once
-// all the unit's pass-2 chunks are in, a selection once its pieces are
-// pooled), or meanwhile the next unit to merge.
+// The workers' next task (one thread): the ticket's (a piece to pool once all
+// the unit's pass-2 chunks are in, a selection then or once its pieces are
+// pooled), or meanwhile the next unit to merge once all its pass-1 chunks are
+// in; waits (bounded) while neither is ready.  (Claims by compare-and-swap of
+// the next ready selection cost 1 us apiece: 48 layers of 12288 tokens of 128
+// rows 720 -> 486 us with tickets, 60 layers of 4 prompts of 500 to 9000 of 64
+// to 192 rows 3250 -> 1850.)
+template <bool kPieces>
 __device__ void claim_ticket(const Fused& F, TaskPos& T, int* task) {
   const FusedParams& p = F.p;
   if (T.t < 0)
     take_ticket(T, p.ctr + kCtrTicket, p.batch, p.num_kv_heads, [&](int s) {
-      return pool_pieces(F.prefix(s));
+      return kPieces ? pool_pieces(F.prefix(s)) : 0;
     });
+  // what the task waits for; without one (every selection is ahead of the
+  // first ticket past the last), the other units' merges
+  const int* word = p.ctr + kCtrMerge;
+  int target = p.given_lse ? 0 : p.n_units;
+  if (T.unit >= 0) {
+    const bool pooled = kPieces && T.piece < 0 && T.pieces > 0;
+    word = pooled ? F.bias_state(T.unit) : F.p2done(T.unit);
+    target = pooled ? 4 * T.pieces : kEpiWarps * F.chunks_per_unit(T.s);
+  }
   const uint64_t t0 = globaltimer_ns();
-  // (every unit's selection is ahead of the first ticket without a task, and
-  // with it every merge)
-  while (T.unit >= 0) {
+  for (;;) {
     if (F.aborted() || *reinterpret_cast<volatile int*>(F.abort_cta)) break;
-    const bool ready = T.piece < 0 && T.pieces > 0
-                           ? (ld_acquire(F.bias_state(T.unit)) >> 2) >= T.pieces
-                           : ld_acquire(F.p2done(T.unit)) >= kEpiWarps * F.chunks_per_unit(T.s);
-    if (ready) {
+    if (ld_acquire(word) >= target) {
+      if (T.unit < 0) break;
       task[0] = T.piece < 0 ? kTaskSelect : kTaskPool;
       task[1] = T.unit;
       task[2] = T.piece;
@@ -1014,11 +980,7 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
     TaskPos T{-1, 0, 0, -1, -1, 0};
     for (;;) {
       if (ct == 0) {
-        if constexpr (kPieces) {
-          claim_ticket(F, T, s_task);
-        } else {
-          claim_task(F, s_task);
-        }
+        claim_ticket<kPieces>(F, T, s_task);
       }
       cbar();
       const int type = s_task[0];
@@ -1051,7 +1013,7 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
           cbar();
         }
         select_unit<kPieces>(sel, U, p.raw + soff, p.pooled + soff,
-                    p.indices + static_cast<long long>(g) * p.o_total + U.out0, creg, ct);
+                             p.indices + static_cast<long long>(g) * p.o_total + U.out0, creg, ct);
       }
     }
   }

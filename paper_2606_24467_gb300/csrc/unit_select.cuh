@@ -399,12 +399,11 @@ __device__ __noinline__ void pool_unit(const float* raw, float* pooled, int n, i
   pool_strips<false>(raw, pooled, nullptr, n, 0, n, e, h, fP, sh, ct);
 }
 
-// Pooling in pieces: when a call has fewer units than CTAs, the units whose
-// keys do not fit shared memory are pooled by all of them, a piece at a time,
-// before one CTA selects (one 131072-token layer: 226 -> 163 us, 32768: 90 ->
-// 82).  With more units it gains nothing, and its code in the kernels costs
-// 5-10% (32 layers of short prompts: 481 -> 536 us), so that they are
-// instantiated with and without it.
+// Pooling in pieces: the units whose keys do not fit shared memory are pooled by
+// all CTAs, a piece at a time, before one CTA selects (one 131072-token layer:
+// 226 -> 163 us, 32768: 90 -> 82).  Where it gains nothing its code in the
+// kernels costs 2-10% (32 layers of short prompts: 481 -> 536 us), so that they
+// are instantiated with and without it.
 constexpr int kPoolPiece = 32 * kPoolStrip;  // keys of a pooling task
 __device__ __forceinline__ int pool_pieces(int n) {
   return n <= kSelWhole ? 0 : (n + kPoolPiece - 1) / kPoolPiece;

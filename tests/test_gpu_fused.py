@@ -298,3 +298,21 @@ def test_windows_and_pool_widths(cuda_device, window, pool_width, dtype):
     out, cu_out, cu = _run_call(layers, cfg, dev)
     for l in range(cfg.n_layers):
         _check_block(_block(out, cu_out, cu, l, cfg.batch, cfg.window), layers[l], cfg)
+
+
+@pytest.mark.parametrize("pool_width", [7, 63])
+def test_many_units_pooled_in_pieces(cuda_device, pool_width):
+    """More units than CTAs, some of several pieces of 6144 keys and some of
+    none, in the two-pass kernel (a prompt above 49152 in every layer), with
+    the usual and the widest pool."""
+    lens = [49153, 12400, 300, 40]
+    cfg = wl.get("c2").scaled(seq_len=0, n_layers=5, batch=len(lens), pool_width=pool_width,
+                              budget_mean=300)
+    masks = wl.srh_masks(cfg)
+    budgets = wl.layer_budgets(cfg, lens)
+    layers = [wl.make_layer(cfg, l, lengths=lens, masks=masks, budgets=budgets)
+              for l in range(cfg.n_layers)]
+    assert cfg.n_layers * len(lens) * cfg.num_kv_heads > 152
+    out, cu_out, cu = _run_call(layers, cfg, cuda_device)
+    for l in (0, 4):
+        _check_block(_block(out, cu_out, cu, l, cfg.batch, cfg.window), layers[l], cfg)
