@@ -238,30 +238,32 @@ int compresskv_compress_layer(const ckv_problem* p, const void* q_win, const voi
  * (both traced as CKV_KERNEL_FUSED): one CTA per SM streams K from the first
  * layer to the last while other warps of the same CTAs select and gather the
  * units whose scores are complete.
- * A call whose layers all have short prompts takes the resident kernel, which
- * reads K once: a unit's K tiles are spread over all SMs, their logits stay in
- * tensor memory while the query rows' sums of exponentials are added up over
- * the SMs, and the normalised probabilities of each key (Eq. 1-2) are then
- * summed in fp32 from the same logits.  "Short": the layer's longest prompt
- * has at most 49152 tokens when its widest group has at most 64 query rows
- * (|S_g| W), 12288 at 96 rows, 8192 at 128, 4096 at 192 (24576, 12288, 12288
- * and 6144 with the LSE given).
- * Other calls take the two-pass kernel, which reads K twice per chunk of 16
+ * A layer with short prompts takes the resident kernel, which reads K once:
+ * a unit's K tiles are spread over all SMs, their logits stay in tensor
+ * memory while the query rows' sums of exponentials are added up over the
+ * SMs, and the normalised probabilities of each key (Eq. 1-2) are then summed
+ * in fp32 from the same logits.  "Short": the layer's longest prompt has at
+ * most 49152 tokens when its widest group has at most 64 query rows (|S_g| W),
+ * 12288 at 96 rows, 8192 at 128, 4096 at 192 (24576, 12288, 12288 and 6144
+ * with the LSE given).
+ * Other layers take the two-pass kernel, which reads K twice per chunk of 16
  * tiles of 128 keys: a first pass sums each query row's exponentials (softmax
  * statistics of the chunk), and once every chunk of the unit is in and the
  * row's denominator merged, a second pass sums the normalised probabilities
  * from K read again (for long calls mostly from DRAM: the step then moves
- * about twice the bytes of K).
- * Neither stores exponentials.  The grid of chunks follows from the layer
- * alone, and neither kernel's scores depend on the order in which chunks
- * complete: compressing a layer alone or among others that take the same
- * kernel gives the same bits.  The kernels take windows W that are multiples
- * of 16, query strides that are multiples of 8 elements, at most 32 query
- * heads per group and SRH lists of at most 192 query rows (two Q buffers of
- * them beside a ring of two K tiles fill the shared memory); other per-group
- * problems use the separate kernels.  The resident kernel is a cooperative
- * launch: it starts when every SM has room for one of its CTAs, and where the
- * stream's context has fewer SMs than the device the two-pass kernel runs.
+ * about twice the bytes of K).  A call with layers of both kinds launches
+ * both kernels, one after the other.
+ * Neither stores exponentials.  The kernel and the grid of chunks follow from
+ * the layer alone, and neither kernel's scores depend on the order in which
+ * chunks complete: compressing a layer alone or among others, with a workspace
+ * or without, gives the same bits.  The kernels take windows W that are
+ * multiples of 16, query strides that are multiples of 8 elements, at most 32
+ * query heads per group and SRH lists of at most 192 query rows (two Q buffers
+ * of them beside a ring of two K tiles fill the shared memory); other
+ * per-group problems use the separate kernels.  The resident kernel is a
+ * cooperative launch: it starts when every SM has room for one of its CTAs,
+ * and where the stream's context has fewer SMs than the device the call
+ * returns CKV_ERR_CUDA.
  * n_masks: 1 <= n_masks, dividing batch (else CKV_ERR_INVALID_ARG); at most
  *   256 under CKV_SELECT_PER_GROUP and 4 under CKV_SELECT_PER_LAYER (or when
  *   the separate kernels run) (else CKV_ERR_UNSUPPORTED).

@@ -130,8 +130,8 @@ struct Info {
   long long T = 0, p_total = 0;
   // SRH masks: sequence s uses mask s / spm (n_masks masks, spm = B / n_masks)
   int n_masks = 1, spm = 1;
-  // the workspace holds neither the resident kernel's area nor the row maxima
-  // (a static scratch too small for them)
+  // the workspace holds neither the resident kernel's area for all units nor the
+  // row maxima (a static scratch too small for them)
   bool lean = false;
   int vgroup(int s, int g) const { return srh_group(s, g, spm, Hkv); }
 };
@@ -346,15 +346,15 @@ struct ResidentLayout {
   size_t raw, pooled, rowmax, acc, pairs, ctr, total;
 };
 
-ResidentLayout resident_layout(const Info& I) {
+ResidentLayout resident_layout(const Info& I, int n_seqs) {
   ResidentLayout F;
   const size_t rows = static_cast<size_t>((std::min(I.G * I.W, kResidentMaxRows) + 31) & ~31);
-  const size_t units = static_cast<size_t>(I.B) * I.Hkv;
+  const size_t units = static_cast<size_t>(n_seqs) * I.Hkv;
   const size_t scores = align256(static_cast<size_t>(I.Hkv) * I.p_total * sizeof(float));
   F.raw = kHeaderBytes;
   F.pooled = F.raw + scores;
   F.rowmax = F.pooled + scores;
-  F.acc = F.rowmax + row_max_bytes(I);
+  F.acc = F.rowmax + (I.lean ? 0 : row_max_bytes(I));
   F.pairs = F.acc + align256(units * kAccWords * rows * 8);
   F.ctr = F.pairs + align256(static_cast<size_t>(kResidentMaxGrid) * kPairRing * rows * sizeof(float2));
   F.total = F.ctr + align256((3 * units + 1) * sizeof(int));
@@ -369,7 +369,7 @@ size_t base_bytes(const Info& I) {
   lean.lean = true;
   const size_t base = std::max(workspace_layout(I).total, fused_layout(lean).total);
   if (I.lean || (I.layer && !I.pool_max)) return base;
-  return std::max({base, fused_layout(I).total, resident_layout(I).total});
+  return std::max({base, fused_layout(I).total, resident_layout(I, I.B).total});
 }
 
 // Max pooling: after these layouts, one raw-score row per SRH head slot (at
@@ -937,12 +937,17 @@ int run_gather(const ckv_problem* p, const Info& I, const int32_t* indices,
   return traced(tr, CKV_KERNEL_GATHER, [&] { return launch_gather(P, rows, stream); });
 }
 
-// Whether a layer is one for the resident kernel (resident_kernel.cu: K read
-// once, the logits kept in tensor memory until the softmax sums are complete):
-// short prompts, by its longest prompt and the query rows of its widest group.
-// A call takes it when all its layers are, else the two-pass kernel
-// (fused_kernel.cu).  (Both kernels for a call with layers of both kinds cost
-// a second tail: 32 layers of 15826 tokens with one such layer 568 -> 665 us.)
+// Which of the two persistent kernels a layer takes: the resident one
+// (resident_kernel.cu: K read once, the logits kept in tensor memory until
+// the softmax sums are complete) for short prompts, else the two-pass one
+// (fused_kernel.cu).  The lines are by the layer's longest prompt and the query
+// rows of its widest group, and by nothing else of the call, so that a layer
+// gives the same bits alone or among others; a call with layers of both kinds
+// launches both, for a second tail (32 layers of 14000 tokens, two of them
+// narrow enough for the resident kernel: 92 + 367 us; four KV heads, three
+// such layers: 81 + 228, all 32 in the two-pass kernel 230).  (The prompts of
+// one layer go together: taking a 28-layer batch's shorter prompts apart cost
+// two tails, 3195 -> 3285 us.)
 // Two-pass / resident time in us (1 layer; 32 layers; 8 KV heads):
 //   32 rows      32768: 89/68, 723/496      49152: 108/84, 1009/725
 //   64 rows      32768: 91/76, 683/661      49152: 111/95, 971/977
@@ -1005,7 +1010,7 @@ constexpr double kUmmaTruncation = 1.2e-7;
 //   2560 units of 64 to 192 rows 32768: 8736/8956
 template <class Params>
 void fill_common(Params& P, const ckv_problem* p, const Info& I, const SrhLists& S,
-                 const std::vector<int>& co, int32_t* indices, const void* k, const void* v,
+                 const int* co, int o_total, int32_t* indices, const void* k, const void* v,
                  void* k_out, void* v_out, const LseInput& lse, bool do_select, bool in_pieces,
                  bool exact_denominators) {
   P.lse = lse.lse;
@@ -1031,7 +1036,7 @@ void fill_common(Params& P, const ckv_problem* p, const Info& I, const SrhLists&
   P.num_kv_heads = I.Hkv;
   P.group_size = I.G;
   P.p_total = static_cast<int>(I.p_total);
-  P.o_total = co[I.B];
+  P.o_total = o_total;
   P.is_bf16 = I.bf16 ? 1 : 0;
   P.n_units = I.B * I.Hkv;
   P.batch = I.B;
@@ -1058,6 +1063,18 @@ void fill_common(Params& P, const ckv_problem* p, const Info& I, const SrhLists&
   }
 }
 
+// Sequences [a, b) of a problem, with the offsets they have in it.
+Info sequences(const Info& I, int a, int b) {
+  Info R = I;
+  R.B = R.spm = b - a;
+  R.n_masks = 1;
+  R.cu.assign(I.cu.begin() + a, I.cu.begin() + b + 1);
+  R.cu_prefix.assign(I.cu_prefix.begin() + a, I.cu_prefix.begin() + b + 1);
+  R.len.assign(I.len.begin() + a, I.len.begin() + b);
+  R.n.assign(I.n.begin() + a, I.n.begin() + b);
+  return R;
+}
+
 // Per-group selection of a (multi-layer) fused call in the persistent kernels
 // (fused_kernel.cu, resident_kernel.cu).  Sets *handled = false, enqueueing
 // nothing, when the problem is outside what they take (the caller then uses
@@ -1067,7 +1084,7 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
               const void* k, const void* v, const std::vector<int>& co, int32_t* indices,
               void* k_out, void* v_out, float* raw_user, float* pooled_user, void* ws,
               size_t ws_bytes, cudaStream_t stream, bool* handled, bool do_select = true,
-              const LseInput& lse = LseInput{}, bool allow_resident = true) {
+              const LseInput& lse = LseInput{}) {
   *handled = false;
   if (I.layer || I.G > 32 || I.n_masks * I.Hkv > kFusedMaxLists || I.B > kFusedMaxSeqs)
     return CKV_OK;
@@ -1081,104 +1098,119 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   DeviceFacts* Fd = nullptr;
   int rc = device_facts(&Fd);
   if (rc != CKV_OK) return rc;
-  // the call's kernel, and the query rows of its widest group
+  // Sequences per launch of the resident kernel: all, but where the static
+  // scratch has no room for all units' sums (many tiny ones; it has for some,
+  // as the separate kernels' tables in the same place are larger).
+  const size_t room = I.pool_max ? maxpool_slots_offset(I) : ws_bytes;
+  int r_seqs = I.B;
+  while (I.lean && r_seqs > 0 && resident_layout(I, r_seqs).total > room) r_seqs /= 2;
+  // the kernel of every layer, and the query rows of each kernel's widest group
   const int r_grid = std::min(Fd->sms, kResidentMaxGrid);
-  std::vector<int> seq_ct(I.B, 0);  // K tiles per chunk
-  bool resident = allow_resident && r_grid >= kResidentMinGrid && !I.lean;
-  int max_rows = 16;
+  std::vector<int> seq_ct(I.B, 0);  // K tiles per chunk; 0: the two-pass kernel
+  int max_rows = 16, r_rows = 16;
+  bool any = false, r_any = false;  // sequences of each kernel
+  long long tiles = 0;
+  int longest = 0;
   for (int s0 = 0; s0 < I.B; s0 += I.spm) {  // layer by layer
-    int rows = 0, longest = 0;
+    int rows = 0;
     for (int g = 0; g < I.Hkv; ++g) rows = std::max(rows, S.rows[I.vgroup(s0, g)]);
-    long long tiles = 0;
-    for (int s_ = s0; s_ < s0 + I.spm; ++s_) {
-      longest = std::max(longest, I.len[s_]);
-      if (I.n[s_] > 0)
-        tiles += static_cast<long long>(I.Hkv) * ((I.len[s_] + kTileTokens - 1) / kTileTokens);
-    }
-    resident = resident && takes_resident(rows, longest, lse.lse != nullptr);
-    max_rows = std::max(max_rows, rows);
-    for (int s_ = s0; s_ < s0 + I.spm; ++s_) seq_ct[s_] = resident_chunk_tiles(rows, tiles);
-  }
-  auto half_bytes = [](int rows) { return ((((rows + 15) & ~15) * 128) + 1023) & ~1023; };
-  const int npad_max = (max_rows + 15) & ~15;
-  const int q_half = half_bytes(max_rows);
-  const int row_stride = (max_rows + 31) & ~31;
-  // TMEM: 512 columns of accumulator buffers, tstride columns each
-  const int tstride = npad_max <= 64 ? 64 : (npad_max <= 128 ? 128 : 256);
-  const int nwg = 2;  // epilogue warpgroups that take tiles
-  const int nbuf = 512 / tstride;
-  // three Q buffers when they fit beside a ring of at least four K tiles,
-  // else two beside at least two
-  auto smem_bytes = [&](int nq, int st) {
-    return resident ? resident_smem_bytes(q_half, nq, st, row_stride)
-                    : fused_smem_bytes(q_half, nq, st, row_stride, nwg);
-  };
-  int stages = 0, q_bufs = 0;
-  for (int nq = 3; nq >= 2 && stages == 0; --nq) {
-    for (int st = 8; st >= (nq == 3 ? 4 : 2); --st) {
-      if (smem_bytes(nq, st) <= static_cast<size_t>(Fd->smem_optin)) {
-        stages = st;
-        q_bufs = nq;
-        break;
+    if (s0 == 0 || !std::equal(I.len.begin() + s0, I.len.begin() + s0 + I.spm,
+                               I.len.begin() + s0 - I.spm)) {  // (else as the layer before)
+      tiles = longest = 0;
+      for (int s_ = s0; s_ < s0 + I.spm; ++s_) {
+        longest = std::max(longest, I.len[s_]);
+        if (I.n[s_] > 0)
+          tiles += static_cast<long long>(I.Hkv) * ((I.len[s_] + kTileTokens - 1) / kTileTokens);
       }
     }
+    const bool res = r_grid >= kResidentMinGrid && r_seqs > 0 &&
+                     takes_resident(rows, longest, lse.lse != nullptr);
+    int& most = res ? r_rows : max_rows;
+    most = std::max(most, rows);
+    (res ? r_any : any) = true;
+    if (res)
+      for (int s_ = s0; s_ < s0 + I.spm; ++s_) seq_ct[s_] = resident_chunk_tiles(rows, tiles);
   }
-  if (stages == 0) return CKV_OK;  // query rows too many for two Q buffers and a ring
+  // Both kernels: three Q buffers when they fit beside a ring of at least four
+  // K tiles, else two beside at least two.
+  const int nwg = 2;  // epilogue warpgroups that take tiles (two-pass kernel)
+  auto half_bytes = [](int rows) { return ((((rows + 15) & ~15) * 128) + 1023) & ~1023; };
+  auto row_stride = [](int rows) { return (rows + 31) & ~31; };
+  auto smem_bytes = [&](bool res, int nq, int st) {
+    const int rows = res ? r_rows : max_rows;
+    return res ? resident_smem_bytes(half_bytes(rows), nq, st, row_stride(rows))
+               : fused_smem_bytes(half_bytes(rows), nq, st, row_stride(rows), nwg);
+  };
+  int stages[2] = {0, 0}, q_bufs[2] = {0, 0};  // two-pass, resident
+  for (int res = 0; res < 2; ++res)
+    for (int nq = 3; nq >= 2 && stages[res] == 0; --nq)
+      for (int st = 8; st >= (nq == 3 ? 4 : 2); --st)
+        if (smem_bytes(res != 0, nq, st) <= static_cast<size_t>(Fd->smem_optin)) {
+          stages[res] = st;
+          q_bufs[res] = nq;
+          break;
+        }
+  // query rows too many for two Q buffers and a ring
+  if ((any && stages[0] == 0) || (r_any && stages[1] == 0)) return CKV_OK;
   *handled = true;
   if (!q_win || !k || !aligned16(q_win) || !aligned16(k)) return CKV_ERR_INVALID_ARG;
   if (do_select && (rc = check_outputs(I, co, indices, k, v, k_out, v_out)) != CKV_OK) return rc;
-  const FusedLayout FL = fused_layout(I);
   if (!ws || ws_bytes < workspace_bytes(I) || (reinterpret_cast<uintptr_t>(ws) & 255u))
     return CKV_ERR_WORKSPACE;
   char* wb = static_cast<char*>(ws);
-
   Tracer tr{p->trace, stream};
-  if (resident) {
-    const ResidentLayout RL = resident_layout(I);
-    static thread_local ResidentParams P;  // large (about 13 KB): kept off the stack
-    std::memset(&P, 0, sizeof(P));
-    if ((rc = make_k_map(I, p, k, &P.tmap_k)) != CKV_OK) return rc;
-    if ((rc = make_q_map(I, p, q_win, &P.tmap_q)) != CKV_OK) return rc;
-    fill_common(P, p, I, S, co, indices, k, v, k_out, v_out, lse, do_select,
-                I.B * I.Hkv <= Fd->sms / 4, true);
-    P.raw = raw_user ? raw_user : reinterpret_cast<float*>(wb + RL.raw);
-    P.raw_scratch = raw_user ? 0 : 1;
-    P.pooled = pooled_user ? pooled_user : reinterpret_cast<float*>(wb + RL.pooled);
-    P.rowmax = reinterpret_cast<uint32_t*>(wb + RL.rowmax);
-    P.status = reinterpret_cast<int*>(wb);
-    P.ctr = reinterpret_cast<int*>(wb + kFusedCtrOffset);
-    P.unit_ctr = reinterpret_cast<int*>(wb + RL.ctr);
-    P.acc = reinterpret_cast<unsigned long long*>(wb + RL.acc);
-    P.acc_rows = row_stride;
-    P.pairs = reinterpret_cast<float2*>(wb + RL.pairs);
-    for (int s_ = 0; s_ < I.B; ++s_) {
-      const int tiles = I.n[s_] > 0 ? (I.len[s_] + kTileTokens - 1) / kTileTokens : 0;
-      P.seq_chunk[s_] = static_cast<uint8_t>(seq_ct[s_]);
-      P.chunk_off[s_ + 1] =
-          P.chunk_off[s_] + I.Hkv * ((tiles + seq_ct[s_] - 1) / seq_ct[s_]);
-    }
-    P.n_chunks = P.chunk_off[I.B];
-    P.q_half_bytes = q_half;
-    P.q_bufs = q_bufs;
-    P.stages = stages;
-    if (P.n_units == 0 || (P.n_chunks == 0 && (!do_select || co[I.B] == 0))) return CKV_OK;
-    cudaError_t e = cudaSuccess;
-    rc = traced(tr, CKV_KERNEL_FUSED, [&] {
-      return e = launch_resident(P, r_grid, smem_bytes(q_bufs, stages), stream);
-    });
-    if (e != cudaErrorCooperativeLaunchTooLarge) return rc;
-    // the stream's context has fewer SMs than the device: the two-pass kernel
-    // runs with any number of CTAs at once
-    (void)cudaGetLastError();
-    return run_fused(p, I, S, q_win, k, v, co, indices, k_out, v_out, raw_user, pooled_user, ws,
-                     ws_bytes, stream, handled, do_select, lse, false);
-  }
 
+  if (r_any) {
+    for (int a = 0; a < I.B; a += r_seqs) {
+      const int b = std::min(I.B, a + r_seqs);
+      const Info part = r_seqs < I.B ? sequences(I, a, b) : Info();
+      const Info& R = r_seqs < I.B ? part : I;
+      const ResidentLayout RL = resident_layout(I, R.B);
+      static thread_local ResidentParams P;  // large (about 13 KB): kept off the stack
+      std::memset(&P, 0, sizeof(P));
+      const char* q = static_cast<const char*>(q_win) + 2 * a * p->q_batch_stride;
+      if ((rc = make_k_map(R, p, k, &P.tmap_k)) != CKV_OK) return rc;
+      if ((rc = make_q_map(R, p, a > 0 ? q : q_win, &P.tmap_q)) != CKV_OK) return rc;
+      fill_common(P, p, R, S, co.data() + a, co[I.B], indices, k, v, k_out, v_out, lse, do_select,
+                  R.B * I.Hkv <= Fd->sms / 4, true);
+      P.raw = raw_user ? raw_user : reinterpret_cast<float*>(wb + RL.raw);
+      P.raw_scratch = raw_user ? 0 : 1;
+      P.pooled = pooled_user ? pooled_user : reinterpret_cast<float*>(wb + RL.pooled);
+      P.rowmax = reinterpret_cast<uint32_t*>(wb + RL.rowmax);
+      P.status = reinterpret_cast<int*>(wb);
+      P.ctr = reinterpret_cast<int*>(wb + kFusedCtrOffset);
+      P.unit_ctr = reinterpret_cast<int*>(wb + RL.ctr);
+      P.acc = reinterpret_cast<unsigned long long*>(wb + RL.acc);
+      P.mixed = any ? 1 : 0;
+      P.acc_rows = row_stride(r_rows);
+      P.pairs = reinterpret_cast<float2*>(wb + RL.pairs);
+      long long out = 0;  // rows of the sequences this launch selects
+      for (int s_ = 0; s_ < R.B; ++s_) {
+        const int ct = seq_ct[a + s_];
+        const int nt = R.n[s_] > 0 ? (R.len[s_] + kTileTokens - 1) / kTileTokens : 0;
+        P.seq_chunk[s_] = static_cast<uint8_t>(ct);
+        P.chunk_off[s_ + 1] = P.chunk_off[s_] + (ct ? I.Hkv * ((nt + ct - 1) / ct) : 0);
+        if (ct) out += co[a + s_ + 1] - co[a + s_];
+      }
+      P.n_chunks = P.chunk_off[R.B];
+      P.q_half_bytes = half_bytes(r_rows);
+      P.q_bufs = q_bufs[1];
+      P.stages = stages[1];
+      if (P.n_chunks == 0 && (!do_select || out == 0)) continue;
+      rc = traced(tr, CKV_KERNEL_FUSED, [&] {
+        return launch_resident(P, r_grid, smem_bytes(true, q_bufs[1], stages[1]), stream);
+      });
+      if (rc != CKV_OK) return rc;
+    }
+  }
+  if (!any) return CKV_OK;
+
+  const FusedLayout FL = fused_layout(I);
   static thread_local FusedParams P;  // large (about 15 KB): kept off the stack
   std::memset(&P, 0, sizeof(P));
   if ((rc = make_k_map(I, p, k, &P.tmap_k)) != CKV_OK) return rc;
   if ((rc = make_q_map(I, p, q_win, &P.tmap_q)) != CKV_OK) return rc;
-  fill_common(P, p, I, S, co, indices, k, v, k_out, v_out, lse, do_select,
+  fill_common(P, p, I, S, co.data(), co[I.B], indices, k, v, k_out, v_out, lse, do_select,
               max_rows <= 64 || I.B * I.Hkv < Fd->sms, lse.lse != nullptr);
   P.raw = raw_user ? raw_user : reinterpret_cast<float*>(wb + FL.raw);
   P.raw_scratch = raw_user ? 0 : 1;
@@ -1189,20 +1221,28 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   P.partials = reinterpret_cast<float2*>(wb + FL.partials);
   P.bias = reinterpret_cast<float*>(wb + FL.bias);
   P.part_stride = FL.part_stride;
-  for (int s_ = 0; s_ < I.B; ++s_)
-    P.chunk_off[s_ + 1] = P.chunk_off[s_] + I.Hkv * chunks_per_unit(I, s_);
+  P.mixed = r_any ? 1 : 0;
+  long long out = 0;  // rows of the sequences this launch selects
+  for (int s_ = 0; s_ < I.B; ++s_) {
+    const bool here = seq_ct[s_] == 0;
+    P.chunk_off[s_ + 1] = P.chunk_off[s_] + (here ? I.Hkv * chunks_per_unit(I, s_) : 0);
+    if (here) out += co[s_ + 1] - co[s_];
+  }
   P.n_chunks = P.chunk_off[I.B];
-  if (P.n_chunks != FL.n_chunks) return CKV_ERR_WORKSPACE;  // cannot happen: same plan
-  P.q_half_bytes = q_half;
-  P.q_bufs = q_bufs;
-  P.row_stride = row_stride;
-  P.stages = stages;
-  P.tstride = tstride;
-  P.nbuf = nbuf;
+  if (P.n_chunks > FL.n_chunks) return CKV_ERR_WORKSPACE;  // cannot happen: same plan
+  const int npad_max = (max_rows + 15) & ~15;
+  P.q_half_bytes = half_bytes(max_rows);
+  P.q_bufs = q_bufs[0];
+  P.row_stride = row_stride(max_rows);
+  P.stages = stages[0];
+  // TMEM: 512 columns of accumulator buffers, tstride columns each
+  P.tstride = npad_max <= 64 ? 64 : (npad_max <= 128 ? 128 : 256);
+  P.nbuf = 512 / P.tstride;
   P.nwg = nwg;
-  if (P.n_units == 0 || (P.n_chunks == 0 && (!do_select || co[I.B] == 0))) return CKV_OK;
-  return traced(tr, CKV_KERNEL_FUSED,
-                [&] { return launch_fused(P, Fd->sms, smem_bytes(q_bufs, stages), stream); });
+  if (P.n_chunks == 0 && (!do_select || out == 0)) return CKV_OK;
+  return traced(tr, CKV_KERNEL_FUSED, [&] {
+    return launch_fused(P, Fd->sms, smem_bytes(false, q_bufs[0], stages[0]), stream);
+  });
 }
 
 }  // namespace

@@ -205,10 +205,13 @@ struct FusedParams {
   int cu_seqlens[kFusedMaxSeqs + 1];
   int cu_prefix[kFusedMaxSeqs + 1];
   int cu_out[kFusedMaxSeqs + 1];
-  int chunk_off[kFusedMaxSeqs + 1];   // first chunk of sequence s (units of s are consecutive)
+  // first chunk of sequence s (units of s are consecutive); a sequence with a
+  // prefix and no chunks is not one of this launch
+  int chunk_off[kFusedMaxSeqs + 1];
   uint32_t srh_bits[kFusedMaxLists];  // per (mask, group): bit i = query head group*G + i is SRH
   uint32_t* rowmax;            // largest pooled score of every 32 keys (row_max_offset)
-  int in_pieces;               // long units are pooled in pieces (few units in the call)
+  int in_pieces;               // long units are pooled in pieces
+  int mixed;                   // some sequences are not of this launch
 };
 
 cudaError_t launch_fused(const FusedParams& p, int grid, size_t smem, cudaStream_t s);
@@ -262,10 +265,11 @@ struct ResidentParams {
   int cu_prefix[kFusedMaxSeqs + 1];
   int cu_out[kFusedMaxSeqs + 1];
   int chunk_off[kFusedMaxSeqs + 1];   // first chunk of sequence s (units of s are consecutive)
-  uint8_t seq_chunk[kFusedMaxSeqs];   // K tiles per chunk
+  uint8_t seq_chunk[kFusedMaxSeqs];   // K tiles per chunk; 0: not a sequence of this launch
   uint32_t srh_bits[kFusedMaxLists];  // per (mask, group): bit i = query head group*G + i is SRH
   uint32_t* rowmax;            // largest pooled score of every 32 keys (row_max_offset)
-  int in_pieces;               // long units are pooled in pieces (few units in the call)
+  int in_pieces;               // long units are pooled in pieces
+  int mixed;                   // some sequences are not of this launch
 };
 
 cudaError_t launch_resident(const ResidentParams& p, int grid, size_t smem, cudaStream_t s);

@@ -152,6 +152,17 @@ struct Fused {
   __device__ int chunks_per_unit(int s) const {
     return (p.chunk_off[s + 1] - p.chunk_off[s]) / p.num_kv_heads;
   }
+  // a sequence of a layer that the resident kernel takes
+  __device__ bool not_here(int s) const {
+    return p.chunk_off[s + 1] == p.chunk_off[s] && prefix(s) > 0;
+  }
+  // unit u, or the first unit after it whose sequence has chunks to merge
+  __device__ int next_merge(int u) const {
+    int s = u / p.num_kv_heads;
+    if (s * p.num_kv_heads != u || s >= p.batch || chunks_per_unit(s) > 0) return u;
+    do ++s; while (s < p.batch && chunks_per_unit(s) == 0);
+    return s * p.num_kv_heads;
+  }
   __device__ int list(int s, int g) const { return srh_group(s, g, p.seqs_per_mask, p.num_kv_heads); }
   __device__ int rows(int s, int g) const { return __popc(p.srh_bits[list(s, g)]) * p.window; }
   __device__ int* ticket(int u) const { return p.ctr + kFusedCtrHead + u; }
@@ -372,22 +383,24 @@ __device__ __noinline__ void merge_unit(const Fused& F, int u, uint8_t* creg, in
 // the next ready selection cost 1 us apiece: 48 layers of 12288 tokens of 128
 // rows 720 -> 486 us with tickets, 60 layers of 4 prompts of 500 to 9000 of 64
 // to 192 rows 3250 -> 1850.)
-template <bool kPieces>
+template <int kKind>
 __device__ void claim_ticket(const Fused& F, TaskPos& T, int* task) {
   const FusedParams& p = F.p;
   if (T.t < 0)
     take_ticket(T, p.ctr + kCtrTicket, p.batch, p.num_kv_heads, [&](int s) {
-      return kPieces ? pool_pieces(F.prefix(s)) : 0;
+      if (kKind == kMixed && F.not_here(s)) return -1;
+      return kKind == kInPieces || (kKind == kMixed && p.in_pieces) ? pool_pieces(F.prefix(s)) : 0;
     });
   // what the task waits for; without one (every selection is ahead of the
   // first ticket past the last), the other units' merges
   const int* word = p.ctr + kCtrMerge;
-  int target = p.given_lse ? 0 : p.n_units;
+  int target = p.given_lse ? 0 : (kKind == kMixed && F.next_merge(0) == p.n_units ? 0 : p.n_units);
   if (T.unit >= 0) {
-    const bool pooled = kPieces && T.piece < 0 && T.pieces > 0;
+    const bool pooled = kKind != kPlain && T.piece < 0 && T.pieces > 0;
     word = pooled ? F.bias_state(T.unit) : F.p2done(T.unit);
     target = pooled ? 4 * T.pieces : kEpiWarps * F.chunks_per_unit(T.s);
   }
+  const int first = kKind == kMixed ? F.next_merge(0) : 0;
   const uint64_t t0 = globaltimer_ns();
   for (;;) {
     if (F.aborted() || *reinterpret_cast<volatile int*>(F.abort_cta)) break;
@@ -396,14 +409,16 @@ __device__ void claim_ticket(const Fused& F, TaskPos& T, int* task) {
       task[0] = T.piece < 0 ? kTaskSelect : kTaskPool;
       task[1] = T.unit;
       task[2] = T.piece;
+      if (kKind == kMixed) task[3] = T.pieces;
       T.t = -1;
       return;
     }
     if (!p.given_lse) {
-      const int m = ld_volatile(p.ctr + kCtrMerge);
+      const int at = ld_volatile(p.ctr + kCtrMerge);
+      const int m = kKind == kMixed ? max(at, first) : at;
       if (m < p.n_units &&
           ld_acquire(F.ticket(m)) >= p.nwg * F.chunks_per_unit(m / p.num_kv_heads)) {
-        if (atomicCAS(p.ctr + kCtrMerge, m, m + 1) == m) {
+        if (atomicCAS(p.ctr + kCtrMerge, at, kKind == kMixed ? F.next_merge(m + 1) : m + 1) == at) {
           task[0] = kTaskMerge;
           task[1] = m;
           return;
@@ -458,7 +473,7 @@ __device__ __forceinline__ void wait_plain(uint32_t bar, uint32_t parity, uint64
   mbar_wait_bounded(bar, parity, &never, nullptr, timeout_ns);
 }
 
-template <bool kPieces>
+template <int kKind>
 __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_constant__ FusedParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -980,7 +995,7 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
     TaskPos T{-1, 0, 0, -1, -1, 0};
     for (;;) {
       if (ct == 0) {
-        claim_ticket<kPieces>(F, T, s_task);
+        claim_ticket<kKind>(F, T, s_task);
       }
       cbar();
       const int type = s_task[0];
@@ -1001,7 +1016,7 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
         U.out0 = p.cu_out[s];
         U.kept = p.cu_out[s + 1] - U.out0;
         const long long soff = static_cast<long long>(g) * p.p_total + p.cu_prefix[s];
-        if constexpr (kPieces) {
+        if constexpr (kKind != kPlain) {
           SelShared& ss = *reinterpret_cast<SelShared*>(creg);
           uint32_t* const rowmax = p.rowmax + row_max_offset(soff, g, s, p.batch);
           if (type == kTaskPool) {
@@ -1009,11 +1024,11 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
                        F.bias_state(idx), 4, ct);
             continue;
           }
-          if (ct == 0) ss.rowmax = rowmax;
+          if (ct == 0) ss.rowmax = kKind == kInPieces || s_task[3] > 0 ? rowmax : nullptr;
           cbar();
         }
-        select_unit<kPieces>(sel, U, p.raw + soff, p.pooled + soff,
-                             p.indices + static_cast<long long>(g) * p.o_total + U.out0, creg, ct);
+        select_unit<kKind>(sel, U, p.raw + soff, p.pooled + soff,
+                           p.indices + static_cast<long long>(g) * p.o_total + U.out0, creg, ct);
       }
     }
   }
@@ -1047,11 +1062,12 @@ size_t fused_smem_bytes(int q_half_bytes, int q_bufs, int stages, int row_stride
 }
 
 cudaError_t fused_set_smem_limit(size_t bytes) {
-  const cudaError_t e = cudaFuncSetAttribute(
-      fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(bytes));
+  for (auto kernel : {fused_kernel<kPlain>, fused_kernel<kInPieces>, fused_kernel<kMixed>}) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_fused(const FusedParams& p, int grid, size_t smem, cudaStream_t stream) {
@@ -1062,7 +1078,11 @@ cudaError_t launch_fused(const FusedParams& p, int grid, size_t smem, cudaStream
   cfg.stream = stream;
   cfg.attrs = nullptr;
   cfg.numAttrs = 0;
-  return cudaLaunchKernelEx(&cfg, p.in_pieces ? fused_kernel<true> : fused_kernel<false>, p);
+  return cudaLaunchKernelEx(&cfg,
+                            p.mixed       ? fused_kernel<kMixed>
+                            : p.in_pieces ? fused_kernel<kInPieces>
+                                          : fused_kernel<kPlain>,
+                            p);
 }
 
 }  // namespace ckv

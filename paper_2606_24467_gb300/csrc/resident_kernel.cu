@@ -195,7 +195,7 @@ struct ResidentShared {
   uint64_t dnfull[2][2], dnempty[2][2];                // denominators of a unit, per warpgroup
   uint64_t startbar;
   uint32_t tmem;
-  int abort_cta, task, piece;
+  int abort_cta, task, piece, pieces;
   int sum_pos;                                         // chunks below have left their pairs
   int p2_unit[kPub];
   ChunkDesc descs[kDescs];
@@ -1185,7 +1185,7 @@ __device__ __noinline__ void denominator_role(ResidentShared& sh, int mine, int 
   __syncwarp();
 }
 
-template <bool kPieces>
+template <int kKind>
 __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_constant__ ResidentParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -1201,6 +1201,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
+  constexpr bool kPieces = kKind != kPlain;
   const int grid = static_cast<int>(gridDim.x);
   auto p2done = [&](int u) { return p.unit_ctr + u; };
 
@@ -1446,15 +1447,18 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
       U.out0 = p.cu_out[s];
       U.kept = p.cu_out[s + 1] - U.out0;
       const long long soff = static_cast<long long>(g) * p.p_total + p.cu_prefix[s];
-      select_unit<false>(sh.call.sel, U, p.raw + soff, p.pooled + soff,
+      select_unit<kPlain>(sh.call.sel, U, p.raw + soff, p.pooled + soff,
                   p.indices + static_cast<long long>(g) * p.o_total + U.out0, creg, ct);
     }
     TaskPos T{-1, 0, 0, -1, -1, 0};
 #pragma unroll 1
-    while (kPieces) {
+    while (kPieces && (kKind != kMixed || p.do_select)) {
       if (ct == 0) {
         take_ticket(T, p.unit_ctr + 3 * p.n_units, p.batch, p.num_kv_heads, [&](int s) {
-          return pool_pieces(p.cu_seqlens[s + 1] - p.cu_seqlens[s] - p.window);
+          if (kKind == kMixed && p.seq_chunk[s] == 0) return -1;
+          return kKind == kInPieces || p.in_pieces
+                     ? pool_pieces(p.cu_seqlens[s + 1] - p.cu_seqlens[s] - p.window)
+                     : 0;
         });
         bool ok = T.unit >= 0;
         if (ok)
@@ -1464,6 +1468,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
                                   (p.chunk_off[T.s + 1] - p.chunk_off[T.s]) / p.num_kv_heads);
         sh.task = ok ? T.unit : -1;
         sh.piece = T.piece;
+        if (kKind == kMixed) sh.pieces = T.pieces;
       }
       cbar();
       const int u = sh.task;
@@ -1487,9 +1492,9 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
                    p.unit_ctr + 2 * p.n_units + u, 1, ct);
         continue;
       }
-      if (ct == 0) ss.rowmax = rowmax;
+      if (ct == 0) ss.rowmax = kKind == kInPieces || sh.pieces > 0 ? rowmax : nullptr;
       cbar();
-      select_unit<true>(sh.call.sel, U, p.raw + soff, p.pooled + soff,
+      select_unit<kKind>(sh.call.sel, U, p.raw + soff, p.pooled + soff,
                         p.indices + static_cast<long long>(g) * p.o_total + U.out0, creg, ct);
     }
   }
@@ -1513,11 +1518,12 @@ size_t resident_smem_bytes(int q_half_bytes, int q_bufs, int stages, int acc_row
 }
 
 cudaError_t resident_set_smem_limit(size_t bytes) {
-  const cudaError_t e = cudaFuncSetAttribute(
-      resident_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(resident_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(bytes));
+  for (auto kernel : {resident_kernel<kPlain>, resident_kernel<kInPieces>, resident_kernel<kMixed>}) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_resident(const ResidentParams& p, int grid, size_t smem, cudaStream_t stream) {
@@ -1532,7 +1538,11 @@ cudaError_t launch_resident(const ResidentParams& p, int grid, size_t smem, cuda
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, p.in_pieces ? resident_kernel<true> : resident_kernel<false>, p);
+  return cudaLaunchKernelEx(&cfg,
+                            p.mixed       ? resident_kernel<kMixed>
+                            : p.in_pieces ? resident_kernel<kInPieces>
+                                          : resident_kernel<kPlain>,
+                            p);
 }
 
 }  // namespace ckv

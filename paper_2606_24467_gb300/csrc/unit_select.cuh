@@ -25,7 +25,7 @@ struct SelShared {
   int wcnt[8], wbase[8];
   int wcnt_ge[8];  // per-warp counts at the best threshold with at least k keys above
   alignas(16) uint32_t cnt[2][2][8];  // per-warp results of a bisection step
-  uint32_t* rowmax;                   // (pooling in pieces) the unit's row maxima
+  uint32_t* rowmax;                   // the unit's row maxima, if it was pooled in pieces
 };
 static_assert(sizeof(SelShared) <= kSelRegion, "select scratch");
 static_assert(kSelSamples <= kFusedCandCap, "samples live in the position array");
@@ -403,7 +403,10 @@ __device__ __noinline__ void pool_unit(const float* raw, float* pooled, int n, i
 // all CTAs, a piece at a time, before one CTA selects (one 131072-token layer:
 // 226 -> 163 us, 32768: 90 -> 82).  Where it gains nothing its code in the
 // kernels costs 2-10% (32 layers of short prompts: 481 -> 536 us), so that they
-// are instantiated with and without it.
+// are instantiated with and without it.  A third instance is for calls whose
+// layers take both kernels: it skips the other's sequences and pools in pieces
+// or not (that code in the others costs 1-3%).
+constexpr int kPlain = 0, kInPieces = 1, kMixed = 2;
 constexpr int kPoolPiece = 32 * kPoolStrip;  // keys of a pooling task
 __device__ __forceinline__ int pool_pieces(int n) {
   return n <= kSelWhole ? 0 : (n + kPoolPiece - 1) / kPoolPiece;
@@ -425,7 +428,7 @@ __device__ __noinline__ void pool_piece(const float* raw, float* pooled, uint32_
 }
 
 // The workers' tasks then, in one order that every CTA takes tickets of: of
-// every unit its pieces, then its selection.  A ticket is taken before its
+// every unit its pieces, then its selection (pieces(s) -1: no tasks).  A ticket is taken before its
 // task is ready: claims by compare-and-swap once a task is ready took 1 us
 // apiece (152 CTAs at one counter).
 struct TaskPos {
@@ -462,7 +465,7 @@ __device__ __forceinline__ void take_ticket(TaskPos& T, int* counter, int batch,
 // order and the bisection among them (a radix search among those in global
 // memory, or all the unit's scores, when the bound keeps too few or too many); then the window and the K/V rows.  Pooled
 // scores are >= 0: their bit patterns order like their values.
-template <bool kPieces>
+template <int kKind>
 __device__ __noinline__ void select_unit(const SelCall& p, const SelUnit U, float* raw,
                                          float* pooled, int32_t* out, uint8_t* creg, int ct) {
   assume_shared(creg);
@@ -477,7 +480,7 @@ __device__ __noinline__ void select_unit(const SelCall& p, const SelUnit U, floa
   while (((n + 31) >> 5) > (kSelGroups << e)) ++e;
   const int nr = (n + 31) >> 5;
   const int ng = (nr + (1 << e) - 1) >> e;
-  if (kPieces && n > kSelWhole) {
+  if (kKind != kPlain && n > kSelWhole && (kKind == kInPieces || sh.rowmax)) {
     const uint32_t* const rowmax = sh.rowmax;
 #pragma unroll 4
     for (int i = ct; i < ng; i += kCThreads) {

@@ -183,10 +183,58 @@ def test_calls_on_two_streams_at_once(cuda_device):
             assert torch.equal(getattr(out, key), getattr(want, key)), key
 
 
+def test_layers_on_both_sides_of_the_line(cuda_device):
+    """Layers of 64 and of 96 query rows at a length that the resident kernel
+    takes for the former only: one call launches both kernels, and every layer
+    has the bits of a call of its own (and, without scores, of the call without
+    a workspace)."""
+    dev = cuda_device
+    lens = [13000, 0, 40, 32, 700]
+    cfg = wl.get("c2").scaled(seq_len=0, n_layers=4, batch=len(lens), budget_mean=300)
+    two = np.asarray(wl.srh_masks(cfg.scaled(srh_per_group=(2, 2))))
+    three = np.asarray(wl.srh_masks(cfg.scaled(srh_per_group=(3, 3))))
+    masks = np.stack([two[0], three[1], three[2], two[3]])
+    budgets = wl.layer_budgets(cfg, lens)
+    layers = [wl.make_layer(cfg, l, lengths=lens, masks=masks, budgets=budgets) for l in range(4)]
+    big, cu_out, cu = _run_call(layers, cfg, dev)
+    for l, lay in enumerate(layers):
+        b = _block(big, cu_out, cu, l, cfg.batch, cfg.window)
+        if l < 2:
+            _check_block(b, lay, cfg)
+        alone, cu_out1, cu1 = _run_call([lay], cfg, dev)
+        a = _block(alone, cu_out1, cu1, 0, cfg.batch, cfg.window)
+        for key in BLOCK_KEYS:
+            assert np.array_equal(a[key], b[key]), (l, key)
+    q, k, v, cu, b, m = _pack(layers, dev)
+    trace = ckv.Trace(8)
+    prob = ckv.Problem(q, k, cu, cfg.window, cfg.pool_width, trace=trace)
+    out = ckv.LayerOutputs(prob, b, 128, k.dtype, dev, scores=False)
+    ws = ckv.workspace(prob, dev)
+    ckv.compress_layers(prob, 4, q, k, v, m, b, out.indices, out.k_out, out.v_out, ws)
+    torch.cuda.synchronize()
+    assert ckv.read_device_status(ws) == 0
+    assert trace.struct.launches == 2
+    assert torch.equal(out.indices, big.indices)
+    for l in (0, 1):
+        one = layers[l]
+        q, k, v = (one[x].to(dev) for x in ("q_win", "k", "v"))
+        prob = ckv.Problem(q, k, np.asarray(one["cu_seqlens"], np.int32), cfg.window, cfg.pool_width)
+        if ckv.workspace_size(prob) <= ckv.compresskv.STATIC_SCRATCH_BYTES:
+            out = ckv.LayerOutputs(prob, one["budgets"], 128, k.dtype, dev, scores=True)
+            ckv.compress_layer_noalloc(prob, q, k, v, masks[l], one["budgets"], out.indices,
+                                       out.k_out, out.v_out, raw=out.raw, pooled=out.pooled)
+            torch.cuda.synchronize()
+            got = _block(out, np.concatenate([[0], np.cumsum(np.minimum(one["budgets"], lens))]),
+                         np.asarray(one["cu_seqlens"]), 0, cfg.batch, cfg.window)
+            want = _block(big, cu_out, cu, l, cfg.batch, cfg.window)
+            for key in ("raw", "pooled", "indices", "k_out", "v_out"):
+                assert np.array_equal(got[key], want[key]), (l, key)
+
+
 def test_static_scratch_without_the_resident_area(cuda_device):
     """Many tiny units: the workspace is larger than the static scratch, which
-    holds the two-pass kernel's share of it, so the call without a workspace
-    takes that kernel; both calls agree (fp32 sums in two orders)."""
+    has no room for all units' sums, so the call without a workspace makes
+    several launches: the same bits."""
     dev = cuda_device
     cfg, layers = _make("c2", [20] * 512, n_layers=1, num_q_heads=32, num_kv_heads=32, window=16,
                         srh_per_group=(1, 1), budget_mean=18)
@@ -200,5 +248,5 @@ def test_static_scratch_without_the_resident_area(cuda_device):
                                raw=out.raw, pooled=out.pooled, device_status=status)
     torch.cuda.synchronize()
     assert int(status) == 0
-    torch.testing.assert_close(out.raw, want.raw, rtol=1e-5, atol=1e-9)
+    assert torch.equal(out.raw, want.raw) and torch.equal(out.pooled, want.pooled)
     assert torch.equal(out.indices, want.indices) and torch.equal(out.k_out, want.k_out)
