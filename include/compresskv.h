@@ -166,7 +166,8 @@ size_t compresskv_workspace_size(const ckv_problem* p);
  * kernels share between their CTAs (about 390 KB, enqueued on `stream`).
  * Call once after allocating a workspace, and after reading a non-zero
  * device status (an aborted call can leave the counters set); every call
- * that completes leaves them zero. */
+ * that completes leaves them ready for the next (zero, but for the number of
+ * calls of the resident kernel). */
 int compresskv_workspace_init(void* workspace, size_t workspace_bytes, void* stream);
 
 /* Host-only: per-sequence offsets of the prefix scores (cu_prefix, [batch+1])
@@ -260,10 +261,11 @@ int compresskv_compress_layer(const ckv_problem* p, const void* q_win, const voi
  * multiples of 16, query strides that are multiples of 8 elements, at most 32
  * query heads per group and SRH lists of at most 192 query rows (two Q buffers
  * of them beside a ring of two K tiles fill the shared memory); other
- * per-group problems use the separate kernels.  The resident kernel is a
- * cooperative launch: it starts when every SM has room for one of its CTAs,
- * and where the stream's context has fewer SMs than the device the call
- * returns CKV_ERR_CUDA.
+ * per-group problems use the separate kernels.  The resident kernel's CTAs
+ * wait for one another, so it runs on the SMs that are free when it starts: all
+ * of them (of a green context's share), but where another kernel holds some
+ * for longer than a millisecond it goes on without these.  On few SMs it
+ * reads K twice; the bits are the same on any number.
  * n_masks: 1 <= n_masks, dividing batch (else CKV_ERR_INVALID_ARG); at most
  *   256 under CKV_SELECT_PER_GROUP and 4 under CKV_SELECT_PER_LAYER (or when
  *   the separate kernels run) (else CKV_ERR_UNSUPPORTED).

@@ -43,7 +43,7 @@ constexpr size_t kTicketOffset = 256;
 constexpr size_t kStatusBytes = kTicketOffset + static_cast<size_t>(kMaxItems) * sizeof(int);
 // ... followed by the persistent kernels' words; the whole header is zeroed by
 // compresskv_workspace_init and left zero by every call that completes, but
-// for the resident kernel's start counter and the number of its last call that
+// for the number of the resident kernel's calls and of the last one that
 // stopped.
 constexpr size_t kFusedCtrOffset = kStatusBytes;
 constexpr size_t kHeaderBytes = ((kFusedCtrOffset + kFusedCtrBytes) + 255) & ~static_cast<size_t>(255);
@@ -77,6 +77,8 @@ struct DeviceFacts {
 std::mutex g_mutex;
 DeviceFacts g_facts[64];
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
+PFN_cuStreamGetGreenCtx_v12040 g_stream_green = nullptr;  // null: a driver without green contexts
+PFN_cuGreenCtxGetDevResource_v12040 g_green_resource = nullptr;
 
 int device_facts(DeviceFacts** out) {
   int dev = 0;
@@ -114,9 +116,30 @@ int device_facts(DeviceFacts** out) {
         q != cudaDriverEntryPointSuccess || !fn)
       return CKV_ERR_CUDA;
     g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+    void *gs = nullptr, *gr = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &gs, 12040, cudaEnableDefault, &q) ==
+            cudaSuccess && q == cudaDriverEntryPointSuccess &&
+        cudaGetDriverEntryPointByVersion("cuGreenCtxGetDevResource", &gr, 12040, cudaEnableDefault,
+                                         &q) == cudaSuccess && q == cudaDriverEntryPointSuccess) {
+      g_stream_green = reinterpret_cast<PFN_cuStreamGetGreenCtx_v12040>(gs);
+      g_green_resource = reinterpret_cast<PFN_cuGreenCtxGetDevResource_v12040>(gr);
+    }
+    (void)cudaGetLastError();
   }
   *out = &f;
   return CKV_OK;
+}
+
+// SMs that kernels on the stream may use (a green context's share of the
+// device's).
+int stream_sms(const DeviceFacts& F, cudaStream_t stream) {
+  CUgreenCtx green = nullptr;
+  CUdevResource r;
+  if (!g_stream_green || g_stream_green(stream, &green) != CUDA_SUCCESS || !green ||
+      g_green_resource(green, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS ||
+      r.sm.smCount == 0)
+    return F.sms;
+  return std::min(F.sms, static_cast<int>(r.sm.smCount));
 }
 
 // ------------------------------------------------------------------ validation
@@ -962,7 +985,7 @@ int run_gather(const ckv_problem* p, const Info& I, const int32_t* indices,
 // The resident kernel loses on long prompts because a unit's logits must all
 // be on the chip at once: beyond a few tiles per SM the chunks of different
 // units no longer overlap.
-constexpr int kResidentMinGrid = 96;  // CTAs that hold a unit of every admitted size
+constexpr int kResidentMinSms = 96;  // SMs of a device that hold a unit of every admitted size
 static_assert(kResidentMaxRows <= kMaxQRows, "resident rows");
 
 bool takes_resident(int rows, int len, bool given_lse) {
@@ -980,7 +1003,7 @@ bool takes_resident(int rows, int len, bool given_lse) {
 // four; a 4096-token one 37.5 with two, 38.9 with four, but 32 of the
 // latter 137 with two, 114 with four) or wide groups (the tensor memory must
 // hold two chunks).  A unit then has at most 128 chunks of two tiles or 96 of
-// four (the tensor memory holds 2 to 8): kResidentMinGrid CTAs hold any.
+// four (the tensor memory holds 2 to 8): kResidentMinSms CTAs hold any.
 int resident_chunk_tiles(int rows, long long layer_tiles) {
   const int most = rows <= 64 ? kResidentChunkTiles : (rows <= 128 ? 2 : 1);
   return std::min(most, layer_tiles <= 64 ? 1 : (layer_tiles <= 256 ? 2 : 4));
@@ -1105,8 +1128,8 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   int r_seqs = I.B;
   while (I.lean && r_seqs > 0 && resident_layout(I, r_seqs).total > room) r_seqs /= 2;
   // the kernel of every layer, and the query rows of each kernel's widest group
-  const int r_grid = std::min(Fd->sms, kResidentMaxGrid);
   std::vector<int> seq_ct(I.B, 0);  // K tiles per chunk; 0: the two-pass kernel
+  std::vector<int> seq_width(I.B, 0);  // columns of a tile of the layer's widest group
   int max_rows = 16, r_rows = 16;
   bool any = false, r_any = false;  // sequences of each kernel
   long long tiles = 0;
@@ -1123,13 +1146,16 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
           tiles += static_cast<long long>(I.Hkv) * ((I.len[s_] + kTileTokens - 1) / kTileTokens);
       }
     }
-    const bool res = r_grid >= kResidentMinGrid && r_seqs > 0 &&
+    const bool res = Fd->sms >= kResidentMinSms && r_seqs > 0 &&
                      takes_resident(rows, longest, lse.lse != nullptr);
     int& most = res ? r_rows : max_rows;
     most = std::max(most, rows);
     (res ? r_any : any) = true;
     if (res)
-      for (int s_ = s0; s_ < s0 + I.spm; ++s_) seq_ct[s_] = resident_chunk_tiles(rows, tiles);
+      for (int s_ = s0; s_ < s0 + I.spm; ++s_) {
+        seq_ct[s_] = resident_chunk_tiles(rows, tiles);
+        seq_width[s_] = (rows + 31) & ~31;
+      }
   }
   // Both kernels: three Q buffers when they fit beside a ring of at least four
   // K tiles, else two beside at least two.
@@ -1161,6 +1187,7 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   Tracer tr{p->trace, stream};
 
   if (r_any) {
+    const int r_grid = std::min(stream_sms(*Fd, stream), kResidentMaxGrid);
     for (int a = 0; a < I.B; a += r_seqs) {
       const int b = std::min(I.B, a + r_seqs);
       const Info part = r_seqs < I.B ? sequences(I, a, b) : Info();
@@ -1184,12 +1211,18 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
       P.mixed = any ? 1 : 0;
       P.acc_rows = row_stride(r_rows);
       P.pairs = reinterpret_cast<float2*>(wb + RL.pairs);
+      P.min_grid = 1;
       long long out = 0;  // rows of the sequences this launch selects
       for (int s_ = 0; s_ < R.B; ++s_) {
         const int ct = seq_ct[a + s_];
         const int nt = R.n[s_] > 0 ? (R.len[s_] + kTileTokens - 1) / kTileTokens : 0;
+        const int nch = ct ? (nt + ct - 1) / ct : 0;
         P.seq_chunk[s_] = static_cast<uint8_t>(ct);
-        P.chunk_off[s_ + 1] = P.chunk_off[s_] + (ct ? I.Hkv * ((nt + ct - 1) / ct) : 0);
+        P.chunk_off[s_ + 1] = P.chunk_off[s_] + I.Hkv * nch;
+        if (nch > 0) {
+          const int hold = 512 / (ct * seq_width[a + s_]);  // chunks in tensor memory
+          P.min_grid = std::max(P.min_grid, (nch + hold - 1) / hold);
+        }
         if (ct) out += co[a + s_ + 1] - co[a + s_];
       }
       P.n_chunks = P.chunk_off[R.B];

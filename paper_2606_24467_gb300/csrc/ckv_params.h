@@ -247,6 +247,7 @@ struct ResidentParams {
   int* unit_ctr;               // per unit: chunks scored; ticket of its second round; pieces pooled;
                                // then the workers' next ticket
   unsigned long long* acc;     // [unit][kAccWords][acc_rows]: the units' sums of exponentials
+  int min_grid;                // CTAs that hold the logits of any unit of the call at once
   int acc_rows;                // row length of the accumulators (a multiple of 32)
   float c;                     // scale * log2(e)
   int window, pool_width, num_kv_heads, group_size, p_total, o_total, is_bf16;

@@ -43,8 +43,11 @@
 // unit of one chunk, of 2^86 in one of 128, or a D below 2^-48 and 2^-27 in
 // these (every logit above about +60 or below about -25).
 //
-// One CTA per SM runs for the whole call (a cooperative launch: the chunks of
-// a unit wait for one another, so all CTAs have to be resident).  Warps:
+// One CTA per SM runs for the whole call.  The chunks of a unit wait for one
+// another, so the CTAs that take part are those that are resident when the call
+// starts (take_part): all, but where another kernel holds SMs for longer than
+// kStartWaitNs.  A unit's sums and scores do not depend on how many they are.
+// Warps:
 //   warp 0      loads each unit's SRH query rows (one TMA box of W rows per
 //               head and 64-column half) into one of two or three Q buffers
 //               and streams the K tiles, by TMA, into a shared-memory ring;
@@ -57,7 +60,7 @@
 //               of pass 2);
 //   warps 8-11  pass 2 (warpgroup 1);
 //   warps 12-19 workers: zero the accumulators when the call starts, then
-//               select and gather the units u = blockIdx, blockIdx + grid...
+//               select and gather the units u = id, id + grid...
 //               as their chunks are scored;
 //   warps 20,22 read the units' complete sums, one unit ahead of pass 2
 //               (alternate units);
@@ -124,20 +127,30 @@ static_assert(kAccMax + 1 == kAccWords, "accumulator words");
 constexpr int kAccE0 = -10;   // sums below 2^kAccE0 share bin 0
 
 // Words of the header's counter block that the two-pass kernel does not use
-// (it zeroes them with its own).  Nothing is reset at the end of a call: the
-// start counter grows by the grid in every call, also in one that stops, and
-// the abort word holds the number of the call that stopped.
+// (it zeroes them with its own).  The last CTA past the start zeroes the
+// start's, also in a call that stops; the number of calls stays, and the abort
+// word holds the number of the call that stopped.
 constexpr int kCtrNever = 6;   // never set: the test hook's stall waits for it
 constexpr int kCtrStop = 8;    // number of the last call in which a wait ran out
-constexpr int kCtrStart = 32;  // (64 bits) CTAs that have zeroed their share, over all calls
+constexpr int kCtrCalls = 9;   // calls so far
+constexpr int kCtrArrive = 32; // CTAs that have started (16 bits); once closed, how many had then
+constexpr int kCtrZeroed = 40; // CTAs taking part that have zeroed their share
+constexpr int kCtrPast = 48;   // CTAs past the start
+constexpr unsigned kClosed = 1u << 31;  // (of kCtrArrive; the 15 bits below: how many take part)
+
+// How long the first CTA waits for the others to start.  A kernel of another
+// stream that ends in this time delays the call by no more than its own time;
+// one that holds SMs for longer leaves the call the others.
+constexpr uint64_t kStartWaitNs = 1000000ull;
 
 constexpr int kModeP1 = 1;    // the chunk's sums of exponentials
 constexpr int kModeP2 = 2;    // the chunk's scores
 
 struct alignas(16) ChunkDesc {
-  int mode, wg, new_q, unit;      // mode 0: no more chunks
+  int mode, wg, new_q, unit;      // mode 0: no more chunks; the unit whose pass 2 is in hand
   int s, g, t0, nt;               // sequence, group, K tiles [t0, t0 + nt)
-  int n_rows, nch, pad0, pad1;    // query rows, chunks of the unit
+  int n_rows, nch;                // query rows, chunks of the unit
+  int tile, sum_unit;             // number of the first tile; the unit that pass 1 adds to
   int n, L, row0, soff;           // prefix, length, first row of K, offset of the scores
   uint32_t bits;                  // SRH heads of the group
   int ct, last_q;                 // tiles per chunk; the Q buffer's last chunk
@@ -176,6 +189,8 @@ struct CallInfo {
   float2* rows;
   uint32_t tbase;
   float c;
+  int id, grid;                    // of this CTA among those that take part (id -1: not one)
+  int ring;                        // chunk sums that each keeps in `pairs`
   int acc_rows, stages, q_bufs, q_half_bytes;
   int window, group_size, is_bf16, given_lse;
   float2* pairs;                   // (M, S) of this CTA's latest chunks, a row each
@@ -199,7 +214,7 @@ struct ResidentShared {
   int sum_pos;                                         // chunks below have left their pairs
   int p2_unit[kPub];
   ChunkDesc descs[kDescs];
-  ListPos list;
+  ListPos list[2];                                     // ([1]: of pass 2 apart from pass 1)
 };
 
 // ... and rows of acc_rows pairs: the chunk sums (M, S) of the four pass-1
@@ -490,7 +505,7 @@ __device__ __noinline__ void p1_slow(ResidentShared& sh, const ChunkDesc& d, int
 __device__ __noinline__ bool slow_denominators(ResidentShared& sh, const ChunkDesc& d, float* out,
                                                int lane) {
   assume_shared(&sh);
-  const int grid = static_cast<int>(gridDim.x);
+  const int grid = sh.call.grid;
   const int nown = (d.x_last - d.x) / grid + 1;
   const int first = d.x / grid;  // this chunk's number among the CTA's
   const int nch = d.nch;
@@ -508,7 +523,7 @@ __device__ __noinline__ bool slow_denominators(ResidentShared& sh, const ChunkDe
     __threadfence_block();
   }
   auto own = [&](int i, int q) -> float2 {
-    return __ldcg(sh.call.pairs + (first + i) % kPairRing * rows + q);
+    return __ldcg(sh.call.pairs + (first + i) % sh.call.ring * rows + q);
   };
 #pragma unroll 1
   for (int q = lane; q < d.n_rows; q += 32) {
@@ -989,7 +1004,8 @@ __device__ __noinline__ void sum_role(ResidentShared& sh, int lane) {
   assume_shared(&sh);
   const CallInfo& p = sh.call;
   const int rows = p.acc_rows;
-  int k1 = 0;  // pass-1 chunks so far
+  int k1 = 0;    // pass-1 chunks so far
+  int slot = 0;  // ... in the ring of their sums
   bool ok = wait_bar(sh, &sh.startbar, 0);
   for (int c = 0; __all_sync(0xffffffffu, ok); ++c) {
     const int ds = c % kDescs;
@@ -1002,8 +1018,8 @@ __device__ __noinline__ void sum_role(ResidentShared& sh, int lane) {
       const Bins B(d.nch);
       const int n_rows = d.n_rows;
       unsigned long long* const acc =
-          p.acc + static_cast<long long>(d.unit) * kAccWords * rows;
-      float2* const keep = p.pairs + k1 % kPairRing * rows;
+          p.acc + static_cast<long long>(d.sum_unit) * kAccWords * rows;
+      float2* const keep = p.pairs + slot * rows;
       const float2* src = pair_row(sh, b * 4);
       ok = wait_all(sh, &sh.p1full[b], static_cast<uint32_t>(k1 >> 1) & 1u);
       if (!ok) break;
@@ -1027,6 +1043,9 @@ __device__ __noinline__ void sum_role(ResidentShared& sh, int lane) {
         *reinterpret_cast<volatile int*>(&sh.sum_pos) = d.x + 1;
       }
       ++k1;
+      slot = slot + 1 == p.ring ? 0 : slot + 1;
+      // (tiles that pass 2 does not read from this copy, at most four: freed here)
+      if (d.mode == kModeP1 && lane < 4 * d.nt) arrive(&sh.tempty[(d.tile + (lane >> 2)) % kTiles]);
     }
     __syncwarp();
     if (lane == 0) arrive(&sh.dempty[ds]);
@@ -1185,6 +1204,122 @@ __device__ __noinline__ void denominator_role(ResidentShared& sh, int mine, int 
   __syncwarp();
 }
 
+// Whether this CTA takes part in the call (one thread, first thing): all do once
+// all have started; when not all have kStartWaitNs after one has, the call is
+// closed to the others, which leave.
+__device__ __forceinline__ void take_part(ResidentShared& sh, int* ctr) {
+  const unsigned all = gridDim.x;
+  unsigned* const word = reinterpret_cast<unsigned*>(ctr + kCtrArrive);
+  const unsigned old = atomicAdd(word, 1u);
+  int id = static_cast<int>(blockIdx.x), grid = static_cast<int>(all);
+  const uint64_t t0 = globaltimer_ns();
+#pragma unroll 1
+  for (unsigned w = old + 1u; w != all; w = static_cast<unsigned>(ld_acquire(ctr + kCtrArrive))) {
+    if (w & kClosed) {
+      id = old & kClosed ? -1 : static_cast<int>(old);
+      grid = static_cast<int>((w >> 16) & 0x7FFFu);
+      break;
+    }
+    if (globaltimer_ns() - t0 > kStartWaitNs) atomicCAS(word, w, kClosed | (w << 16) | w);
+  }
+  sh.call.id = id;
+  sh.call.grid = grid;
+}
+
+// Once every CTA has come here, nothing reads the start's words any more.
+__device__ __forceinline__ void past_start(ResidentShared& sh, int* ctr) {
+  if (atomicAdd(ctr + kCtrPast, 1) == static_cast<int>(gridDim.x) - 1) {
+    ctr[kCtrArrive] = ctr[kCtrZeroed] = ctr[kCtrPast] = 0;
+    ctr[kCtrCalls] = sh.call.number;
+  }
+}
+
+// The list of a CTA's chunks, id, id + grid, ...: what chunk l.x belongs to.
+__device__ __forceinline__ void locate_chunk(const ResidentParams& p, ListPos& l) {
+  if (l.x >= p.n_chunks) return;
+  if (l.x >= l.off_next) {
+    int sq = l.sq, off, off_next = l.off_next;
+#pragma unroll 1
+    do {
+      ++sq;
+      off = off_next;
+      off_next = p.chunk_off[sq + 1];
+    } while (l.x >= off_next);
+    l.sq = sq;
+    l.off = off;
+    l.off_next = off_next;
+    l.row0 = p.cu_seqlens[sq];
+    l.L = p.cu_seqlens[sq + 1] - l.row0;
+    l.nch = (off_next - off) / p.num_kv_heads;
+    l.ct = p.seq_chunk[sq];
+  }
+  const int gr = (l.x - l.off) / l.nch;
+  const int unit = l.sq * p.num_kv_heads + gr;
+  if (unit != l.unit) {
+    l.unit = unit;
+    l.gr = gr;
+    l.unit_end = l.off + (gr + 1) * l.nch;
+    l.bits = p.srh_bits[srh_group(l.sq, gr, p.seqs_per_mask, p.num_kv_heads)];
+    l.n_rows = __popc(l.bits) * p.window;
+    l.width = (l.n_rows + 31) & ~31;
+    l.soff = gr * p.p_total + p.cu_prefix[l.sq];
+  }
+}
+__device__ __forceinline__ void first_chunk(const ResidentParams& p, ListPos& l, int id) {
+  l.x = id;
+  l.sq = l.unit = -1;
+  l.off_next = 0;
+  locate_chunk(p, l);
+}
+// Chunk l.x's descriptor; end: of the last chunk's tensor-memory columns, tile:
+// tiles so far, unit: whose pass 2 is in hand.
+__device__ __forceinline__ void write_chunk(const ResidentParams& p, const ListPos& l, ChunkDesc& d,
+                                            int mode, int wg, int new_q, int grid, int& end,
+                                            int& tile, int& unit) {
+  const int ct = l.ct;
+  const int width = l.width;
+  const int cc = l.x - (l.unit_end - l.nch);
+  const int nt = min(((l.L + kTileTokens - 1) / kTileTokens) - cc * ct, ct);
+  d.new_q = new_q;
+  d.last_q = l.x + grid >= l.unit_end ? 1 : 0;  // this CTA's last chunk of the unit
+  d.mode = mode;
+  d.wg = wg;
+  unit = mode == kModeP1 ? unit : l.unit;
+  d.unit = unit;
+  d.sum_unit = l.unit;
+  d.s = l.sq;
+  d.g = l.gr;
+  d.t0 = cc * ct;
+  d.nt = nt;
+  d.n_rows = l.n_rows;
+  d.nch = l.nch;
+  d.n = l.L - p.window;
+  d.L = l.L;
+  d.row0 = l.row0;
+  d.soff = l.soff;
+  d.bits = l.bits;
+  d.ct = ct;
+  // the chunk's columns: the next multiple of their number, so that
+  // floor(512 / number) chunks of a unit never stand in one another's way
+  const int all = ct * width;
+  int col = (end + all - 1) / all * all;
+  if (col + all > 512) col = 0;
+  end = col + all;
+  d.col = col;
+  d.width = width;
+  d.tile = tile;
+  tile += nt;
+  d.x = l.x;
+  d.x_last = l.x + (l.unit_end - 1 - l.x) / grid * grid;
+}
+// No more chunks: descriptor c.
+__device__ __forceinline__ void write_end(ResidentShared& sh, int c) {
+  const int ds = c % kDescs;
+  wait_bar(sh, &sh.dempty[ds], (static_cast<uint32_t>(c / kDescs) & 1u) ^ 1u);
+  sh.descs[ds].mode = 0;
+  arrive(&sh.dfull[ds]);
+}
+
 template <int kKind>
 __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_constant__ ResidentParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -1202,9 +1337,8 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   constexpr bool kPieces = kKind != kPlain;
-  const int grid = static_cast<int>(gridDim.x);
-  auto p2done = [&](int u) { return p.unit_ctr + u; };
 
+  if (threadIdx.x == kAnnWarp * 32) take_part(sh, p.ctr);
   if (threadIdx.x == 0) {
     auto init = [](uint64_t* b, int n) { mbar_init(smem_u32(b), static_cast<uint32_t>(n)); };
     for (int i = 0; i < nst; ++i) {
@@ -1241,10 +1375,8 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
     sh.call.status = p.status;
     sh.call.sel.status = p.status;
     sh.call.abort_word = p.ctr + kCtrStop;
-    // (this CTA has not added to the start counter yet, so the other CTAs of
-    // this call have not brought it to the next multiple of the grid)
-    sh.call.number = static_cast<int>(
-        ld_relaxed64(reinterpret_cast<unsigned long long*>(p.ctr + kCtrStart)) / gridDim.x + 1ull);
+    // (stays until every CTA is past the start)
+    sh.call.number = ld_volatile(p.ctr + kCtrCalls) + 1;
     sh.call.wait_ns = p.wait_ns;
     sh.call.acc = p.acc;
     sh.call.slow_ticket = p.unit_ctr + p.n_units;
@@ -1267,7 +1399,6 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
     sh.call.is_bf16 = p.is_bf16;
     sh.call.given_lse = p.given_lse;
     sh.call.acc_rows = p.acc_rows;
-    sh.call.pairs = p.pairs + static_cast<long long>(blockIdx.x) * kPairRing * p.acc_rows;
     sh.call.sel.num_kv_heads = p.num_kv_heads;
     sh.call.sel.pool_width = p.pool_width;
     sh.call.sel.raw_scratch = p.raw_scratch;
@@ -1289,97 +1420,86 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = sh.tmem;
-  if (threadIdx.x == 0) sh.call.tbase = tbase;
+  const int id = sh.call.id, grid = sh.call.grid;
+  if (threadIdx.x == 0) {
+    sh.call.tbase = tbase;
+    sh.call.ring = grid == kResidentMaxGrid ? kPairRing : kResidentMaxGrid * kPairRing / grid;
+    sh.call.pairs = p.pairs + static_cast<long long>(id) * sh.call.ring * p.acc_rows;
+  }
   __syncthreads();
 
-  if (warp == kSchedWarp) {
+  if (id < 0) {
+    if (threadIdx.x == 0) past_start(sh, p.ctr);
+  } else if (warp == kSchedWarp) {
     // ------------------------------------------------------------ descriptors
     if (lane == 0) {
       // test hook: a wait that cannot complete, before anything is issued;
       // it runs out after p.wait_ns and stops the call
-      if (p.stall && blockIdx.x == 0) wait_counter(sh, p.ctr + kCtrNever, 1);
-      // this CTA's chunks: blockIdx, blockIdx + grid, ...
-      ListPos& l = sh.list;
-      auto locate = [&]() {
-        if (l.x >= p.n_chunks) return;
-        if (l.x >= l.off_next) {
-          int sq = l.sq, off, off_next = l.off_next;
+      if (p.stall && id == 0) wait_counter(sh, p.ctr + kCtrNever, 1);
+      if (p.given_lse || grid >= p.min_grid) {
+        ListPos& l = sh.list[0];
+        first_chunk(p, l, id);
+        int c = 0, last_unit = -1, end = 0, tile = 0, unit = -1;
 #pragma unroll 1
-          do {
-            ++sq;
-            off = off_next;
-            off_next = p.chunk_off[sq + 1];
-          } while (l.x >= off_next);
-          l.sq = sq;
-          l.off = off;
-          l.off_next = off_next;
-          l.row0 = p.cu_seqlens[sq];
-          l.L = p.cu_seqlens[sq + 1] - l.row0;
-          l.nch = (off_next - off) / p.num_kv_heads;
-          l.ct = p.seq_chunk[sq];
+        for (; l.x < p.n_chunks; ++c) {
+          const int ds = c % kDescs;
+          if (!wait_bar(sh, &sh.dempty[ds], (static_cast<uint32_t>(c / kDescs) & 1u) ^ 1u)) break;
+          const int new_q = l.unit != last_unit ? 1 : 0;
+          last_unit = l.unit;
+          write_chunk(p, l, sh.descs[ds], p.given_lse ? kModeP2 : kModeP1 | kModeP2,
+                      p.given_lse ? (c & 1) : 1, new_q, grid, end, tile, unit);
+          arrive(&sh.dfull[ds]);
+          l.x += grid;
+          locate_chunk(p, l);
         }
-        const int gr = (l.x - l.off) / l.nch;
-        const int unit = l.sq * p.num_kv_heads + gr;
-        if (unit != l.unit) {
-          l.unit = unit;
-          l.gr = gr;
-          l.unit_end = l.off + (gr + 1) * l.nch;
-          l.bits = p.srh_bits[srh_group(l.sq, gr, p.seqs_per_mask, p.num_kv_heads)];
-          l.n_rows = __popc(l.bits) * p.window;
-          l.width = (l.n_rows + 31) & ~31;
-          l.soff = gr * p.p_total + p.cu_prefix[l.sq];
-        }
-      };
-      l.x = blockIdx.x;
-      l.sq = l.unit = -1;
-      l.off_next = 0;
-      locate();
-      int c = 0, last_unit = -1;
-      int end = 0;  // end of the last chunk's tensor-memory columns
+        write_end(sh, c);
+      } else {
+        // Too few CTAs for a unit's logits to be in tensor memory all at once:
+        // its chunks go through pass 1 alone and, after the next unit's pass 1,
+        // through pass 2 with K read again.  (The same sums of the same chunks:
+        // the same bits.  A loop of its own: the two as one cost 1%, this one as
+        // a function 3-6%.)
+        ListPos* l = sh.list;
+        first_chunk(p, sh.list[0], id);
+        first_chunk(p, sh.list[1], id);
+        int mode = kModeP1;
+        int run = l->x < p.n_chunks ? l->unit : -1;  // the unit in hand
+        int prev = -1;                               // and the one before, pass 2 to come
+        int c = 0, last_unit = -1, end = 0, tile = 0, unit = -1;
 #pragma unroll 1
-      for (; l.x < p.n_chunks; ++c) {
-        const int ds = c % kDescs;
-        if (!wait_bar(sh, &sh.dempty[ds], (static_cast<uint32_t>(c / kDescs) & 1u) ^ 1u)) break;
-        ChunkDesc& d = sh.descs[ds];
-        const int ct = l.ct;
-        const int width = l.width;
-        const int cc = l.x - (l.unit_end - l.nch);
-        d.new_q = l.unit != last_unit ? 1 : 0;
-        last_unit = l.unit;
-        d.last_q = l.x + grid >= l.unit_end ? 1 : 0;  // this CTA's last chunk of the unit
-        d.mode = p.given_lse ? kModeP2 : kModeP1 | kModeP2;
-        d.wg = p.given_lse ? (c & 1) : 1;
-        d.unit = l.unit;
-        d.s = l.sq;
-        d.g = l.gr;
-        d.t0 = cc * ct;
-        d.nt = min(((l.L + kTileTokens - 1) / kTileTokens) - cc * ct, ct);
-        d.n_rows = l.n_rows;
-        d.nch = l.nch;
-        d.n = l.L - p.window;
-        d.L = l.L;
-        d.row0 = l.row0;
-        d.soff = l.soff;
-        d.bits = l.bits;
-        d.ct = ct;
-        // the chunk's columns: the next multiple of their number, so that
-        // floor(512 / number) chunks of a unit never stand in one another's way
-        const int all = ct * width;
-        int col = (end + all - 1) / all * all;
-        if (col + all > 512) col = 0;
-        end = col + all;
-        d.col = col;
-        d.width = width;
-        d.x = l.x;
-        d.x_last = l.x + (l.unit_end - 1 - l.x) / grid * grid;
-        arrive(&sh.dfull[ds]);
-        l.x += grid;
-        locate();
+        for (;;) {
+          if (l->x >= p.n_chunks || l->unit != run) {
+            const int next = sh.list[0].x < p.n_chunks ? sh.list[0].unit : -1;
+            if (mode == kModeP2) {
+              if (prev < 0) break;
+              mode = kModeP1;
+              run = next;
+            } else if (prev >= 0) {
+              mode = kModeP2;
+              const int u = run;
+              run = prev;
+              prev = u;
+            } else {
+              prev = run;
+              if (prev < 0) break;
+              run = next;
+            }
+            l = sh.list + (mode == kModeP2 ? 1 : 0);
+            last_unit = -1;
+            continue;
+          }
+          const int ds = c % kDescs;
+          if (!wait_bar(sh, &sh.dempty[ds], (static_cast<uint32_t>(c / kDescs) & 1u) ^ 1u)) break;
+          const int new_q = l->unit != last_unit ? 1 : 0;
+          last_unit = l->unit;
+          write_chunk(p, *l, sh.descs[ds], mode, 1, new_q, grid, end, tile, unit);
+          arrive(&sh.dfull[ds]);
+          l->x += grid;
+          locate_chunk(p, *l);
+          ++c;
+        }
+        write_end(sh, c);
       }
-      const int ds = c % kDescs;
-      wait_bar(sh, &sh.dempty[ds], (static_cast<uint32_t>(c / kDescs) & 1u) ^ 1u);
-      sh.descs[ds].mode = 0;
-      arrive(&sh.dfull[ds]);
     }
     __syncwarp();
   } else if (warp == kProdWarp) {
@@ -1397,7 +1517,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
       pass1_role(sh, warp, lane);
     }
   } else if (warp == kAnnWarp) {
-    announce_role(sh, p2done(0), lane);
+    announce_role(sh, p.unit_ctr, lane);
   } else if (warp == kDenWarp || warp == kDenWarp2) {
     denominator_role(sh, warp == kDenWarp ? 0 : 1, lane);
   } else {
@@ -1405,7 +1525,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
     const int ct = threadIdx.x - kCWarp0 * 32;
     {
       // this CTA's share of the accumulators and counters
-      const long long who = static_cast<long long>(blockIdx.x) * kCThreads + ct;
+      const long long who = static_cast<long long>(id) * kCThreads + ct;
       const long long all = static_cast<long long>(grid) * kCThreads;
       if (!p.given_lse) {
         uint4* a = reinterpret_cast<uint4*>(p.acc);
@@ -1417,24 +1537,20 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
       cbar();
       if (ct == 0) {
         __threadfence();
-        // every call adds `grid` to the counter: it is a multiple of it
-        // before the call's first arrival
-        unsigned long long* const start_ctr =
-            reinterpret_cast<unsigned long long*>(p.ctr + kCtrStart);
-        const unsigned long long old = atomicAdd(start_ctr, 1ull);
-        const unsigned long long target = (old / grid + 1ull) * grid;
+        atomicAdd(p.ctr + kCtrZeroed, 1);
         const uint64_t t0 = globaltimer_ns();
-        while (ld_acquire64(start_ctr) < target && still_waiting(sh, t0)) {
+        while (ld_acquire(p.ctr + kCtrZeroed) < grid && still_waiting(sh, t0)) {
         }
         arrive(&sh.startbar);
+        past_start(sh, p.ctr);
       }
     }
 #pragma unroll 1
-    for (int u = blockIdx.x; !kPieces && p.do_select && u < p.n_units; u += grid) {
+    for (int u = id; !kPieces && p.do_select && u < p.n_units; u += grid) {
       const int s = u / p.num_kv_heads;
       const int g = u - s * p.num_kv_heads;
       const int nch = (p.chunk_off[s + 1] - p.chunk_off[s]) / p.num_kv_heads;
-      if (ct == 0) sh.task = wait_counter(sh, p2done(u), nch) ? 1 : 0;
+      if (ct == 0) sh.task = wait_counter(sh, p.unit_ctr + u, nch) ? 1 : 0;
       cbar();
       const int go = sh.task;
       cbar();
@@ -1532,12 +1648,8 @@ cudaError_t launch_resident(const ResidentParams& p, int grid, size_t smem, cuda
   cfg.blockDim = dim3(kRThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  // the CTAs wait for one another's sums: all of them must be resident
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.attrs = nullptr;
+  cfg.numAttrs = 0;
   return cudaLaunchKernelEx(&cfg,
                             p.mixed       ? resident_kernel<kMixed>
                             : p.in_pieces ? resident_kernel<kInPieces>
