@@ -136,12 +136,15 @@ constexpr int kCtrCalls = 9;   // calls so far
 constexpr int kCtrArrive = 32; // CTAs that have started (16 bits); once closed, how many had then
 constexpr int kCtrZeroed = 40; // CTAs taking part that have zeroed their share
 constexpr int kCtrPast = 48;   // CTAs past the start
-constexpr unsigned kClosed = 1u << 31;  // (of kCtrArrive; the 15 bits below: how many take part)
+constexpr int kCtrSlots = 56;  // (5 words) numbers given by number_by_sm
+constexpr unsigned kClosed = 1u << 31;  // (of kCtrArrive; the 14 bits below kApart: how many take part)
+constexpr unsigned kApart = 1u << 30;   // the CTAs did not start together
 
 // How long the first CTA waits for the others to start.  A kernel of another
 // stream that ends in this time delays the call by no more than its own time;
 // one that holds SMs for longer leaves the call the others.
 constexpr uint64_t kStartWaitNs = 1000000ull;
+constexpr uint64_t kStartApartNs = 8000ull;  // (together: within 2 us)
 
 constexpr int kModeP1 = 1;    // the chunk's sums of exponentials
 constexpr int kModeP2 = 2;    // the chunk's scores
@@ -1204,6 +1207,24 @@ __device__ __noinline__ void denominator_role(ResidentShared& sh, int mine, int 
   __syncwarp();
 }
 
+// A number of its own for every CTA, by the SM it is on: neighbours on one TPC
+// get neighbouring numbers, as in a launch on an idle GPU (chunks of a unit on
+// SMs far apart, as CTAs that start one by one behind another kernel have them,
+// cost 5 to 20%).  A slot taken already (an SM's number may change) goes on to
+// the next free one.
+__device__ __noinline__ int number_by_sm(int* ctr) {
+  uint32_t sm;
+  asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+  const uint32_t all = gridDim.x;
+  sm %= all;
+#pragma unroll 1
+  for (;; sm = sm + 1 == all ? 0 : sm + 1) {
+    const uint32_t bit = 1u << (sm & 31u);
+    if (!(atomicOr(reinterpret_cast<unsigned*>(ctr + kCtrSlots) + (sm >> 5), bit) & bit))
+      return static_cast<int>(sm);
+  }
+}
+
 // Whether this CTA takes part in the call (one thread, first thing): all do once
 // all have started; when not all have kStartWaitNs after one has, the call is
 // closed to the others, which leave.
@@ -1216,11 +1237,21 @@ __device__ __forceinline__ void take_part(ResidentShared& sh, int* ctr) {
 #pragma unroll 1
   for (unsigned w = old + 1u; w != all; w = static_cast<unsigned>(ld_acquire(ctr + kCtrArrive))) {
     if (w & kClosed) {
-      id = old & kClosed ? -1 : static_cast<int>(old);
-      grid = static_cast<int>((w >> 16) & 0x7FFFu);
+      id = old & kClosed ? -1 : static_cast<int>(old & 0xFFFFu);
+      grid = static_cast<int>((w >> 16) & 0x3FFFu);
       break;
     }
-    if (globaltimer_ns() - t0 > kStartWaitNs) atomicCAS(word, w, kClosed | (w << 16) | w);
+    const unsigned n = w & 0xFFFFu;
+    if (n == all) {  // kApart
+      id = number_by_sm(ctr);
+      break;
+    }
+    const uint64_t t = globaltimer_ns() - t0;
+    if (t > kStartWaitNs) {
+      atomicCAS(word, w, kClosed | (n << 16) | n);
+    } else if (t > kStartApartNs && !(w & kApart)) {
+      atomicCAS(word, w, w | kApart);
+    }
   }
   sh.call.id = id;
   sh.call.grid = grid;
@@ -1230,6 +1261,7 @@ __device__ __forceinline__ void take_part(ResidentShared& sh, int* ctr) {
 __device__ __forceinline__ void past_start(ResidentShared& sh, int* ctr) {
   if (atomicAdd(ctr + kCtrPast, 1) == static_cast<int>(gridDim.x) - 1) {
     ctr[kCtrArrive] = ctr[kCtrZeroed] = ctr[kCtrPast] = 0;
+    for (int i = 0; i < (kResidentMaxGrid + 31) / 32; ++i) ctr[kCtrSlots + i] = 0;
     ctr[kCtrCalls] = sh.call.number;
   }
 }
