@@ -1,29 +1,25 @@
-"""A host model of the persistent kernel's in-CTA barrier protocol, run under
-random interleavings (no GPU).
+"""A host model of the two-pass persistent kernel's in-CTA barrier protocol, run
+under random interleavings (no GPU).
 
-The model follows the kernel's roles and mbarriers: the claimer's
-descriptor ring and publish ring, the producer's Q buffers and K stages, two
-UMMA warps (one per epilogue warpgroup, tile t of a chunk to warp t % 2) with
-their TMEM buffers, and eight epilogue warps with their warpgroup and
-all-warp syncs.  Barriers keep an arrival count, a transaction count and a
-phase; a wait on parity P passes when P differs from the parity of the
-current phase (the PTX rule), so a waiter that falls two phases behind -- or
-runs two ahead -- is misled.  TMA copies and UMMA completions are
-asynchronous events.  The model checks that no barrier gets more arrivals
-than its count allows and that every role finishes.
-
-It pins the K-ring layout: with one shared ring (stage = tile % stages), a
-UMMA warp that skipped the other warp's tiles at an odd-sized chunk can wait
-on a stage whose previous fill has not landed and take that older phase for
-its own -- which the model finds; with one sub-ring per UMMA warp (the
-kernel's layout) it finds nothing.
+The model follows the kernel's roles and mbarriers: the claimer's descriptor
+ring and publish ring, the producer's Q buffers and K stages (one ring in tile
+order, of any number of stages), one UMMA warp, each epilogue warpgroup's TMEM
+buffers (tile t of a chunk belongs to warpgroup t % 2), and eight epilogue
+warps with their warpgroup syncs.  Barriers keep an arrival count, a
+transaction count and a phase; a wait on parity P passes when P differs from
+the parity of the current phase (the PTX rule), so a waiter that falls two
+phases behind -- or runs two ahead -- is misled.  TMA copies and UMMA
+completions are asynchronous events.  The model checks that no barrier gets
+more arrivals than its count allows, that every UMMA finds its tile and its
+chunk's queries, that every epilogue warp finds its tile's logits, and that
+every role finishes.
 """
 import random
 
 import pytest
 
 
-class _Bar:
+class Bar:
     def __init__(self, name, count):
         self.name, self.count = name, count
         self.pending, self.tx, self.phase = count, 0, 0
@@ -50,12 +46,59 @@ class _Bar:
         return parity != (self.phase & 1)
 
 
-def _simulate(seed, stages, q_bufs, bufs_per_wg, sub_rings, n_chunks=30, pub=6, descs=4):
-    rng = random.Random(seed)
-    bars = {}
+class Sim:
+    """Roles (generators that yield a condition to wait for, or None) and
+    timed events, interleaved at random."""
+
+    def __init__(self, seed):
+        self.rng = random.Random(seed)
+        self.clock, self.events, self.order = 0, [], 0
+
+    def at(self, time, fn):
+        self.order += 1
+        self.events.append((time, self.order, fn))
+
+    def after(self, fn, lo=1, hi=30):
+        self.at(self.clock + self.rng.randint(lo, hi), fn)
+
+    def run(self, roles, limit=1_000_000):
+        state = {n: None for n in roles}  # the condition each waits for
+        names = sorted(roles)
+        for _ in range(limit):
+            if not names and not self.events:
+                return
+            ready = ()
+            if names and (not self.events or self.rng.random() < 0.8):
+                ready = (self.rng.choice(names),)
+                if not self._ready(state[ready[0]]):
+                    ready = () if self.events else [n for n in names if self._ready(state[n])]
+                    if not ready and not self.events:
+                        raise AssertionError(f"deadlock: {names}")
+            if ready:
+                n = self.rng.choice(ready)
+                try:
+                    state[n] = next(roles[n])
+                except StopIteration:
+                    names.remove(n)
+            elif self.events and (not names or self.rng.random() < 0.5
+                                  or not any(self._ready(state[n]) for n in names)):
+                event = min(self.events, key=lambda e: e[:2])
+                self.events.remove(event)
+                self.clock = max(self.clock, event[0])
+                event[2]()
+        raise AssertionError("no progress (spinning roles only)")
+
+    @staticmethod
+    def _ready(condition):
+        return condition is None or condition()
+
+
+def _simulate(seed, stages, q_bufs, bufs_per_wg, n_chunks=30, pub=6, descs=2, forget=None):
+    sim = Sim(seed)
+    rng, bars = sim.rng, {}
 
     def mk(name, count):
-        bars[name] = _Bar(name, count)
+        bars[name] = Bar(name, count)
 
     for i in range(stages):
         mk(f"full{i}", 1)
@@ -65,27 +108,22 @@ def _simulate(seed, stages, q_bufs, bufs_per_wg, sub_rings, n_chunks=30, pub=6, 
         mk(f"tempty{b}", 4)
     for i in range(descs):
         mk(f"dfull{i}", 1)
-        mk(f"dempty{i}", 3 + 8)
+        mk(f"dempty{i}", 2 + 8)
     for i in range(q_bufs):
         mk(f"qfull{i}", 1)
-        mk(f"qempty{i}", 2)
+        mk(f"qempty{i}", 1)
     for w in range(2):
         mk(f"wg{w}", 4)
-    mk("epi", 8)
     for i in range(pub):
         mk(f"pubfull{i}", 8)
         mk(f"pubempty{i}", 1)
     # chunks: (pass, tiles), with the short and odd-sized ones of ragged units
     chunks = [(rng.choice((1, 2)), rng.choice((1, 1, 2, 3, 5, 7, 16, 16))) for _ in range(n_chunks)]
     ring = [None] * descs
-    events = []
-    clock = [0]
-
-    def after(fn, lo=1, hi=30, at=None):
-        events.append((clock[0] + rng.randint(lo, hi) if at is None else at, fn))
+    k_stage, q_buf, tmem = [None] * stages, [None] * q_bufs, [None] * (2 * bufs_per_wg)
 
     def wait(name, parity):
-        return ("wait", name, parity)
+        return lambda: bars[name].passes(parity)
 
     def claimer():
         issued = nxt = 0
@@ -100,25 +138,20 @@ def _simulate(seed, stages, q_bufs, bufs_per_wg, sub_rings, n_chunks=30, pub=6, 
             ds = c % descs
             while not bars[f"dempty{ds}"].passes(((c // descs) & 1) ^ 1):
                 pump()
-                yield ("spin",)
+                yield None
             while issued - nxt > pub - 1:
                 pump()
-                yield ("spin",)
-            ring[ds] = None if c == n_chunks else chunks[c]
+                yield None
+            ring[ds] = None if c == n_chunks else (c, *chunks[c])
             issued += c < n_chunks
             bars[f"dfull{ds}"].arrive()
-            yield ("spin",)
+            yield None
         while nxt < issued:
             pump()
-            yield ("spin",)
-
-    def stage_of(w, slot):
-        return w + 2 * slot if sub_rings else slot
+            yield None
 
     def producer():
-        slot, ph = [0, 0], [0, 0]
-        shared_slot, shared_ph = 0, 0
-        qb = qph = 0
+        st = ph = qb = qph = 0
         for c in range(n_chunks + 1):
             ds = c % descs
             yield wait(f"dfull{ds}", (c // descs) & 1)
@@ -128,29 +161,29 @@ def _simulate(seed, stages, q_bufs, bufs_per_wg, sub_rings, n_chunks=30, pub=6, 
                 return
             yield wait(f"qempty{qb}", qph ^ 1)
             bars[f"qfull{qb}"].arrive(tx=1)
-            after(lambda q=qb: bars[f"qfull{q}"].land())
-            qb, qph = (0, qph ^ 1) if qb + 1 == q_bufs else (qb + 1, qph)
-            for t in range(d[1]):
-                w = t & 1
-                if sub_rings:
-                    st, p = stage_of(w, slot[w]), ph[w]
-                else:
-                    st, p = shared_slot, shared_ph
-                yield wait(f"empty{st}", p ^ 1)
-                bars[f"full{st}"].arrive(tx=1)
-                after(lambda s=st: bars[f"full{s}"].land())
-                if sub_rings:
-                    slot[w] += 1
-                    if slot[w] == stages // 2:
-                        slot[w], ph[w] = 0, ph[w] ^ 1
-                else:
-                    shared_slot += 1
-                    if shared_slot == stages:
-                        shared_slot, shared_ph = 0, shared_ph ^ 1
 
-    def mma(mw):
-        slot = ph = qb = qph = used = 0
-        busy_until = 0
+            def q_lands(q=qb, c=c):
+                q_buf[q] = c
+                bars[f"qfull{q}"].land()
+
+            sim.after(q_lands)
+            qb, qph = (0, qph ^ 1) if qb + 1 == q_bufs else (qb + 1, qph)
+            for t in range(d[2]):
+                if forget != "empty":
+                    yield wait(f"empty{st}", ph ^ 1)
+                bars[f"full{st}"].arrive(tx=1)
+
+                def lands(s=st, tile=(c, t)):
+                    k_stage[s] = tile
+                    bars[f"full{s}"].land()
+
+                sim.after(lands)
+                st, ph = (0, ph ^ 1) if st + 1 == stages else (st + 1, ph)
+
+    def mma():
+        st = ph = qb = qph = 0
+        used = [0, 0]
+        busy = 0
         for c in range(n_chunks + 1):
             ds = c % descs
             yield wait(f"dfull{ds}", (c // descs) & 1)
@@ -159,29 +192,30 @@ def _simulate(seed, stages, q_bufs, bufs_per_wg, sub_rings, n_chunks=30, pub=6, 
             if d is None:
                 return
             yield wait(f"qfull{qb}", qph)
-            for t in range(d[1]):
-                if (t & 1) != mw:
-                    if not sub_rings:  # the shared ring advances for every tile
-                        slot += 1
-                        if slot == stages:
-                            slot, ph = 0, ph ^ 1
-                    continue
-                b = mw + 2 * (used % bufs_per_wg)
-                yield wait(f"tempty{b}", ((used // bufs_per_wg) & 1) ^ 1)
-                used += 1
-                st = stage_of(mw, slot)
+            for t in range(d[2]):
+                w = t & 1
+                k = used[w]
+                used[w] += 1
+                b = w + 2 * (k % bufs_per_wg)
+                if forget != "tempty":
+                    yield wait(f"tempty{b}", ((k // bufs_per_wg) & 1) ^ 1)
                 yield wait(f"full{st}", ph)
-                busy_until = max(clock[0], busy_until) + rng.randint(1, 10)
-                after(lambda s=st: bars[f"empty{s}"].arrive(), at=busy_until)
-                after(lambda x=b: bars[f"tfull{x}"].arrive(), at=busy_until)
-                slot += 1
-                if slot == (stages // 2 if sub_rings else stages):
-                    slot, ph = 0, ph ^ 1
-            after(lambda q=qb: bars[f"qempty{q}"].arrive(), at=max(clock[0], busy_until) + 1)
+                busy = max(sim.clock, busy) + rng.randint(1, 10)
+
+                def done(s=st, x=b, q=qb, tile=(c, t)):
+                    assert k_stage[s] == tile, "another tile in the K stage"
+                    assert q_buf[q] == tile[0], "another chunk's queries"
+                    tmem[x] = tile
+                    bars[f"tfull{x}"].arrive()
+                    bars[f"empty{s}"].arrive()
+
+                sim.at(busy, done)
+                st, ph = (0, ph ^ 1) if st + 1 == stages else (st + 1, ph)
+            sim.at(max(sim.clock, busy) + 1, lambda q=qb: bars[f"qempty{q}"].arrive())
             qb, qph = (0, qph ^ 1) if qb + 1 == q_bufs else (qb + 1, qph)
 
     def epilogue(wg):
-        used = syncs = syncs8 = 0
+        used = syncs = 0
         for ci in range(n_chunks + 1):
             ds = ci % descs
             yield wait(f"dfull{ds}", (ci // descs) & 1)
@@ -189,67 +223,43 @@ def _simulate(seed, stages, q_bufs, bufs_per_wg, sub_rings, n_chunks=30, pub=6, 
             bars[f"dempty{ds}"].arrive()
             if d is None:
                 return
-            for _ in range(wg, d[1], 2):
+            for t in range(wg, d[2], 2):
                 b = wg + 2 * (used % bufs_per_wg)
                 yield wait(f"tfull{b}", (used // bufs_per_wg) & 1)
                 used += 1
-                yield ("spin",)
+                yield None
+                assert tmem[b] == (ci, t), "another tile's logits"
                 bars[f"tempty{b}"].arrive()
-            if d[0] == 1:  # pass 1: two warpgroup syncs
+            if d[1] == 1:  # pass 1: two warpgroup syncs
                 for _ in range(2):
                     bars[f"wg{wg}"].arrive()
                     yield wait(f"wg{wg}", syncs & 1)
                     syncs += 1
-            else:  # pass 2: one all-epilogue sync
-                bars["epi"].arrive()
-                yield wait("epi", syncs8 & 1)
-                syncs8 += 1
             if ci >= pub:
                 yield wait(f"pubempty{ci % pub}", (ci // pub - 1) & 1)
             bars[f"pubfull{ci % pub}"].arrive()
 
-    roles = {"claimer": claimer(), "producer": producer(), "mma0": mma(0), "mma1": mma(1)}
+    roles = {"claimer": claimer(), "producer": producer(), "mma": mma()}
     for wg in range(2):
         for w in range(4):
             roles[f"epi{wg}.{w}"] = epilogue(wg)
-    state = dict.fromkeys(roles)
-    alive = set(roles)
-    for _ in range(400_000):
-        if not alive and not events:
-            return True
-        runnable = [n for n in alive if state[n] is None or state[n][0] == "spin" or
-                    bars[state[n][1]].passes(state[n][2])]
-        if runnable and (not events or rng.random() < 0.7):
-            n = rng.choice(sorted(runnable))
-            try:
-                state[n] = next(roles[n])
-            except StopIteration:
-                alive.discard(n)
-        elif events:
-            events.sort(key=lambda e: e[0])
-            t, fn = events.pop(0)
-            clock[0] = max(clock[0], t)
-            fn()
-        else:
-            raise AssertionError(f"deadlock: {sorted((n, state[n]) for n in alive)}")
-    raise AssertionError("no progress (spinning roles only)")
+    sim.run(roles)
 
 
-@pytest.mark.parametrize("stages,q_bufs,bufs_per_wg,descs", [(2, 2, 4, 2), (4, 2, 4, 2), (4, 3, 2, 2),
-                                                             (8, 2, 1, 2), (6, 3, 4, 2), (4, 2, 4, 4),
-                                                             (2, 3, 2, 4)])
-def test_sub_rings_survive_random_interleavings(stages, q_bufs, bufs_per_wg, descs):
-    for seed in range(25):
-        assert _simulate(seed, stages, q_bufs, bufs_per_wg, sub_rings=True, descs=descs)
+@pytest.mark.parametrize("stages,q_bufs,bufs_per_wg", [(2, 2, 1), (3, 2, 2), (4, 2, 2), (5, 3, 4),
+                                                       (4, 3, 4), (8, 3, 4), (7, 2, 1)])
+def test_roles_survive_random_interleavings(stages, q_bufs, bufs_per_wg):
+    for seed in range(20):
+        _simulate(seed, stages, q_bufs, bufs_per_wg)
 
 
-def test_shared_ring_with_two_issuers_is_caught():
-    """The layout the kernel does not use: one ring shared by the two UMMA
-    warps.  Some interleaving breaks it (an over-arrived barrier, a deadlock
-    or a role spinning for ever)."""
-    for seed in range(200):
+@pytest.mark.parametrize("forget", ["empty", "tempty"])
+def test_a_forgotten_wait_is_caught(forget):
+    """Planted in the model: the producer or the UMMA warp does not wait for
+    what it overwrites."""
+    for seed in range(50):
         try:
-            _simulate(seed, 3, 2, 4, sub_rings=False)
+            _simulate(seed, 3, 2, 2, forget=forget)
         except AssertionError:
             return
-    raise AssertionError("the shared ring survived every interleaving")
+    raise AssertionError("the forgotten wait went unnoticed")
