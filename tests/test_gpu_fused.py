@@ -1,11 +1,11 @@
-"""The persistent per-group kernel of compresskv_compress_layers against the
+"""The persistent per-group kernels of compresskv_compress_layers against the
 float64 oracle, through the C ABI (needs a GB300).
 
 Besides parity with the oracle (tolerances as in test_gpu_parity.py), the
-kernel's scores depend only on the unit itself: its softmax statistics
-restart on a fixed grid of 16-tile chunks of every unit and each tile of that
-grid always goes to the same epilogue warpgroup, so a layer compressed alone
-and the same layer inside a larger call give identical bits.
+kernels' scores depend only on the layer itself, so a layer compressed alone
+and the same layer inside a larger call give identical bits.  Most lengths here
+are short enough for the resident kernel; test_gpu_two_pass.py has the same
+kinds of calls beyond its line.
 """
 import numpy as np
 import pytest
@@ -144,9 +144,8 @@ def test_repeat_call_is_bit_identical(cuda_device):
 
 def test_full_32_layer_llama8b_32k_in_one_call(cuda_device):
     """The benchmark step itself: all 32 layers of the L=32K Llama-3.1-8B
-    workload in one call (256 units of 16 chunks each, more units than CTAs,
-    so pass-2 chunks wait for merges of units spread over many CTAs).  The
-    first and last layers
+    workload in one call (256 units of 64 chunks each, more units than
+    CTAs).  The first and last layers
     are checked against the oracle unit by unit."""
     dev = cuda_device
     cfg = wl.get("c2")
@@ -157,7 +156,8 @@ def test_full_32_layer_llama8b_32k_in_one_call(cuda_device):
 
 
 def test_bounded_wait_runs_out_and_the_workspace_recovers(cuda_device):
-    """The failure path of the persistent kernel: a wait that cannot complete
+    """The failure path of the resident kernel (of the two-pass one: in
+    test_gpu_two_pass.py): a wait that cannot complete
     (the test hook's counter, before anything is issued) runs out after 2 ms;
     the call returns, every CTA stops, the device status reads
     CKV_ERR_DEVICE_TIMEOUT and, after workspace_init, the same call on the
@@ -191,8 +191,7 @@ def test_bounded_wait_runs_out_and_the_workspace_recovers(cuda_device):
 def test_ragged_odd_chunks_repeated_calls(cuda_device):
     """A Qwen-shaped (7 query heads per group, 4 KV heads) ragged batch over
     several layers, lengths chosen so that many units end in chunks of one or
-    an odd number of K tiles (the two UMMA warps then take unequal shares),
-    compressed repeatedly on one workspace: every call leaves a clean device
+    an odd number of K tiles, compressed repeatedly on one workspace: every call leaves a clean device
     status and the same bits, and one layer matches the oracle."""
     dev = cuda_device
     lens = [2048 * 3 + 128, 2048 + 128 * 5, 128 * 3 + 40, 2048 * 2 + 1, 8000, 128 + 33]
@@ -222,8 +221,8 @@ def test_ragged_odd_chunks_repeated_calls(cuda_device):
 def test_wide_groups_in_a_call_of_many_masks(cuda_device):
     """Six layers of a Llama-70B-shaped problem (8 query heads per group,
     W = 64) with three SRH heads in every group: 192 query rows per unit, the
-    most the persistent kernel's shared memory takes with two Q buffers and a
-    K stage per UMMA warp.  More masks than the separate path takes in one
+    most the persistent kernels' shared memory takes with two Q buffers and two
+    K stages.  More masks than the separate path takes in one
     call, so the call must run in the persistent kernel."""
     dev = cuda_device
     lens = [3000, 2048 + 77]

@@ -130,11 +130,13 @@ def test_exact_ties_break_to_lower_position(cuda_device):
 
 
 def test_selection_full_search_paths(cuda_device):
-    """The fused call's selection lists the keys at or above a sampled lower
-    bound and falls back to a search over all of a unit's keys when that list
-    would exceed 4096 keys.  Equal keys at L = 10000 (about 10000 tied
-    candidates) and a budget of 9000 at L = 12000 take the fallback; both must
-    still equal the oracle (ties to the lowest interior positions)."""
+    """The fused call's selection lists the keys at or above a lower bound (the
+    k-th largest maximum of a group of keys, or a rank among samples) and falls
+    back to a search over all of a unit's keys when that list would exceed 3072
+    keys.  Equal keys at L = 10000 (about 10000 tied candidates) and a budget
+    of 9000 at L = 12000 take the fallback; both must still equal the oracle
+    (ties to the lowest interior positions).  (compresskv_select's own search:
+    tests/test_gpu_select.py.)"""
     cfg = wl.get("c1").scaled(seq_len=10000, dtype="bf16")
     d = wl.make_layer(cfg, 0, sinks=False, needle_gain=0.0)
     d["k"][:] = d["k"][0:1]
@@ -152,12 +154,12 @@ def test_selection_full_search_paths(cuda_device):
 
 
 def test_selection_second_sampled_bound(cuda_device):
-    """A unit whose few top keys sit where the selection samples: strong
-    needles at eleven of the sample positions of the first slice (L = 10000,
-    8 units: a cluster of 10 CTAs -- about 80 CTAs per launch --, 1024
-    positions and 25 evenly spaced samples each) make the first sampled
-    bound the 10th needle, so fewer than k = 96 keys reach it and a second,
-    looser bound is taken.  The result must equal the oracle."""
+    """A unit whose few top keys sit close together, where a cluster of 10 CTAs
+    with slices of 1024 positions and 25 evenly spaced samples each would take
+    samples (L = 10000): eleven strong needles in one slice.  The fused call
+    bounds by the maxima of groups of keys, which needles that share no group
+    leave tight; the cluster select's second bound on such scores is in
+    tests/test_gpu_select.py.  The result must equal the oracle."""
     cfg = wl.get("c1").scaled(seq_len=10000, dtype="bf16")
     d = wl.make_layer(cfg, 0, sinks=False, needle_gain=0.0)
     G = cfg.num_q_heads // cfg.num_kv_heads
