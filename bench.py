@@ -42,7 +42,8 @@ PROFILE_TRAFFIC = os.path.join(ROOT, "profiles", "resident_llama8b_L32k.md")
 # the timed kernel's own sources: a committed traffic figure is shown only
 # while they match
 KERNEL_SOURCES = ["paper_2606_24467_gb300/csrc/" + f
-                  for f in ("resident_kernel.cu", "unit_select.cuh", "tile_math.cuh")]
+                  for f in ("resident_kernel.cu", "unit_select.cuh", "tile_math.cuh",
+                            "select_common.cuh", "ckv_device.cuh")]
 
 
 def parse_args():

@@ -1159,13 +1159,12 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   }
   // Both kernels: three Q buffers when they fit beside a ring of at least four
   // K tiles, else two beside at least two.
-  const int nwg = 2;  // epilogue warpgroups that take tiles (two-pass kernel)
   auto half_bytes = [](int rows) { return ((((rows + 15) & ~15) * 128) + 1023) & ~1023; };
   auto row_stride = [](int rows) { return (rows + 31) & ~31; };
   auto smem_bytes = [&](bool res, int nq, int st) {
     const int rows = res ? r_rows : max_rows;
     return res ? resident_smem_bytes(half_bytes(rows), nq, st, row_stride(rows))
-               : fused_smem_bytes(half_bytes(rows), nq, st, row_stride(rows), nwg);
+               : fused_smem_bytes(half_bytes(rows), nq, st, row_stride(rows));
   };
   int stages[2] = {0, 0}, q_bufs[2] = {0, 0};  // two-pass, resident
   for (int res = 0; res < 2; ++res)
@@ -1271,7 +1270,6 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   // TMEM: 512 columns of accumulator buffers, tstride columns each
   P.tstride = npad_max <= 64 ? 64 : (npad_max <= 128 ? 128 : 256);
   P.nbuf = 512 / P.tstride;
-  P.nwg = nwg;
   if (P.n_chunks == 0 && (!do_select || out == 0)) return CKV_OK;
   return traced(tr, CKV_KERNEL_FUSED, [&] {
     return launch_fused(P, Fd->sms, smem_bytes(false, q_bufs[0], stages[0]), stream);

@@ -143,11 +143,12 @@ struct GatherParams {
 
 // ---------------------------------------------------------------------------
 // Persistent fused layer call (per-group selection of compresskv_compress_layers
-// and compresskv_compress_layers_lse): one kernel streams K for every unit of
-// a call in two passes (softmax statistics, then normalised scores with K
-// re-read from L2), pools, selects and gathers, with work claimed from
-// counters in the workspace.
+// and compresskv_compress_layers_lse), two-pass kernel: it streams K for every
+// unit of its layers in two passes (softmax statistics, then normalised scores
+// from K read again, in long calls mostly from DRAM), pools, selects and
+// gathers, with work claimed from counters in the workspace.
 constexpr int kChunkTiles = 16;         // K tiles per scoring chunk (references restart per chunk)
+constexpr int kFusedPartsPerChunk = 2;  // first-pass pairs per chunk: one per epilogue warpgroup
 constexpr int kFusedMaxSeqs = kMaxBatch;
 constexpr int kFusedMaxLists = 1024;    // (mask, group) SRH lists of one call
 constexpr int kFusedMaxUnits = kMaxBatch * kMaxKvHeads;
@@ -200,7 +201,6 @@ struct FusedParams {
   int row_stride;              // floats per epilogue warp row (>= max query rows, multiple of 32)
   int stages;                  // K tiles in the shared-memory ring
   int tstride, nbuf;           // TMEM columns per accumulator buffer, buffers
-  int nwg;                     // epilogue warpgroups taking tiles (nbuf / nwg buffers each)
   int seqs_per_mask;
   int cu_seqlens[kFusedMaxSeqs + 1];
   int cu_prefix[kFusedMaxSeqs + 1];
@@ -215,8 +215,7 @@ struct FusedParams {
 };
 
 cudaError_t launch_fused(const FusedParams& p, int grid, size_t smem, cudaStream_t s);
-size_t fused_smem_bytes(int q_half_bytes, int q_bufs, int stages, int row_stride, int nwg);
-constexpr int kFusedPartsPerChunk = 4;  // first-pass pairs per chunk (epilogue warpgroups)
+size_t fused_smem_bytes(int q_half_bytes, int q_bufs, int stages, int row_stride);
 cudaError_t fused_set_smem_limit(size_t bytes);
 
 // ---------------------------------------------------------------------------

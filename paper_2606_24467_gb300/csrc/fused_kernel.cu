@@ -39,7 +39,7 @@
 //               their UMMAs, so that both warpgroups' tiles came late and at
 //               the same time, and tensor-memory loads queued behind them.)
 //   warps 4-11  two epilogue warpgroups; tile t of a chunk belongs to
-//               warpgroup t % nwg (nwg = 2), each with its own TMEM buffers;
+//               warpgroup t % 2, each with its own TMEM buffers;
 //   warps 12-19 workers: they merge a unit's pass-1 pairs into its
 //               denominators once all its chunks are in, and select and
 //               gather a unit once all its pass-2 chunks are in (one CTA per
@@ -59,7 +59,7 @@
 // 649 us, 567 and 911 with one logit per register and key-per-lane sums and
 // two UMMA issuers).
 // References restart at every chunk and tile t of a chunk always goes to
-// warpgroup t % nwg, so the scores depend only on the chunk grid (fixed per
+// warpgroup t % 2, so the scores depend only on the chunk grid (fixed per
 // unit), not on which CTA ran a chunk or what else the call holds.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -83,7 +83,7 @@ constexpr int kEpiWarp0 = 4;  // warps 4..11: two warpgroups (TMEM lane quarter 
 constexpr int kEpiWarps = 8;
 constexpr int kCWarp0 = 12;   // warps 12..19
 constexpr int kDescs = 2;     // chunk descriptors in flight (claimed ahead; 2 measured faster than 4)
-constexpr int kNwg = 2;       // epilogue warpgroups that take tiles (tile t of a chunk: t % 2)
+constexpr int kNwg = kFusedPartsPerChunk;  // epilogue warpgroups (tile t of a chunk: t % kNwg)
 constexpr int kPub = 6;       // chunks written, not yet published (publish ring)
 constexpr float kShift = 7.0f;
 constexpr float kRaiseSum = 18446744073709551616.0f;  // 2^64: fp32 column sums stay below it before R is raised
@@ -417,7 +417,7 @@ __device__ void claim_ticket(const Fused& F, TaskPos& T, int* task) {
       const int at = ld_volatile(p.ctr + kCtrMerge);
       const int m = kKind == kMixed ? max(at, first) : at;
       if (m < p.n_units &&
-          ld_acquire(F.ticket(m)) >= p.nwg * F.chunks_per_unit(m / p.num_kv_heads)) {
+          ld_acquire(F.ticket(m)) >= kNwg * F.chunks_per_unit(m / p.num_kv_heads)) {
         if (atomicCAS(p.ctr + kCtrMerge, at, kKind == kMixed ? F.next_merge(m + 1) : m + 1) == at) {
           task[0] = kTaskMerge;
           task[1] = m;
@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
       mbar_init(qfull(i), 1);
       mbar_init(qempty(i), 1);
     }
-    for (int i = 0; i < 4; ++i) mbar_init(wgbar(i), 4);
+    for (int i = 0; i < kNwg; ++i) mbar_init(wgbar(i), 4);
     for (int i = 0; i < kPub; ++i) {
       mbar_init(pubfull(i), kEpiWarps);
       mbar_init(pubempty(i), 1);
@@ -760,9 +760,8 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
     const int qd = warp & 3;  // TMEM lane quarter of this warp
     const int tw = (ew & 3) * 32 + lane;
     constexpr int nwg = kNwg;
-    const bool takes = wg < nwg;  // this warpgroup takes tiles
-    float* ref = sRef + (takes ? ew : 0) * rstride;
-    float* acc_s = sAcc + (takes ? ew : 0) * rstride;
+    float* ref = sRef + ew * rstride;
+    float* acc_s = sAcc + ew * rstride;
     const float c = p.c;
     const uint64_t c2 = pack2(c, c);
     const int bcol = block_col(lane);
@@ -809,7 +808,6 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
         // ---------------------------------------- pass 1: softmax statistics
         // Per query row q the warp keeps a reference R_q and sums
         // 2^(z c - R_q) over its keys, reduced across the lanes every tile.
-        if (!takes) continue;  // warpgroups beyond nwg take no first-pass work
         for (int q = lane; q < N; q += 32) {
           ref[q] = kNegInf;
           acc_s[q] = 0.f;
@@ -937,7 +935,7 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
           for (int q = lane; q < N; q += 32) ref[q] = __ldcg(bias + q);
         }
         __syncwarp();
-        for (int tile = d.t0 + wg; takes && tile < d.t1; tile += nwg) {
+        for (int tile = d.t0 + wg; tile < d.t1; tile += nwg) {
           const int kk = kc++;
           const int b = wg + nwg * (kk & (bpw - 1));
           const uint32_t use = static_cast<uint32_t>(kk >> lbpw) & 1u;
@@ -1055,10 +1053,10 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
 
 }  // namespace
 
-size_t fused_smem_bytes(int q_half_bytes, int q_bufs, int stages, int row_stride, int nwg) {
+size_t fused_smem_bytes(int q_half_bytes, int q_bufs, int stages, int row_stride) {
   return 1024 + static_cast<size_t>(stages) * kTileBytes +
          2 * static_cast<size_t>(q_bufs) * q_half_bytes +
-         2 * static_cast<size_t>(4 * nwg) * row_stride * 4 + kFixedBytes + kSelRegion;
+         2 * static_cast<size_t>(4 * kNwg) * row_stride * 4 + kFixedBytes + kSelRegion;
 }
 
 cudaError_t fused_set_smem_limit(size_t bytes) {
