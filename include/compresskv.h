@@ -253,7 +253,7 @@ int compresskv_compress_layer(const ckv_problem* p, const void* q_win, const voi
  * row's denominator merged, a second pass sums the normalised probabilities
  * from K read again (for long calls mostly from DRAM: the step then moves
  * about twice the bytes of K).  A call with layers of both kinds launches
- * both kernels, one after the other.
+ * both kernels.
  * Neither stores exponentials.  The kernel and the grid of chunks follow from
  * the layer alone, and neither kernel's scores depend on the order in which
  * chunks complete: compressing a layer alone or among others, with a workspace

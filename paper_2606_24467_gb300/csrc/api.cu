@@ -156,6 +156,7 @@ struct Info {
   // the workspace holds neither the resident kernel's area for all units nor the
   // row maxima (a static scratch too small for them)
   bool lean = false;
+  bool one_layer = false;  // known to be one layer: one persistent kernel
   int vgroup(int s, int g) const { return srh_group(s, g, spm, Hkv); }
 };
 
@@ -326,9 +327,11 @@ WorkspaceLayout workspace_layout(const Info& I) {
   return W;
 }
 
-// Layout of the fused call's workspace (after the header; it aliases the
+// Layout of the two-pass kernel's workspace (after the header; it aliases the
 // layout above, which the other entry points use).  A function of the problem
-// alone: rows are bounded with every head of a group counted as SRH.
+// alone: rows are bounded with every head of a group counted as SRH.  In a call
+// that runs both persistent kernels it lies `after` the resident kernel's, with
+// the same scores: the two overlap in time.
 struct FusedLayout {
   size_t raw, pooled, rowmax, partials, bias, total;
   long long n_chunks;
@@ -347,7 +350,7 @@ size_t row_max_bytes(const Info& I) {
                   sizeof(uint32_t));
 }
 
-FusedLayout fused_layout(const Info& I) {
+FusedLayout fused_layout(const Info& I, size_t after = 0) {
   FusedLayout F;
   F.part_stride = (std::min(I.G * I.W, kMaxQRows) + 3) & ~3;
   F.n_chunks = 0;
@@ -356,7 +359,7 @@ FusedLayout fused_layout(const Info& I) {
   const size_t scores = align256(static_cast<size_t>(I.Hkv) * I.p_total * sizeof(float));
   F.raw = kHeaderBytes;
   F.pooled = F.raw + scores;
-  F.partials = F.pooled + scores;
+  F.partials = std::max(F.pooled + scores, after);
   F.bias = F.partials + align256(static_cast<size_t>(F.n_chunks) * kFusedPartsPerChunk *
                                  F.part_stride * sizeof(float2));
   F.rowmax = F.bias + align256(static_cast<size_t>(units) * F.part_stride * sizeof(float));
@@ -392,7 +395,8 @@ size_t base_bytes(const Info& I) {
   lean.lean = true;
   const size_t base = std::max(workspace_layout(I).total, fused_layout(lean).total);
   if (I.lean || (I.layer && !I.pool_max)) return base;
-  return std::max({base, fused_layout(I).total, resident_layout(I, I.B).total});
+  const size_t resident = resident_layout(I, I.B).total;
+  return std::max({base, resident, fused_layout(I, I.B > 1 && !I.one_layer ? resident : 0).total});
 }
 
 // Max pooling: after these layouts, one raw-score row per SRH head slot (at
@@ -966,9 +970,10 @@ int run_gather(const ckv_problem* p, const Info& I, const int32_t* indices,
 // (fused_kernel.cu).  The lines are by the layer's longest prompt and the query
 // rows of its widest group, and by nothing else of the call, so that a layer
 // gives the same bits alone or among others; a call with layers of both kinds
-// launches both, for a second tail (32 layers of 14000 tokens, two of them
-// narrow enough for the resident kernel: 92 + 367 us; four KV heads, three
-// such layers: 81 + 228, all 32 in the two-pass kernel 230).  (The prompts of
+// launches both, the second's CTAs starting where the first's have ended (32
+// layers of 14000 tokens, two of them narrow enough for the resident kernel:
+// 375 us, 449 one after the other, 357 all in the two-pass kernel; four KV
+// heads, three such layers: 245, 306 and 230).  (The prompts of
 // one layer go together: taking a 28-layer batch's shorter prompts apart cost
 // two tails, 3195 -> 3285 us.)
 // Two-pass / resident time in us (1 layer; 32 layers; 8 KV heads):
@@ -1237,7 +1242,7 @@ int run_fused(const ckv_problem* p, const Info& I, const SrhLists& S, const void
   }
   if (!any) return CKV_OK;
 
-  const FusedLayout FL = fused_layout(I);
+  const FusedLayout FL = fused_layout(I, r_any ? resident_layout(I, I.B).total : 0);
   static thread_local FusedParams P;  // large (about 15 KB): kept off the stack
   std::memset(&P, 0, sizeof(P));
   if ((rc = make_k_map(I, p, k, &P.tmap_k)) != CKV_OK) return rc;
@@ -1758,6 +1763,7 @@ extern "C" int compresskv_compress_layer_noalloc(
   Info I;
   int rc = validate(p, I);
   if (rc != CKV_OK) return rc;
+  I.one_layer = true;
   // (many tiny units need more for the resident kernel than without it)
   I.lean = workspace_bytes(I) > static_cast<size_t>(CKV_STATIC_SCRATCH_BYTES);
   if (workspace_bytes(I) > static_cast<size_t>(CKV_STATIC_SCRATCH_BYTES))

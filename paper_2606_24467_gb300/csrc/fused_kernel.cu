@@ -1039,6 +1039,9 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_kernel(const __grid_consta
     tmem_dealloc(tbase, 512);
   }
   if (threadIdx.x == 0) {
+    // (the resident kernel of the same call may still run: its words are among
+    // those zeroed below, and the next kernel waits for this one alone)
+    if (kKind == kMixed) pdl_wait();
     __threadfence();
     *s_last = atomicAdd(p.ctr + kCtrExit, 1) == static_cast<int>(gridDim.x) - 1 ? 1 : 0;
   }
@@ -1074,8 +1077,13 @@ cudaError_t launch_fused(const FusedParams& p, int grid, size_t smem, cudaStream
   cfg.blockDim = dim3(kFThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cfg.attrs = nullptr;
-  cfg.numAttrs = 0;
+  // After the resident kernel of the same call: its CTAs start where that
+  // kernel's have ended (the two share nothing but the call's inputs).
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = p.mixed ? 1 : 0;
   return cudaLaunchKernelEx(&cfg,
                             p.mixed       ? fused_kernel<kMixed>
                             : p.in_pieces ? fused_kernel<kInPieces>

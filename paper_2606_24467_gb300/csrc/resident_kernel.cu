@@ -1460,6 +1460,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(const __grid_con
   }
   __syncthreads();
 
+  if (kKind == kMixed) pdl_launch_dependents();  // the two-pass kernel of the same call
   if (id < 0) {
     if (threadIdx.x == 0) past_start(sh, p.ctr);
   } else if (warp == kSchedWarp) {
