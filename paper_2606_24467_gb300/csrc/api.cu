@@ -887,17 +887,27 @@ int run_select(const ckv_problem* p, const Info& I, const float* raw, const floa
     P.cu_out[s] = cu_out[s];
     if (s < I.B) max_n = std::max(max_n, I.n[s]);
   }
-  if (!I.layer && max_n <= 32 * 1024 && (pooled_in || max_n > 8192)) {
+  const int units = I.B * I.Hkv;
+  // From raw scores the sampled select pools first, and gains where select_kernel
+  // has few or many units of long prefixes; us of compresskv_select by
+  // select_kernel / by the sampled one, pooling width 7:
+  //   prefix      4 units    8 units    16 units   48 units   80 units   256
+  //    8193       13/13      13/13      13/14      15/18      22/21      42/39
+  //   12000       15/14      15/14      15/15      18/20      28/25      55/48
+  //   16384       15/14      15/14      15/16      22/21      36/30      69/58
+  //   20000       14/15      14/15      15/18      24/24      46/41      95/85
+  //   32768       15/15      15/18      19/22      34/31      66/56
+  // (width 31 at 80 and more units: 0.96 to 1.0 below 12000, then 1.01 to 1.1)
+  const bool from_raw =
+      units <= 4 ? max_n > 8192 && max_n <= 16384 : units >= 80 && max_n >= 12000;
+  if (!I.layer && max_n <= 32 * 1024 && (pooled_in || from_raw)) {
     // per-group selection: sampled select, one cluster of
     // C CTAs per unit (longer prefixes list too many keys above the sampled
-    // bound).  From raw scores for long units only (score, select and gather
-    // of four units of 16001 tokens 33.9 -> 31.4 us, of 18984 68 -> 64 with
-    // the host's part; 32 units of up to 892 33.9 -> 35.7).  C gives about kScTargetCtas CTAs per launch -- few, busy CTAs
+    // bound).  C gives about kScTargetCtas CTAs per launch -- few, busy CTAs
     // leave the SMs to the other calls' kernels (measured on the 32-layer
     // bench: 8 units per launch best with C = 8 of 4/8/16, 32 units with
     // C = 2-4 of 2-16) -- but at least slices of kScMaxSlice positions and
     // at most the device's cluster limit.
-    const int units = I.B * I.Hkv;
     const int c_min = (max_n + kScMaxSlice - 1) / kScMaxSlice;
     const int C = std::max(std::max(1, c_min),
                            std::min(F->sampled_cluster, (kScTargetCtas + units - 1) / units));

@@ -1,9 +1,10 @@
 """compresskv_select on given raw scores: pooled scores and indices bit by bit
 against fp32 arithmetic in the kernel's order (the taps from the left, then one
 division) and an exact top-k, on both sides of the lengths between which one
-cluster of CTAs per unit pools and selects (8192 < n <= 32768), where a CTA's
-bound keeps too few or too many candidates and the search reads what the other
-CTAs of the cluster pooled (needs a GB300)."""
+cluster of CTAs per unit pools and selects (up to 4 units: 8192 < n <= 16384; 80
+and more: 12000 <= n <= 32768), where a CTA's bound keeps too few or too many
+candidates and the search reads what the other CTAs of the cluster pooled (needs
+a GB300)."""
 import math
 
 import numpy as np
@@ -74,30 +75,40 @@ def _select(lens, n_kv, P, kind, budgets, dev, pooled_out=True, seed=0):
             assert np.array_equal(got[g, out0[s]:out0[s + 1]], sel), (s, g)
 
 
-@pytest.mark.parametrize("n", [8192, 8193, 16001, 32768, 32769])
+@pytest.mark.parametrize("n", [8192, 8193, 16001, 16384, 16385])
 @pytest.mark.parametrize("P,pooled_out", [(1, True), (7, False), (63, True), (63, False)])
 def test_lengths_and_widths(cuda_device, n, P, pooled_out):
-    _select([n + W, 0, W, W + 1, 700, n // 2 + W], 2, P, "decades", [512, 40, 40, 40, 300, W],
+    for rest in ([700], [0], [W], [W + 1], [n // 2 + W]):
+        _select([n + W, *rest], 2, P, "decades", [512, 300], cuda_device, pooled_out)
+    _select([n + W], 1, P, "decades", [W], cuda_device, pooled_out)
+
+
+@pytest.mark.parametrize("n", [11999, 12000, 32768, 32769])
+@pytest.mark.parametrize("P,pooled_out", [(7, True), (63, False)])
+def test_many_units(cuda_device, n, P, pooled_out):
+    """Clusters of one CTA and of two (slices of 16384 keys and their raw scores
+    in shared memory), with short and empty sequences among them."""
+    _select([n + W, 0, W + 1, 700, n // 2 + W], 16, P, "decades", [600, 40, 40, 300, 900],
             cuda_device, pooled_out)
 
 
 @pytest.mark.parametrize("kind", ["levels", "equal", "few"])
 @pytest.mark.parametrize("budget", [W + 1, 128, 4096 + W, 9000, 11999])
 def test_bounds_that_keep_too_few_or_too_many(cuda_device, kind, budget):
-    _select([12000, 10000], 3, 7, kind, [budget, min(budget, 9999)], cuda_device, budget != 128)
+    _select([12000, 10000], 2, 7, kind, [budget, min(budget, 9999)], cuda_device, budget != 128)
 
 
 def test_second_sampled_bound(cuda_device):
     """Strong scores at eleven of the positions that the first CTA of a cluster
-    samples (8 units of 9968 keys: ten CTAs, slices of 1024 keys, 25 evenly
+    samples (4 units of 9968 keys: 16 CTAs, slices of 640 keys, 16 evenly
     spaced samples each): the first bound is one of them, fewer than k = 96 keys
     reach it, and a second, looser one is taken."""
-    n, n_kv, C, S = 10000 - W, 8, 10, 1024
-    at = [(t * S) // 25 for t in range(1, 12)]
+    n, n_kv, C, S = 10000 - W, 4, 16, 640
+    at = [(t * S) // 16 for t in range(1, 12)]
     samples = []
     for c in range(C):
         lo, hi = min(n, c * S), min(n, (c + 1) * S)
-        samples += [lo + (t * (hi - lo)) // 25 for t in range(25)]
+        samples += [lo + (t * (hi - lo)) // 16 for t in range(16)]
     mu = 96 * len(samples) / n
     rank = min(len(samples), math.ceil(mu + 3 * math.sqrt(mu)) + 2)
 
@@ -108,10 +119,3 @@ def test_second_sampled_bound(cuda_device):
         return x
 
     _select([n + W], n_kv, 1, planted, [96 + W], cuda_device)
-
-
-@pytest.mark.parametrize("n", [12000, 32768])
-def test_many_units(cuda_device, n):
-    """Clusters of two CTAs (slices of 16384 keys and their raw scores in shared
-    memory) and of one."""
-    _select([n + W, n + W - 5], 48, 7, "decades", [600, 900], cuda_device)
