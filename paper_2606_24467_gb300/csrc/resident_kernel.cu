@@ -74,12 +74,12 @@
 // query rows (pass 2) 3 shuffles a tile, where one lane per key takes 31
 // shuffles per block for the first.
 // What bounds it: a short call the chain of its steps (one 777-token layer,
-// 24 us against 67 in the two-pass kernel before it: start 4, scores 9,
-// selection 8), a full one the time that tensor memory is held: a chunk's
-// logits wait for the sums of the unit's slowest chunk, and the memory holds
-// few chunks (32 layers of 32768 tokens: 619 us, 3.5 TB/s of the K that is
-// read once; 32 layers of 8 prompts of 300 to 4000 tokens: 0.48 ms against
-// 3.5).
+// 29 us a call against 73 in the two-pass kernel before it: start 4, scores 9,
+// selection 8, the rest the host's), a full one the time that tensor memory is
+// held: a chunk's logits wait for the sums of the unit's slowest chunk, and the
+// memory holds few chunks (32 layers of 32768 tokens: 622 us, 3.5 TB/s of the K
+// that is read once; 32 layers of 8 prompts of 300 to 4000 tokens: 0.48 ms
+// against 3.5).
 // Every wait is bounded (ResidentParams::wait_ns, kWaitTimeoutNs unless a test
 // shortens it) and on expiry records CKV_ERR_DEVICE_TIMEOUT and stops the
 // call.  A wait depends only on chunks of the same or earlier units, which
@@ -1211,23 +1211,27 @@ __device__ __noinline__ void denominator_role(ResidentShared& sh, int mine, int 
 // get neighbouring numbers, as in a launch on an idle GPU (chunks of a unit on
 // SMs far apart, as CTAs that start one by one behind another kernel have them,
 // cost 5 to 20%).  A slot taken already (an SM's number may change) goes on to
-// the next free one.
+// the next free one; -1 (the CTA leaves) when none is, in a workspace that was
+// not initialised.
 __device__ __noinline__ int number_by_sm(int* ctr) {
   uint32_t sm;
   asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
   const uint32_t all = gridDim.x;
   sm %= all;
 #pragma unroll 1
-  for (;; sm = sm + 1 == all ? 0 : sm + 1) {
+  for (uint32_t left = all; left; --left) {
     const uint32_t bit = 1u << (sm & 31u);
     if (!(atomicOr(reinterpret_cast<unsigned*>(ctr + kCtrSlots) + (sm >> 5), bit) & bit))
       return static_cast<int>(sm);
+    if (++sm == all) sm = 0;
   }
+  return -1;
 }
 
 // Whether this CTA takes part in the call (one thread, first thing): all do once
 // all have started; when not all have kStartWaitNs after one has, the call is
-// closed to the others, which leave.
+// closed to the others, which leave.  Whatever the words held before, a CTA ends
+// with a number below a grid of at most gridDim.x, or leaves.
 __device__ __forceinline__ void take_part(ResidentShared& sh, int* ctr) {
   const unsigned all = gridDim.x;
   unsigned* const word = reinterpret_cast<unsigned*>(ctr + kCtrArrive);
@@ -1253,6 +1257,7 @@ __device__ __forceinline__ void take_part(ResidentShared& sh, int* ctr) {
       atomicCAS(word, w, w | kApart);
     }
   }
+  if (id >= grid || grid > static_cast<int>(all)) id = -1;
   sh.call.id = id;
   sh.call.grid = grid;
 }

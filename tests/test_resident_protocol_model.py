@@ -405,11 +405,17 @@ def test_a_mistake_is_caught(kw):
 CLOSED, APART = 1 << 31, 1 << 30
 
 
-def _start(seed, n, held):
+def _start(seed, n, held, stale=False):
     """n CTAs of which the last `held` start only when an earlier one has left;
-    every atomic operation is one step.  Returns what each became."""
+    every atomic operation is one step.  Returns what each became.  stale: the
+    words hold anything at first."""
     rng = random.Random(seed)
     word = {"arrive": 0, "past": 0, "zeroed": 0, "slots": 0}
+    if stale:
+        word = {"arrive": rng.choice((rng.getrandbits(32), rng.randrange(2 * n),
+                                      CLOSED | rng.getrandbits(18))),
+                "past": rng.getrandbits(32), "zeroed": rng.getrandbits(32),
+                "slots": rng.choice((rng.getrandbits(n), (1 << n) - 1))}
     sms = list(range(n))
     rng.shuffle(sms)
     out = {}
@@ -418,8 +424,8 @@ def _start(seed, n, held):
 
     def cta(block):
         old = word["arrive"]
-        word["arrive"] += 1
-        me, grid, w, polls = block, n, old + 1, 0
+        word["arrive"] = (old + 1) % 2**32
+        me, grid, w, polls = block, n, (old + 1) % 2**32, 0
         yield
         while w != n:
             if w & CLOSED:
@@ -429,7 +435,8 @@ def _start(seed, n, held):
             count = w & 0xFFFF
             if count == n:
                 slot = sms[block] if rng.random() < 0.9 else rng.randrange(n)  # may have changed
-                while True:
+                me = None
+                for _ in range(n):
                     yield
                     if not word["slots"] >> slot & 1:
                         word["slots"] |= 1 << slot
@@ -447,11 +454,15 @@ def _start(seed, n, held):
             yield
             w = word["arrive"]
             yield
+        if me is not None and (me >= grid or grid > n):
+            me = None
         out[block] = (me, grid)
         if me is not None:
             word["zeroed"] += 1
             yield
-            while word["zeroed"] < grid:
+            polls = 0
+            while word["zeroed"] < grid and not (stale and polls > 300):  # the wait runs out
+                polls += 1
                 yield
         word["past"] += 1
         if word["past"] == n:
@@ -470,7 +481,7 @@ def _start(seed, n, held):
             if waiting:  # its SM is free
                 running.append(waiting.pop(0))
     assert not running and not waiting, "the start does not end"
-    assert not any(word.values()), "the words are not ready for the next call"
+    assert stale or not any(word.values()), "the words are not ready for the next call"
     return out
 
 
@@ -483,3 +494,12 @@ def test_the_ctas_agree_on_who_takes_part(n, held):
         assert parts == list(range(len(parts))) and parts
         assert {grid for _, grid in out.values()} == {len(parts)}
         assert len(parts) <= n - held or not held
+
+
+@pytest.mark.parametrize("n", [1, 2, 7, 40, 152])
+def test_a_start_on_stale_words_ends_within_bounds(n):
+    """A workspace that was never initialised: no number beyond the grid (the
+    CTAs index their scratch by it), and no CTA that stays."""
+    for seed in range(100):
+        for me, grid in _start(seed, n, 0, stale=True).values():
+            assert me is None or 0 <= me < grid <= n
